@@ -206,8 +206,10 @@ def run(state):
             out[f] = L["sum_" + f].astype(real)
         out["conserved"] = np.concatenate([G["mass"][:, None], G["momentum"]], axis=1).astype(real)
         if c["hist"]:
+            # every block level below the whole system, whose order parameter is
+            # zero by conservation (its bin would record rounding alone)
             out["hist"] = np.concatenate([ens.histogram(k, l)[0] for k in range(len(ens.systems))
-                                          for l in range(first[k + 1] - first[k])]).astype(np.int64)
+                                          for l in range(1, first[k + 1] - first[k])]).astype(np.int64)
     if c["sk"]:
         sk = [ens.structure_factor(k, nbins_of(s)) for k, s in enumerate(ens.systems)]
         out["sk"] = np.concatenate([v[0] for v in sk]).astype(real)
