@@ -24,6 +24,9 @@ using namespace lbf;
 namespace {
 
 constexpr size_t kAlign = 256;
+// Ensembles of fewer sites than this get site and block items of one element
+// per thread: 1,024-site items would leave SMs idle (2^20 sites = 1,024 items).
+constexpr int64_t kSpreadSites = int64_t(1) << 20;
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
 struct LevelHost {
@@ -43,8 +46,8 @@ struct SysHost {
 
 // Byte offsets of every region inside the workspace.
 struct Plan {
-    size_t sys, phys, tiles, pop0, pop1, step, status, d, dbar, site_items, site_partial, spans, red4, glob, levels,
-        S, E, bottom_items, up_items, rec, acc, hist, field_tmp, sk_sys, sk_tw, sk_acc, sk_b0, sk_b1, sk_bins, jk_j,
+    size_t sys, phys, tiles, pop0, pop1, step, status, d, dbar, site_items, site_partial, spans, glob, levels,
+        S, E, bottom_items, part_items, block_items, parts, up_items, tops, rec, acc, hist, field_tmp, sk_sys, sk_tw, sk_acc, sk_b0, sk_b1, sk_bins, jk_j,
         jk_lap, jk_F, jk_acc, total;
     bool jk = false;
     int hist_bins = 0;
@@ -55,6 +58,10 @@ struct Plan {
     std::vector<SysSpan> spans_h;
     std::vector<LevelDev> levels_h;
     std::vector<ObsItem> bottom_h, up_h;
+    std::vector<ObsPart> part_h;
+    std::vector<ObsBlocks> block_h;
+    std::vector<ObsTop> top_h;
+    int n_parts = 0;
     std::vector<int> up_first;   // up items of depth u: [up_first[u-1], up_first[u])
     // structure factor
     bool sk = false;
@@ -268,7 +275,9 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
     P.n_tiles = int(P.tiles_h.size());
 
     // site chunks
-    const int chunk = AUX_THREADS * SITES_PER_THREAD;
+    // (small ensembles: one site per thread, so that their few items spread over the GPU)
+    const bool spread = site_off < kSpreadSites;
+    const int chunk = AUX_THREADS * (spread ? 1 : SITES_PER_THREAD);
     for (int k = 0; k < n; ++k) {
         SysSpan sp{int(P.site_items_h.size()), 0};
         for (int64_t b = 0; b < sys[k].n; b += chunk)
@@ -279,7 +288,7 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
     P.n_site_items = int(P.site_items_h.size());
 
     // observable levels, items and records
-    const int bchunk = OBS_THREADS * BLOCKS_PER_THREAD;
+    const int bchunk = OBS_THREADS * (spread ? 1 : BLOCKS_PER_THREAD);
     int64_t blk_off = 0;
     P.levels_h.resize(lv_count);
     for (int k = 0; k < n; ++k) {
@@ -304,57 +313,72 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
     }
     P.n_blocks_pyr = blk_off;
     int rec = 0;
-    // bottom items (records of the bottom level, then of the unit level)
+    // records of a level are numbered in the order they are asked for
+    auto new_rec = [&](LevelDev& D) {
+        if (D.rec_count++ == 0) D.rec_first = rec;
+        return rec++;
+    };
+    // bottom items: one thread per block where the blocks are small, else a
+    // warp per block or a CTA per range of its sites (the record of the bottom
+    // level, then of the single-site level)
     for (int k = 0; k < n; ++k) {
         SysHost& h = sys[k];
-        LevelDev& B = P.levels_h[h.lv_first + h.imax];
-        const int first = int(P.bottom_h.size());
-        for (int64_t b = 0; b < B.nblocks; b += bchunk) {
-            ObsItem it;
-            it.level = h.lv_first + h.imax;
-            it.unit_level = h.unit_sep ? h.lv_first + h.imax + 1 : -1;
-            it.b0 = b;
-            it.b1 = std::min<int64_t>(b + bchunk, B.nblocks);
-            it.rec = -1;
-            it.rec2 = -1;
-            P.bottom_h.push_back(it);
+        const int lb = h.lv_first + h.imax, lu = h.unit_sep ? lb + 1 : -1;
+        LevelDev& B = P.levels_h[lb];
+        const int64_t bvol = int64_t(B.bx) * B.by * B.bz;
+        int items = 0;
+        const int part_first = int(P.part_h.size()), bottom_first = int(P.bottom_h.size());
+        if (bvol <= kThreadSites) {
+            for (int64_t b = 0; b < B.nblocks; b += bchunk, ++items)
+                P.bottom_h.push_back(ObsItem{lb, lu, b, std::min<int64_t>(b + bchunk, B.nblocks), new_rec(B), -1});
+        } else if (bvol <= kWarpSites && B.nblocks > 1) {
+            constexpr int64_t wchunk = 4 * (OBS_THREADS / 32);
+            for (int64_t b = 0; b < B.nblocks; b += wchunk, ++items) {
+                const int64_t e = std::min<int64_t>(b + wchunk, B.nblocks);
+                P.part_h.push_back(ObsPart{lb, lu, int(b), int(e), 0, int(bvol), -1, new_rec(B), -1});
+            }
+        } else {
+            const int per = int((bvol + kPartSites - 1) / kPartSites), part0 = P.n_parts;
+            for (int64_t b = 0; b < B.nblocks; ++b)
+                for (int r = 0; r < per; ++r, ++items) {
+                    const int64_t i0 = bvol * r / per, i1 = bvol * (r + 1) / per;
+                    P.part_h.push_back(ObsPart{lb, lu, int(b), int(b) + 1, int(i0), int(i1), per > 1 ? P.n_parts++ : -1,
+                                               per > 1 ? -1 : new_rec(B), -1});
+                }
+            if (per > 1)
+                for (int64_t b = 0; b < B.nblocks; b += OBS_THREADS / 32) {
+                    const int e = int(std::min<int64_t>(b + OBS_THREADS / 32, B.nblocks));
+                    P.block_h.push_back(ObsBlocks{lb, int(b), e, part0, per, new_rec(B)});
+                }
         }
-        const int cnt = int(P.bottom_h.size()) - first;
-        B.rec_first = rec;
-        B.rec_count = cnt;
-        for (int j = 0; j < cnt; ++j) P.bottom_h[first + j].rec = rec + j;
-        rec += cnt;
         if (h.unit_sep) {
-            LevelDev& U = P.levels_h[h.lv_first + h.imax + 1];
-            U.rec_first = rec;
-            U.rec_count = cnt;
-            for (int j = 0; j < cnt; ++j) P.bottom_h[first + j].rec2 = rec + j;
-            rec += cnt;
+            LevelDev& U = P.levels_h[lu];
+            for (int j = 0; j < items; ++j) {
+                const int r = new_rec(U);
+                if (bvol <= kThreadSites) P.bottom_h[bottom_first + j].rec2 = r;
+                else P.part_h[part_first + j].rec2 = r;
+            }
         }
     }
-    // up items grouped by depth u = 1..max_depth (level imax - u of each system)
+    // up items grouped by depth u = 1..max_depth (level imax - u of each
+    // system) down to levels of kTopBlocks blocks; the rest go to the top kernel
     int max_depth = 0;
-    for (auto& h : sys) max_depth = std::max(max_depth, h.imax);
+    for (auto& h : sys) {
+        int top = h.imax;
+        while (top > 0 && h.lv[top - 1].nblocks > kTopBlocks) --top;
+        P.top_h.push_back(ObsTop{h.lv_first, int(h.lv.size()), top});
+        max_depth = std::max(max_depth, h.imax - top);
+    }
     P.max_depth = max_depth;
     P.up_first.push_back(0);
     for (int u = 1; u <= max_depth; ++u) {
         for (int k = 0; k < n; ++k) {
-            SysHost& h = sys[k];
-            const int l = h.imax - u;
-            if (l < 0) continue;
-            LevelDev& D = P.levels_h[h.lv_first + l];
-            D.rec_first = rec;
-            for (int64_t b = 0; b < D.nblocks; b += bchunk) {
-                ObsItem it;
-                it.level = h.lv_first + l;
-                it.unit_level = -1;
-                it.b0 = b;
-                it.b1 = std::min<int64_t>(b + bchunk, D.nblocks);
-                it.rec = rec++;
-                it.rec2 = -1;
-                P.up_h.push_back(it);
-            }
-            D.rec_count = rec - D.rec_first;
+            const int l = sys[k].imax - u;
+            if (l < P.top_h[k].top) continue;
+            LevelDev& D = P.levels_h[sys[k].lv_first + l];
+            for (int64_t b = 0; b < D.nblocks; b += bchunk)
+                P.up_h.push_back(ObsItem{sys[k].lv_first + l, -1, b, std::min<int64_t>(b + bchunk, D.nblocks),
+                                         new_rec(D), -1});
         }
         P.up_first.push_back(int(P.up_h.size()));
     }
@@ -425,13 +449,16 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
     P.site_items = take(sizeof(int4) * P.n_site_items);
     P.site_partial = take(sizeof(double) * 4 * P.n_site_items);
     P.spans = take(sizeof(SysSpan) * n);
-    P.red4 = take(sizeof(double) * 4 * n);
     P.glob = take(sizeof(double) * 8 * n);
     P.levels = take(sizeof(LevelDev) * P.n_levels);
     P.S = take(sizeof(double) * P.n_blocks_pyr);
     P.E = take(sizeof(double) * P.n_blocks_pyr);
     P.bottom_items = take(sizeof(ObsItem) * P.n_bottom);
+    P.part_items = take(sizeof(ObsPart) * P.part_h.size());
+    P.block_items = take(sizeof(ObsBlocks) * P.block_h.size());
+    P.parts = take(sizeof(double2) * P.n_parts);
     P.up_items = take(sizeof(ObsItem) * P.n_up);
+    P.tops = take(sizeof(ObsTop) * n);
     P.rec = take(sizeof(double) * REC * P.n_rec);
     P.acc = take(sizeof(double) * 7 * P.n_levels);
     P.hist_bins = o->hist_bins;
@@ -579,32 +606,38 @@ cudaError_t sample_obs(lb_ctx* c, int buf, bool set_mass0, bool count, bool want
             : launch_obs_site_d3q19(c->fp32, sys, c->at<int4>(P.site_items), P.n_site_items, c->pop(buf),
                                     c->at<double>(P.d), c->at<double>(P.site_partial), jout, P.n_sites, c->stream);
     if (e != cudaSuccess) return e;
-    e = launch_reduce_sys(c->at<SysSpan>(P.spans), c->n_sys, c->at<double>(P.site_partial), 4, c->at<double>(P.red4),
-                          c->stream);
-    if (e != cudaSuccess) return e;
-    e = launch_obs_globals(sys, c->n_sys, c->at<double>(P.red4), c->at<double>(P.dbar), c->at<double>(P.glob),
-                           set_mass0 ? 1 : 0, count ? 1 : 0, c->stream);
-    c->launches += 3;
+    e = launch_reduce_globals(sys, c->at<SysSpan>(P.spans), c->n_sys, c->at<double>(P.site_partial),
+                              c->at<double>(P.dbar), c->at<double>(P.glob), set_mass0 ? 1 : 0, count ? 1 : 0,
+                              c->stream);
+    c->launches += 2;
     if (e != cudaSuccess || !count) return e;
-    c->launches += 2 + P.max_depth;
     HistDev H;
     H.counts = c->at<unsigned long long>(P.hist);
     H.nbins = P.hist_bins;
     H.lo = -P.hist_range;
     H.inv_w = P.hist_bins > 0 ? double(P.hist_bins) / (P.hist_range - (-P.hist_range)) : 0.0;
-    e = launch_pyr_bottom(sys, c->at<LevelDev>(P.levels), c->at<ObsItem>(P.bottom_items), P.n_bottom,
-                          c->at<double>(P.d), c->at<double>(P.dbar), c->at<double>(P.S), c->at<double>(P.E),
-                          c->at<double>(P.rec), H, c->stream);
+    const LevelDev* lv = c->at<LevelDev>(P.levels);
+    double* S = c->at<double>(P.S);
+    double* E = c->at<double>(P.E);
+    double* rec = c->at<double>(P.rec);
+    const int dims3 = c->lattice == LB_D3Q19 ? 1 : 0;
+    e = launch_pyr_bottom(sys, lv, c->at<ObsItem>(P.bottom_items), P.n_bottom, c->at<double>(P.d),
+                          c->at<double>(P.dbar), S, E, rec, H, c->stream);
+    if (e != cudaSuccess) return e;
+    e = launch_pyr_part(sys, lv, c->at<ObsPart>(P.part_items), int(P.part_h.size()), c->at<double>(P.d),
+                        c->at<double>(P.dbar), S, E, c->at<double2>(P.parts), rec, H, c->stream);
+    if (e != cudaSuccess) return e;
+    e = launch_pyr_blocks(lv, c->at<ObsBlocks>(P.block_items), int(P.block_h.size()), c->at<double2>(P.parts), S, E,
+                          rec, H, c->stream);
     if (e != cudaSuccess) return e;
     for (int u = 1; u <= P.max_depth; ++u) {
         const int first = P.up_first[u - 1], cnt = P.up_first[u] - first;
-        e = launch_pyr_up(sys, c->at<LevelDev>(P.levels), c->at<ObsItem>(P.up_items) + first, cnt,
-                          c->lattice == LB_D3Q19 ? 1 : 0, c->at<double>(P.S), c->at<double>(P.E),
-                          c->at<double>(P.rec), H, c->stream);
+        e = launch_pyr_up(lv, c->at<ObsItem>(P.up_items) + first, cnt, dims3, S, E, rec, H, c->stream);
         if (e != cudaSuccess) return e;
     }
-    return launch_obs_accum(c->at<LevelDev>(P.levels), P.n_levels, c->at<double>(P.rec), c->at<double>(P.acc),
-                            c->at<int>(P.status), c->stream);
+    c->launches += (P.n_bottom > 0) + !P.part_h.empty() + !P.block_h.empty() + P.max_depth + 1;
+    return launch_pyr_top(lv, c->at<ObsTop>(P.tops), c->n_sys, dims3, S, E, rec, c->at<double>(P.acc),
+                          c->at<int>(P.status), H, c->stream);
 }
 
 // Momentum spectra of the momentum field the site pass just wrote: Guo
@@ -902,6 +935,14 @@ lb_status lb_create(const lb_system_desc* systems, int n_systems, const lb_run_o
     if (P.n_bottom)
         ok = ok && cudaMemcpyAsync(c->ws + P.bottom_items, P.bottom_h.data(), sizeof(ObsItem) * P.n_bottom,
                                    cudaMemcpyHostToDevice, c->stream) == cudaSuccess;
+    if (!P.part_h.empty())
+        ok = ok && cudaMemcpyAsync(c->ws + P.part_items, P.part_h.data(), sizeof(ObsPart) * P.part_h.size(),
+                                   cudaMemcpyHostToDevice, c->stream) == cudaSuccess;
+    if (!P.block_h.empty())
+        ok = ok && cudaMemcpyAsync(c->ws + P.block_items, P.block_h.data(), sizeof(ObsBlocks) * P.block_h.size(),
+                                   cudaMemcpyHostToDevice, c->stream) == cudaSuccess;
+    ok = ok && cudaMemcpyAsync(c->ws + P.tops, P.top_h.data(), sizeof(ObsTop) * P.top_h.size(),
+                               cudaMemcpyHostToDevice, c->stream) == cudaSuccess;
     if (P.n_up)
         ok = ok && cudaMemcpyAsync(c->ws + P.up_items, P.up_h.data(), sizeof(ObsItem) * P.n_up,
                                    cudaMemcpyHostToDevice, c->stream) == cudaSuccess;
@@ -982,11 +1023,9 @@ lb_status lb_init(lb_ctx* c, int mode, double amplitude, const double* h_rho) {
     if (mode == LB_INIT_UNIFORM_NOISE) {
         LB_CHECK(launch_init_noise(sys, c->at<int4>(P.site_items), P.n_site_items, amplitude, c->at<double>(P.d),
                                    c->at<double>(P.site_partial), c->stream));
-        LB_CHECK(launch_reduce_sys(c->at<SysSpan>(P.spans), c->n_sys, c->at<double>(P.site_partial), 4,
-                                   c->at<double>(P.red4), c->stream));
         // dbar = sum d / n via the globals kernel (its mass fields are overwritten below)
-        LB_CHECK(launch_obs_globals(sys, c->n_sys, c->at<double>(P.red4), c->at<double>(P.dbar),
-                                    c->at<double>(P.glob), 1, 0, c->stream));
+        LB_CHECK(launch_reduce_globals(sys, c->at<SysSpan>(P.spans), c->n_sys, c->at<double>(P.site_partial),
+                                       c->at<double>(P.dbar), c->at<double>(P.glob), 1, 0, c->stream));
     } else {
         LB_CHECK(cudaMemcpyAsync(c->at<double>(P.d), h_rho, sizeof(double) * P.n_sites,
                                  mode == LB_INIT_FROM_DEVICE_RHO ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,

@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(AUX_THREADS)
     obs_site_kernel(const SysDev* __restrict__ sysv, const int4* __restrict__ items, const Real* __restrict__ fbuf,
                     double* __restrict__ d, double* __restrict__ partial, double* __restrict__ jout,
                     int64_t jstride) {
-    __shared__ double sh[4 * AUX_THREADS];
+    __shared__ double sh[4 * AUX_THREADS / 32];
     const int4 it = items[blockIdx.x];
     const SysDev& S = sysv[it.x];
     const int nx = S.nx, ny = S.ny, nz = S.nz;

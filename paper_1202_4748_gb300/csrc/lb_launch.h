@@ -80,6 +80,22 @@ struct ObsItem {            // a range of blocks of one level
     int32_t rec, rec2;      // partial records written (rec2 for the unit level)
 };
 
+struct ObsPart {            // bottom blocks [b0, b1) of one level, sites [i0, i1) of each
+    int32_t level, unit_level;
+    int32_t b0, b1;         // more than one block: whole blocks, one warp each
+    int32_t i0, i1;         // range of the block's sites in (x, y, z) order
+    int32_t part;           // >= 0: the block has several ranges, this range's sums go there
+    int32_t rec, rec2;      // records of the level (part < 0) and of the single-site level
+};
+
+struct ObsBlocks {          // bottom blocks [b0, b1) made of per_block parts each
+    int32_t level, b0, b1, part0, per_block, rec;
+};
+
+struct ObsTop {             // levels of one system: top - 1 .. 0 by the top kernel, the others have records
+    int32_t lv_first, n_levels, top;
+};
+
 // Order-parameter histograms: per level (nbins + 2) counts [under, bins, over]
 // at counts + level * (nbins + 2); nbins = 0 disables them.
 struct HistDev {
@@ -95,22 +111,33 @@ cudaError_t launch_selftest_wait(int* status, cudaStream_t st);
 
 cudaError_t launch_init_noise(const SysDev* sys, const int4* items, int n_items, double amp, double* d,
                               double* partial, cudaStream_t st);
-cudaError_t launch_reduce_sys(const SysSpan* spans, int n_sys, const double* partial, int K, double* out,
-                              cudaStream_t st);
-cudaError_t launch_obs_globals(const SysDev* sys, int n_sys, const double* red4, double* dbar, double* glob,
-                               int set_mass0, int count_sample, cudaStream_t st);
+cudaError_t launch_reduce_globals(const SysDev* sys, const SysSpan* spans, int n_sys, const double* partial,
+                                  double* dbar, double* glob, int set_mass0, int count_sample, cudaStream_t st);
 cudaError_t launch_set_dbar(const SysDev* sys, int n_sys, double* dbar, cudaStream_t st);
 cudaError_t launch_pyr_bottom(const SysDev* sys, const LevelDev* lv, const ObsItem* items, int n_items,
                               const double* d, const double* dbar, double* S, double* E, double* rec,
                               const HistDev& hist, cudaStream_t st);
-cudaError_t launch_pyr_up(const SysDev* sys, const LevelDev* lv, const ObsItem* items, int n_items, int dims3,
+cudaError_t launch_pyr_part(const SysDev* sys, const LevelDev* lv, const ObsPart* items, int n_items,
+                            const double* d, const double* dbar, double* S, double* E, double2* parts, double* rec,
+                            const HistDev& hist, cudaStream_t st);
+cudaError_t launch_pyr_blocks(const LevelDev* lv, const ObsBlocks* items, int n_items, const double2* parts,
+                              double* S, double* E, double* rec, const HistDev& hist, cudaStream_t st);
+cudaError_t launch_pyr_up(const LevelDev* lv, const ObsItem* items, int n_items, int dims3,
                           double* S, double* E, double* rec, const HistDev& hist, cudaStream_t st);
-cudaError_t launch_obs_accum(const LevelDev* lv, int n_levels_total, const double* rec, double* acc,
-                             int* status, cudaStream_t st);
+cudaError_t launch_pyr_top(const LevelDev* lv, const ObsTop* tops, int n_sys, int dims3, double* S, double* E,
+                           const double* rec, double* acc, int* status, const HistDev& hist, cudaStream_t st);
+cudaError_t launch_obs_accum(const LevelDev* lv, int n_levels, const double* rec, double* acc, int* status,
+                             cudaStream_t st);
 cudaError_t launch_advance(int64_t* step, int64_t n, cudaStream_t st);
 
 constexpr int OBS_THREADS = 256;
 constexpr int BLOCKS_PER_THREAD = 4;
+constexpr int TOP_THREADS = 512;        // pyr_top_kernel: one CTA per system
+// Bottom blocks of more than kThreadSites sites take a warp or a CTA instead of
+// a thread (a thread's sites are a serial chain of row loads), those of more
+// than kWarpSites a CTA, in ranges of kPartSites sites (16 per thread).
+constexpr int kThreadSites = 32, kWarpSites = 1024, kPartSites = 4096;
+constexpr int kTopBlocks = 4096;        // levels of at most this many blocks go to the top kernel (8 per thread)
 constexpr int REC = 6;      // per record: sum m, m^2, |m|, m^4, e, e^2
 
 }  // namespace lbf

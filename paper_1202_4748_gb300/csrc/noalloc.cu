@@ -131,7 +131,7 @@ __host__ __device__ inline bool na_plan(int nx, int ny, int nz, bool dims3, NaPl
 }
 
 struct NaLayout {                  // byte offsets of the scratch regions
-    size_t sys, lv, bot, up, items, span, part, red, dbar, glob, stat, S, E, rec, acc, end;
+    size_t sys, lv, bot, up, items, span, part, dbar, glob, stat, S, E, rec, acc, end;
 };
 
 NaLayout na_layout(const NaPlan& P) {
@@ -149,7 +149,6 @@ NaLayout na_layout(const NaPlan& P) {
     o.items = take(sizeof(int4) * P.n_items);
     o.span = take(sizeof(SysSpan));
     o.part = take(sizeof(double) * 4 * P.n_items);
-    o.red = take(sizeof(double) * 4);
     o.dbar = take(sizeof(double));
     o.glob = take(sizeof(double) * 8);
     o.stat = take(sizeof(int));
@@ -292,7 +291,6 @@ extern "C" lb_status lb_block_moments_noalloc(const double* d_rho, int nx, int n
     const SysDev* dsys = reinterpret_cast<const SysDev*>(base + o.sys);
     const LevelDev* dlv = reinterpret_cast<const LevelDev*>(base + o.lv);
     double* part = reinterpret_cast<double*>(base + o.part);
-    double* red4 = reinterpret_cast<double*>(base + o.red);
     double* dbar = reinterpret_cast<double*>(base + o.dbar);
     double* S = reinterpret_cast<double*>(base + o.S);
     double* E = reinterpret_cast<double*>(base + o.E);
@@ -303,14 +301,14 @@ extern "C" lb_status lb_block_moments_noalloc(const double* d_rho, int nx, int n
     rho_partial_kernel<<<P.n_items, AUX_THREADS, 0, st>>>(reinterpret_cast<const int4*>(base + o.items), d_rho,
                                                            part);
     NA_CHECK(cudaGetLastError());
-    NA_CHECK(launch_reduce_sys(reinterpret_cast<const SysSpan*>(base + o.span), 1, part, 4, red4, st));
-    NA_CHECK(launch_obs_globals(dsys, 1, red4, dbar, reinterpret_cast<double*>(base + o.glob), 1, 0, st));
+    NA_CHECK(launch_reduce_globals(dsys, reinterpret_cast<const SysSpan*>(base + o.span), 1, part, dbar,
+                                   reinterpret_cast<double*>(base + o.glob), 1, 0, st));
     const HistDev no_hist{nullptr, 0, 0.0, 0.0};
     NA_CHECK(launch_pyr_bottom(dsys, dlv, reinterpret_cast<const ObsItem*>(base + o.bot), P.n_bottom, d_rho, dbar, S,
                                E, recs, no_hist, st));
     for (int u = 1; u <= P.imax; ++u) {
         const int first = P.up_first[u - 1], cnt = P.up_first[u] - first;
-        NA_CHECK(launch_pyr_up(dsys, dlv, reinterpret_cast<const ObsItem*>(base + o.up) + first, cnt, dims3 ? 1 : 0,
+        NA_CHECK(launch_pyr_up(dlv, reinterpret_cast<const ObsItem*>(base + o.up) + first, cnt, dims3 ? 1 : 0,
                                S, E, recs, no_hist, st));
     }
     NA_CHECK(launch_obs_accum(dlv, P.nl, recs, acc, stat, st));

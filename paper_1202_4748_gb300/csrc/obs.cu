@@ -5,8 +5,23 @@
 // block sums of phi and phi^2 are taken from the sites, every coarser level
 // sums the 2^d children of the next finer one.  Per block the nonlinear terms
 // m, m^2, |m|, m^4, E, E^2 (m = sum phi / V, E = sum phi^2 / 2V) are formed and
-// reduced per item into a record; one thread per level then sums its records
-// in order into the FP64 accumulators.  Every sum has a fixed order.
+// reduced per item into a record; one warp per level then sums its records
+// into the FP64 accumulators.  Every sum has a fixed order.
+//
+// Who sums what (launches of one sample, each skipped when empty):
+//   pyr_bottom_kernel  bottom levels of small blocks: one thread per block
+//   pyr_part_kernel    bottom levels of larger blocks (sides whose odd factor
+//                      is not small): a warp per block, or a CTA per range of
+//                      up to kPartSites sites of a block; with one thread per
+//                      block an odd-sided system was a serial sum over all its
+//                      sites (57.6 ms a sample for 32 systems of up to 141,000
+//                      sites; 0.1 ms with this kernel)
+//   pyr_blocks_kernel  bottom levels whose blocks have several ranges
+//   pyr_up_kernel      coarser levels of more than kTopBlocks blocks
+//   pyr_top_kernel     one CTA per system: its remaining coarser levels, one
+//                      after another behind CTA barriers (a launch per level
+//                      before: these levels are microseconds of latency each),
+//                      and the sums of the records the kernels above wrote
 #include "lattice_kernels.cuh"
 #include "lb_launch.h"
 
@@ -17,7 +32,7 @@ namespace {
 __global__ void __launch_bounds__(AUX_THREADS)
     init_noise_kernel(const SysDev* __restrict__ sysv, const int4* __restrict__ items, double amp,
                       double* __restrict__ d, double* __restrict__ partial) {
-    __shared__ double sh[AUX_THREADS];
+    __shared__ double sh[AUX_THREADS / 32];
     const int4 it = items[blockIdx.x];
     const SysDev& S = sysv[it.x];
     double acc[1] = {0.0};
@@ -34,34 +49,28 @@ __global__ void __launch_bounds__(AUX_THREADS)
     if (threadIdx.x == 0) partial[int64_t(blockIdx.x) * 4] = acc[0];
 }
 
-// out[s * K + k] = sum over the items of system s of partial[item * 4 + k], in order.
+// Per system: the sums over its items of partial[item * 4 + (0..3)] in a fixed
+// order (sum d, sum jx, sum jy, sum jz), then the mean deviation and the
+// global bookkeeping.  glob layout per system (8 doubles): n_samples, mass0,
+// mass, jx, jy, jz, rho_mean, spare.
 __global__ void __launch_bounds__(AUX_THREADS)
-    reduce_sys_kernel(const SysSpan* __restrict__ spans, const double* __restrict__ partial, int K,
-                      double* __restrict__ out) {
-    __shared__ double sh[4 * AUX_THREADS];
-    const SysSpan sp = spans[blockIdx.x];
+    reduce_globals_kernel(const SysDev* __restrict__ sysv, const SysSpan* __restrict__ spans,
+                          const double* __restrict__ partial, double* __restrict__ dbar, double* __restrict__ glob,
+                          int set_mass0, int count_sample) {
+    __shared__ double sh[4 * AUX_THREADS / 32];
+    const int s = blockIdx.x;
+    const SysSpan sp = spans[s];
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
     for (int it = threadIdx.x; it < sp.count; it += AUX_THREADS) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if (k < K) acc[k] += partial[int64_t(sp.first + it) * 4 + k];
+        for (int k = 0; k < 4; ++k) acc[k] += partial[int64_t(sp.first + it) * 4 + k];
     }
     block_sum<4, AUX_THREADS>(acc, sh);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < K; ++k) out[blockIdx.x * K + k] = acc[k];
-}
-
-// glob layout per system (8 doubles): n_samples, mass0, mass, jx, jy, jz, rho_mean, spare
-__global__ void obs_globals_kernel(const SysDev* __restrict__ sysv, int n_sys, const double* __restrict__ red4,
-                                   double* __restrict__ dbar, double* __restrict__ glob, int set_mass0,
-                                   int count_sample) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n_sys) return;
+    if (threadIdx.x != 0) return;
     const SysDev& S = sysv[s];
-    const double sum_d = red4[s * 4 + 0];
     const double n = double(S.n_sites);
-    const double mass = S.rho_c * n + sum_d;
-    dbar[s] = sum_d / n;
+    const double mass = S.rho_c * n + acc[0];
+    dbar[s] = acc[0] / n;
     double* g = glob + s * 8;
     if (set_mass0) {
         g[0] = 0.0;
@@ -69,9 +78,9 @@ __global__ void obs_globals_kernel(const SysDev* __restrict__ sysv, int n_sys, c
     }
     if (count_sample) g[0] += 1.0;
     g[2] = mass;
-    g[3] = red4[s * 4 + 1];
-    g[4] = red4[s * 4 + 2];
-    g[5] = red4[s * 4 + 3];
+    g[3] = acc[1];
+    g[4] = acc[2];
+    g[5] = acc[3];
     g[6] = mass / n;
 }
 
@@ -111,6 +120,14 @@ __device__ __forceinline__ void hist_flush(const unsigned* sh, int n, unsigned l
         if (sh[k]) atomicAdd(g + k, (unsigned long long)sh[k]);
 }
 
+// Block coordinates of block b of a pyramid level: 2^k blocks per axis.
+__device__ __forceinline__ void block_coords(const LevelDev& lv, int b, int& X, int& Y, int& Z) {
+    const int kx = 31 - __clz(lv.gx), ky = 31 - __clz(lv.gy);
+    X = b & (lv.gx - 1);
+    Y = (b >> kx) & (lv.gy - 1);
+    Z = b >> (kx + ky);
+}
+
 // Bottom pyramid level: block sums of phi, phi^2 straight from the sites; the
 // separate single-site level (if any) is fed from the same loop.  With
 // histograms on, each block value m (and each site value of the single-site
@@ -120,7 +137,7 @@ __global__ void __launch_bounds__(OBS_THREADS)
                       const ObsItem* __restrict__ items, const double* __restrict__ d,
                       const double* __restrict__ dbar, double* __restrict__ Sg, double* __restrict__ Eg,
                       double* __restrict__ rec, const HistDev H) {
-    __shared__ double sh[REC * OBS_THREADS];
+    __shared__ double sh[REC * OBS_THREADS / 32];
     extern __shared__ unsigned shist[];          // [block level | single-site level], nbins + 2 each
     const ObsItem it = items[blockIdx.x];
     const LevelDev lv = lvv[it.level];
@@ -138,23 +155,28 @@ __global__ void __launch_bounds__(OBS_THREADS)
     }
     double tb[REC] = {0, 0, 0, 0, 0, 0};
     double tu[REC] = {0, 0, 0, 0, 0, 0};
-    for (int j = 0; j < BLOCKS_PER_THREAD; ++j) {
-        const int64_t b = it.b0 + int64_t(j) * OBS_THREADS + threadIdx.x;
-        if (b >= it.b1) break;
-        const int X = int(b % lv.gx), Y = int((b / lv.gx) % lv.gy), Z = int(b / (int64_t(lv.gx) * lv.gy));
+    const int nx = S.nx, ny = S.ny;
+    const bool sites = lv.bx == 1 && lv.by == 1 && lv.bz == 1;   // blocks are the sites, in site order
+    for (int b = int(it.b0) + threadIdx.x; b < int(it.b1); b += OBS_THREADS) {
         double s = 0.0, e = 0.0;
-        for (int z = 0; z < lv.bz; ++z)
-            for (int y = 0; y < lv.by; ++y) {
-                const int64_t row = int64_t(X) * lv.bx + int64_t(S.nx) * (int64_t(Y) * lv.by + y +
-                                                                           int64_t(S.ny) * (int64_t(Z) * lv.bz + z));
-                for (int x = 0; x < lv.bx; ++x) {
-                    const double phi = (ds[row + x] - db) * inv_rbar;
-                    s += phi;
-                    e += phi * phi;
-                    if (it.unit_level >= 0) add_terms(tu, phi, phi * phi, 1.0);
-                    if (hist_u) atomicAdd(shist + nh + hist_bin(phi, H), 1u);
+        if (sites) {
+            s = (ds[b] - db) * inv_rbar;
+            e = s * s;
+        } else {
+            int X, Y, Z;
+            block_coords(lv, b, X, Y, Z);
+            for (int z = 0; z < lv.bz; ++z)
+                for (int y = 0; y < lv.by; ++y) {
+                    const int row = X * lv.bx + nx * (Y * lv.by + y + ny * (Z * lv.bz + z));
+                    for (int x = 0; x < lv.bx; ++x) {
+                        const double phi = (ds[row + x] - db) * inv_rbar;
+                        s += phi;
+                        e += phi * phi;
+                        if (it.unit_level >= 0) add_terms(tu, phi, phi * phi, 1.0);
+                        if (hist_u) atomicAdd(shist + nh + hist_bin(phi, H), 1u);
+                    }
                 }
-            }
+        }
         Sg[lv.off + b] = s;
         Eg[lv.off + b] = e;
         add_terms(tb, s, e, inv_v);
@@ -176,11 +198,152 @@ __global__ void __launch_bounds__(OBS_THREADS)
     }
 }
 
+// Bottom level of blocks too large for one thread each.  Items either hold
+// several whole blocks, one warp each (warp w takes blocks b0 + w, b0 + w + 8,
+// ...), or a range [i0, i1) of one block's sites, summed by the whole CTA: then
+// the block is complete when the range is all of it (part < 0), else the CTA
+// leaves its sums of phi and phi^2 in parts[part] for pyr_blocks_kernel.
+__global__ void __launch_bounds__(OBS_THREADS)
+    pyr_part_kernel(const SysDev* __restrict__ sysv, const LevelDev* __restrict__ lvv,
+                    const ObsPart* __restrict__ items, const double* __restrict__ d, const double* __restrict__ dbar,
+                    double* __restrict__ Sg, double* __restrict__ Eg, double2* __restrict__ parts,
+                    double* __restrict__ rec, const HistDev H) {
+    constexpr int NW = OBS_THREADS / 32;
+    __shared__ double sh[REC * NW];
+    extern __shared__ unsigned shist[];          // [block level | single-site level], nbins + 2 each
+    const ObsPart it = items[blockIdx.x];
+    const LevelDev lv = lvv[it.level];
+    const SysDev& S = sysv[lv.sys];
+    const double* ds = d + S.site_offset;
+    const double db = dbar[lv.sys];
+    const double inv_rbar = 1.0 / (S.rho_c + db);
+    const double inv_v = 1.0 / (double(lv.bx) * lv.by * lv.bz);
+    const int nh = H.nbins + 2;
+    const bool hist = H.nbins > 0;
+    if (hist) {
+        hist_clear(shist, 2 * nh);
+        __syncthreads();
+    }
+    double tb[REC] = {0, 0, 0, 0, 0, 0};
+    double tu[REC] = {0, 0, 0, 0, 0, 0};
+    const int nx = S.nx, ny = S.ny;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool by_warp = it.b1 - it.b0 > 1;
+    const int step = by_warp ? 32 : OBS_THREADS;
+    auto block_done = [&](int b, double s, double e) {
+        Sg[lv.off + b] = s;
+        Eg[lv.off + b] = e;
+        add_terms(tb, s, e, inv_v);
+        if (hist) atomicAdd(shist + hist_bin(s * inv_v, H), 1u);
+    };
+    for (int b = it.b0 + (by_warp ? warp : 0); b < it.b1; b += by_warp ? NW : 1) {
+        int X, Y, Z;
+        block_coords(lv, b, X, Y, Z);
+        const double* corner = ds + (X * lv.bx + nx * (Y * lv.by + int64_t(ny) * (Z * lv.bz)));
+        double v[2] = {0.0, 0.0};
+        for (int i = it.i0 + (by_warp ? lane : int(threadIdx.x)); i < it.i1; i += step) {
+            const int r = i / lv.bx, x = i - r * lv.bx, z = r / lv.by, y = r - z * lv.by;
+            const double phi = (corner[x + nx * (y + int64_t(ny) * z)] - db) * inv_rbar;
+            v[0] += phi;
+            v[1] += phi * phi;
+            add_terms(tu, phi, phi * phi, 1.0);
+            if (hist) atomicAdd(shist + nh + hist_bin(phi, H), 1u);
+        }
+        if (by_warp) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                v[0] += __shfl_down_sync(0xffffffffu, v[0], o);
+                v[1] += __shfl_down_sync(0xffffffffu, v[1], o);
+            }
+            if (lane == 0) block_done(b, v[0], v[1]);
+        } else {
+            block_sum<2, OBS_THREADS>(v, sh);
+            if (threadIdx.x == 0) {
+                if (it.part < 0) block_done(b, v[0], v[1]);
+                else parts[it.part] = make_double2(v[0], v[1]);
+            }
+            __syncthreads();
+        }
+    }
+    if (it.part < 0) {
+        block_sum<REC, OBS_THREADS>(tb, sh);
+        if (threadIdx.x == 0)
+            for (int k = 0; k < REC; ++k) rec[int64_t(it.rec) * REC + k] = tb[k];
+        __syncthreads();
+    }
+    block_sum<REC, OBS_THREADS>(tu, sh);
+    if (threadIdx.x == 0)
+        for (int k = 0; k < REC; ++k) rec[int64_t(it.rec2) * REC + k] = tu[k];
+    if (hist) {
+        __syncthreads();
+        if (it.part < 0) hist_flush(shist, nh, H.counts + int64_t(it.level) * nh);
+        hist_flush(shist + nh, nh, H.counts + int64_t(it.unit_level) * nh);
+    }
+}
+
+// Blocks of several ranges: one warp per block sums its parts (parts of a
+// block are consecutive, part0 + b * per_block on).
+__global__ void __launch_bounds__(OBS_THREADS)
+    pyr_blocks_kernel(const LevelDev* __restrict__ lvv, const ObsBlocks* __restrict__ items,
+                      const double2* __restrict__ parts, double* __restrict__ Sg, double* __restrict__ Eg,
+                      double* __restrict__ rec, const HistDev H) {
+    constexpr int NW = OBS_THREADS / 32;
+    __shared__ double sh[REC * NW];
+    const ObsBlocks it = items[blockIdx.x];
+    const LevelDev lv = lvv[it.level];
+    const double inv_v = 1.0 / (double(lv.bx) * lv.by * lv.bz);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double tb[REC] = {0, 0, 0, 0, 0, 0};
+    for (int b = it.b0 + warp; b < it.b1; b += NW) {
+        const double2* p = parts + it.part0 + int64_t(b) * it.per_block;
+        double s = 0.0, e = 0.0;
+        for (int k = lane; k < it.per_block; k += 32) {
+            const double2 v = p[k];
+            s += v.x;
+            e += v.y;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            s += __shfl_down_sync(0xffffffffu, s, o);
+            e += __shfl_down_sync(0xffffffffu, e, o);
+        }
+        if (lane == 0) {
+            Sg[lv.off + b] = s;
+            Eg[lv.off + b] = e;
+            add_terms(tb, s, e, inv_v);
+            if (H.nbins > 0)
+                atomicAdd(H.counts + int64_t(it.level) * (H.nbins + 2) + hist_bin(s * inv_v, H), 1ull);
+        }
+    }
+    block_sum<REC, OBS_THREADS>(tb, sh);
+    if (threadIdx.x == 0)
+        for (int k = 0; k < REC; ++k) rec[int64_t(it.rec) * REC + k] = tb[k];
+}
+
+// Sums of phi and phi^2 of block b of level lv over its 2^d children (level
+// ch), in the order x, y, z.
+__device__ __forceinline__ void children_sum(const LevelDev& lv, const LevelDev& ch, int b, int dims3,
+                                             const double* Sg, const double* Eg, double& s, double& e) {
+    int X, Y, Z;
+    block_coords(lv, b, X, Y, Z);
+    s = e = 0.0;
+    const int nz = dims3 ? 2 : 1;
+    for (int dz = 0; dz < nz; ++dz)
+#pragma unroll
+        for (int dy = 0; dy < 2; ++dy) {
+            const int64_t c = ch.off + 2 * X + ch.gx * (2 * Y + dy + int64_t(ch.gy) * (nz * Z + dz));
+            s += Sg[c];
+            e += Eg[c];
+            s += Sg[c + 1];
+            e += Eg[c + 1];
+        }
+}
+
 // One coarser level: each block sums its 2^d children of the next finer level.
 __global__ void __launch_bounds__(OBS_THREADS)
     pyr_up_kernel(const LevelDev* __restrict__ lvv, const ObsItem* __restrict__ items, int dims3,
                   double* __restrict__ Sg, double* __restrict__ Eg, double* __restrict__ rec, const HistDev H) {
-    __shared__ double sh[REC * OBS_THREADS];
+    __shared__ double sh[REC * OBS_THREADS / 32];
     extern __shared__ unsigned shist[];
     const ObsItem it = items[blockIdx.x];
     const LevelDev lv = lvv[it.level];
@@ -193,20 +356,9 @@ __global__ void __launch_bounds__(OBS_THREADS)
         __syncthreads();
     }
     double tb[REC] = {0, 0, 0, 0, 0, 0};
-    for (int j = 0; j < BLOCKS_PER_THREAD; ++j) {
-        const int64_t b = it.b0 + int64_t(j) * OBS_THREADS + threadIdx.x;
-        if (b >= it.b1) break;
-        const int X = int(b % lv.gx), Y = int((b / lv.gx) % lv.gy), Z = int(b / (int64_t(lv.gx) * lv.gy));
-        double s = 0.0, e = 0.0;
-        const int nz = dims3 ? 2 : 1;
-        for (int dz = 0; dz < nz; ++dz)
-            for (int dy = 0; dy < 2; ++dy)
-                for (int dx = 0; dx < 2; ++dx) {
-                    const int64_t cb = int64_t(2 * X + dx) +
-                                       int64_t(ch.gx) * (int64_t(2 * Y + dy) + int64_t(ch.gy) * (int64_t(nz * Z + dz)));
-                    s += Sg[ch.off + cb];
-                    e += Eg[ch.off + cb];
-                }
+    for (int b = int(it.b0) + threadIdx.x; b < int(it.b1); b += OBS_THREADS) {
+        double s, e;
+        children_sum(lv, ch, b, dims3, Sg, Eg, s, e);
         Sg[lv.off + b] = s;
         Eg[lv.off + b] = e;
         add_terms(tb, s, e, inv_v);
@@ -222,22 +374,77 @@ __global__ void __launch_bounds__(OBS_THREADS)
 }
 
 // acc layout per level (7 doubles): n, sum m, m^2, |m|, m^4, e, e^2
-__global__ void obs_accum_kernel(const LevelDev* __restrict__ lvv, int n_levels, const double* __restrict__ rec,
-                                 double* __restrict__ acc, int* status) {
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= n_levels) return;
-    const LevelDev lv = lvv[l];
-    double t[REC] = {0, 0, 0, 0, 0, 0};
-    for (int r = 0; r < lv.rec_count; ++r)
-        for (int k = 0; k < REC; ++k) t[k] += rec[int64_t(lv.rec_first + r) * REC + k];
-    double* a = acc + int64_t(l) * 7;
-    a[0] += double(lv.nblocks);
+__device__ __forceinline__ void accumulate_level(double* a, double nblocks, const double (&t)[REC], int* status) {
+    a[0] += nblocks;
     bool finite = true;
     for (int k = 0; k < REC; ++k) {
         a[1 + k] += t[k];
         finite = finite && isfinite(t[k]);
     }
     if (!finite) atomicOr(status, ST_NONFINITE);
+}
+
+// One warp: the records of a level, summed by lanes 32 apart and a shuffle
+// tree, into its accumulators.  (One thread in order before: 0.1 ms of
+// dependent loads for the 256 records of a 64^3 system.)
+__device__ __forceinline__ void accumulate_records(const LevelDev& lv, const double* __restrict__ rec, double* a,
+                                                   int* status) {
+    const int lane = threadIdx.x & 31;
+    double t[REC] = {0, 0, 0, 0, 0, 0};
+    for (int r = lane; r < lv.rec_count; r += 32)
+#pragma unroll
+        for (int k = 0; k < REC; ++k) t[k] += rec[int64_t(lv.rec_first + r) * REC + k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < REC; ++k) t[k] += __shfl_down_sync(0xffffffffu, t[k], o);
+    if (lane == 0) accumulate_level(a, double(lv.nblocks), t, status);
+}
+
+// The coarsest levels of one system per CTA: levels top - 1 .. 0 (level `top`
+// is complete), each behind a CTA barrier because it reads the block sums that
+// other threads of the CTA wrote; level l's six sums go straight into its
+// accumulators.  The other levels' records are accumulated by a warp each.
+__global__ void __launch_bounds__(TOP_THREADS)
+    pyr_top_kernel(const LevelDev* __restrict__ lvv, const ObsTop* __restrict__ tops, int dims3, double* Sg,
+                   double* Eg, const double* __restrict__ rec, double* __restrict__ acc, int* status,
+                   const HistDev H) {
+    constexpr int NW = TOP_THREADS / 32;
+    __shared__ double sh[REC * NW];
+    extern __shared__ unsigned shist[];
+    const ObsTop T = tops[blockIdx.x];
+    const int nh = H.nbins + 2;
+    const bool hist = H.nbins > 0;
+    for (int l = T.top + int(threadIdx.x >> 5); l < T.n_levels; l += NW)
+        accumulate_records(lvv[T.lv_first + l], rec, acc + int64_t(T.lv_first + l) * 7, status);
+    for (int l = T.top - 1; l >= 0; --l) {
+        const LevelDev lv = lvv[T.lv_first + l];
+        const LevelDev ch = lvv[T.lv_first + l + 1];
+        const double inv_v = 1.0 / (double(lv.bx) * lv.by * lv.bz);
+        if (hist) {
+            hist_clear(shist, nh);
+            __syncthreads();
+        }
+        double tb[REC] = {0, 0, 0, 0, 0, 0};
+        for (int b = threadIdx.x; b < int(lv.nblocks); b += TOP_THREADS) {
+            double s, e;
+            children_sum(lv, ch, b, dims3, Sg, Eg, s, e);
+            Sg[lv.off + b] = s;
+            Eg[lv.off + b] = e;
+            add_terms(tb, s, e, inv_v);
+            if (hist) atomicAdd(shist + hist_bin(s * inv_v, H), 1u);
+        }
+        block_sum<REC, TOP_THREADS>(tb, sh);      // its barrier also orders this level's block sums
+        if (threadIdx.x == 0) accumulate_level(acc + int64_t(T.lv_first + l) * 7, double(lv.nblocks), tb, status);
+        if (hist) hist_flush(shist, nh, H.counts + int64_t(T.lv_first + l) * nh);
+        __syncthreads();
+    }
+}
+
+// One warp per level (the allocation-free entry point, whose levels all have records).
+__global__ void obs_accum_kernel(const LevelDev* __restrict__ lvv, const double* __restrict__ rec,
+                                 double* __restrict__ acc, int* status) {
+    accumulate_records(lvv[blockIdx.x], rec, acc + int64_t(blockIdx.x) * 7, status);
 }
 
 __global__ void advance_kernel(int64_t* step, int64_t n) { *step += n; }
@@ -268,15 +475,9 @@ cudaError_t launch_init_noise(const SysDev* sys, const int4* items, int n_items,
     return cudaGetLastError();
 }
 
-cudaError_t launch_reduce_sys(const SysSpan* spans, int n_sys, const double* partial, int K, double* out,
-                              cudaStream_t st) {
-    reduce_sys_kernel<<<n_sys, AUX_THREADS, 0, st>>>(spans, partial, K, out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_obs_globals(const SysDev* sys, int n_sys, const double* red4, double* dbar, double* glob,
-                               int set_mass0, int count_sample, cudaStream_t st) {
-    obs_globals_kernel<<<(n_sys + 127) / 128, 128, 0, st>>>(sys, n_sys, red4, dbar, glob, set_mass0, count_sample);
+cudaError_t launch_reduce_globals(const SysDev* sys, const SysSpan* spans, int n_sys, const double* partial,
+                                  double* dbar, double* glob, int set_mass0, int count_sample, cudaStream_t st) {
+    reduce_globals_kernel<<<n_sys, AUX_THREADS, 0, st>>>(sys, spans, partial, dbar, glob, set_mass0, count_sample);
     return cudaGetLastError();
 }
 
@@ -294,7 +495,30 @@ cudaError_t launch_pyr_bottom(const SysDev* sys, const LevelDev* lv, const ObsIt
     return cudaGetLastError();
 }
 
-cudaError_t launch_pyr_up(const SysDev*, const LevelDev* lv, const ObsItem* items, int n_items, int dims3,
+cudaError_t launch_pyr_part(const SysDev* sys, const LevelDev* lv, const ObsPart* items, int n_items,
+                            const double* d, const double* dbar, double* S, double* E, double2* parts, double* rec,
+                            const HistDev& hist, cudaStream_t st) {
+    if (n_items == 0) return cudaSuccess;
+    const size_t shm = hist.nbins > 0 ? 2 * sizeof(unsigned) * (hist.nbins + 2) : 0;
+    pyr_part_kernel<<<n_items, OBS_THREADS, shm, st>>>(sys, lv, items, d, dbar, S, E, parts, rec, hist);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pyr_blocks(const LevelDev* lv, const ObsBlocks* items, int n_items, const double2* parts,
+                              double* S, double* E, double* rec, const HistDev& hist, cudaStream_t st) {
+    if (n_items == 0) return cudaSuccess;
+    pyr_blocks_kernel<<<n_items, OBS_THREADS, 0, st>>>(lv, items, parts, S, E, rec, hist);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pyr_top(const LevelDev* lv, const ObsTop* tops, int n_sys, int dims3, double* S, double* E,
+                           const double* rec, double* acc, int* status, const HistDev& hist, cudaStream_t st) {
+    const size_t shm = hist.nbins > 0 ? sizeof(unsigned) * (hist.nbins + 2) : 0;
+    pyr_top_kernel<<<n_sys, TOP_THREADS, shm, st>>>(lv, tops, dims3, S, E, rec, acc, status, hist);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pyr_up(const LevelDev* lv, const ObsItem* items, int n_items, int dims3,
                           double* S, double* E, double* rec, const HistDev& hist, cudaStream_t st) {
     if (n_items == 0) return cudaSuccess;
     const size_t shm = hist.nbins > 0 ? sizeof(unsigned) * (hist.nbins + 2) : 0;
@@ -302,9 +526,9 @@ cudaError_t launch_pyr_up(const SysDev*, const LevelDev* lv, const ObsItem* item
     return cudaGetLastError();
 }
 
-cudaError_t launch_obs_accum(const LevelDev* lv, int n_levels_total, const double* rec, double* acc, int* status,
+cudaError_t launch_obs_accum(const LevelDev* lv, int n_levels, const double* rec, double* acc, int* status,
                              cudaStream_t st) {
-    obs_accum_kernel<<<(n_levels_total + 127) / 128, 128, 0, st>>>(lv, n_levels_total, rec, acc, status);
+    obs_accum_kernel<<<n_levels, 32, 0, st>>>(lv, rec, acc, status);
     return cudaGetLastError();
 }
 
