@@ -48,7 +48,8 @@ struct SysHost {
 struct Plan {
     size_t sys, phys, tiles, pop0, pop1, step, status, d, dbar, site_items, site_partial, spans, glob, levels,
         S, E, bottom_items, part_items, block_items, parts, up_items, tops, rec, acc, hist, field_tmp, sk_sys, sk_tw, sk_acc, sk_b0, sk_b1, sk_bins, jk_j,
-        jk_lap, jk_F, jk_acc, total;
+        jk_lap, jk_F, jk_acc, mom, total;
+    int tdim[3] = {0, 0, 0};      // tile shape of the step kernel
     bool jk = false;
     int hist_bins = 0;
     double hist_range = 0.0;
@@ -184,6 +185,12 @@ lb_status choose_tile(int lattice, int coupling, const lb_run_opts* o, int& tile
     return LB_OK;
 }
 
+bool split_row(int lattice, int tile_id) {
+    int t[32][kVariantCols];
+    tile_table(lattice, t);
+    return t[tile_id][5] == 4;
+}
+
 // Number of step tiles (CTAs) of a tile shape over the ensemble.
 int64_t tiles_of(const lb_system_desc* s, int n, const int tdim[3]) {
     int64_t c = 0;
@@ -193,24 +200,27 @@ int64_t tiles_of(const lb_system_desc* s, int n, const int tdim[3]) {
     return c;
 }
 
-// Default variant: among the rows that differ from the default row only in
-// the z-chunk, the longest chunk whose CTAs still fill the GPU at least twice
-// over (resident CTAs per SM x SMs of the current device; 152 SMs when no
-// device is visible), else the default row.  Longer chunks re-read fewer
-// halo planes (4 per chunk; 2 for the modified equilibrium on D3Q19), but
-// too few CTAs leave SMs idle in the last
-// wave: on GB300 the 64-plane chunks win on the 160-system ensemble (1,184
-// CTAs) and on 256^3 (1,024), the 32-plane ones on 32 systems of 64^3 (512).
-void prefer_longer_chunk(const lb_system_desc* s, int n, int& tile_id, int tdim[3]) {
-    int t[32][kVariantCols];
-    const int nt = tile_table(s[0].lattice, t);
-    int sms = 0;
-    int dev = 0;
+// SMs of the current device (152 when none is visible).
+int sm_count() {
+    int sms = 0, dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) {
         cudaGetLastError();
         sms = 152;
     }
+    return sms;
+}
+
+// Default variant: among the rows that differ from the default row only in
+// the z-chunk, the longest chunk whose CTAs still fill the GPU at least twice
+// over (resident CTAs per SM x SMs), else the row given.  Longer chunks re-read fewer
+// halo planes (4 per chunk; 2 for the modified equilibrium on D3Q19), but
+// too few CTAs leave SMs idle in the last
+// wave: on GB300 the 64-plane chunks win on the 160-system ensemble (1,184
+// CTAs) and on 256^3 (1,024), the 32-plane ones on 32 systems of 64^3 (512).
+bool prefer_longer_chunk(const lb_system_desc* s, int n, int sms, int& tile_id) {
+    int t[32][kVariantCols];
+    const int nt = tile_table(s[0].lattice, t);
     const int* d = t[tile_id];
     int best = tile_id;
     for (int k = 0; k < nt; ++k) {
@@ -221,8 +231,62 @@ void prefer_longer_chunk(const lb_system_desc* s, int n, int& tile_id, int tdim[
         const int occ = t[k][3] > 0 ? t[k][3] : 1;
         if (tiles_of(s, n, t[k]) >= int64_t(2) * occ * sms) best = k;
     }
+    const bool found = best != tile_id;
     tile_id = best;
-    for (int k = 0; k < 3; ++k) tdim[k] = t[best][k];
+    return found;
+}
+
+// Estimated step time (us) of a D3Q19 row on the fully relaxed FP32 path, from
+// timings on GB300 (152 SMs) of ensembles of 512 to 8.4 M sites; it only has
+// to rank the rows.
+//  * paired kernel (staging 3): a resident CTA advances one plane per 1.53 us
+//    alone on its SM, 2.2 us beside one other, 3.1 us beside two; zc planes
+//    plus the halo planes of its chunk; CTAs in waves of 3 per SM.
+//  * split step (staging 4): the moment pass (quads of sites, or single sites
+//    where some nx is not a multiple of 4), then collision columns that occupy
+//    their SM for 0.51 us per plane plus 0.43 us (half of it for the 8 x 8
+//    columns) and take 0.87 us per plane plus 2 us however idle the SM is.
+// Measured against the 32- and 64-plane paired rows that were the default of
+// every ensemble: 16^3 28.9 -> 5.3 us, 64^3 52 -> 14.4, 4 x 64^3 55 -> 46,
+// 16 x 64^3 157 -> 147 us per step; 2.6 M sites with odd sides 332 -> 137 us.
+double estimated_step_us(const lb_system_desc* s, int n, const int* row, int sms, bool quads) {
+    const double ctas = double(tiles_of(s, n, row)), zc = row[2];
+    int64_t sites = 0;
+    int nz = 0;
+    for (int k = 0; k < n; ++k) {
+        sites += int64_t(s[k].nx) * s[k].ny * s[k].nz;
+        nz = std::max(nz, s[k].nz);
+    }
+    const double planes = std::min<double>(zc, nz);
+    if (row[5] == 3) {
+        const double per = planes + (s[0].coupling == LB_MODEQ ? 2 : 4), slots = 3.0 * sms;
+        const double full = std::floor(ctas / slots), rest = ctas - full * slots;
+        const double plane_us[4] = {0.0, 1.53, 2.2, 3.1};
+        return 3.0 + per * (3.1 * full + plane_us[int(std::ceil(rest / sms))]);
+    }
+    const double cost = (0.51 * planes + 0.43) * (row[0] == 8 ? 0.5 : 1.0);
+    const double load = ctas / sms, filled = load <= 4.0 ? std::ceil(load) : load + 0.5;
+    return 3.0 + sites * (quads ? 1.6e-5 : 2.2e-5) + std::max(2.0 + 0.87 * planes, filled * cost);
+}
+
+// Default row of the fully relaxed FP32 path on D3Q19: the 64-plane paired row
+// while the ensemble fills the GPU twice over with it, else the cheapest of
+// the paired rows (every nx a multiple of 4) and the split rows.
+void choose_d3q19_row(const lb_system_desc* s, int n, bool quads, int& tile_id) {
+    const int sms = sm_count();
+    if (quads && prefer_longer_chunk(s, n, sms, tile_id)) return;
+    int t[32][kVariantCols];
+    const int nt = tile_table(LB_D3Q19, t);
+    double best_us = quads ? estimated_step_us(s, n, t[tile_id], sms, quads) : INFINITY;
+    for (int k = 0; k < nt; ++k) {
+        const bool paired = t[k][5] == 3 && t[k][0] == t[0][0] && quads;
+        if (!paired && t[k][5] != 4) continue;
+        const double us = estimated_step_us(s, n, t[k], sms, quads);
+        if (us < best_us) {
+            best_us = us;
+            tile_id = k;
+        }
+    }
 }
 
 lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::vector<SysHost>& sys, Plan& P,
@@ -230,15 +294,22 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
     lb_status st = validate(s, n, o);
     if (st != LB_OK) return st;
     int tdim[3];
-    bool paired_runs = o->precision == LB_FP32_DEVIATION;
+    bool relaxed32 = o->precision == LB_FP32_DEVIATION, quads = true;
     for (int k = 0; k < n; ++k) {
-        if (s[k].nx % 4 != 0) paired_runs = false;
+        if (s[k].nx % 4 != 0) quads = false;
         for (int a = s[k].lattice == LB_D2Q9 ? 3 : 4; a < q_of(s[k].lattice); ++a)
-            if (s[k].tau[a] != 1.0) paired_runs = false;
+            if (s[k].tau[a] != 1.0) relaxed32 = false;
     }
-    st = choose_tile(s[0].lattice, s[0].coupling, o, tile_id, tdim, !paired_runs);
+    st = choose_tile(s[0].lattice, s[0].coupling, o, tile_id, tdim, !(relaxed32 && quads));
     if (st != LB_OK) return st;
-    if (o->variant == 0 && o->tile[0] <= 0 && o->occupancy <= 0) prefer_longer_chunk(s, n, tile_id, tdim);
+    if (o->variant == 0 && o->tile[0] <= 0 && o->occupancy <= 0) {
+        if (s[0].lattice == LB_D3Q19 && relaxed32) choose_d3q19_row(s, n, quads, tile_id);
+        else prefer_longer_chunk(s, n, sm_count(), tile_id);
+        int t[32][kVariantCols];
+        tile_table(s[0].lattice, t);
+        for (int k = 0; k < 3; ++k) tdim[k] = t[tile_id][k];
+    }
+    for (int k = 0; k < 3; ++k) P.tdim[k] = tdim[k];
     const int q = q_of(s[0].lattice);
     const size_t es = o->precision == LB_FP64 ? 8 : 4;
     sys.assign(n, SysHost());
@@ -480,6 +551,8 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
     P.jk_lap = take(sizeof(double) * jkn);
     P.jk_F = take(sizeof(double) * 6 * jkn);
     P.jk_acc = take(sizeof(double) * 3 * jkn);
+    // density and momentum of the split step
+    P.mom = take(split_row(s[0].lattice, tile_id) && relaxed32 ? es * 4 * P.n_sites : 0);
     P.total = off;
     return LB_OK;
 }
@@ -554,7 +627,7 @@ SysDev to_dev(const SysHost& h) {
 
 struct lb_ctx {
     int lattice = 0, coupling = 0, fp32 = 0, q = 9, n_sys = 0, tile_id = 0, bgk_only = 0, bulk_ok = 0,
-        pair_ok = 0;
+        pair_ok = 0, step_kernels = 1;
     lb_run_opts opts{};
     std::vector<SysHost> sys;
     Plan P;
@@ -766,12 +839,18 @@ cudaError_t launch_steps(lb_ctx* c, int64_t n) {
         a.k = int(k);
         a.status = c->at<int>(P.status);
         a.tile_id = c->tile_id;
+        a.zc = P.tdim[2];
+        a.mom = c->ws + P.mom;
+        a.n_sites = P.n_sites;
+        a.site_items = c->at<int4>(P.site_items);
+        a.n_site_items = P.n_site_items;
+        a.small_items = P.n_sites < kSpreadSites ? 1 : 0;
         a.bgk_only = c->bgk_only;
         a.bulk_ok = c->bulk_ok;
         a.pair_ok = c->pair_ok;
         cudaError_t e = launch_step_any(c, a);
         if (e != cudaSuccess) return e;
-        c->launches += 1;
+        c->launches += c->step_kernels;
         const int64_t t1 = t + 1;
         const bool obs_due = c->opts.obs_every > 0 && t1 % c->opts.obs_every == 0;
         if (c->fault_kind != 0 && t1 == c->fault_step) {
@@ -898,6 +977,7 @@ lb_status lb_create(const lb_system_desc* systems, int n_systems, const lb_run_o
         if (!s.bgk) c->bgk_only = 0;
         else if (s.lam_bgk != 1.0 && c->bgk_only == 2) c->bgk_only = 1;
     }
+    if (split_row(c->lattice, c->tile_id) && c->fp32 && c->bgk_only == 2) c->step_kernels = 2;
     // bulk-copy staging: 16-byte aligned rows (nx % 4 == 0, so every system's
     // populations start 16-byte aligned too), at most 4 seam pieces per staged
     // row (nx >= 8) and single periodic wraps (every side >= 3)

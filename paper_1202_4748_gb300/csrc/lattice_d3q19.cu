@@ -19,13 +19,18 @@ namespace {
 // aligned quads in registers (0) or with cp.async in shared memory (3).  Two sites per consumer
 // thread: the paired kernel (x-adjacent site pairs, paired FP32 arithmetic;
 // ensembles with an odd nx run the one-site warp-specialised kernel of the
-// same tile).  The first entry is the default.
+// same tile).  Staging 4: the split step (a moment pass, then collision columns
+// of the tile, two sites stacked in z per thread; FP32 with every mode at
+// tau = 1, else the plain z-marching kernel of the same tile).  The first entry is the default.
 constexpr int kTiles[][kVariantCols] = {
     {32, 8, 32, 3, 4, 3, 2}, {32, 8, 64, 3, 4, 3, 2}, {16, 16, 32, 3, 4, 3, 2}, {16, 16, 64, 3, 4, 3, 2},
     {32, 8, 32, 2, 4, 0, 2}, {16, 16, 32, 2, 4, 0, 2},
     {32, 8, 64, 2, 4, 0, 2}, {16, 8, 32, 3, 4, 0, 1},  {16, 8, 64, 3, 4, 0, 1},  {16, 8, 16, 3, 4, 0, 1},
     {16, 8, 32, 3, 4, 1, 1}, {16, 8, 16, 6, 0, 0, 1},  {16, 8, 32, 6, 0, 0, 1},  {16, 16, 16, 4, 0, 0, 1},
-    {16, 16, 32, 4, 0, 0, 1}};
+    {16, 16, 32, 4, 0, 0, 1},
+    {32, 8, 16, 3, 4, 3, 2}, {32, 8, 8, 3, 4, 3, 2},
+    {16, 8, 2, 4, 0, 4, 2},  {16, 8, 4, 4, 0, 4, 2},   {16, 8, 8, 4, 0, 4, 2},   {16, 8, 16, 4, 0, 4, 2},
+    {16, 8, 32, 4, 0, 4, 2}, {8, 8, 2, 8, 0, 4, 2}};
 constexpr int kNumTiles = int(sizeof(kTiles) / sizeof(kTiles[0]));
 // ring planes of the paired kernel: 8 with register staging (2 CTAs per SM),
 // 4 with cp.async staging (the staging areas share the shared memory)
@@ -34,35 +39,39 @@ constexpr int pair_ring(int stg) { return stg == 3 ? 4 : 8; }
 template <int CP, class Real, int I>
 cudaError_t step_variant(const StepLaunch& a, cudaStream_t st) {
     constexpr int PW = kTiles[I][4];
+    if constexpr (kTiles[I][5] == 4 && std::is_same<Real, float>::value) {
+        if (a.bgk_only == 2)
+            return step_split<CP, kTiles[I][0], kTiles[I][1], kTiles[I][3]>(a, st);
+    }
     if constexpr (CP == MODEQ) {
         // the modified equilibrium: the paired kernel on the paired rows (FP32,
         // every mode at tau = 1, every nx a multiple of 4), else the radius-1
         // z-marching kernel of the same tile
         if constexpr (PW > 0 && kTiles[I][5] == 3 && kTiles[I][6] == 2 && std::is_same<Real, float>::value) {
             if (a.bgk_only == 2 && a.pair_ok)
-                return step_pair<kTiles[I][0], kTiles[I][1], kTiles[I][2], PW, kTiles[I][3], pair_ring(kTiles[I][5]),
+                return step_pair<kTiles[I][0], kTiles[I][1], PW, kTiles[I][3], pair_ring(kTiles[I][5]),
                                  kTiles[I][5], MODEQ>(a, st);
         }
-        return step_zm<D3Q19, Real, kTiles[I][0], kTiles[I][1], kTiles[I][2], kTiles[I][3]>(a, st);
+        return step_zm<D3Q19, Real, kTiles[I][0], kTiles[I][1], kTiles[I][3]>(a, st);
     } else {
         if constexpr (PW > 0 && std::is_same<Real, float>::value) {
             if (a.bgk_only == 2) {
                 if constexpr (kTiles[I][6] == 2) {
                     if (a.pair_ok)
-                        return step_pair<kTiles[I][0], kTiles[I][1], kTiles[I][2], PW, kTiles[I][3],
+                        return step_pair<kTiles[I][0], kTiles[I][1], PW, kTiles[I][3],
                                          pair_ring(kTiles[I][5]), kTiles[I][5]>(a, st);
-                    return step_ws<D3Q19, kTiles[I][0], kTiles[I][1], kTiles[I][2], PW, 1, 0>(a, st);
+                    return step_ws<D3Q19, kTiles[I][0], kTiles[I][1], PW, 1, 0>(a, st);
                 } else {
                     if constexpr (kTiles[I][5] == 1) {
                         if (a.bulk_ok)
-                            return step_ws<D3Q19, kTiles[I][0], kTiles[I][1], kTiles[I][2], PW, kTiles[I][3], 1>(a,
+                            return step_ws<D3Q19, kTiles[I][0], kTiles[I][1], PW, kTiles[I][3], 1>(a,
                                                                                                               st);
                     }
-                    return step_ws<D3Q19, kTiles[I][0], kTiles[I][1], kTiles[I][2], PW, kTiles[I][3], 0>(a, st);
+                    return step_ws<D3Q19, kTiles[I][0], kTiles[I][1], PW, kTiles[I][3], 0>(a, st);
                 }
             }
         }
-        return step_z<D3Q19, CP, Real, kTiles[I][0], kTiles[I][1], kTiles[I][2], kTiles[I][3]>(a, st);
+        return step_z<D3Q19, CP, Real, kTiles[I][0], kTiles[I][1], kTiles[I][3]>(a, st);
     }
 }
 

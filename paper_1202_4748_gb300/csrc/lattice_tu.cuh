@@ -6,13 +6,14 @@
 #include "lb_launch.h"
 #include "step_kernel_modeq3.cuh"
 #include "step_kernel_pair.cuh"
+#include "step_kernel_split.cuh"
 #include "step_kernel_strip_pair.cuh"
 #include "step_kernels.cuh"
 
 namespace lbf {
 
-template <class L, int CP, class Real, int TX, int TY, int TZ, int MODE>
-cudaError_t step_one_mode(const StepLaunch& a, cudaStream_t st) {
+template <class Real>
+StepArgs<Real> step_args(const StepLaunch& a) {
     StepArgs<Real> A;
     A.sys = a.sys;
     A.phys = static_cast<const SysPhys<Real>*>(a.phys);
@@ -22,6 +23,13 @@ cudaError_t step_one_mode(const StepLaunch& a, cudaStream_t st) {
     A.step_ptr = a.step_ptr;
     A.k = a.k;
     A.status = a.status;
+    A.zc = a.zc;
+    return A;
+}
+
+template <class L, int CP, class Real, int TX, int TY, int TZ, int MODE>
+cudaError_t step_one_mode(const StepLaunch& a, cudaStream_t st) {
+    const StepArgs<Real> A = step_args<Real>(a);
     step_kernel<L, CP, Real, TX, TY, TZ, MODE><<<a.n_tiles, TX * TY * TZ, 0, st>>>(A);
     return cudaGetLastError();
 }
@@ -30,15 +38,7 @@ cudaError_t step_one_mode(const StepLaunch& a, cudaStream_t st) {
 // of SW sites x YC rows, one warp per 32 sites of a tile.
 template <class L, int CP, class Real, int YC, int WPC, int MINB, int MODE, int SW>
 cudaError_t step_strip_mode(const StepLaunch& a, cudaStream_t st) {
-    StepArgs<Real> A;
-    A.sys = a.sys;
-    A.phys = static_cast<const SysPhys<Real>*>(a.phys);
-    A.tiles = a.tiles;
-    A.fin = static_cast<const Real*>(a.fin);
-    A.fout = static_cast<Real*>(a.fout);
-    A.step_ptr = a.step_ptr;
-    A.k = a.k;
-    A.status = a.status;
+    const StepArgs<Real> A = step_args<Real>(a);
     const int warps = a.n_tiles * (SW / 32);
     const int grid = (warps + WPC - 1) / WPC;
     step_kernel_strip<L, CP, Real, YC, WPC, MINB, MODE, SW><<<grid, 32 * WPC, 0, st>>>(A, a.n_tiles);
@@ -59,15 +59,7 @@ template <class L, int CP, class Real, int YC, int WPC, int MINB>
 cudaError_t step_strip2(const StepLaunch& a, cudaStream_t st) {
     if constexpr (sizeof(Real) == 4 && CP == MODEQ) {
         if (a.bgk_only == 2 && a.pair_ok) {
-            StepArgs<float> A;
-            A.sys = a.sys;
-            A.phys = static_cast<const SysPhys<float>*>(a.phys);
-            A.tiles = a.tiles;
-            A.fin = static_cast<const float*>(a.fin);
-            A.fout = static_cast<float*>(a.fout);
-            A.step_ptr = a.step_ptr;
-            A.k = a.k;
-            A.status = a.status;
+            const StepArgs<float> A = step_args<float>(a);
             const int grid = (a.n_tiles + WPC - 1) / WPC;
             step_kernel_strip_pair<YC, WPC, MINB><<<grid, 32 * WPC, 0, st>>>(A, a.n_tiles);
             return cudaGetLastError();
@@ -76,75 +68,51 @@ cudaError_t step_strip2(const StepLaunch& a, cudaStream_t st) {
     return step_strip<L, CP, Real, YC, WPC, MINB, 64>(a, st);
 }
 
-template <class L, int CP, class Real, int TX, int TY, int ZC, int MINB, int MODE>
+template <class L, int CP, class Real, int TX, int TY, int MINB, int MODE>
 cudaError_t step_z_mode(const StepLaunch& a, cudaStream_t st) {
-    StepArgs<Real> A;
-    A.sys = a.sys;
-    A.phys = static_cast<const SysPhys<Real>*>(a.phys);
-    A.tiles = a.tiles;
-    A.fin = static_cast<const Real*>(a.fin);
-    A.fout = static_cast<Real*>(a.fout);
-    A.step_ptr = a.step_ptr;
-    A.k = a.k;
-    A.status = a.status;
-    step_kernel_z<L, CP, Real, TX, TY, ZC, MINB, MODE><<<a.n_tiles, TX * TY, 0, st>>>(A);
+    const StepArgs<Real> A = step_args<Real>(a);
+    step_kernel_z<L, CP, Real, TX, TY, MINB, MODE><<<a.n_tiles, TX * TY, 0, st>>>(A);
     return cudaGetLastError();
 }
 
 // z-marching launch: tile = (TX, TY, z-chunk), register budget for MINB resident
 // CTAs per SM (the FP64 instances use the natural register count).
-template <class L, int CP, class Real, int TX, int TY, int ZC, int MINB>
+template <class L, int CP, class Real, int TX, int TY, int MINB>
 cudaError_t step_z(const StepLaunch& a, cudaStream_t st) {
     constexpr int MB = sizeof(Real) == 4 ? MINB : 1;
-    if (a.bgk_only == 2) return step_z_mode<L, CP, Real, TX, TY, ZC, MB, 2>(a, st);
-    if (a.bgk_only == 1) return step_z_mode<L, CP, Real, TX, TY, ZC, MB, 1>(a, st);
-    return step_z_mode<L, CP, Real, TX, TY, ZC, MB, 0>(a, st);
+    if (a.bgk_only == 2) return step_z_mode<L, CP, Real, TX, TY, MB, 2>(a, st);
+    if (a.bgk_only == 1) return step_z_mode<L, CP, Real, TX, TY, MB, 1>(a, st);
+    return step_z_mode<L, CP, Real, TX, TY, MB, 0>(a, st);
 }
 
 // z-marching launch of the D3Q19 modified equilibrium (density footprint of
 // radius 1); the FP64 instances use the natural register count.
-template <class L, class Real, int TX, int TY, int ZC, int MINB, int MODE>
+template <class L, class Real, int TX, int TY, int MINB, int MODE>
 cudaError_t step_zm_mode(const StepLaunch& a, cudaStream_t st) {
-    StepArgs<Real> A;
-    A.sys = a.sys;
-    A.phys = static_cast<const SysPhys<Real>*>(a.phys);
-    A.tiles = a.tiles;
-    A.fin = static_cast<const Real*>(a.fin);
-    A.fout = static_cast<Real*>(a.fout);
-    A.step_ptr = a.step_ptr;
-    A.k = a.k;
-    A.status = a.status;
-    step_kernel_zm<L, Real, TX, TY, ZC, MINB, MODE><<<a.n_tiles, TX * TY, 0, st>>>(A);
+    const StepArgs<Real> A = step_args<Real>(a);
+    step_kernel_zm<L, Real, TX, TY, MINB, MODE><<<a.n_tiles, TX * TY, 0, st>>>(A);
     return cudaGetLastError();
 }
-template <class L, class Real, int TX, int TY, int ZC, int MINB>
+template <class L, class Real, int TX, int TY, int MINB>
 cudaError_t step_zm(const StepLaunch& a, cudaStream_t st) {
     constexpr int MB = sizeof(Real) == 4 ? (MINB < 2 ? 2 : MINB) : 1;
-    if (a.bgk_only == 2) return step_zm_mode<L, Real, TX, TY, ZC, MB, 2>(a, st);
-    if (a.bgk_only == 1) return step_zm_mode<L, Real, TX, TY, ZC, MB, 1>(a, st);
-    return step_zm_mode<L, Real, TX, TY, ZC, MB, 0>(a, st);
+    if (a.bgk_only == 2) return step_zm_mode<L, Real, TX, TY, MB, 2>(a, st);
+    if (a.bgk_only == 1) return step_zm_mode<L, Real, TX, TY, MB, 1>(a, st);
+    return step_zm_mode<L, Real, TX, TY, MB, 0>(a, st);
 }
 
 // Warp-specialised launch (fully relaxed Guo path, FP32): TX x TY consumer
 // threads and PW producer warps per CTA; STG = 1 stages the footprint with
 // bulk copies (a dynamic shared-memory stage), 0 with plain loads.
-template <class L, int TX, int TY, int ZC, int PW, int MINB, int STG>
+template <class L, int TX, int TY, int PW, int MINB, int STG>
 cudaError_t step_ws(const StepLaunch& a, cudaStream_t st) {
-    StepArgs<float> A;
-    A.sys = a.sys;
-    A.phys = static_cast<const SysPhys<float>*>(a.phys);
-    A.tiles = a.tiles;
-    A.fin = static_cast<const float*>(a.fin);
-    A.fout = static_cast<float*>(a.fout);
-    A.step_ptr = a.step_ptr;
-    A.k = a.k;
-    A.status = a.status;
+    const StepArgs<float> A = step_args<float>(a);
     size_t dyn = 0;
     if constexpr (STG == 1) {
-        dyn = BulkStage<L, TX, TY, ZC, PW>::bytes;
+        dyn = BulkStage<L, TX, TY, PW>::bytes;
         static bool attr = false;              // once per instantiation
         if (!attr) {
-            auto k = step_kernel_ws<L, TX, TY, ZC, PW, MINB, STG>;
+            auto k = step_kernel_ws<L, TX, TY, PW, MINB, STG>;
             cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dyn));
             if (e == cudaSuccess)
                 e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -153,7 +121,7 @@ cudaError_t step_ws(const StepLaunch& a, cudaStream_t st) {
             attr = true;
         }
     }
-    step_kernel_ws<L, TX, TY, ZC, PW, MINB, STG><<<a.n_tiles, TX * TY + 32 * PW, dyn, st>>>(A);
+    step_kernel_ws<L, TX, TY, PW, MINB, STG><<<a.n_tiles, TX * TY + 32 * PW, dyn, st>>>(A);
     return cudaGetLastError();
 }
 
@@ -162,21 +130,13 @@ cudaError_t step_ws(const StepLaunch& a, cudaStream_t st) {
 // equilibrium): TX TY / 2 consumer threads and PW producer warps
 // per CTA, rings of R planes (and, STG = 3, the producers' staging area) in
 // dynamic shared memory.
-template <int TX, int TY, int ZC, int PW, int MINB, int R, int STG, int CP = GUO>
+template <int TX, int TY, int PW, int MINB, int R, int STG, int CP = GUO>
 cudaError_t step_pair(const StepLaunch& a, cudaStream_t st) {
-    StepArgs<float> A;
-    A.sys = a.sys;
-    A.phys = static_cast<const SysPhys<float>*>(a.phys);
-    A.tiles = a.tiles;
-    A.fin = static_cast<const float*>(a.fin);
-    A.fout = static_cast<float*>(a.fout);
-    A.step_ptr = a.step_ptr;
-    A.k = a.k;
-    A.status = a.status;
+    const StepArgs<float> A = step_args<float>(a);
     constexpr size_t dyn = PairSmem<TX, TY, PW, R, STG, CP>::bytes;
     static int state = 0;                      // once per instantiation: 1 usable, -1 not
     if (state == 0) {
-        auto k = step_kernel_pair<TX, TY, ZC, PW, MINB, R, STG, CP>;
+        auto k = step_kernel_pair<TX, TY, PW, MINB, R, STG, CP>;
         cudaFuncAttributes fa;
         cudaError_t e = cudaFuncGetAttributes(&fa, k);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dyn));
@@ -187,11 +147,56 @@ cudaError_t step_pair(const StepLaunch& a, cudaStream_t st) {
         state = (!PairRegs<TX, TY, PW, MINB, STG>::split || fa.numRegs == PairRegs<TX, TY, PW, MINB, STG>::launch) ? 1 : -1;
     }
     if (state < 0) {
-        if constexpr (CP == MODEQ) return step_zm<D3Q19, float, TX, TY, ZC, MINB>(a, st);
-        else return step_ws<D3Q19, TX, TY, ZC, PW, 1, 0>(a, st);
+        if constexpr (CP == MODEQ) return step_zm<D3Q19, float, TX, TY, MINB>(a, st);
+        else return step_ws<D3Q19, TX, TY, PW, 1, 0>(a, st);
     }
-    step_kernel_pair<TX, TY, ZC, PW, MINB, R, STG, CP><<<a.n_tiles, TX * TY / 2 + 32 * PW, dyn, st>>>(A);
+    step_kernel_pair<TX, TY, PW, MINB, R, STG, CP><<<a.n_tiles, TX * TY / 2 + 32 * PW, dyn, st>>>(A);
     return cudaGetLastError();
+}
+
+// Launch with programmatic stream serialisation: the kernel may start before
+// its predecessor on the stream has ended and orders itself with grid_wait.
+template <class... P, class... A>
+cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigned block, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = st;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// Moment pass of the split step: quads of sites where every nx is a multiple of
+// 4, else single sites; small CTAs when the items are small (few of them).
+template <class L, class Real>
+cudaError_t step_moments(const StepLaunch& a, cudaStream_t st) {
+    const Real* f = static_cast<const Real*>(a.fin);
+    Real* mom = static_cast<Real*>(a.mom);
+    if constexpr (sizeof(Real) == 4) {
+        if (a.pair_ok) {
+            if (a.small_items)
+                return launch_dependent(moments_quad_kernel<L, 64>, a.n_site_items, 64, st, a.sys, a.site_items, f, mom,
+                                        a.n_sites);
+            return launch_dependent(moments_quad_kernel<L, 256>, a.n_site_items, 256, st, a.sys, a.site_items, f, mom,
+                                    a.n_sites);
+        }
+    }
+    return launch_dependent(moments_kernel<L, Real, 256>, a.n_site_items, 256, st, a.sys, a.site_items, f, mom,
+                            a.n_sites);
+}
+
+// Split step (D3Q19, FP32, every mode at tau = 1): the moment pass over the
+// site items, then the collision of TX x TY columns in chunks of a.zc planes.
+template <int CP, int TX, int TY, int MINB>
+cudaError_t step_split(const StepLaunch& a, cudaStream_t st) {
+    const cudaError_t e = step_moments<D3Q19, float>(a, st);
+    if (e != cudaSuccess) return e;
+    return launch_dependent(collide_march_kernel<CP, TX, TY, MINB>, a.n_tiles, TX * TY, st, step_args<float>(a),
+                            static_cast<const float*>(a.mom), a.n_sites);
 }
 
 template <class L, int CP, class Real, int TX, int TY, int TZ>

@@ -23,6 +23,12 @@ struct StepLaunch {
     int k;
     int* status;
     int tile_id;            // index into the lattice's tile-shape table
+    int zc;                 // z extent of its tiles (planes per chunk of the z-marching kernels)
+    void* mom;              // split step: density and momentum fields, one per n_sites values
+    int64_t n_sites;        // sites of the ensemble
+    const int4* site_items; // split step: the moment pass's work list
+    int n_site_items;
+    int small_items;        // the items hold AUX_THREADS sites (else SITES_PER_THREAD times as many)
     int bgk_only;           // 0: per-mode rates; 1: one rate per system; 2: one rate, equal to 1
     int bulk_ok;            // every system allows bulk-copy staging (nx % 4 == 0, nx >= 8, sides >= 3)
     int pair_ok;            // every system has nx % 4 == 0 (the paired-site kernel can run)

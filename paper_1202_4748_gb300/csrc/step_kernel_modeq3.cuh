@@ -147,7 +147,7 @@ __device__ __forceinline__ void collide_modeq3(Real (&f)[L::Q], const Real drho,
 }
 
 // z-marching step for the modified equilibrium on D3Q19: a CTA owns a TX x TY
-// column and walks a chunk of ZC planes; iteration zz forms the density of
+// column and walks a chunk of A.zc planes; iteration zz forms the density of
 // footprint plane zz (tile + 1 site, from the pulled populations; with every
 // mode at tau = 1 also the momentum of the tile sites, so the collision needs
 // no second pull) into a ring of 4 planes, and after one barrier collides plane
@@ -155,7 +155,7 @@ __device__ __forceinline__ void collide_modeq3(Real (&f)[L::Q], const Real drho,
 // next iteration writes the slot of plane zz - 3, which no collision of
 // iteration zz reads, and no thread starts it before every thread has passed
 // the barrier of iteration zz.
-template <class L, class Real, int TX, int TY, int ZC, int MINB, int MODE>
+template <class L, class Real, int TX, int TY, int MINB, int MODE>
 __global__ void __launch_bounds__(TX* TY, MINB) step_kernel_zm(const StepArgs<Real> A) {
     static_assert(L::D == 3, "z-marching is for 3-D lattices");
     constexpr int Q = L::Q;
@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(TX* TY, MINB) step_kernel_zm(const StepArgs<Re
     const int N = S.ns;
     const Real* __restrict__ fb = A.fin + S.pop_offset;
     Real* __restrict__ fo = A.fout + S.pop_offset;
-    const int z0 = tl.w, z1 = min(z0 + ZC, nz);
+    const int z0 = tl.w, z1 = min(z0 + A.zc, nz);
     const int64_t step = *A.step_ptr + A.k;
     const int tid = threadIdx.x;
     const int tx = tid % TX, ty = tid / TX;

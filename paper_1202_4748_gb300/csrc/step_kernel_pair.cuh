@@ -1,7 +1,7 @@
 // Warp-specialised z-marching D3Q19 step with two x-adjacent sites per
 // consumer thread (fully relaxed Guo path, FP32, every nx a multiple of 4).
 //
-// Per CTA a TX x TY column of sites walks a chunk of ZC planes.  PW producer
+// Per CTA a TX x TY column of sites walks a chunk of A.zc planes.  PW producer
 // warps stage each plane into shared-memory rings of R planes:
 //   * density deviation on the footprint (columns x0 - 4 .. x0 + TX + 3, rows
 //     y0 - 2 .. y0 + TY + 1; y0 - 1 .. y0 + TY for the modified equilibrium,
@@ -178,7 +178,7 @@ struct PairSmem {
     static constexpr size_t bytes = PairLayout<TX, TY, R, CP == MODEQ ? 1 : 2>::bytes + stage;
 };
 
-template <int TX, int TY, int ZC, int PW, int MINB, int R, int STG, int CP = GUO>
+template <int TX, int TY, int PW, int MINB, int R, int STG, int CP = GUO>
 __global__ void __launch_bounds__(TX* TY / 2 + 32 * PW, MINB) step_kernel_pair(const StepArgs<float> A) {
     using RG = PairRegs<TX, TY, PW, MINB, STG>;
     using L = D3Q19;
@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(TX* TY / 2 + 32 * PW, MINB) step_kernel_pair(c
     const SysDev S = A.sys[tl.x];          // register copy: not re-read after the stores
     const int nx = S.nx, ny = S.ny, nz = S.nz;
     const int N = S.ns;
-    const int z0 = tl.w, z1 = min(z0 + ZC, nz);
+    const int z0 = tl.w, z1 = min(z0 + A.zc, nz);
     const int tid = threadIdx.x;
     if (tid == 0) {
         for (int r = 0; r < R; ++r) {

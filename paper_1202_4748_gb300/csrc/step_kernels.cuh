@@ -32,6 +32,7 @@ struct StepArgs {
     const int64_t* step_ptr;  // device step counter at the start of the chunk
     int k;                    // offset of this step inside the chunk
     int* status;
+    int zc;                   // planes per tile of the z-marching kernels
 };
 
 template <class L, int CP>
@@ -741,19 +742,14 @@ __global__ void __launch_bounds__(32 * WPC, MINB) step_kernel_strip(const StepAr
 namespace lbf {
 
 // z-marching variant for 3-D lattices.  A CTA owns a TX x TY column of sites
-// and walks a chunk of ZC planes.  (Keeping each thread's own populations in
+// and walks a chunk of A.zc planes.  (Keeping each thread's own populations in
 // shared memory instead of re-reading them was measured slower: the carve-out
 // takes the L1 space that serves the overlapping footprint pulls.)  The density deviation of each plane is
 // computed once on the column's footprint (halo H in x and y) into a ring of
 // 2H+1 planes in shared memory, the Laplacian (Guo force) into a ring of 3
 // planes, so every footprint value is formed once per chunk instead of once
 // per tile, and the collision of plane z follows two planes behind.
-template <class L, int CP, class Real, int TX, int TY, int ZC>
-struct ZLayout {
-    static constexpr size_t bytes = 0;     // static shared memory only
-};
-
-template <class L, int CP, class Real, int TX, int TY, int ZC, int MINB, int MODE>
+template <class L, int CP, class Real, int TX, int TY, int MINB, int MODE>
 __global__ void __launch_bounds__(TX* TY, MINB)
     step_kernel_z(const StepArgs<Real> A) {
     static_assert(L::D == 3, "z-marching is for 3-D lattices");
@@ -787,7 +783,7 @@ __global__ void __launch_bounds__(TX* TY, MINB)
     const int N = S.ns;
     const Real* __restrict__ fb = A.fin + S.pop_offset;
     Real* __restrict__ fo = A.fout + S.pop_offset;
-    const int z0 = tl.w, z1 = min(z0 + ZC, nz);
+    const int z0 = tl.w, z1 = min(z0 + A.zc, nz);
     const int64_t step = *A.step_ptr + A.k;
 
     const int tid = threadIdx.x;
@@ -937,7 +933,7 @@ __device__ __forceinline__ int foot_slot(int s) {
     return (H + r) * SX + (c < H ? c : TX + c);
 }
 
-template <class L, int TX, int TY, int ZC, int PW>
+template <class L, int TX, int TY, int PW>
 struct BulkStage {
     static constexpr int H = HaloOf<L, GUO>::H;
     static constexpr int BW = TX + 8;              // staged row: x0 - 4 .. x0 + TX + 3
@@ -948,7 +944,7 @@ struct BulkStage {
     static constexpr size_t bytes = 2 * size_t(BSTAGE) * sizeof(float);
 };
 
-template <class L, int TX, int TY, int ZC, int PW, int MINB, int STG>
+template <class L, int TX, int TY, int PW, int MINB, int STG>
 __global__ void __launch_bounds__(TX* TY + 32 * PW, MINB) step_kernel_ws(const StepArgs<float> A) {
     using Real = float;
     static_assert(L::D == 3, "z-marching is for 3-D lattices");
@@ -965,7 +961,7 @@ __global__ void __launch_bounds__(TX* TY + 32 * PW, MINB) step_kernel_ws(const S
     __shared__ Real sj[R * 3 * NC];
     __shared__ uint64_t full[R], empty[R];
     __shared__ int abort_flag;
-    using BS = BulkStage<L, TX, TY, ZC, PW>;
+    using BS = BulkStage<L, TX, TY, PW>;
     static_assert(STG == 0 || TX % 4 == 0, "staged rows start 16-byte aligned");
     extern __shared__ __align__(128) float stage_smem[];
     __shared__ uint64_t tfull[2];                  // bulk-copy stages
@@ -976,7 +972,7 @@ __global__ void __launch_bounds__(TX* TY + 32 * PW, MINB) step_kernel_ws(const S
     const SysDev S = A.sys[tl.x];          // register copy: not re-read after the stores
     const int nx = S.nx, ny = S.ny, nz = S.nz;
     const int N = S.ns;
-    const int z0 = tl.w, z1 = min(z0 + ZC, nz);
+    const int z0 = tl.w, z1 = min(z0 + A.zc, nz);
     const int tid = threadIdx.x;
     if (tid == 0) {
         for (int r = 0; r < R; ++r) {
