@@ -69,10 +69,11 @@ struct Plan {
     std::vector<SkSys> sk_h;
     std::vector<int> tw_sides, tw_offs;
     int tw_total = 0, tw_max = 0, sk_max_bins = 0;
-    // line-FFT work list of the structure factor (every side 2^a 3^b), else the direct sums
+    // line-FFT work lists of the spectra (every side up to kSkFftMaxElems), else the direct sums
     bool sk_fft = false;
     std::vector<int4> fft_items_h;
-    int n_fft_items = 0, fft_max_elems = 0;
+    int n_fft_x = 0, n_fft_y = 0, n_fft_last = 0, fft_max_x = 0, fft_max_y = 0, fft_max_last = 0, n_fields = 1;
+    int64_t half_total = 0;     // values of one field's half spectra
     size_t fft_items = 0;
 };
 
@@ -479,6 +480,8 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
             k.tw_z = table_of(h.d.nz);
             k.site_offset = h.site_off;
             k.inv_n = 1.0 / double(h.n);
+            k.half_offset = P.half_total;
+            P.half_total += h.n / h.d.nx * (h.d.nx / 2 + 1);
             P.sk_h.push_back(k);
             const int side = h.d.nx;
             P.sk_max_bins = std::max(P.sk_max_bins, int(std::ceil(std::sqrt(3.0) * side / 2.0)) + 2);
@@ -487,17 +490,35 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
         for (auto& h : sys)
             if (!sk_fft_side(h.d.nx)) P.sk_fft = false;
         if (P.sk_fft) {
-            for (int k = 0; k < n; ++k) {
-                const int side = sys[k].d.nx;
-                const int lines = int(sys[k].n / side);
-                const int per = std::max(1, kSkFftMaxElems / side);
-                for (int l = 0; l < lines; l += per) {
+            // lines per item: eight (whole warps of butterflies, 128-byte runs of
+            // kx), more where that leaves several items per SM, in kSkFftMaxElems
+            const bool d3 = s[0].lattice == LB_D3Q19;
+            P.n_fields = o->jk_spectra == 1 ? (d3 ? 4 : 3) : 1;
+            int64_t lines_all = 0;
+            for (auto& h : sys) lines_all += h.n / h.d.nx * P.n_fields;
+            const int want = int(std::min<int64_t>(64, std::max<int64_t>(8, lines_all / (8 * 152))));
+            auto add = [&](int k, int lines, int len, int field, int in_cta, int& count, int& mx) {
+                const int per = std::max(1, std::min(std::max(want / in_cta, 2), kSkFftMaxElems / (len * in_cta)));
+                for (int l = 0; l < lines; l += per, ++count) {
                     const int cnt = std::min(per, lines - l);
-                    P.fft_items_h.push_back(make_int4(k, l, cnt, 0));
-                    P.fft_max_elems = std::max(P.fft_max_elems, cnt * side);
+                    P.fft_items_h.push_back(make_int4(k, l, cnt, field));
+                    mx = std::max(mx, cnt * len * in_cta);
                 }
+            };
+            for (int k = 0; k < n; ++k)
+                for (int f = 0; f < P.n_fields; ++f) {
+                    const int S = sys[k].d.nx;
+                    add(k, int(sys[k].n / S), S % 2 == 0 ? S / 2 : S, f, 1, P.n_fft_x, P.fft_max_x);
+                }
+            for (int k = 0; k < n && d3; ++k)
+                for (int f = 0; f < P.n_fields; ++f) {
+                    const int S = sys[k].d.nx;
+                    add(k, (S / 2 + 1) * S, S, f, 1, P.n_fft_y, P.fft_max_y);
+                }
+            for (int k = 0; k < n; ++k) {
+                const int S = sys[k].d.nx;
+                add(k, (S / 2 + 1) * (d3 ? S : 1), S, 0, P.n_fields, P.n_fft_last, P.fft_max_last);
             }
-            P.n_fft_items = int(P.fft_items_h.size());
         }
     }
 
@@ -539,17 +560,18 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
     const int64_t skn = P.sk ? P.n_sites : 0;
     P.sk_sys = take(sizeof(SkSys) * (P.sk ? n : 0));
     P.sk_tw = take(sizeof(double) * 2 * P.tw_total);
-    P.fft_items = take(sizeof(int4) * P.n_fft_items);
+    P.fft_items = take(sizeof(int4) * P.fft_items_h.size());
     P.sk_acc = take(sizeof(double) * skn);
-    P.sk_b0 = take(sizeof(double) * 2 * skn);
-    P.sk_b1 = take(sizeof(double) * 2 * skn);
-    P.sk_bins = take(sizeof(double) * 2 * P.sk_max_bins);
+    // half spectra of every field (line FFTs), or two complex fields (direct sums)
+    P.sk_b0 = take(sizeof(double) * 2 * (P.sk_fft ? P.half_total * P.n_fields : skn));
+    P.sk_b1 = take(sizeof(double) * 2 * (P.sk_fft ? 0 : skn));
+    P.sk_bins = take(sizeof(double) * 6 * P.sk_max_bins);
     // momentum spectra: j (3 fields), Laplacian scratch (Guo), transforms (3 complex fields), accumulators
     P.jk = P.sk && o->jk_spectra == 1;
     const int64_t jkn = P.jk ? P.n_sites : 0;
     P.jk_j = take(sizeof(double) * 3 * jkn);
     P.jk_lap = take(sizeof(double) * jkn);
-    P.jk_F = take(sizeof(double) * 6 * jkn);
+    P.jk_F = take(sizeof(double) * 6 * (P.sk_fft ? 0 : jkn));
     P.jk_acc = take(sizeof(double) * 3 * jkn);
     // density and momentum of the split step
     P.mom = take(split_row(s[0].lattice, tile_id) && relaxed32 ? es * 4 * P.n_sites : 0);
@@ -713,58 +735,49 @@ cudaError_t sample_obs(lb_ctx* c, int buf, bool set_mass0, bool count, bool want
                           c->at<int>(P.status), H, c->stream);
 }
 
-// Momentum spectra of the momentum field the site pass just wrote: Guo
-// half-force, then per component x, y (and z) transforms, then accumulation.
-cudaError_t sample_jk(lb_ctx* c) {
+// Guo half-force on the momentum field the site pass just wrote.
+cudaError_t add_half_force(lb_ctx* c) {
     const Plan& P = c->P;
-    cudaError_t e;
+    if (!P.jk || c->coupling != LB_GUO) return cudaSuccess;
+    c->launches += 2;
+    return launch_jk_guo_force(c->lattice == LB_D3Q19 ? 1 : 0, c->at<SysDev>(P.sys), c->at<int4>(P.site_items),
+                               P.n_site_items, c->at<double>(P.d), c->at<double>(P.jk_lap), c->at<double>(P.jk_j),
+                               P.n_sites, c->stream);
+}
+
+// Spectra by direct sums (a side beyond the line FFTs): the structure factor,
+// then per momentum component the x, y (and z) transforms and the accumulation.
+cudaError_t sample_sk_direct(lb_ctx* c) {
+    const Plan& P = c->P;
+    cudaError_t e = cudaSuccess;
     const SysDev* sys = c->at<SysDev>(P.sys);
     const SkSys* sk = c->at<SkSys>(P.sk_sys);
     const int4* items = c->at<int4>(P.site_items);
     const int n_items = P.n_site_items;
     const int64_t ns = P.n_sites;
-    double* j = c->at<double>(P.jk_j);
-    double* F = c->at<double>(P.jk_F);
     double* b0 = c->at<double>(P.sk_b0);
     double* b1 = c->at<double>(P.sk_b1);
     const double* tw = c->at<double>(P.sk_tw);
     const bool d3 = c->lattice == LB_D3Q19;
+    // in: real field (with dbar: the order parameter); the transform lands in b0 (3-D) or out
+    auto transform = [&](const double* in, const double* dbar, double* out) {
+        cudaError_t r = launch_sk_x(sys, sk, items, n_items, in, dbar, tw, b0, c->stream);
+        if (r == cudaSuccess) r = launch_sk_pass(sk, items, n_items, 1, tw, b0, d3 ? b1 : out, c->stream);
+        if (r == cudaSuccess && d3) r = launch_sk_pass(sk, items, n_items, 2, tw, b1, out, c->stream);
+        c->launches += d3 ? 3 : 2;
+        return r;
+    };
+    double* fin = d3 ? b0 : b1;
+    e = transform(c->at<double>(P.d), c->at<double>(P.dbar), fin);
+    if (e != cudaSuccess) return e;
+    c->launches += 1;
+    e = launch_sk_accum(sk, items, n_items, fin, c->at<double>(P.sk_acc), c->stream);
+    if (e != cudaSuccess || !P.jk) return e;
     const int dims = d3 ? 3 : 2;
-    if (c->coupling == LB_GUO) {
-        e = launch_jk_guo_force(d3 ? 1 : 0, sys, items, n_items, c->at<double>(P.d), c->at<double>(P.jk_lap), j, ns,
-                                c->stream);
-        if (e != cudaSuccess) return e;
-        c->launches += 2;
-    }
+    double* F = c->at<double>(P.jk_F);
     for (int a = 0; a < dims; ++a) {
-        double* Fa = F + 2 * ns * a;
-        if (P.sk_fft) {
-            const int4* fi = c->at<int4>(P.fft_items);
-            e = launch_sk_fft(sys, sk, fi, P.n_fft_items, 0, j + ns * a, nullptr, nullptr, tw, b0, P.fft_max_elems,
-                              c->stream);
-            if (e != cudaSuccess) return e;
-            e = launch_sk_fft(sys, sk, fi, P.n_fft_items, 1, nullptr, nullptr, b0, tw, d3 ? b1 : Fa,
-                              P.fft_max_elems, c->stream);
-            if (e != cudaSuccess) return e;
-            c->launches += 2;
-            if (d3) {
-                e = launch_sk_fft(sys, sk, fi, P.n_fft_items, 2, nullptr, nullptr, b1, tw, Fa, P.fft_max_elems,
-                                  c->stream);
-                if (e != cudaSuccess) return e;
-                c->launches += 1;
-            }
-            continue;
-        }
-        e = launch_sk_x(sys, sk, items, n_items, j + ns * a, nullptr, tw, b0, c->stream);
+        e = transform(c->at<double>(P.jk_j) + ns * a, nullptr, F + 2 * ns * a);
         if (e != cudaSuccess) return e;
-        e = launch_sk_pass(sk, items, n_items, 1, tw, b0, d3 ? b1 : Fa, c->stream);
-        if (e != cudaSuccess) return e;
-        c->launches += 2;
-        if (d3) {
-            e = launch_sk_pass(sk, items, n_items, 2, tw, b1, Fa, c->stream);
-            if (e != cudaSuccess) return e;
-            c->launches += 1;
-        }
     }
     c->launches += 1;
     return launch_jk_accum(sk, items, n_items, dims, F, F + 2 * ns, d3 ? F + 4 * ns : nullptr,
@@ -781,46 +794,32 @@ cudaError_t sample_sk(lb_ctx* c, int buf, bool have_d) {
         e = sample_obs(c, buf, false, false, true);
         if (e != cudaSuccess) return e;
     }
-    const SysDev* sys = c->at<SysDev>(P.sys);
-    const SkSys* sk = c->at<SkSys>(P.sk_sys);
-    const int4* items = c->at<int4>(P.site_items);
-    double* b0 = c->at<double>(P.sk_b0);
-    double* b1 = c->at<double>(P.sk_b1);
-    const double* tw = c->at<double>(P.sk_tw);
-    const double* fin = b1;
-    if (P.sk_fft) {
-        const int4* fi = c->at<int4>(P.fft_items);
-        e = launch_sk_fft(sys, sk, fi, P.n_fft_items, 0, c->at<double>(P.d), c->at<double>(P.dbar), nullptr, tw, b0,
-                          P.fft_max_elems, c->stream);
-        if (e != cudaSuccess) return e;
-        e = launch_sk_fft(sys, sk, fi, P.n_fft_items, 1, nullptr, nullptr, b0, tw, b1, P.fft_max_elems, c->stream);
-        if (e != cudaSuccess) return e;
-        c->launches += 2;
-        if (c->lattice == LB_D3Q19) {
-            e = launch_sk_fft(sys, sk, fi, P.n_fft_items, 2, nullptr, nullptr, b1, tw, b0, P.fft_max_elems,
-                              c->stream);
-            if (e != cudaSuccess) return e;
-            fin = b0;
-            c->launches += 1;
-        }
-    } else {
-        e = launch_sk_x(sys, sk, items, P.n_site_items, c->at<double>(P.d), c->at<double>(P.dbar), tw, b0,
-                        c->stream);
-        if (e != cudaSuccess) return e;
-        e = launch_sk_pass(sk, items, P.n_site_items, 1, tw, b0, b1, c->stream);
-        if (e != cudaSuccess) return e;
-        c->launches += 2;
-        if (c->lattice == LB_D3Q19) {
-            e = launch_sk_pass(sk, items, P.n_site_items, 2, tw, b1, b0, c->stream);
-            if (e != cudaSuccess) return e;
-            fin = b0;
-            c->launches += 1;
-        }
-    }
-    c->launches += 1;
-    e = launch_sk_accum(sk, items, P.n_site_items, fin, c->at<double>(P.sk_acc), c->stream);
-    if (e != cudaSuccess || !P.jk) return e;
-    return sample_jk(c);
+    e = add_half_force(c);
+    if (e != cudaSuccess) return e;
+    if (!P.sk_fft) return sample_sk_direct(c);
+    FftLaunch a;
+    a.sys = c->at<SysDev>(P.sys);
+    a.sk = c->at<SkSys>(P.sk_sys);
+    a.items = c->at<int4>(P.fft_items);
+    a.n_x = P.n_fft_x;
+    a.n_y = P.n_fft_y;
+    a.n_last = P.n_fft_last;
+    a.max_x = P.fft_max_x;
+    a.max_y = P.fft_max_y;
+    a.max_last = P.fft_max_last;
+    a.dims = c->lattice == LB_D3Q19 ? 3 : 2;
+    a.nf = P.n_fields;
+    a.d = c->at<double>(P.d);
+    a.dbar = c->at<double>(P.dbar);
+    a.j = c->at<double>(P.jk_j);
+    a.tw = c->at<double>(P.sk_tw);
+    a.F = c->at<double>(P.sk_b0);
+    a.fstride = P.half_total;
+    a.n_sites = P.n_sites;
+    a.acc = c->at<double>(P.sk_acc);
+    a.jacc = c->at<double>(P.jk_acc);
+    c->launches += a.dims;
+    return launch_sk_fft(a, c->stream);
 }
 
 // Launch `n` steps starting at host step c->step (device counter must equal it).
@@ -1037,9 +1036,10 @@ lb_status lb_create(const lb_system_desc* systems, int n_systems, const lb_run_o
                                    c->stream) == cudaSuccess;
         ok = ok && launch_sk_twiddles(c->at<double>(P.sk_tw), dmeta, dmeta + P.tw_sides.size(),
                                       int(P.tw_sides.size()), P.tw_max, c->stream) == cudaSuccess;
-        if (P.n_fft_items)
-            ok = ok && cudaMemcpyAsync(c->ws + P.fft_items, P.fft_items_h.data(), sizeof(int4) * P.n_fft_items,
-                                       cudaMemcpyHostToDevice, c->stream) == cudaSuccess;
+        if (!P.fft_items_h.empty())
+            ok = ok && cudaMemcpyAsync(c->ws + P.fft_items, P.fft_items_h.data(),
+                                       sizeof(int4) * P.fft_items_h.size(), cudaMemcpyHostToDevice,
+                                       c->stream) == cudaSuccess;
     }
     ok = ok && cudaMemsetAsync(c->ws + P.step, 0, sizeof(int64_t), c->stream) == cudaSuccess;
     ok = ok && reset_accumulators(c) == LB_OK;
@@ -1416,17 +1416,17 @@ lb_status lb_structure_factor(lb_ctx* c, int sys, double* h_sum, int64_t* h_coun
     const Plan& P = c->P;
     if (!P.sk) return LB_ERR_UNSUPPORTED;
     if (nbins > P.sk_max_bins) return LB_ERR_ARG;
-    double* bins = c->at<double>(P.sk_bins);
-    LB_CHECK(launch_sk_bin(c->at<SkSys>(P.sk_sys), sys, c->at<double>(P.sk_acc), nbins, bins, bins + P.sk_max_bins,
-                           c->stream));
-    std::vector<double> hb(2 * size_t(P.sk_max_bins));
-    if (nbins > 0)
-        LB_CHECK(cudaMemcpyAsync(hb.data(), bins, sizeof(double) * 2 * P.sk_max_bins, cudaMemcpyDeviceToHost,
-                                 c->stream));
+    double* bins = c->at<double>(P.sk_bins);       // sums, then counts
+    std::vector<double> hb(2 * size_t(nbins));
+    if (nbins > 0) {
+        LB_CHECK(launch_sk_bin(c->at<SkSys>(P.sk_sys), sys, c->at<double>(P.sk_acc), 0, 1, nbins, bins, bins + nbins,
+                               c->stream));
+        LB_CHECK(cudaMemcpyAsync(hb.data(), bins, sizeof(double) * hb.size(), cudaMemcpyDeviceToHost, c->stream));
+    }
     lb_status s = sync_and_check(c);
     for (int j = 0; j < nbins; ++j) {
         h_sum[j] = hb[j];
-        h_count[j] = int64_t(hb[P.sk_max_bins + j]);
+        h_count[j] = int64_t(hb[nbins + j]);
     }
     if (n_samples) *n_samples = c->step / c->opts.sk_every;
     return s;
@@ -1437,20 +1437,18 @@ lb_status lb_momentum_spectra(lb_ctx* c, int sys, double* h_sum, int64_t* h_coun
     const Plan& P = c->P;
     if (!P.jk) return LB_ERR_UNSUPPORTED;
     if (nbins > P.sk_max_bins) return LB_ERR_ARG;
-    double* bins = c->at<double>(P.sk_bins);
-    std::vector<double> hb(2 * size_t(P.sk_max_bins));
-    for (int comp = 0; comp < 3 && nbins > 0; ++comp) {
-        LB_CHECK(launch_sk_bin(c->at<SkSys>(P.sk_sys), sys, c->at<double>(P.jk_acc) + int64_t(comp) * P.n_sites,
-                               nbins, bins, bins + P.sk_max_bins, c->stream));
-        LB_CHECK(cudaMemcpyAsync(hb.data(), bins, sizeof(double) * 2 * P.sk_max_bins, cudaMemcpyDeviceToHost,
-                                 c->stream));
-        LB_CHECK(cudaStreamSynchronize(c->stream));
-        for (int j = 0; j < nbins; ++j) {
-            h_sum[int64_t(comp) * nbins + j] = hb[j];
-            h_count[j] = int64_t(hb[P.sk_max_bins + j]);
-        }
+    double* bins = c->at<double>(P.sk_bins);       // sums of the three spectra, then counts
+    std::vector<double> hb(6 * size_t(nbins));
+    if (nbins > 0) {
+        LB_CHECK(launch_sk_bin(c->at<SkSys>(P.sk_sys), sys, c->at<double>(P.jk_acc), P.n_sites, 3, nbins, bins,
+                               bins + 3 * nbins, c->stream));
+        LB_CHECK(cudaMemcpyAsync(hb.data(), bins, sizeof(double) * hb.size(), cudaMemcpyDeviceToHost, c->stream));
     }
     lb_status st = sync_and_check(c);
+    for (int j = 0; j < nbins; ++j) {
+        for (int comp = 0; comp < 3; ++comp) h_sum[int64_t(comp) * nbins + j] = hb[size_t(comp) * nbins + j];
+        h_count[j] = int64_t(hb[size_t(3) * nbins + j]);
+    }
     if (n_samples) *n_samples = c->step / c->opts.sk_every;
     return st;
 }

@@ -10,32 +10,38 @@
 namespace lbf {
 
 // Work item of a site pass: (system, first site, end site, unused).
-// Deterministic sum of K doubles over the CTA; result valid in thread 0.
+// Deterministic sum of K doubles over the CTA; result valid in thread 0, and
+// (after its last barrier) in res.  A warp instruction occupies the FP64 unit
+// for 16 cycles whatever its mask, so the sum is packed: warp k adds the warps'
+// values lane by lane and reduces the 32 sums by shuffles, 12 additions per
+// value instead of 5 per value and warp.  Only threads below `active` (a
+// multiple of 32 or the CTA size) bring values.
 template <int K, int NT>
-__device__ __forceinline__ void block_sum(double (&v)[K], double* sh /* >= K * NT / 32 */) {
+struct BlockSum {
     static_assert(NT % 32 == 0 && NT <= 1024, "whole warps");
+    double v[K][NT];
+    double res[K];
+};
+template <int K, int NT>
+__device__ __forceinline__ void block_sum(double (&v)[K], BlockSum<K, NT>& sh, int active = NT) {
     constexpr int NW = NT / 32;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    // within each warp: shuffle-down tree (fixed order, so the sum is reproducible)
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (active + 31) >> 5;
+    if (w < nw) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-    }
-    if (lane == 0) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) sh[k * NW + w] = v[k];
+        for (int k = 0; k < K; ++k) sh.v[k][threadIdx.x] = v[k];
     }
     __syncthreads();
-    // across warps: warp 0 reduces the NW partial sums the same way
-    if (w == 0) {
+    for (int k = w; k < K; k += NW) {
+        double s = sh.v[k][lane];
+        for (int u = 1; u < nw; ++u) s += sh.v[k][32 * u + lane];
 #pragma unroll
-        for (int k = 0; k < K; ++k) v[k] = lane < NW ? sh[k * NW + lane] : 0.0;
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (lane == 0) sh.res[k] = s;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-            for (int k = 0; k < K; ++k) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-        }
+        for (int k = 0; k < K; ++k) v[k] = sh.res[k];
     }
 }
 
@@ -198,7 +204,7 @@ __global__ void __launch_bounds__(AUX_THREADS)
     obs_site_kernel(const SysDev* __restrict__ sysv, const int4* __restrict__ items, const Real* __restrict__ fbuf,
                     double* __restrict__ d, double* __restrict__ partial, double* __restrict__ jout,
                     int64_t jstride) {
-    __shared__ double sh[4 * AUX_THREADS / 32];
+    __shared__ BlockSum<4, AUX_THREADS> sh;
     const int4 it = items[blockIdx.x];
     const SysDev& S = sysv[it.x];
     const int nx = S.nx, ny = S.ny, nz = S.nz;
@@ -233,7 +239,7 @@ __global__ void __launch_bounds__(AUX_THREADS)
         acc[2] += m[1].value();
         acc[3] += m[2].value();
     }
-    block_sum<4, AUX_THREADS>(acc, sh);
+    block_sum(acc, sh);
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) partial[int64_t(blockIdx.x) * 4 + k] = acc[k];

@@ -143,7 +143,10 @@ constexpr int TOP_THREADS = 512;        // pyr_top_kernel: one CTA per system
 // a thread (a thread's sites are a serial chain of row loads), those of more
 // than kWarpSites a CTA, in ranges of kPartSites sites (16 per thread).
 constexpr int kThreadSites = 32, kWarpSites = 1024, kPartSites = 4096;
-constexpr int kTopBlocks = 4096;        // levels of at most this many blocks go to the top kernel (8 per thread)
+// Levels of at most this many blocks go to the top kernel.  Its one CTA per
+// system has one SM's FP64 unit (two operations per clock): 4,096 blocks cost
+// it 30 us, 512 blocks 4 us, about a launch.
+constexpr int kTopBlocks = 512;
 constexpr int REC = 6;      // per record: sum m, m^2, |m|, m^4, e, e^2
 
 }  // namespace lbf
@@ -155,6 +158,7 @@ struct SkSys {             // per system: sides, twiddle-table offsets, site off
     int32_t nx, ny, nz;
     int32_t tw_x, tw_y, tw_z;   // offsets of W_n^j = exp(-2 pi i j / n) tables (complex)
     int64_t site_offset;
+    int64_t half_offset;        // first value of the system's half spectrum (kx <= nx/2)
     double inv_n;               // 1 / sites
 };
 
@@ -165,14 +169,28 @@ cudaError_t launch_sk_x(const SysDev* sys, const SkSys* sk, const int4* items, i
                         const double* dbar, const double* tw, double* out, cudaStream_t st);
 cudaError_t launch_sk_pass(const SkSys* sk, const int4* items, int n_items, int axis, const double* tw,
                            const double* in, double* out, cudaStream_t st);
-// Line FFTs along `axis` for systems with equal sides 2^a 3^b (see sk.cu):
-// items (system, first line, line count, 0) with line count * side <= max_elems
-// <= kSkFftMaxElems; in == nullptr: real input from d (and dbar) as launch_sk_x.
+// Line FFTs of every field of a sample and accumulation of its spectra, for
+// systems with sides up to kSkFftMaxElems (see sk.cu).  Work lists in `items`:
+// n_x items (system, first line, count, field) of the x pass, n_y of the y pass
+// (3-D only), n_last (system, first line, count, 0) of the last pass; max_* are
+// the largest line count x line length of an item, in complex values (of all
+// fields in the last pass).
 constexpr int kSkFftMaxElems = 2048;
-bool sk_fft_side(int n);   // n = 2^a 3^b and n <= kSkFftMaxElems
-cudaError_t launch_sk_fft(const SysDev* sys, const SkSys* sk, const int4* items, int n_items, int axis,
-                          const double* d, const double* dbar, const double* in, const double* tw, double* out,
-                          int max_elems, cudaStream_t st);
+constexpr int FFT_THREADS = 128;
+bool sk_fft_side(int n);
+struct FftLaunch {
+    const SysDev* sys;
+    const SkSys* sk;
+    const int4* items;
+    int n_x, n_y, n_last, max_x, max_y, max_last;
+    int dims, nf;               // fields: phi, then the momentum components (nf = 1: phi alone)
+    const double *d, *dbar, *j; // j_a at j + a n_sites
+    const double* tw;
+    double* F;                  // half spectra, field f at F + 2 f fstride
+    int64_t fstride, n_sites;
+    double *acc, *jacc;         // accumulated spectra (jacc: three, n_sites apart)
+};
+cudaError_t launch_sk_fft(const FftLaunch& a, cudaStream_t st);
 cudaError_t launch_sk_accum(const SkSys* sk, const int4* items, int n_items, const double* F, double* acc,
                             cudaStream_t st);
 // per-shell sums of the accumulated C(k) of one system (one CTA per shell)
@@ -183,7 +201,8 @@ cudaError_t launch_jk_accum(const SkSys* sk, const int4* items, int n_items, int
 // Guo variant: lap = Laplacian of d, then j_a += kappa rho d_a(lap) / 2 (j at jf + a * stride).
 cudaError_t launch_jk_guo_force(int lattice, const SysDev* sys, const int4* items, int n_items, const double* d,
                                 double* lap, double* jf, int64_t stride, cudaStream_t st);
-cudaError_t launch_sk_bin(const SkSys* sk, int sys, const double* acc, int nbins, double* sums, double* counts,
-                          cudaStream_t st);
+// Shell sums (and point counts) of nspec spectra of one system, `stride` apart: [spectrum][shell].
+cudaError_t launch_sk_bin(const SkSys* sk, int sys, const double* acc, int64_t stride, int nspec, int nbins,
+                          double* sums, double* counts, cudaStream_t st);
 
 }  // namespace lbf

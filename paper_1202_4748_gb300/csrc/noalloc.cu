@@ -50,7 +50,7 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratch
 // Sum of rho over each site item; partial[item * 4 + 0] = sum, the rest 0.
 __global__ void __launch_bounds__(AUX_THREADS)
     rho_partial_kernel(const int4* __restrict__ items, const double* __restrict__ rho, double* __restrict__ partial) {
-    __shared__ double sh[AUX_THREADS];
+    __shared__ BlockSum<1, AUX_THREADS> sh;
     const int4 it = items[blockIdx.x];
     double acc[1] = {0.0};
     for (int j = 0; j < SITES_PER_THREAD; ++j) {
@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(AUX_THREADS)
         if (site >= it.z) break;
         acc[0] += rho[site];
     }
-    block_sum<1, AUX_THREADS>(acc, sh);
+    block_sum(acc, sh);
     if (threadIdx.x == 0) {
         partial[int64_t(blockIdx.x) * 4 + 0] = acc[0];
         partial[int64_t(blockIdx.x) * 4 + 1] = 0.0;

@@ -32,7 +32,7 @@ namespace {
 __global__ void __launch_bounds__(AUX_THREADS)
     init_noise_kernel(const SysDev* __restrict__ sysv, const int4* __restrict__ items, double amp,
                       double* __restrict__ d, double* __restrict__ partial) {
-    __shared__ double sh[AUX_THREADS / 32];
+    __shared__ BlockSum<1, AUX_THREADS> sh;
     const int4 it = items[blockIdx.x];
     const SysDev& S = sysv[it.x];
     double acc[1] = {0.0};
@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(AUX_THREADS)
         d[S.site_offset + site] = v;
         acc[0] += v;
     }
-    block_sum<1, AUX_THREADS>(acc, sh);
+    block_sum(acc, sh);
     if (threadIdx.x == 0) partial[int64_t(blockIdx.x) * 4] = acc[0];
 }
 
@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(AUX_THREADS)
     reduce_globals_kernel(const SysDev* __restrict__ sysv, const SysSpan* __restrict__ spans,
                           const double* __restrict__ partial, double* __restrict__ dbar, double* __restrict__ glob,
                           int set_mass0, int count_sample) {
-    __shared__ double sh[4 * AUX_THREADS / 32];
+    __shared__ BlockSum<4, AUX_THREADS> sh;
     const int s = blockIdx.x;
     const SysSpan sp = spans[s];
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(AUX_THREADS)
 #pragma unroll
         for (int k = 0; k < 4; ++k) acc[k] += partial[int64_t(sp.first + it) * 4 + k];
     }
-    block_sum<4, AUX_THREADS>(acc, sh);
+    block_sum(acc, sh);
     if (threadIdx.x != 0) return;
     const SysDev& S = sysv[s];
     const double n = double(S.n_sites);
@@ -99,6 +99,19 @@ __device__ __forceinline__ void add_terms(double (&t)[REC], double s, double e, 
     t[3] += m2 * m2;
     t[4] += E;
     t[5] += E * E;
+}
+
+// The same for single sites (V = 1: E = m^2 / 2, so its sums are halves and
+// quarters of those of m^2 and m^4, exactly): t = sum m, m^2, |m|, m^4.
+__device__ __forceinline__ void add_site_terms(double (&t)[REC], double m, double m2) {
+    t[0] += m;
+    t[1] += m2;
+    t[2] += fabs(m);
+    t[3] += m2 * m2;
+}
+__device__ __forceinline__ void finish_site_terms(double (&t)[REC]) {
+    t[4] = 0.5 * t[1];
+    t[5] = 0.25 * t[3];
 }
 
 // Histogram bin of a block value m: 1 + floor(t), t = (m - lo) * inv_w, with
@@ -137,7 +150,7 @@ __global__ void __launch_bounds__(OBS_THREADS)
                       const ObsItem* __restrict__ items, const double* __restrict__ d,
                       const double* __restrict__ dbar, double* __restrict__ Sg, double* __restrict__ Eg,
                       double* __restrict__ rec, const HistDev H) {
-    __shared__ double sh[REC * OBS_THREADS / 32];
+    __shared__ BlockSum<REC, OBS_THREADS> sh;
     extern __shared__ unsigned shist[];          // [block level | single-site level], nbins + 2 each
     const ObsItem it = items[blockIdx.x];
     const LevelDev lv = lvv[it.level];
@@ -172,22 +185,25 @@ __global__ void __launch_bounds__(OBS_THREADS)
                         const double phi = (ds[row + x] - db) * inv_rbar;
                         s += phi;
                         e += phi * phi;
-                        if (it.unit_level >= 0) add_terms(tu, phi, phi * phi, 1.0);
+                        if (it.unit_level >= 0) add_site_terms(tu, phi, phi * phi);
                         if (hist_u) atomicAdd(shist + nh + hist_bin(phi, H), 1u);
                     }
                 }
         }
         Sg[lv.off + b] = s;
         Eg[lv.off + b] = e;
-        add_terms(tb, s, e, inv_v);
+        if (sites) add_site_terms(tb, s, e);
+        else add_terms(tb, s, e, inv_v);
         if (hist) atomicAdd(shist + hist_bin(s * inv_v, H), 1u);
     }
-    block_sum<REC, OBS_THREADS>(tb, sh);
+    if (sites) finish_site_terms(tb);
+    finish_site_terms(tu);
+    block_sum(tb, sh);
     if (threadIdx.x == 0)
         for (int k = 0; k < REC; ++k) rec[int64_t(it.rec) * REC + k] = tb[k];
     if (it.unit_level >= 0) {
         __syncthreads();
-        block_sum<REC, OBS_THREADS>(tu, sh);
+        block_sum(tu, sh);
         if (threadIdx.x == 0)
             for (int k = 0; k < REC; ++k) rec[int64_t(it.rec2) * REC + k] = tu[k];
     }
@@ -209,7 +225,8 @@ __global__ void __launch_bounds__(OBS_THREADS)
                     double* __restrict__ Sg, double* __restrict__ Eg, double2* __restrict__ parts,
                     double* __restrict__ rec, const HistDev H) {
     constexpr int NW = OBS_THREADS / 32;
-    __shared__ double sh[REC * NW];
+    __shared__ BlockSum<REC, OBS_THREADS> sh;
+    auto& sh2 = reinterpret_cast<BlockSum<2, OBS_THREADS>&>(sh);   // used before sh, a barrier apart
     extern __shared__ unsigned shist[];          // [block level | single-site level], nbins + 2 each
     const ObsPart it = items[blockIdx.x];
     const LevelDev lv = lvv[it.level];
@@ -246,7 +263,7 @@ __global__ void __launch_bounds__(OBS_THREADS)
             const double phi = (corner[x + nx * (y + int64_t(ny) * z)] - db) * inv_rbar;
             v[0] += phi;
             v[1] += phi * phi;
-            add_terms(tu, phi, phi * phi, 1.0);
+            add_site_terms(tu, phi, phi * phi);
             if (hist) atomicAdd(shist + nh + hist_bin(phi, H), 1u);
         }
         if (by_warp) {
@@ -257,7 +274,7 @@ __global__ void __launch_bounds__(OBS_THREADS)
             }
             if (lane == 0) block_done(b, v[0], v[1]);
         } else {
-            block_sum<2, OBS_THREADS>(v, sh);
+            block_sum(v, sh2);
             if (threadIdx.x == 0) {
                 if (it.part < 0) block_done(b, v[0], v[1]);
                 else parts[it.part] = make_double2(v[0], v[1]);
@@ -265,13 +282,14 @@ __global__ void __launch_bounds__(OBS_THREADS)
             __syncthreads();
         }
     }
+    finish_site_terms(tu);
     if (it.part < 0) {
-        block_sum<REC, OBS_THREADS>(tb, sh);
+        block_sum(tb, sh);
         if (threadIdx.x == 0)
             for (int k = 0; k < REC; ++k) rec[int64_t(it.rec) * REC + k] = tb[k];
         __syncthreads();
     }
-    block_sum<REC, OBS_THREADS>(tu, sh);
+    block_sum(tu, sh);
     if (threadIdx.x == 0)
         for (int k = 0; k < REC; ++k) rec[int64_t(it.rec2) * REC + k] = tu[k];
     if (hist) {
@@ -288,7 +306,7 @@ __global__ void __launch_bounds__(OBS_THREADS)
                       const double2* __restrict__ parts, double* __restrict__ Sg, double* __restrict__ Eg,
                       double* __restrict__ rec, const HistDev H) {
     constexpr int NW = OBS_THREADS / 32;
-    __shared__ double sh[REC * NW];
+    __shared__ BlockSum<REC, OBS_THREADS> sh;
     const ObsBlocks it = items[blockIdx.x];
     const LevelDev lv = lvv[it.level];
     const double inv_v = 1.0 / (double(lv.bx) * lv.by * lv.bz);
@@ -315,7 +333,7 @@ __global__ void __launch_bounds__(OBS_THREADS)
                 atomicAdd(H.counts + int64_t(it.level) * (H.nbins + 2) + hist_bin(s * inv_v, H), 1ull);
         }
     }
-    block_sum<REC, OBS_THREADS>(tb, sh);
+    block_sum(tb, sh);
     if (threadIdx.x == 0)
         for (int k = 0; k < REC; ++k) rec[int64_t(it.rec) * REC + k] = tb[k];
 }
@@ -343,7 +361,7 @@ __device__ __forceinline__ void children_sum(const LevelDev& lv, const LevelDev&
 __global__ void __launch_bounds__(OBS_THREADS)
     pyr_up_kernel(const LevelDev* __restrict__ lvv, const ObsItem* __restrict__ items, int dims3,
                   double* __restrict__ Sg, double* __restrict__ Eg, double* __restrict__ rec, const HistDev H) {
-    __shared__ double sh[REC * OBS_THREADS / 32];
+    __shared__ BlockSum<REC, OBS_THREADS> sh;
     extern __shared__ unsigned shist[];
     const ObsItem it = items[blockIdx.x];
     const LevelDev lv = lvv[it.level];
@@ -364,7 +382,7 @@ __global__ void __launch_bounds__(OBS_THREADS)
         add_terms(tb, s, e, inv_v);
         if (hist) atomicAdd(shist + hist_bin(s * inv_v, H), 1u);
     }
-    block_sum<REC, OBS_THREADS>(tb, sh);
+    block_sum(tb, sh);
     if (threadIdx.x == 0)
         for (int k = 0; k < REC; ++k) rec[int64_t(it.rec) * REC + k] = tb[k];
     if (hist) {
@@ -410,7 +428,7 @@ __global__ void __launch_bounds__(TOP_THREADS)
                    double* Eg, const double* __restrict__ rec, double* __restrict__ acc, int* status,
                    const HistDev H) {
     constexpr int NW = TOP_THREADS / 32;
-    __shared__ double sh[REC * NW];
+    __shared__ BlockSum<REC, TOP_THREADS> sh;
     extern __shared__ unsigned shist[];
     const ObsTop T = tops[blockIdx.x];
     const int nh = H.nbins + 2;
@@ -434,7 +452,7 @@ __global__ void __launch_bounds__(TOP_THREADS)
             add_terms(tb, s, e, inv_v);
             if (hist) atomicAdd(shist + hist_bin(s * inv_v, H), 1u);
         }
-        block_sum<REC, TOP_THREADS>(tb, sh);      // its barrier also orders this level's block sums
+        block_sum(tb, sh, int(min(int64_t(TOP_THREADS), lv.nblocks)));      // its barrier also orders this level's block sums
         if (threadIdx.x == 0) accumulate_level(acc + int64_t(T.lv_first + l) * 7, double(lv.nblocks), tb, status);
         if (hist) hist_flush(shist, nh, H.counts + int64_t(T.lv_first + l) * nh);
         __syncthreads();

@@ -31,7 +31,7 @@ template <class L>
 __global__ void __launch_bounds__(AUX_THREADS)
     pt_prop_kernel(const int4* __restrict__ items, SkSys K, double m, double kappa, double* __restrict__ G,
                    double* __restrict__ partial) {
-    __shared__ double sh[2 * AUX_THREADS];
+    __shared__ BlockSum<2, AUX_THREADS> sh;
     const int4 it = items[blockIdx.x];
     double acc[2] = {0.0, 0.0};
     for (int j = 0; j < SITES_PER_THREAD; ++j) {
@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(AUX_THREADS)
         acc[0] += g;
         acc[1] += g * g;
     }
-    block_sum<2, AUX_THREADS>(acc, sh);
+    block_sum(acc, sh);
     if (threadIdx.x == 0) {
         partial[2 * blockIdx.x] = acc[0];
         partial[2 * blockIdx.x + 1] = acc[1];
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(AUX_THREADS)
 __global__ void __launch_bounds__(AUX_THREADS)
     pt_cube_kernel(const int4* __restrict__ items, double inv_n, const double* __restrict__ F,
                    double* __restrict__ partial) {
-    __shared__ double sh[AUX_THREADS];
+    __shared__ BlockSum<1, AUX_THREADS> sh;
     const int4 it = items[blockIdx.x];
     double acc[1] = {0.0};
     for (int j = 0; j < SITES_PER_THREAD; ++j) {
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(AUX_THREADS)
         const double g = F[2 * int64_t(e)] * inv_n;
         acc[0] += g * g * g;
     }
-    block_sum<1, AUX_THREADS>(acc, sh);
+    block_sum(acc, sh);
     if (threadIdx.x == 0) partial[blockIdx.x] = acc[0];
 }
 

@@ -1,11 +1,19 @@
 // Structure factor C(k) = N^-1 |sum_r phi(r) exp(-i k.r)|^2 (Eq. 80), accumulated
 // in FP64 over samples for every k of every system.  The discrete Fourier
 // transform is taken one axis at a time (x: real -> complex, then y, z) with
-// per-side twiddle tables W_n^j = exp(-2 pi i j / n).  Sides of the form
-// 2^a 3^b (every workload's) are transformed by a mixed-radix (4, 2, 3)
-// Stockham FFT, one CTA per group of lines in shared memory; other sides sum
-// each output element's line directly in a fixed order.  Shell binning
-// (j(j-1) < |n|^2 <= j(j+1)) happens only when the accumulated spectrum is read.
+// per-side twiddle tables W_n^j = exp(-2 pi i j / n).  Sides up to
+// kSkFftMaxElems are transformed by a mixed-radix Stockham FFT, one CTA per
+// group of lines in shared memory; longer sides sum each output element's line
+// directly in a fixed order.  Shell binning (j(j-1) < |n|^2 <= j(j+1)) happens
+// only when the accumulated spectrum is read.
+//
+// GB300's FP64 units do two operations per clock and SM, so the transforms are
+// bound by their arithmetic, and what is left out counts: the fields are real,
+// so the x pass of an even side is a complex FFT of half the length, only the
+// kx <= S/2 half of the spectrum is carried through the other axes, and the
+// last pass adds both of a mode's squared moduli (k and -k) to the accumulated
+// spectra.  All fields of a sample (order parameter, momentum components) go
+// through each pass in one launch: 3 launches on D3Q19 instead of 15.
 #include "lattice_kernels.cuh"
 #include "lb_launch.h"
 
@@ -110,92 +118,71 @@ __device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_doub
 // -i a
 __device__ __forceinline__ double2 cmi(double2 a) { return make_double2(a.y, -a.x); }
 
-// Line FFT along `axis` (0 x, 1 y, 2 z) of systems with equal sides S = 2^a 3^b:
-// item = (system, first line, line count, unused); line l of a system is the
-// l-th line along the axis with the other two coordinates in [z][y][x] order
-// (x lines: l = y + S z; y lines: l = x + S z; z lines: l = x + S y).  REAL_IN:
-// the input is phi = (d - dbar)/(rho_c + dbar) (or d itself without dbar),
-// else the complex field `in`.  Stockham autosort: stage with radix R after
-// sub-transforms of length Ns takes, for butterfly j of a line, the R inputs
-// a[j + r S/R] times W^(k r S/(Ns R)), k = j mod Ns, and writes their R-point
-// DFT to b[(j / Ns) Ns R + k + s Ns]; after the last stage the line is in
-// natural order.  F(k) = sum_x a(x) exp(-2 pi i k x / S), as the direct sums.
-template <bool REAL_IN>
-__global__ void __launch_bounds__(AUX_THREADS)
-    sk_fft_kernel(const SysDev* __restrict__ sysv, const SkSys* __restrict__ skv, const int4* __restrict__ items,
-                  int axis, const double* __restrict__ d, const double* __restrict__ dbar,
-                  const double2* __restrict__ in, const double2* __restrict__ tw, double2* __restrict__ out) {
-    extern __shared__ double2 fft_buf[];
-    const int4 it = items[blockIdx.x];
-    const SkSys K = skv[it.x];
-    const int S = K.nx;
-    const int nl = it.z, line0 = it.y;
-    const int toff = axis == 0 ? K.tw_x : (axis == 1 ? K.tw_y : K.tw_z);
-    double2* A = fft_buf;
-    double2* B = fft_buf + nl * S;
-    auto elem = [&](int line, int t) -> int64_t {
-        if (axis == 0) return int64_t(line) * S + t;
-        const int u = line % S, v = line / S;
-        if (axis == 1) return u + int64_t(S) * (t + int64_t(S) * v);
-        return u + int64_t(S) * (v + int64_t(S) * t);
-    };
-    // element (line l, position t) <-> index: x lines contiguous per line, the
-    // other axes with consecutive lines (consecutive x) in consecutive threads
-    auto lt = [&](int idx, int& l, int& t) {
-        if (axis == 0) {
-            l = idx / S;
-            t = idx - l * S;
-        } else {
-            t = idx / nl;
-            l = idx - t * nl;
-        }
-    };
-    double db = 0.0, inv_rbar = 1.0;
-    if constexpr (REAL_IN) {
-        if (dbar) {
-            db = dbar[it.x];
-            inv_rbar = 1.0 / (sysv[it.x].rho_c + db);
-        }
-    }
-    for (int idx = threadIdx.x; idx < nl * S; idx += AUX_THREADS) {
-        int l, t;
-        lt(idx, l, t);
-        const int64_t g = K.site_offset + elem(line0 + l, t);
-        if constexpr (REAL_IN) A[l * S + t] = make_double2((d[g] - db) * inv_rbar, 0.0);
-        else A[l * S + t] = in[g];
-    }
-    __syncthreads();
+// Complex FFTs of nl lines of length n in shared memory (line l at A + l n),
+// with B as the other buffer; returns the one that holds the result.  tw is
+// the table of W_S^j, S = n * mul.  Stockham autosort: the stage with radix R
+// after sub-transforms of length Ns takes, for butterfly j of a line, the R
+// inputs a[j + r n/R] times W_n^(k r n/(Ns R)), k = j mod Ns, and writes their
+// R-point DFT to b[(j / Ns) Ns R + k + s Ns]; after the last stage the line is
+// in natural order.  Radices 4, 2 and 3, then the odd primes left, whose
+// outputs are summed one per thread.
+__device__ __forceinline__ double2* fft_lines(double2* A, double2* B, int nl, int n, int mul,
+                                              const double2* __restrict__ tw) {
     int Ns = 1;
-    for (int m = S; m > 1;) {
-        const int R = (m % 4 == 0) ? 4 : ((m % 2 == 0) ? 2 : 3);
+    for (int m = n; m > 1;) {
+        int R = (m % 4 == 0) ? 4 : ((m % 2 == 0) ? 2 : 3);
+        while (m % R) R += 2;
         m /= R;
-        const int nb = S / R, tstep = S / (Ns * R);
-        for (int b = threadIdx.x; b < nl * nb; b += AUX_THREADS) {
-            const int l = b / nb, j = b - l * nb, k = j % Ns;
-            const double2* src = A + l * S;
-            double2* dst = B + l * S + (j / Ns) * Ns * R + k;
-            double2 v[4];
-            v[0] = src[j];
-            for (int r = 1; r < R; ++r) v[r] = cmul(src[j + r * nb], tw[toff + k * r * tstep]);
-            if (R == 4) {
-                const double2 s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]);
-                const double2 s13 = cadd(v[1], v[3]), d13 = cmi(csub(v[1], v[3]));
-                dst[0] = cadd(s02, s13);
-                dst[Ns] = cadd(d02, d13);
-                dst[2 * Ns] = csub(s02, s13);
-                dst[3 * Ns] = csub(d02, d13);
-            } else if (R == 2) {
-                dst[0] = cadd(v[0], v[1]);
-                dst[Ns] = csub(v[0], v[1]);
-            } else {
-                // w = exp(-2 pi i / 3): X1,2 = v0 - (v1 + v2)/2 -+ i (sqrt(3)/2)(v1 - v2)
-                const double2 t1 = cadd(v[1], v[2]), t2 = csub(v[1], v[2]);
-                const double2 m0 = make_double2(v[0].x - 0.5 * t1.x, v[0].y - 0.5 * t1.y);
-                const double h = 0.86602540378443864676;
-                const double2 rt = make_double2(h * t2.y, -h * t2.x);      // -i (sqrt(3)/2) t2
-                dst[0] = cadd(v[0], t1);
-                dst[Ns] = cadd(m0, rt);
-                dst[2 * Ns] = csub(m0, rt);
+        const int nb = n / R, tstep = mul * (n / (Ns * R));
+        if (R > 4) {
+            const int S = n * mul, sstep = S / R;
+            for (int b = threadIdx.x; b < nl * n; b += blockDim.x) {
+                const int l = b / n, o = b - l * n, s = o / nb, j = o - s * nb, k = j % Ns;
+                const double2* src = A + l * n + j;
+                const int e = k * tstep + s * sstep;          // exponent per input, < 2 S
+                double2 v = src[0];
+                int idx = 0;
+                for (int r = 1; r < R; ++r) {
+                    idx += e;
+                    while (idx >= S) idx -= S;
+                    const double2 w = tw[idx], a = src[r * nb];
+                    v.x += a.x * w.x - a.y * w.y;
+                    v.y += a.x * w.y + a.y * w.x;
+                }
+                B[l * n + (j / Ns) * Ns * R + k + s * Ns] = v;
+            }
+        } else {
+            for (int b = threadIdx.x; b < nl * nb; b += blockDim.x) {
+                const int l = b / nb, j = b - l * nb, k = j % Ns;
+                const double2* src = A + l * n;
+                double2* dst = B + l * n + (j / Ns) * Ns * R + k;
+                double2 v[4];
+                v[0] = src[j];
+                if (Ns == 1) {
+                    for (int r = 1; r < R; ++r) v[r] = src[j + r * nb];
+                } else {
+                    for (int r = 1; r < R; ++r) v[r] = cmul(src[j + r * nb], tw[k * r * tstep]);
+                }
+                if (R == 4) {
+                    const double2 s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]);
+                    const double2 s13 = cadd(v[1], v[3]), d13 = cmi(csub(v[1], v[3]));
+                    dst[0] = cadd(s02, s13);
+                    dst[Ns] = cadd(d02, d13);
+                    dst[2 * Ns] = csub(s02, s13);
+                    dst[3 * Ns] = csub(d02, d13);
+                } else if (R == 2) {
+                    dst[0] = cadd(v[0], v[1]);
+                    dst[Ns] = csub(v[0], v[1]);
+                } else {
+                    // w = exp(-2 pi i / 3): X1,2 = v0 - (v1 + v2)/2 -+ i (sqrt(3)/2)(v1 - v2)
+                    const double2 t1 = cadd(v[1], v[2]), t2 = csub(v[1], v[2]);
+                    const double2 m0 = make_double2(v[0].x - 0.5 * t1.x, v[0].y - 0.5 * t1.y);
+                    const double h = 0.86602540378443864676;
+                    const double2 rt = make_double2(h * t2.y, -h * t2.x);      // -i (sqrt(3)/2) t2
+                    dst[0] = cadd(v[0], t1);
+                    dst[Ns] = cadd(m0, rt);
+                    dst[2 * Ns] = csub(m0, rt);
+                }
             }
         }
         __syncthreads();
@@ -204,14 +191,163 @@ __global__ void __launch_bounds__(AUX_THREADS)
         B = tmp;
         Ns *= R;
     }
-    for (int idx = threadIdx.x; idx < nl * S; idx += AUX_THREADS) {
+    return A;
+}
+
+// x pass: item = (system, first line, line count, field); line l of a system
+// is row l in [z][y] order.  Field 0 is phi = (d - dbar)/(rho_c + dbar), field
+// f > 0 the momentum component j_(f-1).  Writes the half spectrum kx = 0 .. S/2
+// of each line, rows of hx = S/2 + 1 values.  An even side S packs its samples
+// as z_j = a_2j + i a_(2j+1), j < S/2 = h: with Z the transform of z,
+// F(k) = E + W_S^k O, E = (Z_k + conj Z_(h-k))/2, O = -i (Z_k - conj Z_(h-k))/2.
+__global__ void __launch_bounds__(FFT_THREADS)
+    fft_x_kernel(const SysDev* __restrict__ sysv, const SkSys* __restrict__ skv, const int4* __restrict__ items,
+                 const double* __restrict__ d, const double* __restrict__ dbar, const double* __restrict__ jf,
+                 int64_t jstride, const double2* __restrict__ twv, double2* __restrict__ F, int64_t fstride) {
+    extern __shared__ double2 fft_buf[];
+    const int4 it = items[blockIdx.x];
+    const SkSys K = skv[it.x];
+    const int S = K.nx, hx = S / 2 + 1, nl = it.z;
+    const double2* tw = twv + K.tw_x;
+    const bool even = S % 2 == 0;
+    const int n = even ? S / 2 : S;
+    double db = 0.0, inv = 1.0;
+    const double* src = it.w == 0 ? d : jf + (it.w - 1) * jstride;
+    if (it.w == 0) {
+        db = dbar[it.x];
+        inv = 1.0 / (sysv[it.x].rho_c + db);
+    }
+    src += K.site_offset + int64_t(it.y) * S;
+    // the samples in order: interleaved they are the packed complex line
+    if (even) {
+        double* a = reinterpret_cast<double*>(fft_buf);
+        for (int i = threadIdx.x; i < nl * S; i += FFT_THREADS) a[i] = it.w == 0 ? (src[i] - db) * inv : src[i];
+    } else {
+        for (int i = threadIdx.x; i < nl * S; i += FFT_THREADS)
+            fft_buf[i] = make_double2(it.w == 0 ? (src[i] - db) * inv : src[i], 0.0);
+    }
+    __syncthreads();
+    const double2* Z = fft_lines(fft_buf, fft_buf + nl * n, nl, n, even ? 2 : 1, tw);
+    double2* out = F + it.w * fstride + K.half_offset + int64_t(it.y) * hx;
+    for (int i = threadIdx.x; i < nl * hx; i += FFT_THREADS) {
+        const int l = i / hx, k = i - l * hx;
+        const double2* z = Z + l * n;
+        if (even) {
+            const double2 p = z[k == n ? 0 : k], q = z[k == 0 ? 0 : n - k];
+            const double2 e = make_double2(0.5 * (p.x + q.x), 0.5 * (p.y - q.y));
+            const double2 o = make_double2(0.5 * (p.y + q.y), -0.5 * (p.x - q.x));
+            const double2 w = k == 0 ? make_double2(1.0, 0.0) : (k == n ? make_double2(-1.0, 0.0) : tw[k]);
+            out[i] = cadd(e, cmul(w, o));
+        } else {
+            out[i] = z[k];
+        }
+    }
+}
+
+// y pass of a 3-D system, in place on the half spectrum: item = (system, first
+// line, line count, field); line l is kx + hx z.
+__global__ void __launch_bounds__(FFT_THREADS)
+    fft_y_kernel(const SkSys* __restrict__ skv, const int4* __restrict__ items, const double2* __restrict__ twv,
+                 double2* __restrict__ F, int64_t fstride) {
+    extern __shared__ double2 fft_buf[];
+    const int4 it = items[blockIdx.x];
+    const SkSys K = skv[it.x];
+    const int S = K.ny, hx = K.nx / 2 + 1, nl = it.z;
+    double2* f = F + it.w * fstride + K.half_offset;
+    // consecutive lines are consecutive kx: a warp reads rows of lines
+    auto elem = [&](int i, int& l, int& t) -> int64_t {
+        t = i / nl;
+        l = i - t * nl;
+        const int g = it.y + l, z = g / hx, kx = g - z * hx;
+        return kx + int64_t(hx) * (t + int64_t(S) * z);
+    };
+    for (int i = threadIdx.x; i < nl * S; i += FFT_THREADS) {
         int l, t;
-        lt(idx, l, t);
-        out[K.site_offset + elem(line0 + l, t)] = A[l * S + t];
+        const int64_t e = elem(i, l, t);
+        fft_buf[l * S + t] = f[e];
+    }
+    __syncthreads();
+    const double2* Z = fft_lines(fft_buf, fft_buf + nl * S, nl, S, 1, twv + K.tw_y);
+    for (int i = threadIdx.x; i < nl * S; i += FFT_THREADS) {
+        int l, t;
+        const int64_t e = elem(i, l, t);
+        f[e] = Z[l * S + t];
     }
 }
 
 __device__ __forceinline__ int wrapk(int k, int n) { return 2 * k < n ? k : k - n; }
+
+// What the spectra of one mode add: |J_x|^2, |n . J|^2 / |n|^2 and the
+// transverse rest per component, all over N (0 for the projections at n = 0).
+struct ModeSpectra {
+    double x, lon, tra;
+};
+__device__ __forceinline__ ModeSpectra mode_spectra(double a, double b, double c, double2 X, double2 Y, double2 Z,
+                                                    int dims, double inv_n) {
+    ModeSpectra m{0.0, 0.0, 0.0};
+    const double jx2 = X.x * X.x + X.y * X.y;
+    m.x = jx2 * inv_n;
+    const double nn2 = a * a + b * b + c * c;
+    if (nn2 > 0.0) {
+        const double pr = a * X.x + b * Y.x + c * Z.x, pi = a * X.y + b * Y.y + c * Z.y;
+        const double p2 = (pr * pr + pi * pi) / nn2;
+        const double tot = jx2 + Y.x * Y.x + Y.y * Y.y + Z.x * Z.x + Z.y * Z.y;
+        m.lon = p2 * inv_n;
+        m.tra = (tot - p2) * (dims == 3 ? 0.5 * inv_n : inv_n);
+    }
+    return m;
+}
+
+// Last pass (y in 2-D, z in 3-D) and accumulation: item = (system, first line,
+// line count, -); line l is l = kx + hx ky (3-D) or kx.  All nf fields of a
+// line are in the CTA, so every mode's spectra are formed where its transforms
+// end: acc[k] += |phi(k)|^2 / N, and with momentum components (nf > 1)
+// jacc + c stride as ModeSpectra.  A mode with 0 < kx < S/2 stands for -k too:
+// its moduli are the same, and so are the projections unless a wrapped
+// component is -S/2, whose sign does not flip (n is formed again for it).
+__global__ void __launch_bounds__(FFT_THREADS)
+    fft_last_kernel(const SkSys* __restrict__ skv, const int4* __restrict__ items, int nf,
+                    const double2* __restrict__ twv, const double2* __restrict__ F, int64_t fstride,
+                    double* __restrict__ acc, double* __restrict__ jacc, int64_t jstride, int dims) {
+    extern __shared__ double2 fft_buf[];
+    const int4 it = items[blockIdx.x];
+    const SkSys K = skv[it.x];
+    const int S = K.nx, hx = S / 2 + 1, nl = it.z;
+    const int64_t tstride = dims == 3 ? int64_t(hx) * S : hx;     // along the transformed axis
+    const double2* f = F + K.half_offset + it.y;
+    for (int i = threadIdx.x; i < nf * nl * S; i += FFT_THREADS) {
+        const int fl = i / (nl * S), r = i - fl * (nl * S), t = r / nl, l = r - t * nl;
+        fft_buf[(fl * nl + l) * S + t] = f[fl * fstride + l + tstride * t];
+    }
+    __syncthreads();
+    const double2* Z = fft_lines(fft_buf, fft_buf + nf * nl * S, nf * nl, S, 1, twv + K.tw_y);
+    auto neg = [&](int k) { return k == 0 ? 0 : S - k; };
+    for (int i = threadIdx.x; i < nl * S; i += FFT_THREADS) {
+        const int t = i / nl, l = i - t * nl, g = it.y + l;
+        const int kx = g % hx, ky = dims == 3 ? g / hx : t, kz = dims == 3 ? t : 0;
+        const int64_t at = K.site_offset + kx + int64_t(S) * (ky + int64_t(S) * kz);
+        const bool both = kx > 0 && 2 * kx < S;
+        const int64_t at2 = K.site_offset + neg(kx) + int64_t(S) * (neg(ky) + int64_t(S) * neg(kz));
+        const double2 p = Z[l * S + t];
+        const double c = (p.x * p.x + p.y * p.y) * K.inv_n;
+        acc[at] += c;
+        if (both) acc[at2] += c;
+        if (nf == 1) continue;
+        const double2 X = Z[(nl + l) * S + t], Y = Z[(2 * nl + l) * S + t];
+        const double2 W = dims == 3 ? Z[(3 * nl + l) * S + t] : make_double2(0.0, 0.0);
+        ModeSpectra m = mode_spectra(wrapk(kx, S), wrapk(ky, S), dims == 3 ? wrapk(kz, S) : 0, X, Y, W, dims, K.inv_n);
+        jacc[at] += m.x;
+        jacc[jstride + at] += m.lon;
+        jacc[2 * jstride + at] += m.tra;
+        if (both) {
+            if (2 * ky == S || (dims == 3 && 2 * kz == S))
+                m = mode_spectra(-kx, wrapk(neg(ky), S), dims == 3 ? wrapk(neg(kz), S) : 0, X, Y, W, dims, K.inv_n);
+            jacc[at2] += m.x;
+            jacc[jstride + at2] += m.lon;
+            jacc[2 * jstride + at2] += m.tra;
+        }
+    }
+}
 
 // Momentum spectra of one sample (Eq. 69 diagnostics): from the transforms
 // J_a(k) (complex, one field per component) accumulate per k
@@ -230,21 +366,13 @@ __global__ void __launch_bounds__(AUX_THREADS)
         if (e >= it.z) break;
         const int64_t g = K.site_offset + e;
         const int kx = e % K.nx, ky = (e / K.nx) % K.ny, kz = e / (K.nx * K.ny);
-        const double a = wrapk(kx, K.nx), b = wrapk(ky, K.ny), c = dims == 3 ? wrapk(kz, K.nz) : 0;
-        const double xr = F0[2 * g], xi = F0[2 * g + 1];
-        const double yr = F1[2 * g], yi = F1[2 * g + 1];
-        const double zr = dims == 3 ? F2[2 * g] : 0.0, zi = dims == 3 ? F2[2 * g + 1] : 0.0;
-        const double jx2 = xr * xr + xi * xi;
-        acc[g] += jx2 * K.inv_n;
-        const double nn2 = a * a + b * b + c * c;
-        if (nn2 > 0.0) {
-            const double inv = 1.0 / sqrt(nn2);
-            const double pr = (a * xr + b * yr + c * zr) * inv, pi = (a * xi + b * yi + c * zi) * inv;
-            const double p2 = pr * pr + pi * pi;
-            const double tot = jx2 + yr * yr + yi * yi + zr * zr + zi * zi;
-            acc[stride + g] += p2 * K.inv_n;
-            acc[2 * stride + g] += (tot - p2) * K.inv_n / double(dims - 1);
-        }
+        const double2 X = make_double2(F0[2 * g], F0[2 * g + 1]), Y = make_double2(F1[2 * g], F1[2 * g + 1]);
+        const double2 Z = dims == 3 ? make_double2(F2[2 * g], F2[2 * g + 1]) : make_double2(0.0, 0.0);
+        const ModeSpectra m = mode_spectra(wrapk(kx, K.nx), wrapk(ky, K.ny), dims == 3 ? wrapk(kz, K.nz) : 0, X, Y, Z,
+                                           dims, K.inv_n);
+        acc[g] += m.x;
+        acc[stride + g] += m.lon;
+        acc[2 * stride + g] += m.tra;
     }
 }
 
@@ -306,28 +434,49 @@ __global__ void __launch_bounds__(AUX_THREADS)
     }
 }
 
+// Shell sums of one system's accumulated spectra: CTA (j - 1, c) adds the
+// points of shell j, j (j - 1) < |n|^2 <= j (j + 1), of spectrum c (at acc + c
+// stride) in a fixed order, one row (ky, kz) per thread at a time: the row's
+// points of the shell are the two runs kx = +-(a .. b).  (Every CTA tested
+// every k point before: 0.5 ms for 32 shells of 64^3.)
 __global__ void __launch_bounds__(AUX_THREADS)
-    sk_bin_kernel(const SkSys* __restrict__ skv, int sys, const double* __restrict__ acc, double* __restrict__ sums,
-                  double* __restrict__ counts) {
-    __shared__ double sh[2 * AUX_THREADS];
+    sk_bin_kernel(const SkSys* __restrict__ skv, int sys, const double* __restrict__ acc, int64_t stride,
+                  double* __restrict__ sums, double* __restrict__ counts) {
+    __shared__ BlockSum<2, AUX_THREADS> sh;
     const SkSys K = skv[sys];
-    const int bin = blockIdx.x + 1;                    // shells j = 1 .. nbins
-    const int64_t n = int64_t(K.nx) * K.ny * K.nz;
+    const int64_t j = blockIdx.x + 1, lo = j * (j - 1), hi = j * (j + 1);
+    const int S = K.nx;
+    const double* row0 = acc + blockIdx.y * stride + K.site_offset;
     double v[2] = {0.0, 0.0};
-    const int64_t lo = int64_t(bin) * (bin - 1), hi = int64_t(bin) * (bin + 1);
-    for (int64_t e = threadIdx.x; e < n; e += AUX_THREADS) {
-        const int kx = int(e % K.nx), ky = int((e / K.nx) % K.ny), kz = int(e / (int64_t(K.nx) * K.ny));
-        const int64_t a = wrapk(kx, K.nx), b = wrapk(ky, K.ny), c = wrapk(kz, K.nz);
-        const int64_t n2 = a * a + b * b + c * c;
-        if (n2 > lo && n2 <= hi) {
-            v[0] += acc[K.site_offset + e];
-            v[1] += 1.0;
+    for (int r = threadIdx.x; r < K.ny * K.nz; r += AUX_THREADS) {
+        const int64_t ny = wrapk(r % K.ny, K.ny), nz = wrapk(r / K.ny, K.nz), m = ny * ny + nz * nz;
+        if (m > hi) continue;
+        // smallest and largest x >= 0 with lo < x^2 + m <= hi
+        int b = int(sqrt(double(hi - m)));
+        while (int64_t(b) * b > hi - m) --b;
+        while (int64_t(b + 1) * (b + 1) <= hi - m) ++b;
+        int a = 0;
+        if (m <= lo) {
+            a = int(sqrt(double(lo - m)));
+            while (int64_t(a) * a > lo - m) --a;
+            while (int64_t(a) * a + m <= lo) ++a;
+        }
+        const double* row = row0 + int64_t(S) * r;
+        for (int x = a; x <= b && 2 * x <= S; ++x) {
+            if (2 * x < S) {                              // wrapped components -S/2 .. (S - 1)/2
+                v[0] += row[x];
+                v[1] += 1.0;
+            }
+            if (x > 0) {
+                v[0] += row[S - x];
+                v[1] += 1.0;
+            }
         }
     }
-    block_sum<2, AUX_THREADS>(v, sh);
+    block_sum(v, sh);
     if (threadIdx.x == 0) {
-        sums[blockIdx.x] = v[0];
-        counts[blockIdx.x] = v[1];
+        sums[blockIdx.y * gridDim.x + blockIdx.x] = v[0];
+        counts[blockIdx.y * gridDim.x + blockIdx.x] = v[1];
     }
 }
 
@@ -355,35 +504,36 @@ cudaError_t launch_sk_pass(const SkSys* sk, const int4* items, int n_items, int 
     return cudaGetLastError();
 }
 
-bool sk_fft_side(int n) {
-    if (n < 1 || n > kSkFftMaxElems) return false;
-    while (n % 2 == 0) n /= 2;
-    while (n % 3 == 0) n /= 3;
-    return n == 1;
-}
+bool sk_fft_side(int n) { return n >= 1 && n <= kSkFftMaxElems; }
 
-cudaError_t launch_sk_fft(const SysDev* sys, const SkSys* sk, const int4* items, int n_items, int axis,
-                          const double* d, const double* dbar, const double* in, const double* tw, double* out,
-                          int max_elems, cudaStream_t st) {
-    if (n_items == 0) return cudaSuccess;
-    const size_t dyn = size_t(2) * max_elems * sizeof(double2);
+cudaError_t launch_sk_fft(const FftLaunch& a, cudaStream_t st) {
+    // two buffers of kSkFftMaxElems values; the last pass holds every field of a
+    // line, three of kSkFftMaxElems in 2-D (192 KB), four of at most 483 in 3-D
+    constexpr int kMaxBytes = int(2 * kSkFftMaxElems * sizeof(double2));
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(sk_fft_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             int(2 * kSkFftMaxElems * sizeof(double2)));
+        cudaError_t e = cudaFuncSetAttribute(fft_x_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxBytes);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(sk_fft_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     int(2 * kSkFftMaxElems * sizeof(double2)));
+            e = cudaFuncSetAttribute(fft_y_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxBytes);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(fft_last_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * kMaxBytes);
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    const double2* tw2 = reinterpret_cast<const double2*>(tw);
-    double2* out2 = reinterpret_cast<double2*>(out);
-    if (in == nullptr)
-        sk_fft_kernel<true><<<n_items, AUX_THREADS, dyn, st>>>(sys, sk, items, axis, d, dbar, nullptr, tw2, out2);
-    else
-        sk_fft_kernel<false><<<n_items, AUX_THREADS, dyn, st>>>(sys, sk, items, axis, nullptr, nullptr,
-                                                                reinterpret_cast<const double2*>(in), tw2, out2);
+    const double2* tw = reinterpret_cast<const double2*>(a.tw);
+    double2* F = reinterpret_cast<double2*>(a.F);
+    // both line buffers of the largest item
+    const size_t line = 2 * sizeof(double2);
+    fft_x_kernel<<<a.n_x, FFT_THREADS, line * a.max_x, st>>>(a.sys, a.sk, a.items, a.d, a.dbar, a.j, a.n_sites, tw, F,
+                                                            a.fstride);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess && a.dims == 3) {
+        fft_y_kernel<<<a.n_y, FFT_THREADS, line * a.max_y, st>>>(a.sk, a.items + a.n_x, tw, F, a.fstride);
+        e = cudaGetLastError();
+    }
+    if (e != cudaSuccess) return e;
+    fft_last_kernel<<<a.n_last, FFT_THREADS, line * a.max_last, st>>>(a.sk, a.items + a.n_x + a.n_y, a.nf, tw, F,
+                                                                      a.fstride, a.acc, a.jacc, a.n_sites, a.dims);
     return cudaGetLastError();
 }
 
@@ -414,10 +564,10 @@ cudaError_t launch_jk_guo_force(int lattice, const SysDev* sys, const int4* item
     return cudaGetLastError();
 }
 
-cudaError_t launch_sk_bin(const SkSys* sk, int sys, const double* acc, int nbins, double* sums, double* counts,
-                          cudaStream_t st) {
+cudaError_t launch_sk_bin(const SkSys* sk, int sys, const double* acc, int64_t stride, int nspec, int nbins,
+                          double* sums, double* counts, cudaStream_t st) {
     if (nbins <= 0) return cudaSuccess;
-    sk_bin_kernel<<<nbins, AUX_THREADS, 0, st>>>(sk, sys, acc, sums, counts);
+    sk_bin_kernel<<<dim3(nbins, nspec), AUX_THREADS, 0, st>>>(sk, sys, acc, stride, sums, counts);
     return cudaGetLastError();
 }
 
