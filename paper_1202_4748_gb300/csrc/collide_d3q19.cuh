@@ -179,8 +179,7 @@ __device__ __forceinline__ void draw4(const NoiseKey& k, uint2 site, uint32_t d,
     n[3] = need3 ? vmul(rr1, make_float2(sfu_sin(t1.x), sfu_sin(t1.y))) : make_float2(0.0f, 0.0f);
 }
 
-// FP64: U = (x + 1/2) 2^-32 exactly, R = sqrt(-2 ln U), angle 2 pi U_b, with
-// the library's correctly rounded functions.
+// FP64: U = (x + 1/2) 2^-32 exactly, R = sqrt(-2 ln U), angle 2 pi U_b.
 __device__ __forceinline__ void draw4(const NoiseKey& k, uint32_t site, uint32_t d, double sc0, double sc1,
                                       double (&n)[4], bool need3) {
     const uint4 w = philox_draw(k, site, d);

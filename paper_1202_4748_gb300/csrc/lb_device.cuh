@@ -9,6 +9,8 @@
 #include <type_traits>
 #include <cuda_runtime.h>
 
+#include "normal64.cuh"
+
 namespace lbf {
 
 constexpr int LB_MAX_Q_DEV = 19;
@@ -220,13 +222,19 @@ __device__ __forceinline__ uint4 site_draw(const SysDev& s, uint32_t site, int64
 }
 
 // Uniform in (0,1): (x + 1/2) 2^-32, then Box-Muller (R = sqrt(-2 ln U_a),
-// angle 2 pi U_b).  Float and double versions.
+// angle 2 pi U_b).  Double: in 64-bit fixed point (normal64.cuh), the table in
+// the read-only cache.
+static __device__ __align__(16) const LogEntry kLogTable[64] = {LB_LOG_TABLE};
+struct LogTable {
+    __device__ __forceinline__ LogEntry operator()(int i) const {
+        const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(kLogTable) + i);
+        return LogEntry{uint32_t(v.x), v.y};
+    }
+};
 __device__ __forceinline__ void box_muller(uint32_t wa, uint32_t wb, double& n0, double& n1) {
-    const double ua = (double(wa) + 0.5) * 2.3283064365386962890625e-10;
-    const double ub = (double(wb) + 0.5) * 2.3283064365386962890625e-10;
-    const double r = sqrt(-2.0 * log(ua));
     double s, c;
-    sincospi(2.0 * ub, &s, &c);
+    const double r = n64_radius(wa, LogTable());
+    n64_angle(wb, c, s);
     n0 = r * c;
     n1 = r * s;
 }
