@@ -380,10 +380,11 @@ lb_status lb_load(lb_ctx* ctx, const char* path);
  * sites (x sites per tile) of y rows, densities in registers and warp
  * shuffles, 3 = (paired D3Q19 kernel) producers stage their 16-byte quads of
  * pulled populations in shared memory with cp.async instead of holding them
- * in registers, 4 = (D3Q19, FP32 with every mode at tau = 1, else the
- * scheme-0 kernel of the same tile) split step: one kernel forms the density
- * and momentum of every site, a second collides tile columns with two sites
- * stacked in z per thread; sites per thread: 1, or 2 = two x-adjacent sites per thread
+ * in registers, 4 = (D3Q19) split step: one kernel forms the density and
+ * momentum of every site, a second collides tile columns with two sites stacked
+ * in z per thread (on D3Q19, FP64 runs and runs with a relaxation time other
+ * than 1 take the split step whatever the row, in 16 x 8 columns with the row's
+ * z-chunk); sites per thread: 1, or 2 = two x-adjacent sites per thread
  * with paired FP32 arithmetic (D3Q19: per consumer thread of the
  * warp-specialised kernel; D2Q9: per lane of 64-site strips, every mode at
  * tau = 1), when the run is FP32 and every system has nx % 4 == 0, else the
@@ -401,9 +402,9 @@ int lb_kernel_variants(int lattice, int32_t* out, int max_rows);
  * default row, or a row that differs from it only in a longer z-chunk when
  * the ensemble still has at least twice as many tiles as the GPU holds
  * resident CTAs (fewer halo planes per site, no idle SMs in the last wave);
- * on D3Q19 in FP32 with every mode at tau = 1, ensembles too small for that
- * (and those with an nx that is not a multiple of 4) take the row of the
- * lowest estimated step time among the paired and the split rows.
+ * on D3Q19, ensembles too small for that, those with an nx that is not a
+ * multiple of 4, FP64 runs and runs with a relaxation time other than 1 take
+ * the row of the lowest estimated step time among the paired and split rows.
  * Errors: LB_ERR_ARG. */
 lb_status lb_kernel_variant(lb_ctx* ctx, int* row);
 

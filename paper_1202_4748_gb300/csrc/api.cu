@@ -50,6 +50,7 @@ struct Plan {
         S, E, bottom_items, part_items, block_items, parts, up_items, tops, rec, acc, hist, field_tmp, sk_sys, sk_tw, sk_acc, sk_b0, sk_b1, sk_bins, jk_j,
         jk_lap, jk_F, jk_acc, mom, total;
     int tdim[3] = {0, 0, 0};      // tile shape of the step kernel
+    bool split = false, narrow = false;   // D3Q19: the split step (in 8 x 8 columns)
     bool jk = false;
     int hist_bins = 0;
     double hist_range = 0.0;
@@ -149,47 +150,25 @@ int tile_table(int lattice, int (*t)[kVariantCols]) {
 // The variant given by index, else the first compiled variant matching the
 // requested shape (and occupancy, if given), else the default: the first
 // variant the coupling runs (row-marching strips, scheme 2, are compiled for
-// the modified equilibrium only).  zm_default: the modified equilibrium on
-// D3Q19 where the paired kernel cannot run (FP64, a rate other than 1, an nx
-// that is not a multiple of 4) runs the radius-1 z-marching kernel whatever
-// the row, so its default is the first row of the plain z-marching kernel
-// (no producer warps), whose tile shape and budget suit it best (16 x 8
-// columns at 6 CTAs per SM: 0.563 ms on the 160-system ensemble against
-// 0.645 ms with the paired kernel's tile).
-lb_status choose_tile(int lattice, int coupling, const lb_run_opts* o, int& tile_id, int tdim[3],
-                      bool zm_default = false) {
+// the modified equilibrium only).
+lb_status choose_tile(int lattice, int coupling, const lb_run_opts* o, int& tile_id) {
     int t[32][kVariantCols];
     const int nt = tile_table(lattice, t);
     auto runs = [&](int k) { return t[k][5] != 2 || coupling == LB_MODEQ; };
-    const bool defaults = o->tile[0] <= 0 && o->occupancy <= 0;
-    auto preferred = [&](int k) {
-        if (!defaults || !zm_default || lattice != LB_D3Q19 || coupling != LB_MODEQ) return true;
-        return t[k][4] == 0 && t[k][5] == 0 && t[k][6] == 1;
-    };
-    tile_id = 0;
     if (o->variant < 0) return LB_ERR_ARG;
     if (o->variant > 0) {
         if (o->variant > nt || !runs(o->variant - 1)) return LB_ERR_UNSUPPORTED;
         tile_id = o->variant - 1;
-    } else {
-        tile_id = -1;
-        for (int pass = 0; pass < 2 && tile_id < 0; ++pass)
-            for (int k = 0; k < nt && tile_id < 0; ++k) {
-                const bool shape = o->tile[0] <= 0 || (t[k][0] == o->tile[0] && t[k][1] == o->tile[1] &&
-                                                       t[k][2] == (o->tile[2] > 0 ? o->tile[2] : 1));
-                const bool occ = o->occupancy <= 0 || t[k][3] == o->occupancy;
-                if (shape && occ && runs(k) && (pass == 1 || preferred(k))) tile_id = k;
-            }
-        if (tile_id < 0) return LB_ERR_UNSUPPORTED;
+        return LB_OK;
     }
-    for (int k = 0; k < 3; ++k) tdim[k] = t[tile_id][k];
-    return LB_OK;
-}
-
-bool split_row(int lattice, int tile_id) {
-    int t[32][kVariantCols];
-    tile_table(lattice, t);
-    return t[tile_id][5] == 4;
+    tile_id = -1;
+    for (int k = 0; k < nt && tile_id < 0; ++k) {
+        const bool shape = o->tile[0] <= 0 || (t[k][0] == o->tile[0] && t[k][1] == o->tile[1] &&
+                                               t[k][2] == (o->tile[2] > 0 ? o->tile[2] : 1));
+        const bool occ = o->occupancy <= 0 || t[k][3] == o->occupancy;
+        if (shape && occ && runs(k)) tile_id = k;
+    }
+    return tile_id < 0 ? LB_ERR_UNSUPPORTED : LB_OK;
 }
 
 // Number of step tiles (CTAs) of a tile shape over the ensemble.
@@ -237,52 +216,67 @@ bool prefer_longer_chunk(const lb_system_desc* s, int n, int sms, int& tile_id) 
     return found;
 }
 
-// Estimated step time (us) of a D3Q19 row on the fully relaxed FP32 path, from
-// timings on GB300 (152 SMs) of ensembles of 512 to 8.4 M sites; it only has
-// to rank the rows.
+// What a split step costs, by what it runs (FP32 at tau = 1; FP32 with other
+// rates, which pulls the populations again; FP64, bound by the FP64 units):
+// time (us) that a 16 x 8 column occupies its SM per plane and per chunk, that
+// it takes per plane and chunk on an idle SM, and of the moment pass per site.
+struct SplitCost {
+    double plane, chunk, alone_plane, alone_chunk, moment;
+};
+SplitCost split_cost(int kind, bool quads) {
+    if (kind == 2) return {11.4, 2.0, 14.7, 4.0, 7.4e-5};
+    if (kind == 1) return {0.72, 0.6, 1.15, 2.0, quads ? 1.6e-5 : 2.2e-5};
+    return {0.51, 0.43, 0.87, 2.0, quads ? 1.6e-5 : 2.2e-5};
+}
+
+// Estimated step time (us) of a D3Q19 row, from timings on GB300 (152 SMs) of
+// ensembles of 512 to 8.4 M sites; it only has to rank the rows.
 //  * paired kernel (staging 3): a resident CTA advances one plane per 1.53 us
 //    alone on its SM, 2.2 us beside one other, 3.1 us beside two; zc planes
 //    plus the halo planes of its chunk; CTAs in waves of 3 per SM.
-//  * split step (staging 4): the moment pass (quads of sites, or single sites
-//    where some nx is not a multiple of 4), then collision columns that occupy
-//    their SM for 0.51 us per plane plus 0.43 us (half of it for the 8 x 8
-//    columns) and take 0.87 us per plane plus 2 us however idle the SM is.
+//  * split step: SplitCost; an 8 x 8 column occupies its SM half as long.
 // Measured against the 32- and 64-plane paired rows that were the default of
 // every ensemble: 16^3 28.9 -> 5.3 us, 64^3 52 -> 14.4, 4 x 64^3 55 -> 46,
-// 16 x 64^3 157 -> 147 us per step; 2.6 M sites with odd sides 332 -> 137 us.
-double estimated_step_us(const lb_system_desc* s, int n, const int* row, int sms, bool quads) {
-    const double ctas = double(tiles_of(s, n, row)), zc = row[2];
+// 16 x 64^3 157 -> 147 us per step; 2.6 M sites with odd sides 332 -> 137 us;
+// against the z-marching kernels that ran the other settings: 4 x 64^3 with a
+// rate per mode 181 -> 71 us, FP64 256^3 29.2 -> 11.1 ms (of which the integer
+// noise 29.2 -> 14).
+double estimated_step_us(const lb_system_desc* s, int n, const int tdim[3], bool paired, int kind, int sms, bool quads) {
+    const double ctas = double(tiles_of(s, n, tdim));
     int64_t sites = 0;
     int nz = 0;
     for (int k = 0; k < n; ++k) {
         sites += int64_t(s[k].nx) * s[k].ny * s[k].nz;
         nz = std::max(nz, s[k].nz);
     }
-    const double planes = std::min<double>(zc, nz);
-    if (row[5] == 3) {
+    const double planes = std::min(tdim[2], nz);
+    if (paired) {
         const double per = planes + (s[0].coupling == LB_MODEQ ? 2 : 4), slots = 3.0 * sms;
         const double full = std::floor(ctas / slots), rest = ctas - full * slots;
         const double plane_us[4] = {0.0, 1.53, 2.2, 3.1};
         return 3.0 + per * (3.1 * full + plane_us[int(std::ceil(rest / sms))]);
     }
-    const double cost = (0.51 * planes + 0.43) * (row[0] == 8 ? 0.5 : 1.0);
+    const SplitCost c = split_cost(kind, quads);
+    const double cost = (c.plane * planes + c.chunk) * (tdim[0] == 8 ? 0.5 : 1.0);
     const double load = ctas / sms, filled = load <= 4.0 ? std::ceil(load) : load + 0.5;
-    return 3.0 + sites * (quads ? 1.6e-5 : 2.2e-5) + std::max(2.0 + 0.87 * planes, filled * cost);
+    return 3.0 + sites * c.moment + std::max(c.alone_chunk + c.alone_plane * planes, filled * cost);
 }
 
-// Default row of the fully relaxed FP32 path on D3Q19: the 64-plane paired row
-// while the ensemble fills the GPU twice over with it, else the cheapest of
-// the paired rows (every nx a multiple of 4) and the split rows.
-void choose_d3q19_row(const lb_system_desc* s, int n, bool quads, int& tile_id) {
+// Default row on D3Q19.  FP32 with every mode at tau = 1 (kind 0): the 64-plane
+// paired row while the ensemble fills the GPU twice over with it, else the
+// cheapest of the paired rows (every nx a multiple of 4) and the split rows.
+// Otherwise the cheapest z-chunk of the split step.
+void choose_d3q19_row(const lb_system_desc* s, int n, int kind, bool quads, int& tile_id) {
     const int sms = sm_count();
-    if (quads && prefer_longer_chunk(s, n, sms, tile_id)) return;
+    if (kind == 0 && quads && prefer_longer_chunk(s, n, sms, tile_id)) return;
     int t[32][kVariantCols];
     const int nt = tile_table(LB_D3Q19, t);
-    double best_us = quads ? estimated_step_us(s, n, t[tile_id], sms, quads) : INFINITY;
+    double best_us = INFINITY;
     for (int k = 0; k < nt; ++k) {
-        const bool paired = t[k][5] == 3 && t[k][0] == t[0][0] && quads;
-        if (!paired && t[k][5] != 4) continue;
-        const double us = estimated_step_us(s, n, t[k], sms, quads);
+        const bool paired = t[k][5] == 3 && t[k][0] == t[0][0] && quads && kind == 0;
+        const bool split = t[k][5] == 4 && (kind == 0 || t[k][0] == 16);
+        if (!paired && !split) continue;
+        const double us = estimated_step_us(s, n, t[k], paired, kind, sms, quads);
         if (us < best_us) {
             best_us = us;
             tile_id = k;
@@ -294,21 +288,32 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
                     int& tile_id) {
     lb_status st = validate(s, n, o);
     if (st != LB_OK) return st;
-    int tdim[3];
-    bool relaxed32 = o->precision == LB_FP32_DEVIATION, quads = true;
+    const bool fp32 = o->precision == LB_FP32_DEVIATION, d3 = s[0].lattice == LB_D3Q19;
+    bool relaxed = true, quads = fp32;
     for (int k = 0; k < n; ++k) {
         if (s[k].nx % 4 != 0) quads = false;
-        for (int a = s[k].lattice == LB_D2Q9 ? 3 : 4; a < q_of(s[k].lattice); ++a)
-            if (s[k].tau[a] != 1.0) relaxed32 = false;
+        for (int a = d3 ? 4 : 3; a < q_of(s[k].lattice); ++a)
+            if (s[k].tau[a] != 1.0) relaxed = false;
     }
-    st = choose_tile(s[0].lattice, s[0].coupling, o, tile_id, tdim, !(relaxed32 && quads));
+    st = choose_tile(s[0].lattice, s[0].coupling, o, tile_id);
     if (st != LB_OK) return st;
     if (o->variant == 0 && o->tile[0] <= 0 && o->occupancy <= 0) {
-        if (s[0].lattice == LB_D3Q19 && relaxed32) choose_d3q19_row(s, n, quads, tile_id);
+        if (d3) choose_d3q19_row(s, n, !fp32 ? 2 : (relaxed ? 0 : 1), quads, tile_id);
         else prefer_longer_chunk(s, n, sm_count(), tile_id);
+    }
+    int tdim[3];
+    {
         int t[32][kVariantCols];
         tile_table(s[0].lattice, t);
         for (int k = 0; k < 3; ++k) tdim[k] = t[tile_id][k];
+        // the split step: its own rows, and every D3Q19 run that the marching
+        // kernels are not compiled for (FP64, other rates), in 16 x 8 columns
+        P.split = d3 && (t[tile_id][5] == 4 || !fp32 || !relaxed);
+        P.narrow = P.split && t[tile_id][5] == 4 && tdim[0] == 8 && fp32 && relaxed;
+        if (P.split && !P.narrow) {
+            tdim[0] = 16;
+            tdim[1] = 8;
+        }
     }
     for (int k = 0; k < 3; ++k) P.tdim[k] = tdim[k];
     const int q = q_of(s[0].lattice);
@@ -536,15 +541,19 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
     P.pop1 = take(es * q * P.n_sites);
     P.step = take(sizeof(int64_t));
     P.status = take(sizeof(int));
-    P.d = take(sizeof(double) * P.n_sites);
     P.dbar = take(sizeof(double) * n);
     P.site_items = take(sizeof(int4) * P.n_site_items);
     P.site_partial = take(sizeof(double) * 4 * P.n_site_items);
     P.spans = take(sizeof(SysSpan) * n);
     P.glob = take(sizeof(double) * 8 * n);
     P.levels = take(sizeof(LevelDev) * P.n_levels);
+    // scratch of a sample (density deviation and block sums), which the density
+    // and momentum field of the split step shares: it lives within one step
+    P.mom = off;
+    P.d = take(sizeof(double) * P.n_sites);
     P.S = take(sizeof(double) * P.n_blocks_pyr);
     P.E = take(sizeof(double) * P.n_blocks_pyr);
+    if (P.split) off = std::max(off, align_up(P.mom + es * 4 * P.n_sites));
     P.bottom_items = take(sizeof(ObsItem) * P.n_bottom);
     P.part_items = take(sizeof(ObsPart) * P.part_h.size());
     P.block_items = take(sizeof(ObsBlocks) * P.block_h.size());
@@ -573,8 +582,6 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
     P.jk_lap = take(sizeof(double) * jkn);
     P.jk_F = take(sizeof(double) * 6 * (P.sk_fft ? 0 : jkn));
     P.jk_acc = take(sizeof(double) * 3 * jkn);
-    // density and momentum of the split step
-    P.mom = take(split_row(s[0].lattice, tile_id) && relaxed32 ? es * 4 * P.n_sites : 0);
     P.total = off;
     return LB_OK;
 }
@@ -839,6 +846,8 @@ cudaError_t launch_steps(lb_ctx* c, int64_t n) {
         a.status = c->at<int>(P.status);
         a.tile_id = c->tile_id;
         a.zc = P.tdim[2];
+        a.split = P.split ? 1 : 0;
+        a.narrow = P.narrow ? 1 : 0;
         a.mom = c->ws + P.mom;
         a.n_sites = P.n_sites;
         a.site_items = c->at<int4>(P.site_items);
@@ -976,7 +985,7 @@ lb_status lb_create(const lb_system_desc* systems, int n_systems, const lb_run_o
         if (!s.bgk) c->bgk_only = 0;
         else if (s.lam_bgk != 1.0 && c->bgk_only == 2) c->bgk_only = 1;
     }
-    if (split_row(c->lattice, c->tile_id) && c->fp32 && c->bgk_only == 2) c->step_kernels = 2;
+    if (c->P.split) c->step_kernels = 2;
     // bulk-copy staging: 16-byte aligned rows (nx % 4 == 0, so every system's
     // populations start 16-byte aligned too), at most 4 seam pieces per staged
     // row (nx >= 8) and single periodic wraps (every side >= 3)

@@ -251,6 +251,50 @@ __device__ __forceinline__ void grad_lap12_d3q19(const LapV& lv, V& gx, V& gy, V
     }
 }
 
+// f_i = 36 t_i sum_a T_ai h_a.
+template <class V>
+__device__ __forceinline__ void d3q19_populations(const V (&h)[19], V (&f)[19]) {
+    // rest: 12 (h0 - h4 + h16)
+    f[0] = vmul(vadd(vsub(h[0], h[4]), h[16]), vk<V>(12.0));
+    // faces (36 t = 2): even parts G + 2 D5, G - D5 +- D6; odd parts h_a - 2 h_{a+9}
+    {
+        const V G = vfma(h[16], vk<V>(-2.0), h[0]);
+        const V D5 = vsub(h[5], h[17]), D6 = vsub(h[6], h[18]);
+        const V Ex = vfma(D5, vk<V>(2.0), G);
+        const V GD = vsub(G, D5);
+        const V Ey = vadd(GD, D6), Ez = vsub(GD, D6);
+        const V Ox = vfma(h[10], vk<V>(-2.0), h[1]);
+        const V Oy = vfma(h[11], vk<V>(-2.0), h[2]);
+        const V Oz = vfma(h[12], vk<V>(-2.0), h[3]);
+        V s;
+        s = vadd(Ex, Ox); f[1] = vadd(s, s);
+        s = vsub(Ex, Ox); f[2] = vadd(s, s);
+        s = vadd(Ey, Oy); f[3] = vadd(s, s);
+        s = vsub(Ey, Oy); f[4] = vadd(s, s);
+        s = vadd(Ez, Oz); f[5] = vadd(s, s);
+        s = vsub(Ez, Oz); f[6] = vadd(s, s);
+    }
+    // edges (36 t = 1): even parts C + P5 +- P6 (xy, xz), C - 2 P5 (yz), plus the
+    // off-diagonal stress mode of the plane; odd parts from X+-, Y+-, Z+-
+    {
+        const V C = vadd(vadd(h[0], h[4]), h[16]);
+        const V P5 = vadd(h[5], h[17]), P6 = vadd(h[6], h[18]);
+        const V CP5 = vadd(C, P5);
+        const V Bxy = vadd(CP5, P6), Bxz = vsub(CP5, P6), Byz = vfma(P5, vk<V>(-2.0), C);
+        const V X = vadd(h[1], h[10]), Y = vadd(h[2], h[11]), Z = vadd(h[3], h[12]);
+        const V Xp = vadd(X, h[13]), Xm = vsub(X, h[13]);
+        const V Yp = vadd(Y, h[14]), Ym = vsub(Y, h[14]);
+        const V Zp = vadd(Z, h[15]), Zm = vsub(Z, h[15]);
+        V E, O;
+        E = vadd(Bxy, h[7]); O = vadd(Xp, Ym); f[7] = vadd(E, O); f[8] = vsub(E, O);
+        E = vsub(Bxy, h[7]); O = vsub(Xp, Ym); f[9] = vadd(E, O); f[10] = vsub(E, O);
+        E = vadd(Bxz, h[9]); O = vadd(Xm, Zp); f[11] = vadd(E, O); f[12] = vsub(E, O);
+        E = vsub(Bxz, h[9]); O = vsub(Xm, Zp); f[13] = vadd(E, O); f[14] = vsub(E, O);
+        E = vadd(Byz, h[8]); O = vadd(Yp, Zm); f[15] = vadd(E, O); f[16] = vsub(E, O);
+        E = vsub(Byz, h[8]); O = vsub(Yp, Zm); f[17] = vadd(E, O); f[18] = vsub(E, O);
+    }
+}
+
 // The part every fully relaxed D3Q19 collision shares: given h_a = w_a /
 // (36 N_a) of the equilibrium moments (h[0..9] and h[16]; h[10..15], h[17],
 // h[18] are set here), adds the noise of Eq. 68 in its lattice-general form
@@ -322,46 +366,7 @@ __device__ __forceinline__ void d3q19_tau1_noise_and_populations(V (&h)[19], V (
         h[17] = vk<V>(0.0);
         h[18] = vk<V>(0.0);
     }
-
-    // f_i = 36 t_i sum_a T_ai h_a.  Rest: 12 (h0 - h4 + h16).
-    f[0] = vmul(vadd(vsub(h[0], h[4]), h[16]), vk<V>(12.0));
-    // faces (36 t = 2): even parts G + 2 D5, G - D5 +- D6; odd parts h_a - 2 h_{a+9}
-    {
-        const V G = vfma(h[16], vk<V>(-2.0), h[0]);
-        const V D5 = vsub(h[5], h[17]), D6 = vsub(h[6], h[18]);
-        const V Ex = vfma(D5, vk<V>(2.0), G);
-        const V GD = vsub(G, D5);
-        const V Ey = vadd(GD, D6), Ez = vsub(GD, D6);
-        const V Ox = vfma(h[10], vk<V>(-2.0), h[1]);
-        const V Oy = vfma(h[11], vk<V>(-2.0), h[2]);
-        const V Oz = vfma(h[12], vk<V>(-2.0), h[3]);
-        V s;
-        s = vadd(Ex, Ox); f[1] = vadd(s, s);
-        s = vsub(Ex, Ox); f[2] = vadd(s, s);
-        s = vadd(Ey, Oy); f[3] = vadd(s, s);
-        s = vsub(Ey, Oy); f[4] = vadd(s, s);
-        s = vadd(Ez, Oz); f[5] = vadd(s, s);
-        s = vsub(Ez, Oz); f[6] = vadd(s, s);
-    }
-    // edges (36 t = 1): even parts C + P5 +- P6 (xy, xz), C - 2 P5 (yz), plus the
-    // off-diagonal stress mode of the plane; odd parts from X+-, Y+-, Z+-
-    {
-        const V C = vadd(vadd(h[0], h[4]), h[16]);
-        const V P5 = vadd(h[5], h[17]), P6 = vadd(h[6], h[18]);
-        const V CP5 = vadd(C, P5);
-        const V Bxy = vadd(CP5, P6), Bxz = vsub(CP5, P6), Byz = vfma(P5, vk<V>(-2.0), C);
-        const V X = vadd(h[1], h[10]), Y = vadd(h[2], h[11]), Z = vadd(h[3], h[12]);
-        const V Xp = vadd(X, h[13]), Xm = vsub(X, h[13]);
-        const V Yp = vadd(Y, h[14]), Ym = vsub(Y, h[14]);
-        const V Zp = vadd(Z, h[15]), Zm = vsub(Z, h[15]);
-        V E, O;
-        E = vadd(Bxy, h[7]); O = vadd(Xp, Ym); f[7] = vadd(E, O); f[8] = vsub(E, O);
-        E = vsub(Bxy, h[7]); O = vsub(Xp, Ym); f[9] = vadd(E, O); f[10] = vsub(E, O);
-        E = vadd(Bxz, h[9]); O = vadd(Xm, Zp); f[11] = vadd(E, O); f[12] = vsub(E, O);
-        E = vsub(Bxz, h[9]); O = vsub(Xm, Zp); f[13] = vadd(E, O); f[14] = vsub(E, O);
-        E = vadd(Byz, h[8]); O = vadd(Yp, Zm); f[15] = vadd(E, O); f[16] = vsub(E, O);
-        E = vsub(Byz, h[8]); O = vsub(Yp, Zm); f[17] = vadd(E, O); f[18] = vsub(E, O);
-    }
+    d3q19_populations<V>(h, f);
 }
 
 // f[i] <- post-collision deviations of the site(s) with density deviation
@@ -424,6 +429,58 @@ __device__ __forceinline__ void collide_d3q19_tau1(V (&f)[19], const V drho, con
     d3q19_tau1_noise_and_populations<V>(h, f, rho, cs2, P, key, site, status);
 }
 
+// g_a = 3 sum_i t_i c_ia rho(r + c_i) = (face difference) / 6 + (edge differences) / 12
+template <class V, class RhoV>
+__device__ __forceinline__ void d3q19_gradient(const RhoV& rv, V (&g)[3]) {
+    const V dfx = vsub(rv.template at<1, 0, 0>(), rv.template at<-1, 0, 0>());
+    const V dfy = vsub(rv.template at<0, 1, 0>(), rv.template at<0, -1, 0>());
+    const V dfz = vsub(rv.template at<0, 0, 1>(), rv.template at<0, 0, -1>());
+    const V exy = vsub(rv.template at<1, 1, 0>(), rv.template at<-1, -1, 0>());
+    const V exm = vsub(rv.template at<1, -1, 0>(), rv.template at<-1, 1, 0>());
+    const V exz = vsub(rv.template at<1, 0, 1>(), rv.template at<-1, 0, -1>());
+    const V ezm = vsub(rv.template at<1, 0, -1>(), rv.template at<-1, 0, 1>());
+    const V eyz = vsub(rv.template at<0, 1, 1>(), rv.template at<0, -1, -1>());
+    const V eym = vsub(rv.template at<0, 1, -1>(), rv.template at<0, -1, 1>());
+    // x: (1,1,0), (1,-1,0), (1,0,1), (1,0,-1) minus their opposites
+    g[0] = vfma(dfx, vk<V>(1.0 / 6.0), vmul(vadd(vadd(exy, exm), vadd(exz, ezm)), vk<V>(1.0 / 12.0)));
+    // y: (1,1,0), (-1,1,0) = -exm, (0,1,1), (0,1,-1)
+    g[1] = vfma(dfy, vk<V>(1.0 / 6.0), vmul(vadd(vsub(exy, exm), vadd(eyz, eym)), vk<V>(1.0 / 12.0)));
+    // z: (1,0,1), (-1,0,1) = -ezm, (0,1,1), (0,-1,1) = -eym
+    g[2] = vfma(dfz, vk<V>(1.0 / 6.0), vmul(vadd(vsub(exz, ezm), vsub(eyz, eym)), vk<V>(1.0 / 12.0)));
+}
+
+// h_4 .. h_9 and h_16 (m_a / (36 N_a)) of the modified equilibrium below.
+template <class V>
+__device__ __forceinline__ void d3q19_modeq_second(V (&h)[19], const V drho, const V rho, const V jx, const V jy,
+                                                   const V jz, const V ir, const V p0, const V lap, const V (&g)[3],
+                                                   const SysPhys<typename VT<V>::S>& P) {
+    const V ux = vmul(jx, ir), uy = vmul(jy, ir), uz = vmul(jz, ir);
+    const V iso = vfma(vmul(rho, vbc<V>(-P.kappa)), lap, p0);          // p0 - kappa rho lap rho
+    const V nu = vbc<V>(P.nu);
+    const V udg = vfma(ux, g[0], vfma(uy, g[1], vmul(uz, g[2])));
+    const V Xxx = vfma(jx, ux, vmul(nu, vfma(vadd(ux, ux), g[0], udg)));
+    const V Xyy = vfma(jy, uy, vmul(nu, vfma(vadd(uy, uy), g[1], udg)));
+    const V Xzz = vfma(jz, uz, vmul(nu, vfma(vadd(uz, uz), g[2], udg)));
+    const V Xxy = vfma(jx, uy, vmul(nu, vfma(ux, g[1], vmul(uy, g[0]))));
+    const V Xyz = vfma(jy, uz, vmul(nu, vfma(uy, g[2], vmul(uz, g[1]))));
+    const V Xzx = vfma(jz, ux, vmul(nu, vfma(uz, g[0], vmul(ux, g[2]))));
+    const V kgx = vmul(vbc<V>(P.kappa), g[0]), kgy = vmul(vbc<V>(P.kappa), g[1]), kgz = vmul(vbc<V>(P.kappa), g[2]);
+    const V Kxx = vmul(kgx, g[0]), Kyy = vmul(kgy, g[1]), Kzz = vmul(kgz, g[2]);
+    const V Ksum = vadd(vadd(Kxx, Kyy), Kzz);
+    const V trX = vadd(vadd(Xxx, Xyy), Xzz);
+
+    // h_a = m_a / (36 N_a); N = (1, 1/3 x3, 2/3, 4/3, 4/9, 1/9 x3, ..., 2 for mode 16)
+    h[4] = vmul(vfma(Ksum, vk<V>(-0.5), vfma(iso, vk<V>(3.0), vsub(trX, drho))), vk<V>(1.0 / 24.0));
+    h[5] = vmul(vadd(vfma(Xxx, vk<V>(2.0), vsub(vk<V>(0.0), vadd(Xyy, Xzz))),
+                     vfma(Kxx, vk<V>(2.0), vsub(vk<V>(0.0), vadd(Kyy, Kzz)))),
+                vk<V>(1.0 / 48.0));
+    h[6] = vmul(vadd(vsub(Xyy, Xzz), vsub(Kyy, Kzz)), vk<V>(1.0 / 16.0));
+    h[7] = vmul(vfma(kgx, g[1], Xxy), vk<V>(1.0 / 4.0));
+    h[8] = vmul(vfma(kgy, g[2], Xyz), vk<V>(1.0 / 4.0));
+    h[9] = vmul(vfma(kgz, g[0], Xzx), vk<V>(1.0 / 4.0));
+    h[16] = vmul(vfma(Ksum, vk<V>(-1.5), vfma(iso, vk<V>(-3.0), drho)), vk<V>(1.0 / 72.0));
+}
+
 // The modified equilibrium carried to D3Q19 (Eq. 65's structure with the
 // isotropic weights 3 t_i and the rotation-invariant square-gradient terms),
 // fully relaxed.  Its moments on this basis (deviation form) are
@@ -458,60 +515,212 @@ __device__ __forceinline__ void collide_d3q19_modeq_tau1(V (&f)[19], const V drh
     const V p0 = vsub(vmul(rr, df0), f0);
     const V cs2 = vmul(vmul(rr, vbc<V>(P.inv_rho_c)), vfma(vbc<V>(S(3) * P.b), phi2, vbc<V>(P.a)));
 
-    // g_a = 3 sum_i t_i c_ia rho(r + c_i) = (face difference) / 6 + (edge differences) / 12
     V g[3];
-    {
-        const V dfx = vsub(rv.template at<1, 0, 0>(), rv.template at<-1, 0, 0>());
-        const V dfy = vsub(rv.template at<0, 1, 0>(), rv.template at<0, -1, 0>());
-        const V dfz = vsub(rv.template at<0, 0, 1>(), rv.template at<0, 0, -1>());
-        const V exy = vsub(rv.template at<1, 1, 0>(), rv.template at<-1, -1, 0>());
-        const V exm = vsub(rv.template at<1, -1, 0>(), rv.template at<-1, 1, 0>());
-        const V exz = vsub(rv.template at<1, 0, 1>(), rv.template at<-1, 0, -1>());
-        const V ezm = vsub(rv.template at<1, 0, -1>(), rv.template at<-1, 0, 1>());
-        const V eyz = vsub(rv.template at<0, 1, 1>(), rv.template at<0, -1, -1>());
-        const V eym = vsub(rv.template at<0, 1, -1>(), rv.template at<0, -1, 1>());
-        // x: (1,1,0), (1,-1,0), (1,0,1), (1,0,-1) minus their opposites
-        g[0] = vfma(dfx, vk<V>(1.0 / 6.0), vmul(vadd(vadd(exy, exm), vadd(exz, ezm)), vk<V>(1.0 / 12.0)));
-        // y: (1,1,0), (-1,1,0) = -exm, (0,1,1), (0,1,-1)
-        g[1] = vfma(dfy, vk<V>(1.0 / 6.0), vmul(vadd(vsub(exy, exm), vadd(eyz, eym)), vk<V>(1.0 / 12.0)));
-        // z: (1,0,1), (-1,0,1) = -ezm, (0,1,1), (0,-1,1) = -eym
-        g[2] = vfma(dfz, vk<V>(1.0 / 6.0), vmul(vadd(vsub(exz, ezm), vsub(eyz, eym)), vk<V>(1.0 / 12.0)));
-    }
+    d3q19_gradient<V>(rv, g);
     const V lap = lap_d3q19<V>(rv);
 
     const V ir = vmap(rho, [](S x) { return fast_rcp(x); });
-    const V ux = vmul(jx, ir), uy = vmul(jy, ir), uz = vmul(jz, ir);
-    const V iso = vfma(vmul(rho, vbc<V>(-P.kappa)), lap, p0);          // p0 - kappa rho lap rho
-    const V nu = vbc<V>(P.nu);
-    const V udg = vfma(ux, g[0], vfma(uy, g[1], vmul(uz, g[2])));
-    const V Xxx = vfma(jx, ux, vmul(nu, vfma(vadd(ux, ux), g[0], udg)));
-    const V Xyy = vfma(jy, uy, vmul(nu, vfma(vadd(uy, uy), g[1], udg)));
-    const V Xzz = vfma(jz, uz, vmul(nu, vfma(vadd(uz, uz), g[2], udg)));
-    const V Xxy = vfma(jx, uy, vmul(nu, vfma(ux, g[1], vmul(uy, g[0]))));
-    const V Xyz = vfma(jy, uz, vmul(nu, vfma(uy, g[2], vmul(uz, g[1]))));
-    const V Xzx = vfma(jz, ux, vmul(nu, vfma(uz, g[0], vmul(ux, g[2]))));
-    const V kgx = vmul(vbc<V>(P.kappa), g[0]), kgy = vmul(vbc<V>(P.kappa), g[1]), kgz = vmul(vbc<V>(P.kappa), g[2]);
-    const V Kxx = vmul(kgx, g[0]), Kyy = vmul(kgy, g[1]), Kzz = vmul(kgz, g[2]);
-    const V Ksum = vadd(vadd(Kxx, Kyy), Kzz);
-    const V trX = vadd(vadd(Xxx, Xyy), Xzz);
-
-    // h_a = m_a / (36 N_a); N = (1, 1/3 x3, 2/3, 4/3, 4/9, 1/9 x3, ..., 2 for mode 16)
     V h[19];
+    d3q19_modeq_second<V>(h, drho, rho, jx, jy, jz, ir, p0, lap, g, P);
     h[0] = vmul(drho, vk<V>(1.0 / 36.0));
     h[1] = vmul(jx, vk<V>(1.0 / 12.0));
     h[2] = vmul(jy, vk<V>(1.0 / 12.0));
     h[3] = vmul(jz, vk<V>(1.0 / 12.0));
-    h[4] = vmul(vfma(Ksum, vk<V>(-0.5), vfma(iso, vk<V>(3.0), vsub(trX, drho))), vk<V>(1.0 / 24.0));
-    h[5] = vmul(vadd(vfma(Xxx, vk<V>(2.0), vsub(vk<V>(0.0), vadd(Xyy, Xzz))),
-                     vfma(Kxx, vk<V>(2.0), vsub(vk<V>(0.0), vadd(Kyy, Kzz)))),
-                vk<V>(1.0 / 48.0));
-    h[6] = vmul(vadd(vsub(Xyy, Xzz), vsub(Kyy, Kzz)), vk<V>(1.0 / 16.0));
-    h[7] = vmul(vfma(kgx, g[1], Xxy), vk<V>(1.0 / 4.0));
-    h[8] = vmul(vfma(kgy, g[2], Xyz), vk<V>(1.0 / 4.0));
-    h[9] = vmul(vfma(kgz, g[0], Xzx), vk<V>(1.0 / 4.0));
-    h[16] = vmul(vfma(Ksum, vk<V>(-1.5), vfma(iso, vk<V>(-3.0), drho)), vk<V>(1.0 / 72.0));
-
     d3q19_tau1_noise_and_populations<V>(h, f, rho, cs2, P, key, site, status);
+}
+
+// Collision with any relaxation rates, either coupling: with k_a = w_a / (36 N_a),
+//   w_a = m_a + lambda_a (m^eq_a - m_a) + (1 - lambda_a / 2) S_a + xi_a
+// on the non-conserved modes, m^eq as in the fully relaxed collisions above
+// (Guo: with E_bc = rho u_b u_c alone) and S the Guo source, S_4 = 2 u.F,
+// S_5 = 2 (3 u_x F_x - u.F), S_6 = 2 (u_y F_y - u_z F_z), S_7 = u_x F_y + u_y F_x,
+// S_8, S_9 likewise, 0 on the ghosts.  MODE 0: a rate per mode, m_a from the
+// sums the modes share; MODE 1: one rate lambda, f' = (1 - lambda) f + 36 t_i
+// sum_a T_ai (lambda k^eq + (1 - lambda / 2) k^S + k^xi).  f holds the
+// pre-collision deviations on entry; nv views the density (MODEQ) or its
+// Laplacian (GUO) around the site(s).
+template <int MODE, int CP, class V, class NV>
+__device__ __forceinline__ void collide_d3q19_rates(V (&f)[19], const V drho, const V jx, const V jy, const V jz,
+                                                    const NV& nv, const SysPhys<typename VT<V>::S>& P,
+                                                    const NoiseKey& key, const typename SiteIdx<V>::type site,
+                                                    int* status) {
+    using S = typename VT<V>::S;
+    constexpr int W = VT<V>::W;
+    static_assert(MODE == 0 || MODE == 1, "one rate or a rate per mode");
+    const V rho = vadd(vbc<V>(P.rho_c), drho);
+    bool bad_rho = false;
+#pragma unroll
+    for (int l = 0; l < W; ++l) bad_rho |= !(lane(rho, l) > S(0));
+    if (bad_rho) atomicOr(status, ST_RHO);
+
+    const V phi = vmul(drho, vbc<V>(P.inv_rho_c));
+    const V phi2 = vmul(phi, phi);
+    const V df0 = vmul(phi, vfma(vbc<V>(P.b), phi2, vbc<V>(P.a)));
+    const V f0 = vmul(phi2, vfma(vbc<V>(S(0.25) * P.b), phi2, vbc<V>(S(0.5) * P.a)));
+    const V rr = vmul(rho, vbc<V>(P.inv_rho_c));
+    const V p0 = vsub(vmul(rr, df0), f0);
+    const V cs2 = vmul(vmul(rr, vbc<V>(P.inv_rho_c)), vfma(vbc<V>(S(3) * P.b), phi2, vbc<V>(P.a)));
+    const V ir = vmap(rho, [](S x) { return fast_rcp(x); });
+
+    // k: equilibrium moments over 36 N_a (0 .. 9 and 16); s: the Guo source likewise (4 .. 9)
+    V k[19], s[6] = {}, F[3] = {};
+    if constexpr (CP == GUO) {
+        V gx, gy, gz;
+        grad_lap12_d3q19<V>(nv, gx, gy, gz);
+        const V kr = vmul(rho, vbc<V>(P.kappa * S(1.0 / 12.0)));
+        F[0] = vmul(kr, gx);
+        F[1] = vmul(kr, gy);
+        F[2] = vmul(kr, gz);
+        const V ux = vmul(vfma(F[0], vk<V>(0.5), jx), ir);
+        const V uy = vmul(vfma(F[1], vk<V>(0.5), jy), ir);
+        const V uz = vmul(vfma(F[2], vk<V>(0.5), jz), ir);
+        const V mx = vmul(rho, ux), my = vmul(rho, uy), mz = vmul(rho, uz);
+        const V Exx = vmul(ux, mx), Eyy = vmul(uy, my), Ezz = vmul(uz, mz);
+        const V tr = vadd(vadd(Exx, Eyy), Ezz);
+        const V iso = vfma(p0, vk<V>(-3.0), drho);
+        k[4] = vmul(vsub(tr, iso), vk<V>(1.0 / 24.0));
+        k[5] = vmul(vfma(Exx, vk<V>(3.0), vsub(vk<V>(0.0), tr)), vk<V>(1.0 / 48.0));
+        k[6] = vmul(vsub(Eyy, Ezz), vk<V>(1.0 / 16.0));
+        k[7] = vmul(vmul(ux, my), vk<V>(1.0 / 4.0));
+        k[8] = vmul(vmul(uy, mz), vk<V>(1.0 / 4.0));
+        k[9] = vmul(vmul(uz, mx), vk<V>(1.0 / 4.0));
+        k[16] = vmul(iso, vk<V>(1.0 / 72.0));
+        const V gxx = vmul(ux, F[0]), gyy = vmul(uy, F[1]), gzz = vmul(uz, F[2]);
+        const V uF = vadd(vadd(gxx, gyy), gzz);
+        s[0] = vmul(uF, vk<V>(1.0 / 12.0));
+        s[1] = vmul(vfma(gxx, vk<V>(3.0), vsub(vk<V>(0.0), uF)), vk<V>(1.0 / 24.0));
+        s[2] = vmul(vsub(gyy, gzz), vk<V>(1.0 / 8.0));
+        s[3] = vmul(vfma(ux, F[1], vmul(uy, F[0])), vk<V>(1.0 / 4.0));
+        s[4] = vmul(vfma(uy, F[2], vmul(uz, F[1])), vk<V>(1.0 / 4.0));
+        s[5] = vmul(vfma(uz, F[0], vmul(ux, F[2])), vk<V>(1.0 / 4.0));
+    } else {
+        V g[3];
+        d3q19_gradient<V>(nv, g);
+        const V lap = lap_d3q19<V>(nv);
+        d3q19_modeq_second<V>(k, drho, rho, jx, jy, jz, ir, p0, lap, g, P);
+    }
+    k[0] = vmul(drho, vk<V>(1.0 / 36.0));
+    k[1] = vmul(jx, vk<V>(1.0 / 12.0));
+    k[2] = vmul(jy, vk<V>(1.0 / 12.0));
+    k[3] = vmul(jz, vk<V>(1.0 / 12.0));
+
+    if constexpr (MODE == 1) {
+        const V lam = vbc<V>(P.lam_bgk), half = vbc<V>(S(1) - S(0.5) * P.lam_bgk);
+#pragma unroll
+        for (int a = 0; a < 10; ++a) k[a] = vmul(lam, k[a]);
+        k[16] = vmul(lam, k[16]);
+        if constexpr (CP == GUO) {
+#pragma unroll
+            for (int a = 0; a < 6; ++a) k[4 + a] = vfma(half, s[a], k[4 + a]);
+        }
+#pragma unroll
+        for (int a = 10; a < 16; ++a) k[a] = vk<V>(0.0);
+        k[17] = k[18] = vk<V>(0.0);
+    } else {
+        // m_a / (36 N_a) of f: sums and differences of opposite velocities, faces and edges
+        const V sx = vadd(f[1], f[2]), sy = vadd(f[3], f[4]), sz = vadd(f[5], f[6]);
+        const V dx = vsub(f[1], f[2]), dy = vsub(f[3], f[4]), dz = vsub(f[5], f[6]);
+        const V a1 = vadd(f[7], f[8]), a2 = vadd(f[9], f[10]), e1 = vsub(f[7], f[8]), e2 = vsub(f[9], f[10]);
+        const V b1 = vadd(f[11], f[12]), b2 = vadd(f[13], f[14]), g1 = vsub(f[11], f[12]), g2 = vsub(f[13], f[14]);
+        const V c1 = vadd(f[15], f[16]), c2 = vadd(f[17], f[18]), h1 = vsub(f[15], f[16]), h2 = vsub(f[17], f[18]);
+        const V Sxy = vadd(a1, a2), Sxz = vadd(b1, b2), Syz = vadd(c1, c2);
+        const V xe = vadd(Sxy, Sxz), ee = vadd(xe, Syz);
+        const V e5 = vfma(Syz, vk<V>(-2.0), xe), e6 = vsub(Sxy, Sxz);       // edge parts of modes 5 and 17, 6 and 18
+        const V fyz = vadd(sy, sz), f5 = vfma(sx, vk<V>(2.0), vsub(vk<V>(0.0), fyz)), f6 = vsub(sy, sz);
+        const V Xxy = vadd(e1, e2), Yxy = vsub(e1, e2), Xxz = vadd(g1, g2), Zxz = vsub(g1, g2);
+        const V Yyz = vadd(h1, h2), Zyz = vsub(h1, h2);
+        V m[19];
+        m[4] = vmul(vsub(ee, f[0]), vk<V>(1.0 / 24.0));
+        m[5] = vmul(vadd(f5, e5), vk<V>(1.0 / 48.0));
+        m[6] = vmul(vadd(f6, e6), vk<V>(1.0 / 16.0));
+        m[7] = vmul(vsub(a1, a2), vk<V>(1.0 / 4.0));
+        m[8] = vmul(vsub(c1, c2), vk<V>(1.0 / 4.0));
+        m[9] = vmul(vsub(b1, b2), vk<V>(1.0 / 4.0));
+        m[10] = vmul(vfma(dx, vk<V>(-2.0), vadd(Xxy, Xxz)), vk<V>(1.0 / 24.0));
+        m[11] = vmul(vfma(dy, vk<V>(-2.0), vadd(Yxy, Yyz)), vk<V>(1.0 / 24.0));
+        m[12] = vmul(vfma(dz, vk<V>(-2.0), vadd(Zxz, Zyz)), vk<V>(1.0 / 24.0));
+        m[13] = vmul(vsub(Xxy, Xxz), vk<V>(1.0 / 8.0));
+        m[14] = vmul(vsub(Yyz, Yxy), vk<V>(1.0 / 8.0));
+        m[15] = vmul(vsub(Zxz, Zyz), vk<V>(1.0 / 8.0));
+        m[16] = vmul(vadd(vfma(vadd(sx, fyz), vk<V>(-2.0), f[0]), ee), vk<V>(1.0 / 72.0));
+        m[17] = vmul(vsub(e5, f5), vk<V>(1.0 / 48.0));
+        m[18] = vmul(vsub(e6, f6), vk<V>(1.0 / 16.0));
+        sfor<4, 19>([&](auto A) {
+            constexpr int a = A;
+            const V lam = vbc<V>(P.lam[a]);
+            if constexpr (a < 10 || a == 16) k[a] = vfma(lam, vsub(k[a], m[a]), m[a]);
+            else k[a] = vmul(vbc<V>(S(1) - P.lam[a]), m[a]);
+            if constexpr (CP == GUO && a < 10) k[a] = vfma(vbc<V>(S(1) - S(0.5) * P.lam[a]), s[a - 4], k[a]);
+        });
+    }
+    if constexpr (CP == GUO) {
+        // (T F)_a = F_a on the momentum rows
+        k[1] = vfma(F[0], vk<V>(1.0 / 12.0), k[1]);
+        k[2] = vfma(F[1], vk<V>(1.0 / 12.0), k[2]);
+        k[3] = vfma(F[2], vk<V>(1.0 / 12.0), k[3]);
+    }
+
+    if (P.kT > S(0)) {
+        // as in the fully relaxed collisions, with g_ab = 1 - gamma_a gamma_b on the
+        // amplitudes: M = [[(2/3 + om) g_44, -om g_4,16], [., (2 + om) g_16,16]]
+        const V sc = vsqrt_pos(vmul(vbc<V>(vmul(S(3.0 * DrawScale<S>::v), P.kT)), rho));
+        const V om = vfma(cs2, vk<V>(-3.0), vk<V>(1.0));
+        const V mpp = vmul(vadd(vk<V>(2.0 / 3.0), om), vbc<V>(P.g_diag[4]));
+        const V mpr = vmul(om, vbc<V>(-P.g_pair));
+        const V mrr = vmul(vadd(vk<V>(2.0), om), vbc<V>(P.g_diag[16]));
+        const V det = vsub(vmul(mpp, mrr), vmul(mpr, mpr));
+        const V q = vrsqrt(mpp);
+        V k11 = vmul(vmul(mpp, q), vk<V>(1.0 / 24.0));
+        V k21 = vmul(vmul(mpr, q), vk<V>(1.0 / 72.0));
+        V k22 = vmul(vmul(det, vrsqrt(vmul(det, mpp))), vk<V>(1.0 / 72.0));
+        auto bad = [&](int l) { return !(lane(det, l) > S(0)) || !(lane(mpp, l) > S(0)); };
+        bool bad_noise = false;
+#pragma unroll
+        for (int l = 0; l < W; ++l) bad_noise = bad_noise || bad(l);
+        if (bad_noise) {
+#pragma unroll
+            for (int l = 0; l < W; ++l) {
+                if (bad(l)) {
+                    set_lane(k11, l, S(0));
+                    set_lane(k21, l, S(0));
+                    set_lane(k22, l, S(0));
+                }
+            }
+            atomicOr(status, ST_NOISE);
+        }
+        // sqrt(N_a g_aa) / (36 N_a), 36 N_a as above
+        auto amp = [&](int a, double inv) { return vbc<V>(vmul(P.namp[a], S(inv))); };
+        V n[4];
+        draw4(key, site, 0u, sc, sc, n, true);
+        const V n4 = n[0];
+        k[4] = vfma(k11, n4, k[4]);
+        k[5] = vfma(n[1], amp(5, 1.0 / 48.0), k[5]);
+        k[6] = vfma(n[2], amp(6, 1.0 / 16.0), k[6]);
+        k[7] = vfma(n[3], amp(7, 1.0 / 4.0), k[7]);
+        draw4(key, site, 1u, sc, sc, n, true);
+        k[8] = vfma(n[0], amp(8, 1.0 / 4.0), k[8]);
+        k[9] = vfma(n[1], amp(9, 1.0 / 4.0), k[9]);
+        k[10] = vfma(n[2], amp(10, 1.0 / 24.0), k[10]);
+        k[11] = vfma(n[3], amp(11, 1.0 / 24.0), k[11]);
+        draw4(key, site, 2u, sc, sc, n, true);
+        k[12] = vfma(n[0], amp(12, 1.0 / 24.0), k[12]);
+        k[13] = vfma(n[1], amp(13, 1.0 / 8.0), k[13]);
+        k[14] = vfma(n[2], amp(14, 1.0 / 8.0), k[14]);
+        k[15] = vfma(n[3], amp(15, 1.0 / 8.0), k[15]);
+        draw4(key, site, 3u, sc, sc, n, false);
+        k[16] = vfma(k22, n[0], vfma(k21, n4, k[16]));
+        k[17] = vfma(n[1], amp(17, 1.0 / 48.0), k[17]);
+        k[18] = vfma(n[2], amp(18, 1.0 / 16.0), k[18]);
+    }
+    if constexpr (MODE == 1) {
+        V g[19];
+        d3q19_populations<V>(k, g);
+        const V oml = vbc<V>(S(1) - P.lam_bgk);
+#pragma unroll
+        for (int i = 0; i < 19; ++i) f[i] = vfma(oml, f[i], g[i]);
+    } else {
+        d3q19_populations<V>(k, f);
+    }
 }
 
 }  // namespace lbf

@@ -2,6 +2,8 @@
 // launchers for the step, init, gather/scatter and observable-site kernels.
 #pragma once
 
+#include <type_traits>
+
 #include "lattice_kernels.cuh"
 #include "lb_launch.h"
 #include "step_kernel_modeq3.cuh"
@@ -68,37 +70,19 @@ cudaError_t step_strip2(const StepLaunch& a, cudaStream_t st) {
     return step_strip<L, CP, Real, YC, WPC, MINB, 64>(a, st);
 }
 
-template <class L, int CP, class Real, int TX, int TY, int MINB, int MODE>
-cudaError_t step_z_mode(const StepLaunch& a, cudaStream_t st) {
-    const StepArgs<Real> A = step_args<Real>(a);
-    step_kernel_z<L, CP, Real, TX, TY, MINB, MODE><<<a.n_tiles, TX * TY, 0, st>>>(A);
-    return cudaGetLastError();
-}
-
-// z-marching launch: tile = (TX, TY, z-chunk), register budget for MINB resident
-// CTAs per SM (the FP64 instances use the natural register count).
-template <class L, int CP, class Real, int TX, int TY, int MINB>
+// z-marching launches (FP32, every mode at tau = 1): columns of TX x TY sites,
+// chunks of a.zc planes, a register budget for MINB resident CTAs per SM; the
+// Guo form, and the modified equilibrium on its radius-1 footprint.
+template <class L, int TX, int TY, int MINB>
 cudaError_t step_z(const StepLaunch& a, cudaStream_t st) {
-    constexpr int MB = sizeof(Real) == 4 ? MINB : 1;
-    if (a.bgk_only == 2) return step_z_mode<L, CP, Real, TX, TY, MB, 2>(a, st);
-    if (a.bgk_only == 1) return step_z_mode<L, CP, Real, TX, TY, MB, 1>(a, st);
-    return step_z_mode<L, CP, Real, TX, TY, MB, 0>(a, st);
-}
-
-// z-marching launch of the D3Q19 modified equilibrium (density footprint of
-// radius 1); the FP64 instances use the natural register count.
-template <class L, class Real, int TX, int TY, int MINB, int MODE>
-cudaError_t step_zm_mode(const StepLaunch& a, cudaStream_t st) {
-    const StepArgs<Real> A = step_args<Real>(a);
-    step_kernel_zm<L, Real, TX, TY, MINB, MODE><<<a.n_tiles, TX * TY, 0, st>>>(A);
+    step_kernel_z<L, TX, TY, MINB><<<a.n_tiles, TX * TY, 0, st>>>(step_args<float>(a));
     return cudaGetLastError();
 }
-template <class L, class Real, int TX, int TY, int MINB>
+template <class L, int TX, int TY, int MINB>
 cudaError_t step_zm(const StepLaunch& a, cudaStream_t st) {
-    constexpr int MB = sizeof(Real) == 4 ? (MINB < 2 ? 2 : MINB) : 1;
-    if (a.bgk_only == 2) return step_zm_mode<L, Real, TX, TY, MB, 2>(a, st);
-    if (a.bgk_only == 1) return step_zm_mode<L, Real, TX, TY, MB, 1>(a, st);
-    return step_zm_mode<L, Real, TX, TY, MB, 0>(a, st);
+    constexpr int MB = MINB < 2 ? 2 : MINB;
+    step_kernel_zm<L, TX, TY, MB><<<a.n_tiles, TX * TY, 0, st>>>(step_args<float>(a));
+    return cudaGetLastError();
 }
 
 // Warp-specialised launch (fully relaxed Guo path, FP32): TX x TY consumer
@@ -147,7 +131,7 @@ cudaError_t step_pair(const StepLaunch& a, cudaStream_t st) {
         state = (!PairRegs<TX, TY, PW, MINB, STG>::split || fa.numRegs == PairRegs<TX, TY, PW, MINB, STG>::launch) ? 1 : -1;
     }
     if (state < 0) {
-        if constexpr (CP == MODEQ) return step_zm<D3Q19, float, TX, TY, MINB>(a, st);
+        if constexpr (CP == MODEQ) return step_zm<D3Q19, TX, TY, MINB>(a, st);
         else return step_ws<D3Q19, TX, TY, PW, 1, 0>(a, st);
     }
     step_kernel_pair<TX, TY, PW, MINB, R, STG, CP><<<a.n_tiles, TX * TY / 2 + 32 * PW, dyn, st>>>(A);
@@ -189,14 +173,29 @@ cudaError_t step_moments(const StepLaunch& a, cudaStream_t st) {
                             a.n_sites);
 }
 
-// Split step (D3Q19, FP32, every mode at tau = 1): the moment pass over the
-// site items, then the collision of TX x TY columns in chunks of a.zc planes.
-template <int CP, int TX, int TY, int MINB>
-cudaError_t step_split(const StepLaunch& a, cudaStream_t st) {
-    const cudaError_t e = step_moments<D3Q19, float>(a, st);
+// Split step on D3Q19: the moment pass over the site items, then the collision
+// of TX x TY columns in chunks of a.zc planes.  Resident CTAs: FP32 at tau = 1
+// fits 4 (8 of the 8 x 8 columns) without spills; the pulled populations of the
+// other rates need more registers; the FP64 unit needs no more than 2.
+template <int MODE, int CP, class Real, int TX, int TY>
+cudaError_t step_split_mode(const StepLaunch& a, cudaStream_t st) {
+    using V = typename std::conditional<std::is_same<Real, float>::value, float2, double>::type;
+    constexpr int MINB = (sizeof(Real) == 8 ? 2 : (MODE == 2 ? 4 : 3)) * (TX == 8 ? 2 : 1);
+    const cudaError_t e = step_moments<D3Q19, Real>(a, st);
     if (e != cudaSuccess) return e;
-    return launch_dependent(collide_march_kernel<CP, TX, TY, MINB>, a.n_tiles, TX * TY, st, step_args<float>(a),
-                            static_cast<const float*>(a.mom), a.n_sites);
+    return launch_dependent(collide_march_kernel<MODE, CP, V, TX, TY, MINB>, a.n_tiles, TX * TY, st,
+                            step_args<Real>(a), static_cast<const Real*>(a.mom), a.n_sites);
+}
+template <int CP, class Real>
+cudaError_t step_split(const StepLaunch& a, cudaStream_t st) {
+    if (a.bgk_only == 2) {
+        if constexpr (std::is_same<Real, float>::value) {
+            if (a.narrow) return step_split_mode<2, CP, Real, 8, 8>(a, st);
+        }
+        return step_split_mode<2, CP, Real, 16, 8>(a, st);
+    }
+    if (a.bgk_only == 1) return step_split_mode<1, CP, Real, 16, 8>(a, st);
+    return step_split_mode<0, CP, Real, 16, 8>(a, st);
 }
 
 template <class L, int CP, class Real, int TX, int TY, int TZ>

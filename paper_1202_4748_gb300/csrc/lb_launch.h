@@ -24,6 +24,8 @@ struct StepLaunch {
     int* status;
     int tile_id;            // index into the lattice's tile-shape table
     int zc;                 // z extent of its tiles (planes per chunk of the z-marching kernels)
+    int split;              // D3Q19: run the split step (narrow: in 8 x 8 columns)
+    int narrow;
     void* mom;              // split step: density and momentum fields, one per n_sites values
     int64_t n_sites;        // sites of the ensemble
     const int4* site_items; // split step: the moment pass's work list

@@ -1,14 +1,14 @@
 // Split form of the fused step: a moment pass writes the density and momentum
-// of every site (from the 19 populations pulled to it, once per site), and a
-// collision pass reads that field around each block of sites and writes the
+// of every site (from the populations pulled to it, once per site), and a
+// collision pass reads that field around each column of sites and writes the
 // post-collision populations.  With every mode at tau = 1 the collision needs
 // nothing else; with other rates it pulls the site's populations again.
 //
-// Against the z-marching kernels, which re-form the density on the halo of
-// every column and walk it plane by plane, this trades 16 extra bytes written
-// and about 35 read per site (both from L2 while the ensemble fits there) for
-// having no serial chain: every site of every block is in flight at once.  A
-// marching CTA takes about 1.6 us per plane however few CTAs there are, so an
+// Against the kernels that form the density on the halo of every column, this
+// trades 16 bytes written and about 35 read per FP32 site (from L2 while the
+// ensemble fits there) for forming each density once, which is what the FP64
+// path needs (its units do two operations per clock and SM), and for short
+// chunks: a paired CTA takes 1.53 us per plane however few CTAs there are, so an
 // ensemble that gives it less than a CTA per SM waits for latency alone.
 #pragma once
 
@@ -124,60 +124,70 @@ __global__ void __launch_bounds__(NT)
     grid_release();
 }
 
-// Two sites stacked in z per thread (paired FP32): at<cx, cy, cz>() is the pair
-// of values at (x + cx, y + cy, z + cz) and one plane above, from the four
-// planes z - 1 .. z + 2 of row pitch PX.
-template <int PX>
+// The thread's sites are W = 1 site, or 2 stacked in z (paired FP32):
+// at<cx, cy, cz>() is the value (or pair of values) at (x + cx, y + cy, z + cz)
+// from the planes z - 1 .. z + W of row pitch PX.
+template <class V, int PX>
 struct ZPlanes {
-    const float *m, *o, *p, *q;
+    using S = typename VT<V>::S;
+    const S* p[2 + VT<V>::W];
     int c;
     template <int CX, int CY, int CZ>
-    __device__ __forceinline__ float2 at() const {
+    __device__ __forceinline__ V at() const {
         constexpr int off = CX + PX * CY;
-        if constexpr (CZ == -1) return make_float2(m[c + off], o[c + off]);
-        else if constexpr (CZ == 0) return make_float2(o[c + off], p[c + off]);
-        else return make_float2(p[c + off], q[c + off]);
+        if constexpr (VT<V>::W == 2) return make_float2(p[1 + CZ][c + off], p[2 + CZ][c + off]);
+        else return p[1 + CZ][c + off];
     }
 };
 
-// Collision pass (D3Q19, FP32, every mode at tau = 1): a CTA owns a TX x TY
-// column and walks a chunk of A.zc planes, two planes per iteration, one pair
-// of sites stacked in z per thread.  Every load and store is then a row of
+// Collision pass of the split step on D3Q19: a CTA owns a TX x TY column and
+// walks a chunk of A.zc planes, W per iteration: two with paired FP32, one site
+// per lane of the pair, else one.  Every load and store is then a row of
 // consecutive sites, whatever the parity of the sides.  Density planes come
-// from the moment field by 4-byte cp.async into a ring, two iterations before
-// the Laplacian that needs them; the Laplacian (Guo form) of planes z + 3,
-// z + 4 and the collision of planes z, z + 1 share one phase, so there is one
-// CTA barrier per iteration; the momenta of the next pair are in flight across
-// it.  Rings of 8 planes: the collision of z reads density z, z + 1 (z - 1 ..
-// z + 2 for the modified equilibrium) and Laplacian z - 1 .. z + 2, the
-// Laplacian pass reads density z + 2 .. z + 5 and writes Laplacian z + 3,
-// z + 4, the copies write density z + 6, z + 7, and a warp still in the
-// iteration before reads nothing below density z - 3 and Laplacian z - 3.
-template <int CP, int TX, int TY, int MINB>
+// from the moment field by cp.async into a ring, an iteration before the
+// Laplacian that needs them; the Laplacian (Guo form) of planes z + W + 1 ..
+// z + 2 W and the collision of planes z .. z + W - 1 share one phase, so there
+// is one CTA barrier per iteration; the momenta of the next sites are in flight
+// across it.  With rates other than 1 (MODE 0 and 1) a thread also pulls its
+// sites' populations, requested before the Laplacian pass.
+//
+// Rings of 8 planes: iteration z reads density z .. z + 2 W + 1 (z - 1 .. z + W
+// for the modified equilibrium) and Laplacian z - 1 .. z + W, writes Laplacian
+// up to z + 2 W, and its copies land in density up to z + 3 W + 1 <= z + 7; no
+// warp is in an earlier iteration once they are issued, after the barrier.
+//
+// 16 x 8 columns, 128 threads: the Laplacian's halo costs 1.4, four or five
+// CTAs per SM decouple the phases.  FP32, tau = 1: bound by issue and, below a
+// CTA per SM, by the latency of a chunk (0.87 us per plane).  FP64: bound by
+// the FP64 units (two operations per clock and SM).
+template <int MODE, int CP, class V, int TX, int TY, int MINB>
 __global__ void __launch_bounds__(TX* TY, MINB)
-    collide_march_kernel(const StepArgs<float> A, const float* __restrict__ mom, int64_t stride) {
+    collide_march_kernel(const StepArgs<typename VT<V>::S> A, const typename VT<V>::S* __restrict__ mom,
+                         int64_t stride) {
+    using Real = typename VT<V>::S;
+    using L = D3Q19;
+    constexpr int W = VT<V>::W;
     constexpr int H = CP == GUO ? 2 : 1;
     constexpr int NT = TX * TY, R = 8;
     constexpr int SX = TX + 2 * H, SY = TY + 2 * H, SP = SX * SY;
     constexpr int LX = TX + 2, LY = TY + 2, LP = CP == GUO ? LX * LY : 1;
-    constexpr int PPT = (SP + NT - 1) / NT;           // footprint sites per thread
-    constexpr int AHEAD = CP == GUO ? 5 : 2;          // highest density plane an iteration reads, minus z
-    __shared__ float srho[R * SP];
-    __shared__ float slap[R * LP];
+    constexpr int PPT = (SP + NT - 1) / NT;              // footprint sites per thread
+    constexpr int AHEAD = CP == GUO ? 2 * W + 1 : W;     // highest density plane an iteration reads, minus z
+    __shared__ Real srho[R * SP];
+    __shared__ Real slap[R * LP];
 
     const int4 tl = A.tiles[blockIdx.x];
     const SysDev& S = A.sys[tl.x];
-    const SysPhys<float> P = A.phys[tl.x];
+    const SysPhys<Real>& P = A.phys[tl.x];
     const int nx = S.nx, ny = S.ny, nz = S.nz, N = S.ns, pl = nx * ny;
     const int z0 = tl.w, z1 = min(z0 + A.zc, nz);
     const int tid = threadIdx.x;
     const int lx = tid % TX, ly = tid / TX;
     const int x = tl.y + lx, y = tl.z + ly;
     const bool own = x < nx && y < ny;
-    const float* __restrict__ rho_g = mom + S.site_offset;
-    float* __restrict__ fo = A.fout + S.pop_offset + (y * nx + x);
-    const float* __restrict__ jg = rho_g + stride + (y * nx + x);
-    const int64_t js = stride;
+    const Real* __restrict__ rho_g = mom + S.site_offset;
+    const Real* __restrict__ jg = rho_g + stride + (y * nx + x);
+    Real* __restrict__ fo = A.fout + S.pop_offset + (y * nx + x);
 
     // wrapped in-plane offset of the thread's footprint sites (-1: not needed)
     int foot[PPT];
@@ -188,93 +198,117 @@ __global__ void __launch_bounds__(TX* TY, MINB)
     });
     auto slot = [](int rel) { return rel & (R - 1); };   // rel = plane - z0 + R
     auto fetch = [&](int zz) {                           // density plane zz into its ring slot
-        const float* src = rho_g + wrapm(zz, nz) * pl;
-        float* dst = srho + slot(zz - z0 + R) * SP + tid;
+        const Real* src = rho_g + wrapm(zz, nz) * pl;
+        Real* dst = srho + slot(zz - z0 + R) * SP + tid;
         sfor<0, PPT>([&](auto K) {
             constexpr int k = K;
-            if (foot[k] >= 0) cp_async4(dst + k * NT, src + foot[k]);
+            if (foot[k] >= 0) cp_async_elem(dst + k * NT, src + foot[k]);
         });
     };
     const int zlast = z1 - 1 + H;                        // last density plane any collision of the chunk needs
-    auto laplacian2 = [&](int zl) {                      // Laplacian planes zl, zl + 1
+    auto laplacian = [&](int zl) {                       // Laplacian planes zl .. zl + W - 1
         if constexpr (CP == GUO) {
-            const int r = zl - z0 + R;
-            const float* pm = srho + slot(r - 1) * SP;
-            const float* p0 = srho + slot(r) * SP;
-            const float* p1 = srho + slot(r + 1) * SP;
-            const float* p2 = srho + slot(r + 2) * SP;
-            float* l0 = slap + slot(r) * LP;
-            float* l1 = slap + slot(r + 1) * LP;
+            ZPlanes<V, SX> rv;
+            sfor<0, 2 + W>([&](auto K) {
+                constexpr int k = K;
+                rv.p[k] = srho + slot(zl - z0 + R - 1 + k) * SP;
+            });
+            Real* l0 = slap + slot(zl - z0 + R) * LP;
+            Real* l1 = slap + slot(zl - z0 + R + W - 1) * LP;
             for (int i = tid; i < LP; i += NT) {
-                const int c = (i / LX + 1) * SX + i % LX + 1;
-                const ZPlanes<SX> rv{pm, p0, p1, p2, c};
-                const float2 lap = lap_d3q19<float2>(rv);
-                l0[i] = lap.x;
-                l1[i] = lap.y;
+                rv.c = (i / LX + 1) * SX + i % LX + 1;
+                const V lap = lap_d3q19<V>(rv);
+                l0[i] = lane(lap, 0);
+                if constexpr (W == 2) l1[i] = lane(lap, 1);
             }
         }
     };
-    float2 jn[3];
-    auto momenta = [&](int z) {                          // the pair's momenta (the second site may not exist)
-        sfor<0, 3>([&](auto C) { jn[decltype(C)::value] = make_float2(0.0f, 0.0f); });
+    V jn[3];
+    auto momenta = [&](int z) {                          // of the sites (x, y, z ..); the second may not exist
+        sfor<0, 3>([&](auto C) { jn[decltype(C)::value] = vk<V>(0.0); });
         if (own && z < z1) {
             const int up = z + 1 < z1 ? pl : 0;
             sfor<0, 3>([&](auto C) {
                 constexpr int c = C;
-                const float* q = jg + c * js + z * pl;
-                jn[c] = make_float2(q[0], q[up]);
+                const Real* q = jg + c * stride + z * pl;
+                set_lane(jn[c], 0, q[0]);
+                if constexpr (W == 2) set_lane(jn[c], 1, q[up]);
             });
         }
     };
 
     grid_wait();
     const NoiseKey key = noise_key(S, *A.step_ptr + A.k);
-    for (int zz = z0 - H; zz <= min(z0 + AHEAD - (CP == GUO ? 2 : 0), zlast); ++zz) fetch(zz);
+    for (int zz = z0 - H; zz <= min(z0 + AHEAD - (CP == GUO ? W : 0), zlast); ++zz) fetch(zz);
     cp_async_commit();
     if constexpr (CP == GUO) {
-        for (int zz = z0 + AHEAD - 1; zz <= min(z0 + AHEAD, zlast); ++zz) fetch(zz);
+        for (int zz = z0 + AHEAD - W + 1; zz <= min(z0 + AHEAD, zlast); ++zz) fetch(zz);
         cp_async_commit();
     }
     momenta(z0);
     if constexpr (CP == GUO) {
         cp_async_wait<1>();
         __syncthreads();
-        laplacian2(z0 - 1);
-        laplacian2(z0 + 1);
+        sfor<0, (2 + W) / W>([&](auto K) { laplacian(z0 - 1 + W * int(K)); });   // planes z0 - 1 .. z0 + W
     }
-    for (int z = z0; z < z1; z += 2) {
-        float2 jm[3];
+    for (int z = z0; z < z1; z += W) {
+        V jm[3];
         sfor<0, 3>([&](auto C) { jm[decltype(C)::value] = jn[decltype(C)::value]; });
         cp_async_wait<0>();                              // density up to plane z + AHEAD has landed (this thread's copies)
         __syncthreads();
-        if (z + 2 < z1) {
-            for (int zz = z + AHEAD + 1; zz <= min(z + AHEAD + 2, zlast); ++zz) fetch(zz);
-            momenta(z + 2);
+        const bool more = z + W < z1, two = z + 1 < z1;
+        if (more) {
+            for (int zz = z + AHEAD + 1; zz <= min(z + AHEAD + W, zlast); ++zz) fetch(zz);
+            momenta(z + W);
         }
         cp_async_commit();
-        if (CP == GUO && z + 2 < z1) laplacian2(z + 3);
-        if (z + 2 >= z1) grid_release();
+        V f[19];
+        if constexpr (MODE != 2) {
+            if (own) {
+                const Real* fb = A.fin + S.pop_offset;
+                const Nbr nb(x, y, z, nx, ny, nz, true);
+                const int pu = two && W == 2 ? z + 1 : z;   // past the chunk the second lane repeats the first
+                const int zu[3] = {(pu == 0 ? nz - 1 : pu - 1) * pl, pu * pl, (pu == nz - 1 ? 0 : pu + 1) * pl};
+                sfor<0, 19>([&](auto I) {
+                    constexpr int i = I;
+                    const Real* col = fb + (i * N + nb.X[1 - L::c(i, 0)] + nb.Y[1 - L::c(i, 1)]);
+                    set_lane(f[i], 0, col[nb.Z[1 - L::c(i, 2)]]);
+                    if constexpr (W == 2) set_lane(f[i], 1, col[zu[1 - L::c(i, 2)]]);
+                });
+            }
+        }
+        if (more) laplacian(z + W + 1);
+        else grid_release();
         if (own) {
-            const bool two = z + 1 < z1;
             const int site = y * nx + x + z * pl;
-            const uint2 sites = make_uint2(site, two ? site + pl : site);
             const int r = z - z0 + R;
             const int c = (ly + H) * SX + lx + H;
-            const float* d0 = srho + slot(r) * SP + c;
-            const float* d1 = srho + slot(two ? r + 1 : r) * SP + c;   // past the chunk the second lane repeats the first
-            const float2 drho = make_float2(d0[0], d1[0]);
-            float2 f[19];
-            if constexpr (CP == GUO) {
-                const ZPlanes<LX> lv{slap + slot(r - 1) * LP, slap + slot(r) * LP, slap + slot(r + 1) * LP,
-                                     slap + slot(r + 2) * LP, (ly + 1) * LX + lx + 1};
-                collide_d3q19_tau1<float2>(f, drho, jm[0], jm[1], jm[2], lv, P, key, sites, A.status);
+            typename SiteIdx<V>::type sites;
+            V drho;
+            set_lane(drho, 0, srho[slot(r) * SP + c]);
+            if constexpr (W == 2) {
+                sites = make_uint2(site, two ? site + pl : site);
+                set_lane(drho, 1, srho[slot(two ? r + 1 : r) * SP + c]);
             } else {
-                const ZPlanes<SX> rv{srho + slot(r - 1) * SP, srho + slot(r) * SP, srho + slot(r + 1) * SP,
-                                     srho + slot(r + 2) * SP, c};
-                collide_d3q19_modeq_tau1<float2>(f, drho, jm[0], jm[1], jm[2], rv, P, key, sites, A.status);
+                sites = site;
             }
-            sfor<0, 19>([&](auto I) { fo[decltype(I)::value * N + z * pl] = f[decltype(I)::value].x; });
-            if (two) sfor<0, 19>([&](auto I) { fo[decltype(I)::value * N + (z + 1) * pl] = f[decltype(I)::value].y; });
+            ZPlanes<V, CP == GUO ? LX : SX> nv;
+            nv.c = CP == GUO ? (ly + 1) * LX + lx + 1 : c;
+            sfor<0, 2 + W>([&](auto K) {
+                constexpr int k = K;
+                nv.p[k] = CP == GUO ? slap + slot(r - 1 + k) * LP : srho + slot(r - 1 + k) * SP;
+            });
+            if constexpr (MODE != 2)
+                collide_d3q19_rates<MODE, CP, V>(f, drho, jm[0], jm[1], jm[2], nv, P, key, sites, A.status);
+            else if constexpr (CP == GUO)
+                collide_d3q19_tau1<V>(f, drho, jm[0], jm[1], jm[2], nv, P, key, sites, A.status);
+            else
+                collide_d3q19_modeq_tau1<V>(f, drho, jm[0], jm[1], jm[2], nv, P, key, sites, A.status);
+            sfor<0, 19>([&](auto I) { fo[decltype(I)::value * N + z * pl] = lane(f[decltype(I)::value], 0); });
+            if constexpr (W == 2) {
+                if (two)
+                    sfor<0, 19>([&](auto I) { fo[decltype(I)::value * N + (z + 1) * pl] = lane(f[decltype(I)::value], 1); });
+            }
         }
     }
 }

@@ -741,41 +741,34 @@ __global__ void __launch_bounds__(32 * WPC, MINB) step_kernel_strip(const StepAr
 
 namespace lbf {
 
-// z-marching variant for 3-D lattices.  A CTA owns a TX x TY column of sites
-// and walks a chunk of A.zc planes.  (Keeping each thread's own populations in
-// shared memory instead of re-reading them was measured slower: the carve-out
-// takes the L1 space that serves the overlapping footprint pulls.)  The density deviation of each plane is
-// computed once on the column's footprint (halo H in x and y) into a ring of
-// 2H+1 planes in shared memory, the Laplacian (Guo force) into a ring of 3
-// planes, so every footprint value is formed once per chunk instead of once
-// per tile, and the collision of plane z follows two planes behind.
-template <class L, int CP, class Real, int TX, int TY, int MINB, int MODE>
-__global__ void __launch_bounds__(TX* TY, MINB)
-    step_kernel_z(const StepArgs<Real> A) {
+// z-marching variant for the fully relaxed Guo path (every mode at tau = 1,
+// FP32), any sides.  A CTA owns a TX x TY column of sites and walks a chunk of
+// A.zc planes.  The density deviation of each plane is computed once on the
+// column's footprint (halo H in x and y) into a ring of planes in shared memory,
+// the Laplacian into a ring of 4, so every footprint value is formed once per
+// chunk, and the collision follows H + 1 planes behind.  The footprint pass also
+// sums the momentum of the column's own sites, which with the density is all
+// that the collision needs.
+template <class L, int TX, int TY, int MINB>
+__global__ void __launch_bounds__(TX* TY, MINB) step_kernel_z(const StepArgs<float> A) {
+    using Real = float;
     static_assert(L::D == 3, "z-marching is for 3-D lattices");
-    static_assert(CP == GUO, "the z-marching kernel implements the Guo-forced coupling");
-    constexpr bool BGK_ONLY = MODE >= 1;
-    constexpr bool TAU1 = MODE == 2;
     constexpr int Q = L::Q;
-    constexpr int H = HaloOf<L, CP>::H;
+    constexpr int H = HaloOf<L, GUO>::H;
     constexpr int SX = TX + 2 * H, SY = TY + 2 * H, SP = SX * SY;     // rho footprint plane
     // One barrier per plane: the collision trails the density by H + 1 planes,
     // so the Laplacian planes it reads were written before the iteration's
     // barrier.  Ring sizes: rho planes zz-2..zz are read by the Laplacian while a
-    // thread past the barrier may already write plane zz+1 (4 slots); Laplacian
-    // planes zz-4..zz-2 are read by the collision while plane zz-1 is written (4).
-    // PULLFREE (every mode fully relaxed): the collision needs only the conserved
-    // moments of the site, which the footprint pass already sums; they are kept
-    // in a ring (sj, with the density in srho) instead of pulling the site again.
-    // The collided plane zz - 3 then stays live while plane zz + 1 is written: 5 slots.
-    constexpr bool PULLFREE = MODE == 2;
-    constexpr int NR = PULLFREE ? 5 : 4;                              // rho ring planes
+    // thread past the barrier may already write plane zz+1, and the collided plane
+    // zz - 3 stays live meanwhile (5 slots); Laplacian planes zz-4..zz-2 are read
+    // by the collision while plane zz-1 is written (4).
+    constexpr int NR = 5;                                             // rho ring planes
     constexpr int LX = TX + 2, LY = TY + 2, LP = LX * LY;             // Laplacian plane
     constexpr int NL = 4;
     constexpr int NT = TX * TY;
     __shared__ Real srho[NR * SP];
     __shared__ Real slap[NL * LP];
-    __shared__ Real sj[PULLFREE ? NR * 3 * NT : 1];
+    __shared__ Real sj[NR * 3 * NT];
 
     const int4 tl = A.tiles[blockIdx.x];
     const SysDev& S = A.sys[tl.x];
@@ -790,43 +783,28 @@ __global__ void __launch_bounds__(TX* TY, MINB)
     const int tx = tid % TX, ty = tid / TX;
     const int x = tl.y + tx, y = tl.z + ty;
     const bool valid_xy = x < nx && y < ny;
-
-    // footprint of plane zz: the density at the tile + halo H sites, from the
-    // populations pulled to them; thread tid handles footprint sites tid + s NT
     const bool sm = S.small != 0;
-    auto foot_site = [&](int idx, int zz, int& gxw, int& gyw, int& wz) {
-        const int px = idx % SX, py = idx / SX;
-        const int gx = tl.y + px - H, gy = tl.z + py - H;
-        if (!(gx < nx + H && gy < ny + H)) return false;
-        gxw = sm ? wrapm(gx, nx) : wrap2(gx, nx);
-        gyw = sm ? wrapm(gy, ny) : wrap2(gy, ny);
-        wz = sm ? wrapm(zz, nz) : wrap2(zz, nz);
-        return true;
-    };
 
     // rho planes z0 - H .. z1 + H - 1, Laplacian planes z0 - 1 .. z1, collisions z0 .. z1 - 1
     for (int zz = z0 - H; zz <= z1 + H; ++zz) {
         const int zc = zz - H - 1;
-        const bool collide = zc >= z0 && valid_xy;
         if (zz < z1 + H) {
             const int slot = (zz - z0 + 2 * NR) % NR;
             for (int idx = tid; idx < SP; idx += NT) {
-                int gxw, gyw, wz;
+                const int px = idx % SX, py = idx / SX;
+                const int gx = tl.y + px - H, gy = tl.z + py - H;
                 Real v = Real(0);
-                if (foot_site(idx, zz, gxw, gyw, wz)) {
-                    const Nbr nb(gxw, gyw, wz, nx, ny, nz, true);
+                if (gx < nx + H && gy < ny + H) {
+                    const Nbr nb(sm ? wrapm(gx, nx) : wrap2(gx, nx), sm ? wrapm(gy, ny) : wrap2(gy, ny),
+                                 sm ? wrapm(zz, nz) : wrap2(zz, nz), nx, ny, nz, true);
                     Real g[Q];
                     pull_site<L, Real>(fb, N, nb, g);
                     sfor<0, Q>([&](auto I) { v += g[decltype(I)::value]; });
-                    if constexpr (PULLFREE) {
-                        const int px = idx % SX - H, py = idx / SX - H;
-                        if (px >= 0 && px < TX && py >= 0 && py < TY) {
-                            Real jm[3];
-                            momentum_of<L, Real>(g, jm);
-                            sfor<0, 3>([&](auto A) {
-                                sj[(slot * 3 + int(A)) * NT + py * TX + px] = jm[decltype(A)::value];
-                            });
-                        }
+                    const int ix = px - H, iy = py - H;
+                    if (ix >= 0 && ix < TX && iy >= 0 && iy < TY) {
+                        Real jm[3];
+                        momentum_of<L, Real>(g, jm);
+                        sfor<0, 3>([&](auto C) { sj[(slot * 3 + int(C)) * NT + iy * TX + ix] = jm[decltype(C)::value]; });
                     }
                 }
                 srho[slot * SP + idx] = v;
@@ -848,31 +826,16 @@ __global__ void __launch_bounds__(TX* TY, MINB)
             }
         }
         // collision of plane zc = zz - H - 1
-        if (collide) {
-            Real f[Q];
-            Real drho = Real(0);
-            Real jc[3];
+        if (zc >= z0 && valid_xy) {
+            Real f[Q], jc[3];
             const int cslot = (zc - z0 + 2 * NR) % NR;
-            if constexpr (PULLFREE) {
-                drho = srho[cslot * SP + (ty + H) * SX + (tx + H)];
-                sfor<0, 3>([&](auto A) { jc[decltype(A)::value] = sj[(cslot * 3 + int(A)) * NT + tid]; });
-            } else {
-                pull_site<L, Real>(fb, N, Nbr(x, y, zc, nx, ny, nz, true), f);
-                sfor<0, Q>([&](auto I) { drho += f[decltype(I)::value]; });
-            }
+            const Real drho = srho[cslot * SP + (ty + H) * SX + (tx + H)];
+            sfor<0, 3>([&](auto C) { jc[decltype(C)::value] = sj[(cslot * 3 + int(C)) * NT + tid]; });
             const int site = site_index(x, y, zc, nx, ny);
-            // the Guo collision reads only the Laplacian planes zc-1..zc+1 around the
-            // site (a 3-plane view); the density view is unused by this coupling
-            const RingView<Real, SX> rv{srho, 0, 0, 0, (ty + H) * SX + (tx + H)};
             const RingView<Real, LX> lv{slap, ((zc - 1 - z0 + 2 * NL) % NL) * LP, ((zc - z0 + 2 * NL) % NL) * LP,
                                         ((zc + 1 - z0 + 2 * NL) % NL) * LP, (ty + 1) * LX + (tx + 1)};
-            if constexpr (PULLFREE)
-                collide_d3q19_tau1<Real>(f, drho, jc[0], jc[1], jc[2], lv, A.phys[tl.x], noise_key(S, step),
-                                         uint32_t(site), A.status);
-            else if constexpr (BGK_ONLY)
-                collide_guo_bgk<L, Real, TAU1>(f, drho, lv, S, A.phys[tl.x], uint32_t(site), step, A.status);
-            else
-                collide_site<L, CP, Real, BGK_ONLY>(f, drho, rv, lv, S, A.phys[tl.x], uint32_t(site), step, A.status);
+            collide_d3q19_tau1<Real>(f, drho, jc[0], jc[1], jc[2], lv, A.phys[tl.x], noise_key(S, step),
+                                     uint32_t(site), A.status);
             sfor<0, Q>([&](auto I) {
                 constexpr int i = I;
                 fo[i * N + site] = f[i];

@@ -76,4 +76,4 @@ def test_default_rows_of_small_and_odd_ensembles():
 
     assert scheme(16, 1)[5] == 4 and scheme(64, 1)[5] == 4 and scheme(27, 40)[5] == 4
     assert scheme(64, 16)[5] == 3 and scheme(64, 32)[:3] == rows[0][:3]
-    assert scheme(16, 1, tau=0.8)[5] != 4
+    assert scheme(16, 1, tau=0.8)[5] == 4
