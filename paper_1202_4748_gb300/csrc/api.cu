@@ -14,6 +14,8 @@
 #include <utility>
 #include <vector>
 
+#include <unistd.h>
+
 #include <nvtx3/nvToolsExt.h>
 
 #include "../../include/lbfluct.h"
@@ -47,7 +49,7 @@ struct SysHost {
 // Byte offsets of every region inside the workspace.
 struct Plan {
     size_t sys, phys, tiles, pop0, pop1, step, status, d, dbar, site_items, site_partial, spans, glob, levels,
-        S, E, bottom_items, part_items, block_items, parts, up_items, tops, rec, acc, hist, field_tmp, sk_sys, sk_tw, sk_acc, sk_b0, sk_b1, sk_bins, jk_j,
+        S, E, bottom_items, part_items, block_items, parts, up_items, tops, rec, acc, hist, sk_meta, sk_sys, sk_tw, sk_acc, sk_b0, sk_b1, sk_bins, jk_j,
         jk_lap, jk_F, jk_acc, mom, total;
     int tdim[3] = {0, 0, 0};      // tile shape of the step kernel
     bool split = false, narrow = false;   // D3Q19: the split step (in 8 x 8 columns)
@@ -55,7 +57,7 @@ struct Plan {
     int hist_bins = 0;
     double hist_range = 0.0;
     int n_tiles = 0, n_site_items = 0, n_levels = 0, n_bottom = 0, n_up = 0, n_rec = 0, max_depth = 0;
-    int64_t n_sites = 0, n_blocks_pyr = 0, max_sites = 0;
+    int64_t n_sites = 0, n_blocks_pyr = 0;
     std::vector<int4> tiles_h, site_items_h;
     std::vector<SysSpan> spans_h;
     std::vector<LevelDev> levels_h;
@@ -331,7 +333,6 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
         h.lv = make_levels(s[k], h.imax, h.unit_sep);
         h.lv_first = lv_count;
         lv_count += int(h.lv.size());
-        P.max_sites = std::max(P.max_sites, h.n);
     }
     P.n_sites = site_off;
     P.n_levels = lv_count;
@@ -565,7 +566,7 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
     P.hist_bins = o->hist_bins;
     P.hist_range = o->hist_range;
     P.hist = take(sizeof(uint64_t) * (P.hist_bins > 0 ? (P.hist_bins + 2) * int64_t(P.n_levels) : 0));
-    P.field_tmp = take(sizeof(double) * P.max_sites);
+    P.sk_meta = take(sizeof(int) * 2 * P.tw_sides.size());
     const int64_t skn = P.sk ? P.n_sites : 0;
     P.sk_sys = take(sizeof(SkSys) * (P.sk ? n : 0));
     P.sk_tw = take(sizeof(double) * 2 * P.tw_total);
@@ -952,6 +953,32 @@ lb_status lb_workspace_bytes(const lb_system_desc* systems, int n_systems, const
     *bytes = P.total;
     return LB_OK;
 }
+// Field transfers stage FP64 populations in the population buffer that the next
+// step will write, which between steps holds nothing (the step reads the other
+// one): as many populations of an n-site system at once as fit, at least one
+// (4 q n_sites >= 8 n: q >= 9).
+int staged_populations(const lb_ctx* c, int64_t n) {
+    const int64_t room = int64_t(c->fp32 ? 4 : 8) * c->q * c->P.n_sites / (8 * n);
+    return int(std::min<int64_t>(room, c->q));
+}
+
+// Writes a byte of every page of an output buffer, so that its pages exist
+// before the device copies into them: a copy into untouched pageable memory
+// takes a fault of the device's address translation per page (64^3 populations
+// into a fresh array: 32 ms; touched first, 3.2 ms).  Only plain host memory.
+void touch_pages(void* p, size_t bytes) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    if (at.type != cudaMemoryTypeUnregistered) return;
+    const size_t page = size_t(sysconf(_SC_PAGESIZE));
+    volatile char* q = static_cast<volatile char*>(p);
+    for (size_t i = 0; i < bytes; i += page) q[i] = 0;
+    if (bytes) q[bytes - 1] = 0;
+}
+
 
 lb_status lb_create(const lb_system_desc* systems, int n_systems, const lb_run_opts* opts, void* d_workspace,
                     size_t bytes, void* stream, lb_ctx** out) {
@@ -1037,10 +1064,10 @@ lb_status lb_create(const lb_system_desc* systems, int n_systems, const lb_run_o
     if (P.sk) {
         ok = ok && cudaMemcpyAsync(c->ws + P.sk_sys, P.sk_h.data(), sizeof(SkSys) * P.sk_h.size(),
                                    cudaMemcpyHostToDevice, c->stream) == cudaSuccess;
-        // twiddle tables: sides and offsets staged through the bin scratch (ints fit in it)
+        // twiddle tables from their sides and offsets
         std::vector<int> meta(P.tw_sides);
         meta.insert(meta.end(), P.tw_offs.begin(), P.tw_offs.end());
-        int* dmeta = reinterpret_cast<int*>(c->ws + P.field_tmp);
+        int* dmeta = c->at<int>(P.sk_meta);
         ok = ok && cudaMemcpyAsync(dmeta, meta.data(), sizeof(int) * meta.size(), cudaMemcpyHostToDevice,
                                    c->stream) == cudaSuccess;
         ok = ok && launch_sk_twiddles(c->at<double>(P.sk_tw), dmeta, dmeta + P.tw_sides.size(),
@@ -1544,14 +1571,16 @@ lb_status lb_read_fields(lb_ctx* c, int sys, double* h_f) {
     if (!c || !h_f || sys < 0 || sys >= c->n_sys) return LB_ERR_ARG;
     if (!c->has_state) return LB_ERR_STATE;
     const SysHost& h = c->sys[sys];
-    const int buf = int(c->step & 1);
-    double* tmp = c->at<double>(c->P.field_tmp);
-    for (int i = 0; i < c->q; ++i) {
-        LB_CHECK(c->lattice == LB_D2Q9
-                     ? launch_gather_d2q9(c->fp32, c->at<SysDev>(c->P.sys), sys, i, h.n, c->pop(buf), tmp, c->stream)
-                     : launch_gather_d3q19(c->fp32, c->at<SysDev>(c->P.sys), sys, i, h.n, c->pop(buf), tmp,
-                                           c->stream));
-        LB_CHECK(cudaMemcpyAsync(h_f + int64_t(i) * h.n, tmp, sizeof(double) * h.n, cudaMemcpyDeviceToHost,
+    const int buf = int(c->step & 1), batch = staged_populations(c, h.n);
+    double* tmp = static_cast<double*>(c->pop(1 - buf));
+    touch_pages(h_f, sizeof(double) * c->q * size_t(h.n));
+    for (int i = 0; i < c->q; i += batch) {
+        const int ni = std::min(batch, c->q - i);
+        LB_CHECK(c->lattice == LB_D2Q9 ? launch_gather_d2q9(c->fp32, c->at<SysDev>(c->P.sys), sys, i, ni, h.n,
+                                                            c->pop(buf), tmp, c->stream)
+                                       : launch_gather_d3q19(c->fp32, c->at<SysDev>(c->P.sys), sys, i, ni, h.n,
+                                                             c->pop(buf), tmp, c->stream));
+        LB_CHECK(cudaMemcpyAsync(h_f + int64_t(i) * h.n, tmp, sizeof(double) * ni * h.n, cudaMemcpyDeviceToHost,
                                  c->stream));
     }
     LB_CHECK(cudaStreamSynchronize(c->stream));
@@ -1561,15 +1590,16 @@ lb_status lb_read_fields(lb_ctx* c, int sys, double* h_f) {
 lb_status lb_write_fields(lb_ctx* c, int sys, const double* h_f) {
     if (!c || !h_f || sys < 0 || sys >= c->n_sys) return LB_ERR_ARG;
     const SysHost& h = c->sys[sys];
-    const int buf = int(c->step & 1);
-    double* tmp = c->at<double>(c->P.field_tmp);
-    for (int i = 0; i < c->q; ++i) {
-        LB_CHECK(cudaMemcpyAsync(tmp, h_f + int64_t(i) * h.n, sizeof(double) * h.n, cudaMemcpyHostToDevice,
+    const int buf = int(c->step & 1), batch = staged_populations(c, h.n);
+    double* tmp = static_cast<double*>(c->pop(1 - buf));
+    for (int i = 0; i < c->q; i += batch) {
+        const int ni = std::min(batch, c->q - i);
+        LB_CHECK(cudaMemcpyAsync(tmp, h_f + int64_t(i) * h.n, sizeof(double) * ni * h.n, cudaMemcpyHostToDevice,
                                  c->stream));
-        LB_CHECK(c->lattice == LB_D2Q9
-                     ? launch_scatter_d2q9(c->fp32, c->at<SysDev>(c->P.sys), sys, i, h.n, tmp, c->pop(buf), c->stream)
-                     : launch_scatter_d3q19(c->fp32, c->at<SysDev>(c->P.sys), sys, i, h.n, tmp, c->pop(buf),
-                                            c->stream));
+        LB_CHECK(c->lattice == LB_D2Q9 ? launch_scatter_d2q9(c->fp32, c->at<SysDev>(c->P.sys), sys, i, ni, h.n, tmp,
+                                                             c->pop(buf), c->stream)
+                                       : launch_scatter_d3q19(c->fp32, c->at<SysDev>(c->P.sys), sys, i, ni, h.n, tmp,
+                                                              c->pop(buf), c->stream));
     }
     LB_CHECK(cudaMemsetAsync(c->ws + c->P.status, 0, sizeof(int), c->stream));
     LB_CHECK(cudaStreamSynchronize(c->stream));

@@ -72,15 +72,15 @@ cudaError_t launch_init_feq_d2q9(int coupling, int fp32, const SysDev* sys, cons
     return fp32 ? init_feq_any<D2Q9, float>(coupling, sys, items, n_items, d, dbar, fbuf, st)
                 : init_feq_any<D2Q9, double>(coupling, sys, items, n_items, d, dbar, fbuf, st);
 }
-cudaError_t launch_gather_d2q9(int fp32, const SysDev* sys, int s, int i, int64_t n, const void* fbuf, double* out,
+cudaError_t launch_gather_d2q9(int fp32, const SysDev* sys, int s, int i0, int ni, int64_t n, const void* fbuf, double* out,
                                cudaStream_t st) {
-    return fp32 ? gather_any<D2Q9, float>(sys, s, i, n, fbuf, out, st)
-                : gather_any<D2Q9, double>(sys, s, i, n, fbuf, out, st);
+    return fp32 ? gather_any<D2Q9, float>(sys, s, i0, ni, n, fbuf, out, st)
+                : gather_any<D2Q9, double>(sys, s, i0, ni, n, fbuf, out, st);
 }
-cudaError_t launch_scatter_d2q9(int fp32, const SysDev* sys, int s, int i, int64_t n, const double* in, void* fbuf,
+cudaError_t launch_scatter_d2q9(int fp32, const SysDev* sys, int s, int i0, int ni, int64_t n, const double* in, void* fbuf,
                                 cudaStream_t st) {
-    return fp32 ? scatter_any<D2Q9, float>(sys, s, i, n, in, fbuf, st)
-                : scatter_any<D2Q9, double>(sys, s, i, n, in, fbuf, st);
+    return fp32 ? scatter_any<D2Q9, float>(sys, s, i0, ni, n, in, fbuf, st)
+                : scatter_any<D2Q9, double>(sys, s, i0, ni, n, in, fbuf, st);
 }
 cudaError_t launch_obs_site_d2q9(int fp32, const SysDev* sys, const int4* items, int n_items, const void* fbuf,
                                  double* d, double* partial, double* jout, int64_t jstride, cudaStream_t st) {

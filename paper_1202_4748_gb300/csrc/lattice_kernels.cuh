@@ -133,14 +133,9 @@ __global__ void __launch_bounds__(AUX_THREADS)
     }
 }
 
-// out[site] = f_i(r, t) = buf_i(r - c_i) + rho_c [i == 0], one population.
-template <class L, class Real>
-__global__ void __launch_bounds__(AUX_THREADS)
-    gather_kernel(const SysDev* __restrict__ sysv, int sys, int i, const Real* __restrict__ fbuf,
-                  double* __restrict__ out) {
-    const SysDev& S = sysv[sys];
-    const int64_t site = int64_t(blockIdx.x) * AUX_THREADS + threadIdx.x;
-    if (site >= S.n_sites) return;
+// Element of population i that the pull of site `site` reads: buf_i(r - c_i).
+template <class L>
+__device__ __forceinline__ int64_t pulled_element(const SysDev& S, int site, int i) {
     int x, y, z;
     site_coords(int(site), S.nx, S.ny, x, y, z);
     int cx = 0, cy = 0, cz = 0;
@@ -152,31 +147,34 @@ __global__ void __launch_bounds__(AUX_THREADS)
             cz = L::c(q, 2);
         }
     const int sx = wrapm(x - cx, S.nx), sy = wrapm(y - cy, S.ny), sz = wrapm(z - cz, S.nz);
-    const double v = double(fbuf[S.pop_offset + int64_t(i) * S.n_sites + (sx + S.nx * (sy + S.ny * sz))]);
-    out[site] = v + (i == 0 ? S.rho_c : 0.0);
+    return S.pop_offset + int64_t(i) * S.n_sites + (sx + S.nx * (sy + S.ny * sz));
+}
+
+// out[k][site] = f_i(r, t) = buf_i(r - c_i) + rho_c [i == 0] for the populations
+// i = i0 + k, k the CTA's y index.
+template <class L, class Real>
+__global__ void __launch_bounds__(AUX_THREADS)
+    gather_kernel(const SysDev* __restrict__ sysv, int sys, int i0, const Real* __restrict__ fbuf,
+                  double* __restrict__ out) {
+    const SysDev& S = sysv[sys];
+    const int64_t site = int64_t(blockIdx.x) * AUX_THREADS + threadIdx.x;
+    if (site >= S.n_sites) return;
+    const int i = i0 + blockIdx.y;
+    const double v = double(fbuf[pulled_element<L>(S, int(site), i)]);
+    out[int64_t(blockIdx.y) * S.n_sites + site] = v + (i == 0 ? S.rho_c : 0.0);
 }
 
 // buf_i(r - c_i) = f_i(r) - rho_c [i == 0], one population.
 template <class L, class Real>
 __global__ void __launch_bounds__(AUX_THREADS)
-    scatter_kernel(const SysDev* __restrict__ sysv, int sys, int i, const double* __restrict__ in,
+    scatter_kernel(const SysDev* __restrict__ sysv, int sys, int i0, const double* __restrict__ in,
                    Real* __restrict__ fbuf) {
     const SysDev& S = sysv[sys];
     const int64_t site = int64_t(blockIdx.x) * AUX_THREADS + threadIdx.x;
     if (site >= S.n_sites) return;
-    int x, y, z;
-    site_coords(int(site), S.nx, S.ny, x, y, z);
-    int cx = 0, cy = 0, cz = 0;
-#pragma unroll
-    for (int q = 0; q < L::Q; ++q)
-        if (q == i) {
-            cx = L::c(q, 0);
-            cy = L::c(q, 1);
-            cz = L::c(q, 2);
-        }
-    const int sx = wrapm(x - cx, S.nx), sy = wrapm(y - cy, S.ny), sz = wrapm(z - cz, S.nz);
-    fbuf[S.pop_offset + int64_t(i) * S.n_sites + (sx + S.nx * (sy + S.ny * sz))] =
-        Real(in[site] - (i == 0 ? S.rho_c : 0.0));
+    const int i = i0 + blockIdx.y;
+    fbuf[pulled_element<L>(S, int(site), i)] =
+        Real(in[int64_t(blockIdx.y) * S.n_sites + site] - (i == 0 ? S.rho_c : 0.0));
 }
 
 // Compensated sum (Knuth's TwoSum): s + c carries the exact sum of the added

@@ -218,16 +218,16 @@ cudaError_t init_feq_any(int coupling, const SysDev* sys, const int4* items, int
 }
 
 template <class L, class Real>
-cudaError_t gather_any(const SysDev* sys, int s, int i, int64_t n, const void* fbuf, double* out, cudaStream_t st) {
-    const unsigned grid = unsigned((n + AUX_THREADS - 1) / AUX_THREADS);
-    gather_kernel<L, Real><<<grid, AUX_THREADS, 0, st>>>(sys, s, i, static_cast<const Real*>(fbuf), out);
+cudaError_t gather_any(const SysDev* sys, int s, int i0, int ni, int64_t n, const void* fbuf, double* out, cudaStream_t st) {
+    const dim3 grid(unsigned((n + AUX_THREADS - 1) / AUX_THREADS), unsigned(ni));
+    gather_kernel<L, Real><<<grid, AUX_THREADS, 0, st>>>(sys, s, i0, static_cast<const Real*>(fbuf), out);
     return cudaGetLastError();
 }
 
 template <class L, class Real>
-cudaError_t scatter_any(const SysDev* sys, int s, int i, int64_t n, const double* in, void* fbuf, cudaStream_t st) {
-    const unsigned grid = unsigned((n + AUX_THREADS - 1) / AUX_THREADS);
-    scatter_kernel<L, Real><<<grid, AUX_THREADS, 0, st>>>(sys, s, i, in, static_cast<Real*>(fbuf));
+cudaError_t scatter_any(const SysDev* sys, int s, int i0, int ni, int64_t n, const double* in, void* fbuf, cudaStream_t st) {
+    const dim3 grid(unsigned((n + AUX_THREADS - 1) / AUX_THREADS), unsigned(ni));
+    scatter_kernel<L, Real><<<grid, AUX_THREADS, 0, st>>>(sys, s, i0, in, static_cast<Real*>(fbuf));
     return cudaGetLastError();
 }
 

@@ -50,13 +50,14 @@ cudaError_t launch_init_feq_d2q9(int coupling, int fp32, const SysDev* sys, cons
                                  const double* d, const double* dbar, void* fbuf, cudaStream_t st);
 cudaError_t launch_init_feq_d3q19(int coupling, int fp32, const SysDev* sys, const int4* items, int n_items,
                                   const double* d, const double* dbar, void* fbuf, cudaStream_t st);
-cudaError_t launch_gather_d2q9(int fp32, const SysDev* sys, int s, int i, int64_t n, const void* fbuf, double* out,
+// Populations i0 .. i0 + ni - 1 of one system, [population][site] in out / in.
+cudaError_t launch_gather_d2q9(int fp32, const SysDev* sys, int s, int i0, int ni, int64_t n, const void* fbuf, double* out,
                                cudaStream_t st);
-cudaError_t launch_gather_d3q19(int fp32, const SysDev* sys, int s, int i, int64_t n, const void* fbuf, double* out,
+cudaError_t launch_gather_d3q19(int fp32, const SysDev* sys, int s, int i0, int ni, int64_t n, const void* fbuf, double* out,
                                 cudaStream_t st);
-cudaError_t launch_scatter_d2q9(int fp32, const SysDev* sys, int s, int i, int64_t n, const double* in, void* fbuf,
+cudaError_t launch_scatter_d2q9(int fp32, const SysDev* sys, int s, int i0, int ni, int64_t n, const double* in, void* fbuf,
                                 cudaStream_t st);
-cudaError_t launch_scatter_d3q19(int fp32, const SysDev* sys, int s, int i, int64_t n, const double* in, void* fbuf,
+cudaError_t launch_scatter_d3q19(int fp32, const SysDev* sys, int s, int i0, int ni, int64_t n, const double* in, void* fbuf,
                                  cudaStream_t st);
 // jout (nullable): momentum field j_a at jout + a * jstride.
 cudaError_t launch_obs_site_d2q9(int fp32, const SysDev* sys, const int4* items, int n_items, const void* fbuf,
