@@ -380,17 +380,18 @@ lb_status lb_load(lb_ctx* ctx, const char* path);
  * sites (x sites per tile) of y rows, densities in registers and warp
  * shuffles, 3 = (paired D3Q19 kernel) producers stage their 16-byte quads of
  * pulled populations in shared memory with cp.async instead of holding them
- * in registers, 4 = (D3Q19) split step: one kernel forms the density and
- * momentum of every site, a second collides tile columns with two sites stacked
- * in z per thread (on D3Q19, FP64 runs and runs with a relaxation time other
- * than 1 take the split step whatever the row, in 16 x 8 columns with the row's
- * z-chunk); sites per thread: 1, or 2 = two x-adjacent sites per thread
+ * in registers; sites per thread: 1, or 2 = two x-adjacent sites per thread
  * with paired FP32 arithmetic (D3Q19: per consumer thread of the
  * warp-specialised kernel; D2Q9: per lane of 64-site strips, every mode at
  * tau = 1), when the run is FP32 and every system has nx % 4 == 0, else the
  * one-site kernel of the same tile runs)
  * into out (nullable) and returns the number of variants (negative lb_status
  * on error).
+ * D3Q19 rows of 16 x 8 tiles with 4 resident CTAs are the split step: one
+ * kernel forms the density and momentum of every site, a second collides the
+ * tile columns (in FP32 two sites stacked in z per thread).  On D3Q19, FP64 runs
+ * and runs with a relaxation time other than 1 take the split step whatever the
+ * row, in 16 x 8 columns with the row's z-chunk.
  * Row 0 is the default; where the coupling cannot run it (scheme 2 with the
  * Guo form) the first row it can run is.  Selecting a row the coupling cannot
  * run gives LB_ERR_UNSUPPORTED.  Used by the autotuner; no device call. */

@@ -52,7 +52,7 @@ struct Plan {
         S, E, bottom_items, part_items, block_items, parts, up_items, tops, rec, acc, hist, sk_meta, sk_sys, sk_tw, sk_acc, sk_b0, sk_b1, sk_bins, jk_j,
         jk_lap, jk_F, jk_acc, mom, total;
     int tdim[3] = {0, 0, 0};      // tile shape of the step kernel
-    bool split = false, narrow = false;   // D3Q19: the split step (in 8 x 8 columns)
+    bool split = false;           // D3Q19: the split step
     bool jk = false;
     int hist_bins = 0;
     double hist_range = 0.0;
@@ -193,8 +193,7 @@ int sm_count() {
     return sms;
 }
 
-// Default variant: among the rows that differ from the default row only in
-// the z-chunk, the longest chunk whose CTAs still fill the GPU at least twice
+// Among the rows that differ from the default row only in the z-chunk, the longest chunk whose CTAs still fill the GPU at least twice
 // over (resident CTAs per SM x SMs), else the row given.  Longer chunks re-read fewer
 // halo planes (4 per chunk; 2 for the modified equilibrium on D3Q19), but
 // too few CTAs leave SMs idle in the last
@@ -236,7 +235,7 @@ SplitCost split_cost(int kind, bool quads) {
 //  * paired kernel (staging 3): a resident CTA advances one plane per 1.53 us
 //    alone on its SM, 2.2 us beside one other, 3.1 us beside two; zc planes
 //    plus the halo planes of its chunk; CTAs in waves of 3 per SM.
-//  * split step: SplitCost; an 8 x 8 column occupies its SM half as long.
+//  * split step: SplitCost.
 // Measured against the 32- and 64-plane paired rows that were the default of
 // every ensemble: 16^3 28.9 -> 5.3 us, 64^3 52 -> 14.4, 4 x 64^3 55 -> 46,
 // 16 x 64^3 157 -> 147 us per step; 2.6 M sites with odd sides 332 -> 137 us;
@@ -259,7 +258,7 @@ double estimated_step_us(const lb_system_desc* s, int n, const int tdim[3], bool
         return 3.0 + per * (3.1 * full + plane_us[int(std::ceil(rest / sms))]);
     }
     const SplitCost c = split_cost(kind, quads);
-    const double cost = (c.plane * planes + c.chunk) * (tdim[0] == 8 ? 0.5 : 1.0);
+    const double cost = c.plane * planes + c.chunk;
     const double load = ctas / sms, filled = load <= 4.0 ? std::ceil(load) : load + 0.5;
     return 3.0 + sites * c.moment + std::max(c.alone_chunk + c.alone_plane * planes, filled * cost);
 }
@@ -276,10 +275,44 @@ void choose_d3q19_row(const lb_system_desc* s, int n, int kind, bool quads, int&
     double best_us = INFINITY;
     for (int k = 0; k < nt; ++k) {
         const bool paired = t[k][5] == 3 && t[k][0] == t[0][0] && quads && kind == 0;
-        const bool split = t[k][5] == 4 && (kind == 0 || t[k][0] == 16);
-        if (!paired && !split) continue;
+        if (!paired && !split_row(t[k])) continue;
         const double us = estimated_step_us(s, n, t[k], paired, kind, sms, quads);
         if (us < best_us) {
+            best_us = us;
+            tile_id = k;
+        }
+    }
+}
+
+// Default row of the D2Q9 row-marching strips (modified equilibrium): the
+// number of rows per strip from the estimated step time, rows 0 (32 rows), 1
+// (16) and the shorter ones of the same kernel.  A strip forms the density of
+// two halo rows more than it collides.  A warp of paired FP32 strips takes
+// 0.9 us per row alone on its scheduler, 1.3 beside one other, 1.8 beside two
+// (3 CTAs of 4 warps per SM); the one-site strips (two warps per tile) keep 5
+// CTAs; an FP64 row occupies its SM's FP64 unit for 1.6 us, and CTAs of 4 warps
+// are dealt to the SMs.  32 rows were the default of every ensemble: one 512^2
+// system 33 -> 8 us per step in FP32; in FP64, 64 CTAs on 152 SMs, 293 -> 128.
+void choose_d2q9_row(const lb_system_desc* s, int n, bool fp32, bool paired, int& tile_id) {
+    const int sms = sm_count();
+    int t[32][kVariantCols];
+    const int nt = tile_table(LB_D2Q9, t);
+    const int first = tile_id;
+    constexpr double row_us[6] = {0.0, 0.9, 1.3, 1.8, 1.8, 1.85};      // by warps per scheduler
+    double best_us = INFINITY;
+    for (int k = 0; k < nt; ++k) {
+        if (t[k][5] != 2 || t[k][0] != t[first][0] || t[k][3] != t[first][3] || t[k][1] > t[first][1]) continue;
+        const double warps = double(tiles_of(s, n, t[k])) * (paired ? 1 : 2), rows = t[k][1];
+        double us;
+        if (fp32) {
+            const int ctas = paired ? 3 : 5;
+            const double slots = 4.0 * ctas * sms, full = std::floor(warps / slots), rest = warps - full * slots;
+            us = (rows + 2) * (row_us[ctas] * full + row_us[int(std::ceil(rest / (4.0 * sms)))]);
+        } else {
+            const double ctas = std::ceil(warps / (4.0 * sms));
+            us = std::max(4.0 * ctas * (1.6 * rows + 0.4), 4.0 * (rows + 2));
+        }
+        if (us < 0.98 * best_us) {
             best_us = us;
             tile_id = k;
         }
@@ -301,7 +334,7 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
     if (st != LB_OK) return st;
     if (o->variant == 0 && o->tile[0] <= 0 && o->occupancy <= 0) {
         if (d3) choose_d3q19_row(s, n, !fp32 ? 2 : (relaxed ? 0 : 1), quads, tile_id);
-        else prefer_longer_chunk(s, n, sm_count(), tile_id);
+        else if (s[0].coupling == LB_MODEQ) choose_d2q9_row(s, n, fp32, fp32 && relaxed && quads, tile_id);
     }
     int tdim[3];
     {
@@ -310,9 +343,8 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
         for (int k = 0; k < 3; ++k) tdim[k] = t[tile_id][k];
         // the split step: its own rows, and every D3Q19 run that the marching
         // kernels are not compiled for (FP64, other rates), in 16 x 8 columns
-        P.split = d3 && (t[tile_id][5] == 4 || !fp32 || !relaxed);
-        P.narrow = P.split && t[tile_id][5] == 4 && tdim[0] == 8 && fp32 && relaxed;
-        if (P.split && !P.narrow) {
+        P.split = d3 && (split_row(t[tile_id]) || !fp32 || !relaxed);
+        if (P.split) {
             tdim[0] = 16;
             tdim[1] = 8;
         }
@@ -537,7 +569,9 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
     };
     P.sys = take(sizeof(SysDev) * n);
     P.phys = take(sizeof(SysPhys<double>) * n);
-    P.tiles = take(sizeof(int4) * P.n_tiles);
+    // (room for the shortest default tiles, so that the layout does not depend on the choice)
+    const int short_tile[3] = {d3 ? 16 : 64, d3 ? 8 : 4, d3 ? 2 : 1};
+    P.tiles = take(sizeof(int4) * std::max<int64_t>(P.n_tiles, tiles_of(s, n, short_tile)));
     P.pop0 = take(es * q * P.n_sites);
     P.pop1 = take(es * q * P.n_sites);
     P.step = take(sizeof(int64_t));
@@ -554,7 +588,7 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
     P.d = take(sizeof(double) * P.n_sites);
     P.S = take(sizeof(double) * P.n_blocks_pyr);
     P.E = take(sizeof(double) * P.n_blocks_pyr);
-    if (P.split) off = std::max(off, align_up(P.mom + es * 4 * P.n_sites));
+    if (P.split) off = std::max(off, align_up(P.mom + (fp32 && relaxed ? 16 : es) * P.n_sites));
     P.bottom_items = take(sizeof(ObsItem) * P.n_bottom);
     P.part_items = take(sizeof(ObsPart) * P.part_h.size());
     P.block_items = take(sizeof(ObsBlocks) * P.block_h.size());
@@ -576,12 +610,13 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
     P.sk_b0 = take(sizeof(double) * 2 * (P.sk_fft ? P.half_total * P.n_fields : skn));
     P.sk_b1 = take(sizeof(double) * 2 * (P.sk_fft ? 0 : skn));
     P.sk_bins = take(sizeof(double) * 6 * P.sk_max_bins);
-    // momentum spectra: j (3 fields), Laplacian scratch (Guo), transforms (3 complex fields), accumulators
+    // momentum spectra: j (3 fields), Laplacian scratch (Guo), transforms (3 complex
+    // fields of the direct sums; the layout has them whichever way a side goes), accumulators
     P.jk = P.sk && o->jk_spectra == 1;
     const int64_t jkn = P.jk ? P.n_sites : 0;
     P.jk_j = take(sizeof(double) * 3 * jkn);
     P.jk_lap = take(sizeof(double) * jkn);
-    P.jk_F = take(sizeof(double) * 6 * (P.sk_fft ? 0 : jkn));
+    P.jk_F = take(sizeof(double) * 6 * jkn);
     P.jk_acc = take(sizeof(double) * 3 * jkn);
     P.total = off;
     return LB_OK;
@@ -846,9 +881,8 @@ cudaError_t launch_steps(lb_ctx* c, int64_t n) {
         a.k = int(k);
         a.status = c->at<int>(P.status);
         a.tile_id = c->tile_id;
-        a.zc = P.tdim[2];
+        a.zc = c->lattice == LB_D2Q9 ? P.tdim[1] : P.tdim[2];
         a.split = P.split ? 1 : 0;
-        a.narrow = P.narrow ? 1 : 0;
         a.mom = c->ws + P.mom;
         a.n_sites = P.n_sites;
         a.site_items = c->at<int4>(P.site_items);
@@ -919,6 +953,32 @@ lb_status reset_accumulators(lb_ctx* c) {
     return LB_OK;
 }
 
+// Field transfers stage FP64 populations in the population buffer that the next
+// step will write, which between steps holds nothing (the step reads the other
+// one): as many populations of an n-site system at once as fit, at least one
+// (4 q n_sites >= 8 n: q >= 9).
+int staged_populations(const lb_ctx* c, int64_t n) {
+    const int64_t room = int64_t(c->fp32 ? 4 : 8) * c->q * c->P.n_sites / (8 * n);
+    return int(std::min<int64_t>(room, c->q));
+}
+
+// Writes a byte of every page of an output buffer, so that its pages exist
+// before the device copies into them: a copy into untouched pageable memory
+// takes a fault of the device's address translation per page (64^3 populations
+// into a fresh array: 32 ms; touched first, 2.0 ms).  Only plain host memory.
+void touch_pages(void* p, size_t bytes) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    if (at.type != cudaMemoryTypeUnregistered) return;
+    const size_t page = size_t(sysconf(_SC_PAGESIZE));
+    volatile char* q = static_cast<volatile char*>(p);
+    for (size_t i = 0; i < bytes; i += page) q[i] = 0;
+    if (bytes) q[bytes - 1] = 0;
+}
+
 }  // namespace
 
 extern "C" {
@@ -953,32 +1013,6 @@ lb_status lb_workspace_bytes(const lb_system_desc* systems, int n_systems, const
     *bytes = P.total;
     return LB_OK;
 }
-// Field transfers stage FP64 populations in the population buffer that the next
-// step will write, which between steps holds nothing (the step reads the other
-// one): as many populations of an n-site system at once as fit, at least one
-// (4 q n_sites >= 8 n: q >= 9).
-int staged_populations(const lb_ctx* c, int64_t n) {
-    const int64_t room = int64_t(c->fp32 ? 4 : 8) * c->q * c->P.n_sites / (8 * n);
-    return int(std::min<int64_t>(room, c->q));
-}
-
-// Writes a byte of every page of an output buffer, so that its pages exist
-// before the device copies into them: a copy into untouched pageable memory
-// takes a fault of the device's address translation per page (64^3 populations
-// into a fresh array: 32 ms; touched first, 3.2 ms).  Only plain host memory.
-void touch_pages(void* p, size_t bytes) {
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        cudaGetLastError();
-        return;
-    }
-    if (at.type != cudaMemoryTypeUnregistered) return;
-    const size_t page = size_t(sysconf(_SC_PAGESIZE));
-    volatile char* q = static_cast<volatile char*>(p);
-    for (size_t i = 0; i < bytes; i += page) q[i] = 0;
-    if (bytes) q[bytes - 1] = 0;
-}
-
 
 lb_status lb_create(const lb_system_desc* systems, int n_systems, const lb_run_opts* opts, void* d_workspace,
                     size_t bytes, void* stream, lb_ctx** out) {

@@ -19,31 +19,34 @@ constexpr int kTiles[][kVariantCols] = {{64, 32, 1, 3, 0, 2, 2}, {64, 16, 1, 3, 
                                         {32, 32, 1, 6, 0, 2, 1}, {32, 64, 1, 6, 0, 2, 1}, {32, 16, 1, 6, 0, 2, 1},
                                         {32, 32, 1, 7, 0, 2, 1},
                                         {32, 8, 1, 0, 0, 0, 1},  {64, 4, 1, 0, 0, 0, 1},  {128, 2, 1, 0, 0, 0, 1},
-                                        {32, 4, 1, 0, 0, 0, 1},  {32, 16, 1, 0, 0, 0, 1}, {64, 8, 1, 0, 0, 0, 1}};
+                                        {32, 4, 1, 0, 0, 0, 1},  {32, 16, 1, 0, 0, 0, 1}, {64, 8, 1, 0, 0, 0, 1},
+                                        {64, 8, 1, 3, 0, 2, 2},  {64, 4, 1, 3, 0, 2, 2}};
 constexpr int kNumTiles = int(sizeof(kTiles) / sizeof(kTiles[0]));
 
-template <int CP, class Real, int YC, int MINB>
+template <int CP, class Real, int MINB>
 cudaError_t strip_of(const StepLaunch& a, cudaStream_t st) {
-    if constexpr (CP == MODEQ) return step_strip<D2Q9, CP, Real, YC, 4, MINB>(a, st);
+    if constexpr (CP == MODEQ) return step_strip<D2Q9, CP, Real, 4, MINB>(a, st);
     return cudaErrorInvalidValue;            // the plan admits strips only with Eq. 65
 }
-template <int CP, class Real, int YC, int MINB>
+template <int CP, class Real, int MINB>
 cudaError_t strip2_of(const StepLaunch& a, cudaStream_t st) {
-    if constexpr (CP == MODEQ) return step_strip2<D2Q9, CP, Real, YC, 4, MINB>(a, st);
+    if constexpr (CP == MODEQ) return step_strip2<D2Q9, CP, Real, 4, MINB>(a, st);
     return cudaErrorInvalidValue;
 }
 
 template <int CP, class Real>
 cudaError_t step_tile(const StepLaunch& a, cudaStream_t st) {
     switch (a.tile_id) {
-        case 0: return strip2_of<CP, Real, 32, 3>(a, st);
-        case 1: return strip2_of<CP, Real, 16, 3>(a, st);
-        case 2: return strip2_of<CP, Real, 64, 3>(a, st);
-        case 3: return strip2_of<CP, Real, 32, 4>(a, st);
-        case 4: return strip_of<CP, Real, 32, 6>(a, st);
-        case 5: return strip_of<CP, Real, 64, 6>(a, st);
-        case 6: return strip_of<CP, Real, 16, 6>(a, st);
-        case 7: return strip_of<CP, Real, 32, 7>(a, st);
+        case 0:
+        case 1:
+        case 2:
+        case 14:
+        case 15: return strip2_of<CP, Real, 3>(a, st);
+        case 3: return strip2_of<CP, Real, 4>(a, st);
+        case 4:
+        case 5:
+        case 6: return strip_of<CP, Real, 6>(a, st);
+        case 7: return strip_of<CP, Real, 7>(a, st);
         case 8: return step_one<D2Q9, CP, Real, 32, 8, 1>(a, st);
         case 9: return step_one<D2Q9, CP, Real, 64, 4, 1>(a, st);
         case 10: return step_one<D2Q9, CP, Real, 128, 2, 1>(a, st);

@@ -18,10 +18,10 @@ namespace {
 // memory (3).  Two sites per consumer thread: the paired kernel (x-adjacent
 // site pairs, paired FP32 arithmetic; ensembles with an nx that is not a
 // multiple of 4 run the one-site warp-specialised kernel of the same tile).
-// Staging 4: the split step (a moment pass, then collision columns of the
-// tile, two sites stacked in z per thread).  FP64 and other relaxation rates
-// take the split step whatever the row, in 16 x 8 columns with the row's
-// z-chunk.  The first entry is the default.
+// The 16 x 8 rows with 4 resident CTAs are the split step (a moment pass, then
+// collision columns, two sites stacked in z per thread), which FP64 runs and
+// other relaxation rates take whatever the row, with the row's z-chunk.  The
+// first entry is the default.
 constexpr int kTiles[][kVariantCols] = {
     {32, 8, 32, 3, 4, 3, 2}, {32, 8, 64, 3, 4, 3, 2}, {16, 16, 32, 3, 4, 3, 2}, {16, 16, 64, 3, 4, 3, 2},
     {32, 8, 32, 2, 4, 0, 2}, {16, 16, 32, 2, 4, 0, 2},
@@ -29,8 +29,8 @@ constexpr int kTiles[][kVariantCols] = {
     {16, 8, 32, 3, 4, 1, 1}, {16, 8, 16, 6, 0, 0, 1},  {16, 8, 32, 6, 0, 0, 1},  {16, 16, 16, 4, 0, 0, 1},
     {16, 16, 32, 4, 0, 0, 1},
     {32, 8, 16, 3, 4, 3, 2}, {32, 8, 8, 3, 4, 3, 2},
-    {16, 8, 2, 4, 0, 4, 2},  {16, 8, 4, 4, 0, 4, 2},   {16, 8, 8, 4, 0, 4, 2},   {16, 8, 16, 4, 0, 4, 2},
-    {16, 8, 32, 4, 0, 4, 2}, {8, 8, 2, 8, 0, 4, 2}};
+    {16, 8, 2, 4, 0, 0, 1},  {16, 8, 4, 4, 0, 0, 1},   {16, 8, 8, 4, 0, 0, 1},   {16, 8, 16, 4, 0, 0, 1},
+    {16, 8, 32, 4, 0, 0, 1}};
 constexpr int kNumTiles = int(sizeof(kTiles) / sizeof(kTiles[0]));
 // ring planes of the paired kernel: 8 with register staging (2 CTAs per SM),
 // 4 with cp.async staging (the staging areas share the shared memory)
@@ -41,7 +41,7 @@ template <int CP, int I>
 cudaError_t step_variant(const StepLaunch& a, cudaStream_t st) {
     constexpr int TX = kTiles[I][0], TY = kTiles[I][1], OCC = kTiles[I][3], PW = kTiles[I][4], STG = kTiles[I][5];
     constexpr bool paired = PW > 0 && kTiles[I][6] == 2;
-    if constexpr (STG == 4) {
+    if constexpr (split_row(kTiles[I])) {
         return cudaErrorInvalidValue;        // the plan runs these rows as the split step
     } else if constexpr (CP == MODEQ) {
         // the modified equilibrium: the paired kernel on the paired cp.async rows (every

@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(AUX_THREADS)
 template <class L>
 __device__ __forceinline__ int64_t pulled_element(const SysDev& S, int site, int i) {
     int x, y, z;
-    site_coords(int(site), S.nx, S.ny, x, y, z);
+    site_coords(site, S.nx, S.ny, x, y, z);
     int cx = 0, cy = 0, cz = 0;
 #pragma unroll
     for (int q = 0; q < L::Q; ++q)
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(AUX_THREADS)
     out[int64_t(blockIdx.y) * S.n_sites + site] = v + (i == 0 ? S.rho_c : 0.0);
 }
 
-// buf_i(r - c_i) = f_i(r) - rho_c [i == 0], one population.
+// buf_i(r - c_i) = f_i(r) - rho_c [i == 0] for the populations i = i0 + k.
 template <class L, class Real>
 __global__ void __launch_bounds__(AUX_THREADS)
     scatter_kernel(const SysDev* __restrict__ sysv, int sys, int i0, const double* __restrict__ in,

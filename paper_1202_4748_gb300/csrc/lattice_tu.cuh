@@ -37,37 +37,37 @@ cudaError_t step_one_mode(const StepLaunch& a, cudaStream_t st) {
 }
 
 // Row-marching strips (D2Q9, modified equilibrium): WPC warps per CTA, tiles
-// of SW sites x YC rows, one warp per 32 sites of a tile.
-template <class L, int CP, class Real, int YC, int WPC, int MINB, int MODE, int SW>
+// of SW sites x a.zc rows, one warp per 32 sites of a tile.
+template <class L, int CP, class Real, int WPC, int MINB, int MODE, int SW>
 cudaError_t step_strip_mode(const StepLaunch& a, cudaStream_t st) {
     const StepArgs<Real> A = step_args<Real>(a);
     const int warps = a.n_tiles * (SW / 32);
     const int grid = (warps + WPC - 1) / WPC;
-    step_kernel_strip<L, CP, Real, YC, WPC, MINB, MODE, SW><<<grid, 32 * WPC, 0, st>>>(A, a.n_tiles);
+    step_kernel_strip<L, CP, Real, WPC, MINB, MODE, SW><<<grid, 32 * WPC, 0, st>>>(A, a.n_tiles);
     return cudaGetLastError();
 }
-template <class L, int CP, class Real, int YC, int WPC, int MINB, int SW = 32>
+template <class L, int CP, class Real, int WPC, int MINB, int SW = 32>
 cudaError_t step_strip(const StepLaunch& a, cudaStream_t st) {
     constexpr int MB = sizeof(Real) == 4 && MINB > 0 ? MINB : 1;   // FP64 keeps its registers
-    if (a.bgk_only == 2) return step_strip_mode<L, CP, Real, YC, WPC, MB, 2, SW>(a, st);
-    if (a.bgk_only == 1) return step_strip_mode<L, CP, Real, YC, WPC, MB, 1, SW>(a, st);
-    return step_strip_mode<L, CP, Real, YC, WPC, MB, 0, SW>(a, st);
+    if (a.bgk_only == 2) return step_strip_mode<L, CP, Real, WPC, MB, 2, SW>(a, st);
+    if (a.bgk_only == 1) return step_strip_mode<L, CP, Real, WPC, MB, 1, SW>(a, st);
+    return step_strip_mode<L, CP, Real, WPC, MB, 0, SW>(a, st);
 }
 
 // Two-site strips (D2Q9, modified equilibrium, FP32, every mode at tau = 1,
-// every x side a multiple of 4) on tiles of 64 sites x YC rows; any other run
+// every x side a multiple of 4) on tiles of 64 sites x a.zc rows; any other run
 // of the same tiles takes the one-site strips, two warps per tile.
-template <class L, int CP, class Real, int YC, int WPC, int MINB>
+template <class L, int CP, class Real, int WPC, int MINB>
 cudaError_t step_strip2(const StepLaunch& a, cudaStream_t st) {
     if constexpr (sizeof(Real) == 4 && CP == MODEQ) {
         if (a.bgk_only == 2 && a.pair_ok) {
             const StepArgs<float> A = step_args<float>(a);
             const int grid = (a.n_tiles + WPC - 1) / WPC;
-            step_kernel_strip_pair<YC, WPC, MINB><<<grid, 32 * WPC, 0, st>>>(A, a.n_tiles);
+            step_kernel_strip_pair<WPC, MINB><<<grid, 32 * WPC, 0, st>>>(A, a.n_tiles);
             return cudaGetLastError();
         }
     }
-    return step_strip<L, CP, Real, YC, WPC, MINB, 64>(a, st);
+    return step_strip<L, CP, Real, WPC, MINB, 64>(a, st);
 }
 
 // z-marching launches (FP32, every mode at tau = 1): columns of TX x TY sites,
@@ -155,47 +155,42 @@ cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigned block
 }
 
 // Moment pass of the split step: quads of sites where every nx is a multiple of
-// 4, else single sites; small CTAs when the items are small (few of them).
-template <class L, class Real>
+// 4 (FP32), else single sites; small CTAs when the items are small (few of them).
+template <class L, class Real, bool J>
 cudaError_t step_moments(const StepLaunch& a, cudaStream_t st) {
     const Real* f = static_cast<const Real*>(a.fin);
     Real* mom = static_cast<Real*>(a.mom);
     if constexpr (sizeof(Real) == 4) {
         if (a.pair_ok) {
             if (a.small_items)
-                return launch_dependent(moments_quad_kernel<L, 64>, a.n_site_items, 64, st, a.sys, a.site_items, f, mom,
-                                        a.n_sites);
-            return launch_dependent(moments_quad_kernel<L, 256>, a.n_site_items, 256, st, a.sys, a.site_items, f, mom,
-                                    a.n_sites);
+                return launch_dependent(moments_quad_kernel<L, J, 64>, a.n_site_items, 64, st, a.sys, a.site_items, f,
+                                        mom, a.n_sites);
+            return launch_dependent(moments_quad_kernel<L, J, 256>, a.n_site_items, 256, st, a.sys, a.site_items, f,
+                                    mom, a.n_sites);
         }
     }
-    return launch_dependent(moments_kernel<L, Real, 256>, a.n_site_items, 256, st, a.sys, a.site_items, f, mom,
+    return launch_dependent(moments_kernel<L, Real, J, 256>, a.n_site_items, 256, st, a.sys, a.site_items, f, mom,
                             a.n_sites);
 }
 
 // Split step on D3Q19: the moment pass over the site items, then the collision
-// of TX x TY columns in chunks of a.zc planes.  Resident CTAs: FP32 at tau = 1
-// fits 4 (8 of the 8 x 8 columns) without spills; the pulled populations of the
-// other rates need more registers; the FP64 unit needs no more than 2.
-template <int MODE, int CP, class Real, int TX, int TY>
+// of 16 x 8 columns in chunks of a.zc planes.  Resident CTAs: FP32 at tau = 1
+// fits 4 without spills; the pulled populations of the other rates need more
+// registers; the FP64 unit needs no more than 2.
+template <int MODE, int CP, class Real>
 cudaError_t step_split_mode(const StepLaunch& a, cudaStream_t st) {
     using V = typename std::conditional<std::is_same<Real, float>::value, float2, double>::type;
-    constexpr int MINB = (sizeof(Real) == 8 ? 2 : (MODE == 2 ? 4 : 3)) * (TX == 8 ? 2 : 1);
-    const cudaError_t e = step_moments<D3Q19, Real>(a, st);
+    constexpr int MINB = sizeof(Real) == 8 ? 2 : (MODE == 2 ? 4 : 3);
+    const cudaError_t e = step_moments<D3Q19, Real, MODE == 2 && sizeof(Real) == 4>(a, st);
     if (e != cudaSuccess) return e;
-    return launch_dependent(collide_march_kernel<MODE, CP, V, TX, TY, MINB>, a.n_tiles, TX * TY, st,
+    return launch_dependent(collide_march_kernel<MODE, CP, V, 16, 8, MINB>, a.n_tiles, 128, st,
                             step_args<Real>(a), static_cast<const Real*>(a.mom), a.n_sites);
 }
 template <int CP, class Real>
 cudaError_t step_split(const StepLaunch& a, cudaStream_t st) {
-    if (a.bgk_only == 2) {
-        if constexpr (std::is_same<Real, float>::value) {
-            if (a.narrow) return step_split_mode<2, CP, Real, 8, 8>(a, st);
-        }
-        return step_split_mode<2, CP, Real, 16, 8>(a, st);
-    }
-    if (a.bgk_only == 1) return step_split_mode<1, CP, Real, 16, 8>(a, st);
-    return step_split_mode<0, CP, Real, 16, 8>(a, st);
+    if (a.bgk_only == 2) return step_split_mode<2, CP, Real>(a, st);
+    if (a.bgk_only == 1) return step_split_mode<1, CP, Real>(a, st);
+    return step_split_mode<0, CP, Real>(a, st);
 }
 
 template <class L, int CP, class Real, int TX, int TY, int TZ>

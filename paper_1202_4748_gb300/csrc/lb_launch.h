@@ -23,9 +23,8 @@ struct StepLaunch {
     int k;
     int* status;
     int tile_id;            // index into the lattice's tile-shape table
-    int zc;                 // z extent of its tiles (planes per chunk of the z-marching kernels)
-    int split;              // D3Q19: run the split step (narrow: in 8 x 8 columns)
-    int narrow;
+    int zc;                 // planes per chunk of the z-marching kernels, rows per strip on D2Q9
+    int split;              // D3Q19: run the split step
     void* mom;              // split step: density and momentum fields, one per n_sites values
     int64_t n_sites;        // sites of the ensemble
     const int4* site_items; // split step: the moment pass's work list
@@ -40,6 +39,10 @@ struct StepLaunch {
 // SM, producer warps, staging: 0 plain loads, 1 bulk copies, sites per
 // consumer thread); index = tile_id.
 constexpr int kVariantCols = 7;
+// D3Q19 rows of the split step: 16 x 8 columns, 4 resident CTAs, no producer warps.
+constexpr bool split_row(const int* t) {
+    return t[0] == 16 && t[1] == 8 && t[3] == 4 && t[4] == 0 && t[5] == 0;
+}
 int tile_shapes_d2q9(int (*out)[kVariantCols], int max);
 int tile_shapes_d3q19(int (*out)[kVariantCols], int max);
 

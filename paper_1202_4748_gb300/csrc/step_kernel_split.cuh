@@ -1,8 +1,10 @@
 // Split form of the fused step: a moment pass writes the density and momentum
 // of every site (from the populations pulled to it, once per site), and a
 // collision pass reads that field around each column of sites and writes the
-// post-collision populations.  With every mode at tau = 1 the collision needs
-// nothing else; with other rates it pulls the site's populations again.
+// post-collision populations.  In FP32 with every mode at tau = 1 the collision
+// needs nothing else; with other rates, or in FP64, it pulls the site's
+// populations again and the moment pass writes the density alone (FP64: so that
+// the field fits the scratch of a sample, which it shares).
 //
 // Against the kernels that form the density on the halo of every column, this
 // trades 16 bytes written and about 35 read per FP32 site (from L2 while the
@@ -17,10 +19,10 @@
 
 namespace lbf {
 
-// Density deviation and momentum of every site of the items: mom[site] = drho,
-// mom[(1 + a) stride + site] = j_a, each summed in the order of the fused
+// Density deviation and (J) momentum of every site of the items: mom[site] =
+// drho, mom[(1 + a) stride + site] = j_a, each summed in the order of the fused
 // kernels (from 0, direction by direction).  One site per thread (any sides).
-template <class L, class Real, int NT>
+template <class L, class Real, bool J, int NT>
 __global__ void __launch_bounds__(NT)
     moments_kernel(const SysDev* __restrict__ sysv, const int4* __restrict__ items, const Real* __restrict__ fbuf,
                    Real* __restrict__ mom, int64_t stride) {
@@ -33,13 +35,16 @@ __global__ void __launch_bounds__(NT)
     for (int site = it.y + int(threadIdx.x); site < it.z; site += NT) {
         const int r = site / nx, x = site - r * nx, z = r / ny, y = r - z * ny;
         const Nbr nb(x, y, z, nx, ny, nz, L::D == 3);
-        Real f[L::Q], j[3];
+        Real f[L::Q];
         pull_site<L, Real>(fb, N, nb, f);
         Real v = Real(0);
         sfor<0, L::Q>([&](auto I) { v = vadd(v, f[decltype(I)::value]); });
-        momentum_of<L, Real>(f, j);
         out[site] = v;
-        sfor<0, L::D>([&](auto C) { out[(1 + int(C)) * stride + site] = j[decltype(C)::value]; });
+        if constexpr (J) {
+            Real j[3];
+            momentum_of<L, Real>(f, j);
+            sfor<0, L::D>([&](auto C) { out[(1 + int(C)) * stride + site] = j[decltype(C)::value]; });
+        }
     }
     grid_release();
 }
@@ -49,7 +54,7 @@ __global__ void __launch_bounds__(NT)
 // directions pull across the quad's edge from the neighbouring lane, or loaded
 // where that lane holds another row's quad or none.  A site costs 70
 // instructions instead of 255, and a warp has 9.7 KB of loads in flight.
-template <class L, int NT>
+template <class L, bool J, int NT>
 __global__ void __launch_bounds__(NT)
     moments_quad_kernel(const SysDev* __restrict__ sysv, const int4* __restrict__ items,
                         const float* __restrict__ fbuf, float* __restrict__ mom, int64_t stride) {
@@ -100,7 +105,7 @@ __global__ void __launch_bounds__(NT)
             }
             v01 = vadd(v01, a01);
             v23 = vadd(v23, a23);
-            sfor<0, L::D>([&](auto C) {
+            if constexpr (J) sfor<0, L::D>([&](auto C) {
                 constexpr int c = C;
                 if constexpr (L::c(i, c) == 1) {
                     j01[c] = vadd(j01[c], a01);
@@ -114,7 +119,7 @@ __global__ void __launch_bounds__(NT)
         });
         if (mine) {
             *reinterpret_cast<float4*>(out + site) = make_float4(v01.x, v01.y, v23.x, v23.y);
-            sfor<0, L::D>([&](auto C) {
+            if constexpr (J) sfor<0, L::D>([&](auto C) {
                 constexpr int c = C;
                 *reinterpret_cast<float4*>(out + (1 + c) * stride + site) =
                     make_float4(j01[c].x, j01[c].y, j23[c].x, j23[c].y);
@@ -148,8 +153,8 @@ struct ZPlanes {
 // Laplacian that needs them; the Laplacian (Guo form) of planes z + W + 1 ..
 // z + 2 W and the collision of planes z .. z + W - 1 share one phase, so there
 // is one CTA barrier per iteration; the momenta of the next sites are in flight
-// across it.  With rates other than 1 (MODE 0 and 1) a thread also pulls its
-// sites' populations, requested before the Laplacian pass.
+// across it.  With rates other than 1 (MODE 0 and 1) and in FP64 a thread pulls
+// its sites' populations instead, requested before the Laplacian pass.
 //
 // Rings of 8 planes: iteration z reads density z .. z + 2 W + 1 (z - 1 .. z + W
 // for the modified equilibrium) and Laplacian z - 1 .. z + W, writes Laplacian
@@ -167,6 +172,7 @@ __global__ void __launch_bounds__(TX* TY, MINB)
     using Real = typename VT<V>::S;
     using L = D3Q19;
     constexpr int W = VT<V>::W;
+    constexpr bool PULL = MODE != 2 || sizeof(Real) == 8;
     constexpr int H = CP == GUO ? 2 : 1;
     constexpr int NT = TX * TY, R = 8;
     constexpr int SX = TX + 2 * H, SY = TY + 2 * H, SP = SX * SY;
@@ -226,7 +232,7 @@ __global__ void __launch_bounds__(TX* TY, MINB)
     V jn[3];
     auto momenta = [&](int z) {                          // of the sites (x, y, z ..); the second may not exist
         sfor<0, 3>([&](auto C) { jn[decltype(C)::value] = vk<V>(0.0); });
-        if (own && z < z1) {
+        if (!PULL && own && z < z1) {
             const int up = z + 1 < z1 ? pl : 0;
             sfor<0, 3>([&](auto C) {
                 constexpr int c = C;
@@ -263,7 +269,7 @@ __global__ void __launch_bounds__(TX* TY, MINB)
         }
         cp_async_commit();
         V f[19];
-        if constexpr (MODE != 2) {
+        if constexpr (PULL) {
             if (own) {
                 const Real* fb = A.fin + S.pop_offset;
                 const Nbr nb(x, y, z, nx, ny, nz, true);
@@ -291,6 +297,18 @@ __global__ void __launch_bounds__(TX* TY, MINB)
                 set_lane(drho, 1, srho[slot(two ? r + 1 : r) * SP + c]);
             } else {
                 sites = site;
+            }
+            if constexpr (PULL) {
+                sfor<0, 3>([&](auto C) {
+                    constexpr int cc = C;
+                    V s = vk<V>(0.0);
+                    sfor<1, 19>([&](auto I) {
+                        constexpr int i = I;
+                        if constexpr (L::c(i, cc) == 1) s = vadd(s, f[i]);
+                        if constexpr (L::c(i, cc) == -1) s = vsub(s, f[i]);
+                    });
+                    jm[cc] = s;
+                });
             }
             ZPlanes<V, CP == GUO ? LX : SX> nv;
             nv.c = CP == GUO ? (ly + 1) * LX + lx + 1 : c;

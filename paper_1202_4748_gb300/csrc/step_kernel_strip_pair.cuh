@@ -2,7 +2,7 @@
 // per lane (FP32, every mode at tau = 1).
 //
 // A warp owns 64 consecutive sites of a row (tile (system, x0, y0), x0 a
-// multiple of 64) and walks YC rows; lane l holds the sites x0 + 2l and
+// multiple of 64) and walks A.zc rows; lane l holds the sites x0 + 2l and
 // x0 + 2l + 1 as one float2.  Per footprint row yy each lane loads, for every
 // population, the aligned pair of its own two columns at the pulled row
 // (one 8-byte load, issued one row ahead); the pull's x shift of -c_x is done in registers: the
@@ -55,7 +55,7 @@ struct PairNbr {
     }
 };
 
-template <int YC, int WPC, int MINB>
+template <int WPC, int MINB>
 __global__ void __launch_bounds__(32 * WPC, MINB)
     step_kernel_strip_pair(const StepArgs<float> A, int n_tiles) {
     using L = D2Q9;
@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(32 * WPC, MINB)
     const int xs = wrapm(x, nx);                                   // even: the pair is aligned
     const int xt = wrapm(left ? tl.y - 2 : tl.y + 64, nx);         // the pair just outside the strip
     const NoiseKey key = noise_key(S, *A.step_ptr + A.k);
-    const int y0 = tl.z, y1 = min(y0 + YC, ny);
+    const int y0 = tl.z, y1 = min(y0 + A.zc, ny);
 
     // pulled rows yy - c_y for c_y = -1, 0, 1 (index 1 + c_y), as offsets
     auto rows_of = [&](int yy, int (&ro)[3]) {

@@ -32,7 +32,7 @@ struct StepArgs {
     const int64_t* step_ptr;  // device step counter at the start of the chunk
     int k;                    // offset of this step inside the chunk
     int* status;
-    int zc;                   // planes per tile of the z-marching kernels
+    int zc;                   // planes per tile of the z-marching kernels, rows per tile of the D2Q9 strips
 };
 
 template <class L, int CP>
@@ -631,7 +631,7 @@ struct Nbr9 {
 
 // Row-marching strips for the D2Q9 modified-equilibrium step (Eq. 65 needs
 // the density on the 3 x 3 neighbourhood only).  Each warp owns 32
-// consecutive sites of a row and walks YC rows; a tile (system, x0, y0) is SW
+// consecutive sites of a row and walks A.zc rows; a tile (system, x0, y0) is SW
 // sites wide (32, or 64 for the tiles of the two-site kernel, whose one-site
 // form gives each tile two warps).  Per footprint row yy a lane pulls its
 // site's 9 populations, forms rho, and the neighbours' rho comes by warp
@@ -641,14 +641,13 @@ struct Nbr9 {
 // earlier (with every mode at tau = 1, from its density and momentum only;
 // the collision is collide_d2q9_modeq for every relaxation setting).
 // No shared memory and no CTA barrier: every footprint value is formed once
-// per chunk (halo 2/32 in x, 2/YC in y).  Lanes past the system's last column
+// per chunk (halo 2/32 in x, 2 rows in y).  Lanes past the system's last column
 // form the periodic image of their column for their neighbours and do not
 // collide.  (Colliding two rows behind, to overlap the next row's loads,
 // measured slower: 8 more registers per thread, fewer warps in flight.)
-template <class L, int CP, class Real, int YC, int WPC, int MINB, int MODE, int SW = 32>
+template <class L, int CP, class Real, int WPC, int MINB, int MODE, int SW = 32>
 __global__ void __launch_bounds__(32 * WPC, MINB) step_kernel_strip(const StepArgs<Real> A, int n_tiles) {
     static_assert(L::D == 2 && CP == MODEQ, "row strips: D2Q9 with the modified equilibrium");
-    constexpr bool BGK_ONLY = MODE >= 1;
     constexpr bool TAU1 = MODE == 2;
     constexpr int Q = L::Q;
     constexpr int WPT = SW / 32;                     // warps per tile
@@ -673,7 +672,7 @@ __global__ void __launch_bounds__(32 * WPC, MINB) step_kernel_strip(const StepAr
     const int xo[3] = {wrap1(xs + 1, nx), xs, wrap1(xs - 1, nx)};
     const int ho[3] = {wrap1(xh + 1, nx), xh, wrap1(xh - 1, nx)};
     const int64_t step = *A.step_ptr + A.k;
-    const int y0 = tl.z, y1 = min(y0 + YC, ny);
+    const int y0 = tl.z, y1 = min(y0 + A.zc, ny);
 
     Real fp[TAU1 ? 1 : Q];                           // pulled populations of row yy - 1
     Real pr = Real(0), pjx = Real(0), pjy = Real(0); // tau = 1: (drho, j) of row yy - 1
