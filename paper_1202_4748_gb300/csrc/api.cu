@@ -52,7 +52,7 @@ struct Plan {
         S, E, bottom_items, part_items, block_items, parts, up_items, tops, rec, acc, hist, sk_meta, sk_sys, sk_tw, sk_acc, sk_b0, sk_b1, sk_bins, jk_j,
         jk_lap, jk_F, jk_acc, mom, total;
     int tdim[3] = {0, 0, 0};      // tile shape of the step kernel
-    bool split = false;           // D3Q19: the split step
+    bool split = false, narrow = false;   // D3Q19: the split step (in 8 x 8 columns)
     bool jk = false;
     int hist_bins = 0;
     double hist_range = 0.0;
@@ -290,8 +290,8 @@ void choose_d3q19_row(const lb_system_desc* s, int n, int kind, bool quads, int&
 // two halo rows more than it collides.  A warp of paired FP32 strips takes
 // 0.9 us per row alone on its scheduler, 1.3 beside one other, 1.8 beside two
 // (3 CTAs of 4 warps per SM); the one-site strips (two warps per tile) keep 5
-// CTAs; an FP64 row occupies its SM's FP64 unit for 1.6 us, and CTAs of 4 warps
-// are dealt to the SMs.  32 rows were the default of every ensemble: one 512^2
+// CTAs; in FP64 a CTA of 4 warps takes 8.3 us per row alone on its SM, and 6.4
+// beside others.  32 rows were the default of every ensemble: one 512^2
 // system 33 -> 8 us per step in FP32; in FP64, 64 CTAs on 152 SMs, 293 -> 128.
 void choose_d2q9_row(const lb_system_desc* s, int n, bool fp32, bool paired, int& tile_id) {
     const int sms = sm_count();
@@ -309,8 +309,8 @@ void choose_d2q9_row(const lb_system_desc* s, int n, bool fp32, bool paired, int
             const double slots = 4.0 * ctas * sms, full = std::floor(warps / slots), rest = warps - full * slots;
             us = (rows + 2) * (row_us[ctas] * full + row_us[int(std::ceil(rest / (4.0 * sms)))]);
         } else {
-            const double ctas = std::ceil(warps / (4.0 * sms));
-            us = std::max(4.0 * ctas * (1.6 * rows + 0.4), 4.0 * (rows + 2));
+            const double load = warps / (4.0 * sms), ctas = load <= 4.0 ? std::ceil(load) : load + 0.5;
+            us = (rows + 2) * std::max(8.3, 6.4 * ctas);
         }
         if (us < 0.98 * best_us) {
             best_us = us;
@@ -347,6 +347,14 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
         if (P.split) {
             tdim[0] = 16;
             tdim[1] = 8;
+        }
+        // a lane outside its system costs the FP64 unit as much as one inside: 8 x 8
+        // columns (whose Laplacian halo is 1.56 sites per site against 1.41) where
+        // they cover the systems with fewer (24^3: 0.51 -> 0.43 ms per step)
+        if (P.split && !fp32) {
+            const int narrow[3] = {8, 8, tdim[2]};
+            P.narrow = 1.05 * 64.0 * double(tiles_of(s, n, narrow)) < 128.0 * double(tiles_of(s, n, tdim));
+            if (P.narrow) tdim[0] = 8;
         }
     }
     for (int k = 0; k < 3; ++k) P.tdim[k] = tdim[k];
@@ -883,6 +891,7 @@ cudaError_t launch_steps(lb_ctx* c, int64_t n) {
         a.tile_id = c->tile_id;
         a.zc = c->lattice == LB_D2Q9 ? P.tdim[1] : P.tdim[2];
         a.split = P.split ? 1 : 0;
+        a.narrow = P.narrow ? 1 : 0;
         a.mom = c->ws + P.mom;
         a.n_sites = P.n_sites;
         a.site_items = c->at<int4>(P.site_items);

@@ -30,11 +30,46 @@
 
 namespace lbf {
 
+// Density deviation of one site from its pulled deviations: in FP32 summed in
+// population order from zero, in FP64 by integer additions (FixedSum: the FP64
+// units do two operations per clock and SM).
+template <int Q>
+__device__ __forceinline__ float density_of(const float (&f)[Q]) {
+    float v = 0.0f;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) v = vadd(v, f[i]);
+    return v;
+}
+template <int Q>
+__device__ __forceinline__ double density_of(const double (&f)[Q]) {
+    const FixedSum<Q> s(f);
+    if (s.finite()) {
+        int64_t v = 0;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) v += s.m[i];
+        return s.value(v);
+    }
+    double v = 0.0;
+    for (int i = 0; i < Q; ++i) v += f[i];
+    return v;
+}
+
 // Density deviation and momentum of one site (or a pair) from its pulled
 // deviations: drho = sum_i f_i, j = sum_i c_i f_i, each summed in population
-// order from zero.
+// order from zero (FP64: as density_of).
 template <class V>
 __device__ __forceinline__ void moments_d2q9(const V (&f)[9], V& drho, V& jx, V& jy) {
+    if constexpr (VT<V>::W == 1 && sizeof(V) == 8) {
+        const FixedSum<9> s(f);
+        if (s.finite()) {
+            const int64_t(&m)[9] = s.m;
+            const int64_t a = m[5] - m[6], b = m[7] - m[8];
+            drho = s.value(((m[0] + m[1]) + (m[2] + m[3])) + ((m[4] + m[5]) + (m[6] + m[7])) + m[8]);
+            jx = s.value((m[1] - m[2]) + a + b);
+            jy = s.value((m[3] - m[4]) + a - b);
+            return;
+        }
+    }
     V r = vadd(vk<V>(0.0), f[0]);
 #pragma unroll
     for (int i = 1; i < 9; ++i) r = vadd(r, f[i]);

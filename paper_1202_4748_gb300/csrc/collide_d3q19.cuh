@@ -183,27 +183,29 @@ __device__ __forceinline__ void draw4(const NoiseKey& k, uint2 site, uint32_t d,
 __device__ __forceinline__ void draw4(const NoiseKey& k, uint32_t site, uint32_t d, double sc0, double sc1,
                                       double (&n)[4], bool need3) {
     const uint4 w = philox_draw(k, site, d);
-    double a, b;
-    box_muller(w.x, w.y, a, b);
-    n[0] = vmul(sc0, a);
-    n[1] = vmul(sc0, b);
-    box_muller(w.z, w.w, a, b);
-    n[2] = vmul(sc1, a);
-    n[3] = need3 ? vmul(sc1, b) : 0.0;
+    double c, s;
+    const double r0 = vmul(sc0, n64_radius(w.x, LogTable()));
+    n64_angle(w.y, c, s);
+    n[0] = vmul(r0, c);
+    n[1] = vmul(r0, s);
+    const double r1 = vmul(sc1, n64_radius(w.z, LogTable()));
+    n64_angle(w.w, c, s);
+    n[2] = vmul(r1, c);
+    n[3] = need3 ? vmul(r1, s) : 0.0;
 }
 
 // 1 / sqrt(x) lane by lane.
 __device__ __forceinline__ float vrsqrt(float x) { return sfu_rsqrt(x); }
 __device__ __forceinline__ float2 vrsqrt(float2 x) { return make_float2(sfu_rsqrt(x.x), sfu_rsqrt(x.y)); }
-__device__ __forceinline__ double vrsqrt(double x) { return rsqrt(x); }
+__device__ __forceinline__ double vrsqrt(double x) { return n64_inv_sqrt(x); }
 
 // Noise scale sqrt(max(x, 0)) lane by lane: the special-function square root
-// in float, the library's in double.
+// in float, the integer one in double.
 __device__ __forceinline__ float vsqrt_pos(float x) { return sfu_sqrt(fmaxf(x, 0.0f)); }
 __device__ __forceinline__ float2 vsqrt_pos(float2 x) {
     return make_float2(sfu_sqrt(fmaxf(x.x, 0.0f)), sfu_sqrt(fmaxf(x.y, 0.0f)));
 }
-__device__ __forceinline__ double vsqrt_pos(double x) { return sqrt(x > 0.0 ? x : 0.0); }
+__device__ __forceinline__ double vsqrt_pos(double x) { return n64_sqrt(x > 0.0 ? x : 0.0); }
 
 // Laplacian of the density, lap rho = 6 sum_i t_i (rho(r + c_i) - rho(r))
 // = (1/3) (sum of the 6 face neighbours) + (1/6) (sum of the 12 edge

@@ -174,17 +174,25 @@ cudaError_t step_moments(const StepLaunch& a, cudaStream_t st) {
 }
 
 // Split step on D3Q19: the moment pass over the site items, then the collision
-// of 16 x 8 columns in chunks of a.zc planes.  Resident CTAs: FP32 at tau = 1
+// of 16 x 8 columns (FP64: 8 x 8 where they leave fewer lanes outside the
+// systems) in chunks of a.zc planes.  Resident CTAs: FP32 at tau = 1
 // fits 4 without spills; the pulled populations of the other rates need more
 // registers; the FP64 unit needs no more than 2.
-template <int MODE, int CP, class Real>
-cudaError_t step_split_mode(const StepLaunch& a, cudaStream_t st) {
+template <int MODE, int CP, class Real, int TX>
+cudaError_t step_split_columns(const StepLaunch& a, cudaStream_t st) {
     using V = typename std::conditional<std::is_same<Real, float>::value, float2, double>::type;
-    constexpr int MINB = sizeof(Real) == 8 ? 2 : (MODE == 2 ? 4 : 3);
+    constexpr int MINB = (sizeof(Real) == 8 ? 2 : (MODE == 2 ? 4 : 3)) * (16 / TX);
     const cudaError_t e = step_moments<D3Q19, Real, MODE == 2 && sizeof(Real) == 4>(a, st);
     if (e != cudaSuccess) return e;
-    return launch_dependent(collide_march_kernel<MODE, CP, V, 16, 8, MINB>, a.n_tiles, 128, st,
+    return launch_dependent(collide_march_kernel<MODE, CP, V, TX, 8, MINB>, a.n_tiles, 8 * TX, st,
                             step_args<Real>(a), static_cast<const Real*>(a.mom), a.n_sites);
+}
+template <int MODE, int CP, class Real>
+cudaError_t step_split_mode(const StepLaunch& a, cudaStream_t st) {
+    if constexpr (sizeof(Real) == 8) {
+        if (a.narrow) return step_split_columns<MODE, CP, Real, 8>(a, st);
+    }
+    return step_split_columns<MODE, CP, Real, 16>(a, st);
 }
 template <int CP, class Real>
 cudaError_t step_split(const StepLaunch& a, cudaStream_t st) {

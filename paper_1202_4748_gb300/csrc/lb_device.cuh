@@ -255,15 +255,15 @@ __device__ __forceinline__ void box_muller(uint32_t wa, uint32_t wb, float& n0, 
     n1 = -r * s;
 }
 
-// Reciprocal and reciprocal square root: exact-rounding library calls in
-// double, the special-function unit in float (the FP32 path's error budget is
+// Reciprocal and reciprocal square root: correctly rounded division and the
+// integer root in double, the special-function unit in float (the FP32 path's error budget is
 // ~1e-5 of the populations; these are good to a few ulp).
 __device__ __forceinline__ double fast_rcp(double x) { return 1.0 / x; }
 __device__ __forceinline__ float fast_rcp(float x) { return __fdividef(1.0f, x); }
-__device__ __forceinline__ double fast_rsqrt(double x) { return rsqrt(x); }
+__device__ __forceinline__ double fast_rsqrt(double x) { return n64_inv_sqrt(x); }
 __device__ __forceinline__ float fast_rsqrt(float x) { return rsqrtf(x); }
 // Square root of x >= 0: exact rounding in double; x rsqrt(x) in float (0 at 0).
-__device__ __forceinline__ double fast_sqrt(double x) { return sqrt(x); }
+__device__ __forceinline__ double fast_sqrt(double x) { return n64_sqrt(x); }
 __device__ __forceinline__ float fast_sqrt(float x) { return x > 0.0f ? x * rsqrtf(x) : 0.0f; }
 
 // Periodic wrap of a coordinate in [-n, 2n).

@@ -85,6 +85,107 @@ LB_HD double n64_double(uint64_t m, int e) {
     return n64_bits((uint64_t(e + 1021) << 52) + (m >> 11) + ((m >> 10) & 1));
 }
 
+// y (1 - e)^(-1/2) - y in Q62 terms: for v in [1/4, 1) (Q64) the seed y (Q23,
+// about 22 bits) and c = (1 - e)^(-1/2) - 1 in Q61, e = 1 - v y^2
+LB_HD void n64_seed(uint64_t v, uint32_t& y, int64_t& c) {
+    y = uint32_t(n64_rsqrt(float(uint32_t(v >> 40)) * 5.9604644775390625e-08f) * 8388608.0f);
+    const int64_t e = int64_t((uint64_t(1) << 61) - n64_mulhi(v, (uint64_t(y) * y) << 15));                    // Q61
+    const int64_t eh = e >> 10;
+    c = (e >> 1) + ((3 * ((eh * eh) >> 41)) >> 3);
+}
+
+// sqrt(v / 2^64) as Q64, v in [2^62, 2^64)
+LB_HD uint64_t n64_root(uint64_t v) {
+    uint32_t y;
+    int64_t c;
+    n64_seed(v, y, c);
+    const uint64_t r0 = n64_mulhi(v, uint64_t(y) << 39);                                                       // Q62
+    uint64_t r = r0 + uint64_t(n64_smulhi(int64_t(r0), c * 8));
+    const uint64_t top = (uint64_t(1) << 62) - 1;
+    r = r > top ? top : r;
+    return r << 2;
+}
+
+// sqrt(x) and 1/sqrt(x) of a positive normal x, within 0.51 units in the last
+// place (16 and 10 FP64 operations of the library become integer ones);
+// anything else through the library.
+LB_HD bool n64_split(double x, uint64_t& v, int& h) {
+    uint64_t u;
+    memcpy(&u, &x, 8);
+    const uint32_t eb = uint32_t(u >> 52);
+    if (eb - 1u >= 0x7feu) return false;                       // zero, subnormal, negative, infinite or NaN
+    // x = (m / 2^64) 2^(eb - 1022) = v 2^(2h)
+    const uint64_t m = (u | (uint64_t(1) << 52)) << 11;
+    const int e = int(eb) - 1022;
+    v = (e & 1) ? m >> 1 : m;
+    h = (e + 1) >> 1;
+    return true;
+}
+LB_HD double n64_sqrt(double x) {
+    uint64_t v;
+    int h;
+    if (!n64_split(x, v, h)) return sqrt(x);
+    return n64_double(n64_root(v), h);
+}
+LB_HD double n64_inv_sqrt(double x) {
+    uint64_t v;
+    int h;
+    if (!n64_split(x, v, h)) return 1.0 / sqrt(x);
+    uint32_t y;
+    int64_t c;
+    n64_seed(v, y, c);
+    const uint64_t y62 = uint64_t(y) << 38;                    // y / 2 (y in (1, 2]) as Q62
+    uint64_t r = y62 + uint64_t(n64_smulhi(int64_t(y62), c * 8));
+    const uint64_t top = (uint64_t(1) << 62) - 1;
+    r = r > top ? top : r;
+    return n64_double(r << 2, 1 - h);
+}
+
+// Sums of N doubles to about 2^-57 of the largest: the mantissas aligned to the
+// largest exponent as integers of 58 bits, so that a sum of up to 19 of them
+// fits 63 bits and every sum costs integer additions.  finite() is false when
+// a value is infinite or NaN (the sums are then the caller's in FP64).
+template <int N>
+struct FixedSum {
+    static_assert(N <= 31, "headroom");
+    int64_t m[N];
+    uint32_t top;                  // largest exponent field, in place
+    LB_HD explicit FixedSum(const double (&f)[N]) {
+        uint64_t u[N];
+        top = 0;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int i = 0; i < N; ++i) {
+            memcpy(&u[i], &f[i], 8);
+            const uint32_t e = uint32_t(u[i] >> 32) & 0x7ff00000u;
+            top = e > top ? e : top;
+        }
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int i = 0; i < N; ++i) {
+            const uint32_t hi = uint32_t(u[i] >> 32), e = hi & 0x7ff00000u;
+            const uint32_t sh = (top - e) >> 20;
+            // zeros and subnormals count as 0
+            const uint64_t a = e ? ((u[i] & 0x000fffffffffffffull) | (uint64_t(1) << 52)) << 5 : 0;
+            const uint64_t half = (uint64_t(1) << (sh & 63)) >> 1;
+            const int64_t v = sh > 58 ? 0 : int64_t((a + half) >> (sh & 63));
+            m[i] = int32_t(hi) < 0 ? -v : v;
+        }
+    }
+    LB_HD bool finite() const { return top != 0x7ff00000u; }
+    // the double nearest to s 2^(top - 1023 - 57)
+    LB_HD double value(int64_t s) const {
+        if (s == 0) return 0.0;
+        const uint64_t a = s < 0 ? uint64_t(0) - uint64_t(s) : uint64_t(s);
+        const int nl = n64_clz(a), e = int(top >> 20) - 1022 - 57 + 63 - nl;      // (m / 2^64) 2^e
+        if (e < -1020) return 0.0;
+        const double d = n64_double(a << nl, e);
+        return s < 0 ? -d : d;
+    }
+};
+
 // sqrt(-2 ln U), U = (w + 1/2) 2^-32; tab holds the 64 entries of kLogTable
 template <class Table>
 LB_HD double n64_radius(uint32_t w, const Table& tab) {
@@ -117,16 +218,7 @@ LB_HD double n64_radius(uint32_t w, const Table& tab) {
     L <<= nl;
     // 2 (-ln U) = v 2^(2h), v in [1/4, 1) as Q64
     const int g = 65 - q - nl, h = (g + 1) >> 1;
-    const uint64_t v = (g & 1) ? L >> 1 : L;
-    const uint32_t y = uint32_t(n64_rsqrt(float(uint32_t(v >> 40)) * 5.9604644775390625e-08f) * 8388608.0f);   // Q23
-    const int64_t e = int64_t((uint64_t(1) << 61) - n64_mulhi(v, (uint64_t(y) * y) << 15));                    // Q61
-    const int64_t eh = e >> 10;
-    const int64_t c = (e >> 1) + ((3 * ((eh * eh) >> 41)) >> 3);
-    const uint64_t r0 = n64_mulhi(v, uint64_t(y) << 39);                                                       // Q62
-    uint64_t r = r0 + uint64_t(n64_smulhi(int64_t(r0), c * 8));
-    const uint64_t top = (uint64_t(1) << 62) - 1;
-    r = r > top ? top : r;
-    return n64_double(r << 2, h);
+    return n64_double(n64_root((g & 1) ? L >> 1 : L), h);
 }
 
 // cos and sin of 2 pi U, U = (w + 1/2) 2^-32

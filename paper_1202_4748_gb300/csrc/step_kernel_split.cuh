@@ -14,6 +14,7 @@
 // ensemble that gives it less than a CTA per SM waits for latency alone.
 #pragma once
 
+#include "collide_d2q9.cuh"
 #include "collide_d3q19.cuh"
 #include "step_kernels.cuh"
 
@@ -37,9 +38,7 @@ __global__ void __launch_bounds__(NT)
         const Nbr nb(x, y, z, nx, ny, nz, L::D == 3);
         Real f[L::Q];
         pull_site<L, Real>(fb, N, nb, f);
-        Real v = Real(0);
-        sfor<0, L::Q>([&](auto I) { v = vadd(v, f[decltype(I)::value]); });
-        out[site] = v;
+        out[site] = density_of(f);
         if constexpr (J) {
             Real j[3];
             momentum_of<L, Real>(f, j);
@@ -298,7 +297,22 @@ __global__ void __launch_bounds__(TX* TY, MINB)
             } else {
                 sites = site;
             }
-            if constexpr (PULL) {
+            if constexpr (PULL && sizeof(Real) == 8) {
+                const FixedSum<19> fs(f);                // as density_of
+                sfor<0, 3>([&](auto C) {
+                    constexpr int cc = C;
+                    int64_t s = 0;
+                    double d = 0.0;
+                    sfor<1, 19>([&](auto I) {
+                        constexpr int i = I;
+                        if constexpr (L::c(i, cc) == 1) s += fs.m[i];
+                        if constexpr (L::c(i, cc) == -1) s -= fs.m[i];
+                    });
+                    if (!fs.finite())
+                        sfor<1, 19>([&](auto I) { d += double(L::c(decltype(I)::value, cc)) * f[decltype(I)::value]; });
+                    jm[cc] = fs.finite() ? fs.value(s) : d;
+                });
+            } else if constexpr (PULL) {
                 sfor<0, 3>([&](auto C) {
                     constexpr int cc = C;
                     V s = vk<V>(0.0);

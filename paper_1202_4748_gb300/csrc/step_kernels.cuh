@@ -551,7 +551,7 @@ __global__ void __launch_bounds__(TX* TY* TZ)
     if (valid) {
         const Nbr nb(x, y, z, nx, ny, nz, L::D == 3);
         pull_site<L, Real>(fb, N, nb, f);
-        sfor<0, Q>([&](auto I) { drho += f[decltype(I)::value]; });
+        drho = density_of(f);
     }
     const int cidx = (tz + HZ) * SX * SY + (ty + H) * SX + (tx + H);
 
@@ -572,7 +572,7 @@ __global__ void __launch_bounds__(TX* TY* TZ)
                          L::D == 3 ? (sm ? wrapm(gz, nz) : wrap2(gz, nz)) : 0, nx, ny, nz, L::D == 3);
             Real g[Q];
             pull_site<L, Real>(fb, N, nb, g);
-            sfor<0, Q>([&](auto I) { v += g[decltype(I)::value]; });
+            v = density_of(g);
         }
         srho[idx] = v;
     }
@@ -696,7 +696,7 @@ __global__ void __launch_bounds__(32 * WPC, MINB) step_kernel_strip(const StepAr
                 constexpr int i = I;
                 g[i] = fb[i * N + ro[1 + L::c(i, 1)] + ho[1 + L::c(i, 0)]];
             });
-            sfor<0, Q>([&](auto I) { re = vadd(re, g[decltype(I)::value]); });
+            re = density_of(g);
         }
         Real rc, jx, jy;
         moments_d2q9<Real>(fc, rc, jx, jy);
