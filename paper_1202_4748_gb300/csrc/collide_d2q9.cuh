@@ -218,13 +218,13 @@ __device__ __forceinline__ void collide_d2q9_modeq(V (&f)[9], const V drho, cons
             c67b = vbc<V>(vmul(P.namp[7], S(1.0 / 24.0)));
         }
         V n[4];
-        draw4(key, site, 0u, sc, sc, n, true);
+        draw4<9>(key, site, 0u, sc, sc, n, true);
         const V n3 = n[0];
         k[3] = vfma(k11, n3, k[3]);
         k[4] = vfma(n[1], c4, k[4]);
         k[5] = vfma(n[2], c5, k[5]);
         k[6] = vfma(n[3], c67a, k[6]);
-        draw4(key, site, 1u, sc, sc, n, false);
+        draw4<9>(key, site, 1u, sc, sc, n, false);
         k[7] = vfma(n[0], c67b, k[7]);
         k[8] = vfma(k22, n[1], vfma(k21, n3, k[8]));
     }

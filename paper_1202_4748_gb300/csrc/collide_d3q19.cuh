@@ -141,6 +141,7 @@ struct DrawScale<double> {
 // cosine are accurate; the half turn flips the signs of both, which the
 // negated scales undo) is formed from the word in one rounding.
 // need3 = false skips the sine of the second pair (its normal is not used).
+template <int Q>
 __device__ __forceinline__ void draw4(const NoiseKey& k, uint32_t site, uint32_t d, float sc0, float sc1,
                                       float (&n)[4], bool need3) {
     const uint4 w = philox_draw(k, site, d);
@@ -159,6 +160,7 @@ __device__ __forceinline__ void draw4(const NoiseKey& k, uint32_t site, uint32_t
 }
 
 // Two sites: the same sequence lane by lane, the lane-independent arithmetic paired.
+template <int Q>
 __device__ __forceinline__ void draw4(const NoiseKey& k, uint2 site, uint32_t d, float2 sc0, float2 sc1,
                                       float2 (&n)[4], bool need3) {
     const uint4 wa = philox_draw(k, site.x, d);
@@ -179,19 +181,29 @@ __device__ __forceinline__ void draw4(const NoiseKey& k, uint2 site, uint32_t d,
     n[3] = need3 ? vmul(rr1, make_float2(sfu_sin(t1.x), sfu_sin(t1.y))) : make_float2(0.0f, 0.0f);
 }
 
-// FP64: U = (x + 1/2) 2^-32 exactly, R = sqrt(-2 ln U), angle 2 pi U_b.
+// FP64: U = (x + 1/2) 2^-32 exactly, R = sqrt(-2 ln U), angle 2 pi U_b.  The
+// eight pairs of a D3Q19 site (Q = 19) call one copy of the code, which inlined
+// overflowed the instruction cache (256^3: 9.9 -> 9.1 ms per step); the three of
+// a D2Q9 site do not (512^2: 111 us inlined, 124 called).
+__device__ __forceinline__ double2 normal_pair(uint32_t wa, uint32_t wb, double sc) {
+    double c, s;
+    const double r = vmul(sc, n64_radius(wa, LogTable()));
+    n64_angle(wb, c, s);
+    return make_double2(vmul(r, c), vmul(r, s));
+}
+static __device__ __noinline__ double2 normal_pair_call(uint32_t wa, uint32_t wb, double sc) {
+    return normal_pair(wa, wb, sc);
+}
+template <int Q>
 __device__ __forceinline__ void draw4(const NoiseKey& k, uint32_t site, uint32_t d, double sc0, double sc1,
                                       double (&n)[4], bool need3) {
     const uint4 w = philox_draw(k, site, d);
-    double c, s;
-    const double r0 = vmul(sc0, n64_radius(w.x, LogTable()));
-    n64_angle(w.y, c, s);
-    n[0] = vmul(r0, c);
-    n[1] = vmul(r0, s);
-    const double r1 = vmul(sc1, n64_radius(w.z, LogTable()));
-    n64_angle(w.w, c, s);
-    n[2] = vmul(r1, c);
-    n[3] = need3 ? vmul(r1, s) : 0.0;
+    const double2 a = Q == 19 ? normal_pair_call(w.x, w.y, sc0) : normal_pair(w.x, w.y, sc0);
+    const double2 b = Q == 19 ? normal_pair_call(w.z, w.w, sc1) : normal_pair(w.z, w.w, sc1);
+    n[0] = a.x;
+    n[1] = a.y;
+    n[2] = b.x;
+    n[3] = b.y;
 }
 
 // 1 / sqrt(x) lane by lane.
@@ -342,23 +354,23 @@ __device__ __forceinline__ void d3q19_tau1_noise_and_populations(V (&h)[19], V (
         const double c5 = 1.0 / (36.0 * 1.1547005383792515), c6 = 1.0 / 24.0, c7 = 1.0 / 12.0;
         const double c10 = 1.0 / (36.0 * 0.81649658092772603), c13 = 1.0 / (12.0 * 1.4142135623730951);
         V n[4];
-        draw4(key, site, 0u, sc, sc, n, true);
+        draw4<19>(key, site, 0u, sc, sc, n, true);
         const V n4 = n[0];
         h[4] = vfma(k11, n4, h[4]);
         h[5] = vfma(n[1], vk<V>(c5), h[5]);
         h[6] = vfma(n[2], vk<V>(c6), h[6]);
         h[7] = vfma(n[3], vk<V>(c7), h[7]);
-        draw4(key, site, 1u, sc, vmul(sc, vk<V>(c10)), n, true);
+        draw4<19>(key, site, 1u, sc, vmul(sc, vk<V>(c10)), n, true);
         h[8] = vfma(n[0], vk<V>(c7), h[8]);
         h[9] = vfma(n[1], vk<V>(c7), h[9]);
         h[10] = n[2];
         h[11] = n[3];
-        draw4(key, site, 2u, sc, vmul(sc, vk<V>(c13)), n, true);
+        draw4<19>(key, site, 2u, sc, vmul(sc, vk<V>(c13)), n, true);
         h[12] = vmul(n[0], vk<V>(c10));
         h[13] = vmul(n[1], vk<V>(c13));
         h[14] = n[2];
         h[15] = n[3];
-        draw4(key, site, 3u, sc, sc, n, false);
+        draw4<19>(key, site, 3u, sc, sc, n, false);
         h[16] = vfma(k22, n[0], vfma(k21, n4, h[16]));
         h[17] = vmul(n[1], vk<V>(c5));
         h[18] = vmul(n[2], vk<V>(c6));
@@ -693,23 +705,23 @@ __device__ __forceinline__ void collide_d3q19_rates(V (&f)[19], const V drho, co
         // sqrt(N_a g_aa) / (36 N_a), 36 N_a as above
         auto amp = [&](int a, double inv) { return vbc<V>(vmul(P.namp[a], S(inv))); };
         V n[4];
-        draw4(key, site, 0u, sc, sc, n, true);
+        draw4<19>(key, site, 0u, sc, sc, n, true);
         const V n4 = n[0];
         k[4] = vfma(k11, n4, k[4]);
         k[5] = vfma(n[1], amp(5, 1.0 / 48.0), k[5]);
         k[6] = vfma(n[2], amp(6, 1.0 / 16.0), k[6]);
         k[7] = vfma(n[3], amp(7, 1.0 / 4.0), k[7]);
-        draw4(key, site, 1u, sc, sc, n, true);
+        draw4<19>(key, site, 1u, sc, sc, n, true);
         k[8] = vfma(n[0], amp(8, 1.0 / 4.0), k[8]);
         k[9] = vfma(n[1], amp(9, 1.0 / 4.0), k[9]);
         k[10] = vfma(n[2], amp(10, 1.0 / 24.0), k[10]);
         k[11] = vfma(n[3], amp(11, 1.0 / 24.0), k[11]);
-        draw4(key, site, 2u, sc, sc, n, true);
+        draw4<19>(key, site, 2u, sc, sc, n, true);
         k[12] = vfma(n[0], amp(12, 1.0 / 24.0), k[12]);
         k[13] = vfma(n[1], amp(13, 1.0 / 8.0), k[13]);
         k[14] = vfma(n[2], amp(14, 1.0 / 8.0), k[14]);
         k[15] = vfma(n[3], amp(15, 1.0 / 8.0), k[15]);
-        draw4(key, site, 3u, sc, sc, n, false);
+        draw4<19>(key, site, 3u, sc, sc, n, false);
         k[16] = vfma(k22, n[0], vfma(k21, n4, k[16]));
         k[17] = vfma(n[1], amp(17, 1.0 / 48.0), k[17]);
         k[18] = vfma(n[2], amp(18, 1.0 / 16.0), k[18]);
