@@ -259,7 +259,7 @@ double estimated_step_us(const lb_system_desc* s, int n, const int tdim[3], bool
     }
     const SplitCost c = split_cost(kind, quads);
     const double cost = c.plane * planes + c.chunk;
-    const double load = ctas / sms, filled = load <= 4.0 ? std::ceil(load) : load + 0.5;
+    const double load = ctas / sms, filled = std::max(1.0, load + 0.5);
     return 3.0 + sites * c.moment + std::max(c.alone_chunk + c.alone_plane * planes, filled * cost);
 }
 
@@ -584,7 +584,7 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
     P.pop1 = take(es * q * P.n_sites);
     P.step = take(sizeof(int64_t));
     P.status = take(sizeof(int));
-    P.dbar = take(sizeof(double) * n);
+    P.dbar = take(sizeof(double) * 2 * n);       // mean deviation, 1 / mean density
     P.site_items = take(sizeof(int4) * P.n_site_items);
     P.site_partial = take(sizeof(double) * 4 * P.n_site_items);
     P.spans = take(sizeof(SysSpan) * n);

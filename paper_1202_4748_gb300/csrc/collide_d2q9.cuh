@@ -42,7 +42,7 @@ __device__ __forceinline__ float density_of(const float (&f)[Q]) {
 }
 template <int Q>
 __device__ __forceinline__ double density_of(const double (&f)[Q]) {
-    const FixedSum<Q> s(f);
+    const FixedSum<double, Q> s(f);
     if (s.finite()) {
         int64_t v = 0;
 #pragma unroll
@@ -60,7 +60,7 @@ __device__ __forceinline__ double density_of(const double (&f)[Q]) {
 template <class V>
 __device__ __forceinline__ void moments_d2q9(const V (&f)[9], V& drho, V& jx, V& jy) {
     if constexpr (VT<V>::W == 1 && sizeof(V) == 8) {
-        const FixedSum<9> s(f);
+        const FixedSum<double, 9> s(f);
         if (s.finite()) {
             const int64_t(&m)[9] = s.m;
             const int64_t a = m[5] - m[6], b = m[7] - m[8];

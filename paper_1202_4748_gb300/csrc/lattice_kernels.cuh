@@ -22,15 +22,21 @@ struct BlockSum {
     double v[K][NT];
     double res[K];
 };
-template <int K, int NT>
+// The NT threads are the CTA's first; BAR > 0: only they take part, on that
+// named barrier.
+template <int K, int NT, int BAR = 0>
 __device__ __forceinline__ void block_sum(double (&v)[K], BlockSum<K, NT>& sh, int active = NT) {
     constexpr int NW = NT / 32;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (active + 31) >> 5;
+    auto barrier = [] {
+        if constexpr (BAR > 0) named_barrier(BAR, NT);
+        else __syncthreads();
+    };
     if (w < nw) {
 #pragma unroll
         for (int k = 0; k < K; ++k) sh.v[k][threadIdx.x] = v[k];
     }
-    __syncthreads();
+    barrier();
     for (int k = w; k < K; k += NW) {
         double s = sh.v[k][lane];
         for (int u = 1; u < nw; ++u) s += sh.v[k][32 * u + lane];
@@ -38,7 +44,7 @@ __device__ __forceinline__ void block_sum(double (&v)[K], BlockSum<K, NT>& sh, i
         for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
         if (lane == 0) sh.res[k] = s;
     }
-    __syncthreads();
+    barrier();
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int k = 0; k < K; ++k) v[k] = sh.res[k];
@@ -63,7 +69,7 @@ __global__ void __launch_bounds__(AUX_THREADS)
     const int nx = S.nx, ny = S.ny, nz = S.nz;
     const int64_t N = S.n_sites;
     const double* ds = d + S.site_offset;
-    const double db = dbar[it.x];
+    const double db = dbar[2 * it.x];
     for (int j = 0; j < SITES_PER_THREAD; ++j) {
         const int site = it.y + j * AUX_THREADS + threadIdx.x;
         if (site >= it.z) break;
@@ -177,44 +183,14 @@ __global__ void __launch_bounds__(AUX_THREADS)
         Real(in[int64_t(blockIdx.y) * S.n_sites + site] - (i == 0 ? S.rho_c : 0.0));
 }
 
-// Compensated sum (Knuth's TwoSum): s + c carries the exact sum of the added
-// values up to the rounding of c, i.e. to about eps^2 relative.
-template <class Real>
-struct CompSum {
-    Real s = Real(0), c = Real(0);
-    __device__ __forceinline__ void add(Real v) {
-        const Real t = s + v;
-        const Real bp = t - s;
-        c += (s - (t - bp)) + (v - bp);
-        s = t;
-    }
-    __device__ __forceinline__ double value() const { return double(s) + double(c); }
-};
-
-// Sums of the pulled populations of a site to FP64 accuracy: rv = sum_i f_i,
-// mv = sum_i c_i f_i.  FP32 storage: compensated FP32 sums; FP64 storage:
-// integer additions (FixedSum).  Both keep the per-population work off the FP64
-// units, which do two operations per clock and SM (compensated FP64 sums took
-// 0.39 ms for the 573,440 sites of 64 systems, 340 FP64 operations per site).
-template <class L>
-__device__ __forceinline__ void site_sums(const float (&f)[L::Q], double& rv, double (&mv)[3]) {
-    CompSum<float> r, m[3];
-#pragma unroll
-    for (int i = 0; i < L::Q; ++i) {
-        r.add(f[i]);
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            if (L::c(i, a) == 1) m[a].add(f[i]);
-            if (L::c(i, a) == -1) m[a].add(-f[i]);
-        }
-    }
-    rv = r.value();
-    for (int a = 0; a < L::D; ++a) mv[a] = m[a].value();
-    if (L::D == 2) mv[2] = 0.0;
-}
-template <class L>
-__device__ __forceinline__ void site_sums(const double (&f)[L::Q], double& rv, double (&mv)[3]) {
-    const FixedSum<L::Q> s(f);
+// Sums of the pulled populations of a site to FP64 accuracy, rv = sum_i f_i,
+// mv = sum_i c_i f_i, by integer additions (FixedSum): the per-population work
+// and the conversions stay off the FP64 units, which do two operations per clock
+// and SM.  (Compensated FP64 sums took 0.39 ms for 573,440 FP64 sites; compensated
+// FP32 sums with eight conversions per site 57 us for 2^20 FP32 sites, now 47.)
+template <class L, class Real>
+__device__ __forceinline__ void site_sums(const Real (&f)[L::Q], double& rv, double (&mv)[3]) {
+    const FixedSum<Real, L::Q> s(f);
     int64_t r = 0, m[3] = {0, 0, 0};
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) {
@@ -227,8 +203,8 @@ __device__ __forceinline__ void site_sums(const double (&f)[L::Q], double& rv, d
     if (!s.finite()) {
         rv = mv[0] = mv[1] = mv[2] = 0.0;
         for (int i = 0; i < L::Q; ++i) {
-            rv += f[i];
-            for (int a = 0; a < 3; ++a) mv[a] += L::c(i, a) * f[i];
+            rv += double(f[i]);
+            for (int a = 0; a < 3; ++a) mv[a] += L::c(i, a) * double(f[i]);
         }
     }
 }
@@ -263,7 +239,7 @@ __global__ void __launch_bounds__(AUX_THREADS)
         for (int i = 0; i < L::Q; ++i)
             f[i] = fb[i * S.ns + X[1 + L::c(i, 0)] + Y[1 + L::c(i, 1)] + Z[1 + L::c(i, 2)]];
         double rv, mv[3];
-        site_sums<L>(f, rv, mv);
+        site_sums<L, Real>(f, rv, mv);
         d[S.site_offset + site] = rv;
         if (jout) {
 #pragma unroll

@@ -124,6 +124,7 @@ cudaError_t launch_selftest_wait(int* status, cudaStream_t st);
 
 cudaError_t launch_init_noise(const SysDev* sys, const int4* items, int n_items, double amp, double* d,
                               double* partial, cudaStream_t st);
+// dbar[2 s], dbar[2 s + 1]: mean density deviation of system s and 1 / its mean density.
 cudaError_t launch_reduce_globals(const SysDev* sys, const SysSpan* spans, int n_sys, const double* partial,
                                   double* dbar, double* glob, int set_mass0, int count_sample, cudaStream_t st);
 cudaError_t launch_set_dbar(const SysDev* sys, int n_sys, double* dbar, cudaStream_t st);
@@ -154,6 +155,7 @@ constexpr int kThreadSites = 32, kWarpSites = 1024, kPartSites = 4096;
 // system has one SM's FP64 unit (two operations per clock): 4,096 blocks cost
 // it 30 us, 512 blocks 4 us, about a launch.
 constexpr int kTopBlocks = 512;
+constexpr int kMaxObsLevels = 40;       // block levels of a system (halvings of a side below 2^31, and single sites)
 constexpr int REC = 6;      // per record: sum m, m^2, |m|, m^4, e, e^2
 
 }  // namespace lbf

@@ -149,7 +149,7 @@ NaLayout na_layout(const NaPlan& P) {
     o.items = take(sizeof(int4) * P.n_items);
     o.span = take(sizeof(SysSpan));
     o.part = take(sizeof(double) * 4 * P.n_items);
-    o.dbar = take(sizeof(double));
+    o.dbar = take(2 * sizeof(double));
     o.glob = take(sizeof(double) * 8);
     o.stat = take(sizeof(int));
     o.S = take(sizeof(double) * P.blk);

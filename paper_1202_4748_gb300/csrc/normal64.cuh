@@ -27,6 +27,7 @@
 
 #include <cstdint>
 #include <cstring>
+#include <type_traits>
 
 #ifdef __CUDACC__
 #define LB_HD __host__ __device__ __forceinline__
@@ -141,45 +142,56 @@ LB_HD double n64_inv_sqrt(double x) {
     return n64_double(r << 2, 1 - h);
 }
 
-// Sums of N doubles to about 2^-57 of the largest: the mantissas aligned to the
-// largest exponent as integers of 58 bits, so that a sum of up to 19 of them
-// fits 63 bits and every sum costs integer additions.  finite() is false when
-// a value is infinite or NaN (the sums are then the caller's in FP64).
-template <int N>
+// Sums of N floats or doubles to about 2^-57 of the largest: the mantissas
+// aligned to the largest exponent as integers of 58 bits, so that a sum of up to
+// 31 of them fits 63 bits and every sum costs integer additions (floats within
+// 2^-34 of the largest enter exactly).  finite() is false when a value is
+// infinite or NaN (the sums are then the caller's in FP64).
+template <class T, int N>
 struct FixedSum {
     static_assert(N <= 31, "headroom");
+    using Bits = typename std::conditional<sizeof(T) == 8, uint64_t, uint32_t>::type;
+    static constexpr int kMant = sizeof(T) == 8 ? 52 : 23;            // stored mantissa bits
+    static constexpr int kExp = sizeof(T) == 8 ? 20 : 23;             // exponent's place in the high word
+    static constexpr uint32_t kTop = sizeof(T) == 8 ? 0x7ff00000u : 0x7f800000u;
+    static constexpr int kBias = sizeof(T) == 8 ? 1023 : 127;
     int64_t m[N];
     uint32_t top;                  // largest exponent field, in place
-    LB_HD explicit FixedSum(const double (&f)[N]) {
-        uint64_t u[N];
+    static LB_HD uint32_t high(Bits u) {
+        if constexpr (sizeof(T) == 8) return uint32_t(u >> 32);
+        else return u;
+    }
+    LB_HD explicit FixedSum(const T (&f)[N]) {
+        Bits u[N];
         top = 0;
 #ifdef __CUDACC__
 #pragma unroll
 #endif
         for (int i = 0; i < N; ++i) {
-            memcpy(&u[i], &f[i], 8);
-            const uint32_t e = uint32_t(u[i] >> 32) & 0x7ff00000u;
+            memcpy(&u[i], &f[i], sizeof(T));
+            const uint32_t e = high(u[i]) & kTop;
             top = e > top ? e : top;
         }
 #ifdef __CUDACC__
 #pragma unroll
 #endif
         for (int i = 0; i < N; ++i) {
-            const uint32_t hi = uint32_t(u[i] >> 32), e = hi & 0x7ff00000u;
-            const uint32_t sh = (top - e) >> 20;
+            const uint32_t hi = high(u[i]), e = hi & kTop;
+            const uint32_t sh = (top - e) >> kExp;
             // zeros and subnormals count as 0
-            const uint64_t a = e ? ((u[i] & 0x000fffffffffffffull) | (uint64_t(1) << 52)) << 5 : 0;
+            const Bits one = Bits(1) << kMant;
+            const uint64_t a = e ? uint64_t((u[i] & (one - 1)) | one) << (57 - kMant) : 0;
             const uint64_t half = (uint64_t(1) << (sh & 63)) >> 1;
             const int64_t v = sh > 58 ? 0 : int64_t((a + half) >> (sh & 63));
             m[i] = int32_t(hi) < 0 ? -v : v;
         }
     }
-    LB_HD bool finite() const { return top != 0x7ff00000u; }
-    // the double nearest to s 2^(top - 1023 - 57)
+    LB_HD bool finite() const { return top != kTop; }
+    // the double nearest to s 2^(top - bias - 57)
     LB_HD double value(int64_t s) const {
         if (s == 0) return 0.0;
         const uint64_t a = s < 0 ? uint64_t(0) - uint64_t(s) : uint64_t(s);
-        const int nl = n64_clz(a), e = int(top >> 20) - 1022 - 57 + 63 - nl;      // (m / 2^64) 2^e
+        const int nl = n64_clz(a), e = int(top >> kExp) - kBias + 1 - 57 + 63 - nl;      // (m / 2^64) 2^e
         if (e < -1020) return 0.0;
         const double d = n64_double(a << nl, e);
         return s < 0 ? -d : d;

@@ -70,7 +70,8 @@ __global__ void __launch_bounds__(AUX_THREADS)
     const SysDev& S = sysv[s];
     const double n = double(S.n_sites);
     const double mass = S.rho_c * n + acc[0];
-    dbar[s] = acc[0] / n;
+    dbar[2 * s] = acc[0] / n;
+    dbar[2 * s + 1] = 1.0 / (S.rho_c + acc[0] / n);
     double* g = glob + s * 8;
     if (set_mass0) {
         g[0] = 0.0;
@@ -86,23 +87,33 @@ __global__ void __launch_bounds__(AUX_THREADS)
 
 __global__ void set_dbar_kernel(const SysDev* __restrict__ sysv, int n_sys, double* __restrict__ dbar) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < n_sys) dbar[s] = sysv[s].rho_c;
+    if (s < n_sys) dbar[2 * s] = sysv[s].rho_c;
 }
 
-__device__ __forceinline__ void add_terms(double (&t)[REC], double s, double e, double inv_v) {
-    const double m = s * inv_v;
-    const double E = 0.5 * e * inv_v;
-    const double m2 = m * m;
-    t[0] += m;
-    t[1] += m2;
-    t[2] += fabs(m);
-    t[3] += m2 * m2;
-    t[4] += E;
-    t[5] += E * E;
+// Terms of blocks of volume V from their sums s of phi and e of phi^2: t
+// collects the sums of s, s^2, |s|, s^4, e, e^2, and finish_terms turns them
+// into those of m = s / V, m^2, |m|, m^4, E = e / 2V, E^2.
+__device__ __forceinline__ void add_terms(double (&t)[REC], double s, double e) {
+    const double s2 = s * s;
+    t[0] += s;
+    t[1] += s2;
+    t[2] += fabs(s);
+    t[3] += s2 * s2;
+    t[4] += e;
+    t[5] += e * e;
+}
+__device__ __forceinline__ void finish_terms(double (&t)[REC], double inv_v) {
+    const double v2 = inv_v * inv_v, h = 0.5 * inv_v;
+    t[0] *= inv_v;
+    t[1] *= v2;
+    t[2] *= inv_v;
+    t[3] *= v2 * v2;
+    t[4] *= h;
+    t[5] *= h * h;
 }
 
-// The same for single sites (V = 1: E = m^2 / 2, so its sums are halves and
-// quarters of those of m^2 and m^4, exactly): t = sum m, m^2, |m|, m^4.
+// The same for single sites (V = 1, e = s^2: its sums are halves and quarters
+// of those of m^2 and m^4): t = sum m, m^2, |m|, m^4.
 __device__ __forceinline__ void add_site_terms(double (&t)[REC], double m, double m2) {
     t[0] += m;
     t[1] += m2;
@@ -133,6 +144,26 @@ __device__ __forceinline__ void hist_flush(const unsigned* sh, int n, unsigned l
         if (sh[k]) atomicAdd(g + k, (unsigned long long)sh[k]);
 }
 
+__device__ __forceinline__ double block_volume(const LevelDev& lv) { return double(lv.bx) * lv.by * lv.bz; }
+
+// The CTA's sums of a level's terms as a record (a division occupies the FP64
+// unit like ten additions: one thread's, not every thread's).
+__device__ __forceinline__ void block_record(double (&t)[REC], const LevelDev& lv, BlockSum<REC, OBS_THREADS>& sh,
+                                             double* rec) {
+    block_sum(t, sh);
+    if (threadIdx.x != 0) return;
+    finish_terms(t, 1.0 / block_volume(lv));
+    for (int k = 0; k < REC; ++k) rec[k] = t[k];
+}
+__device__ __forceinline__ void site_record(double (&t)[REC], BlockSum<4, OBS_THREADS>& sh, double* rec) {
+    double v[4] = {t[0], t[1], t[2], t[3]};
+    block_sum(v, sh);
+    if (threadIdx.x != 0) return;
+    for (int k = 0; k < 4; ++k) t[k] = v[k];
+    finish_site_terms(t);
+    for (int k = 0; k < REC; ++k) rec[k] = t[k];
+}
+
 // Block coordinates of block b of a pyramid level: 2^k blocks per axis.
 __device__ __forceinline__ void block_coords(const LevelDev& lv, int b, int& X, int& Y, int& Z) {
     const int kx = 31 - __clz(lv.gx), ky = 31 - __clz(lv.gy);
@@ -151,16 +182,16 @@ __global__ void __launch_bounds__(OBS_THREADS)
                       const double* __restrict__ dbar, double* __restrict__ Sg, double* __restrict__ Eg,
                       double* __restrict__ rec, const HistDev H) {
     __shared__ BlockSum<REC, OBS_THREADS> sh;
+    auto& sh4 = reinterpret_cast<BlockSum<4, OBS_THREADS>&>(sh);   // never between sh's barriers
     extern __shared__ unsigned shist[];          // [block level | single-site level], nbins + 2 each
     const ObsItem it = items[blockIdx.x];
     const LevelDev lv = lvv[it.level];
     const SysDev& S = sysv[lv.sys];
     const double* ds = d + S.site_offset;
-    const double db = dbar[lv.sys];
-    const double inv_rbar = 1.0 / (S.rho_c + db);
-    const double inv_v = 1.0 / (double(lv.bx) * lv.by * lv.bz);
+    const double db = dbar[2 * lv.sys], inv_rbar = dbar[2 * lv.sys + 1];
     const int nh = H.nbins + 2;
     const bool hist = H.nbins > 0;
+    const double inv_v = hist ? 1.0 / block_volume(lv) : 0.0;
     const bool hist_u = hist && it.unit_level >= 0;
     if (hist) {
         hist_clear(shist, hist_u ? 2 * nh : nh);
@@ -193,20 +224,13 @@ __global__ void __launch_bounds__(OBS_THREADS)
         Sg[lv.off + b] = s;
         Eg[lv.off + b] = e;
         if (sites) add_site_terms(tb, s, e);
-        else add_terms(tb, s, e, inv_v);
+        else add_terms(tb, s, e);
         if (hist) atomicAdd(shist + hist_bin(s * inv_v, H), 1u);
     }
-    if (sites) finish_site_terms(tb);
-    finish_site_terms(tu);
-    block_sum(tb, sh);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < REC; ++k) rec[int64_t(it.rec) * REC + k] = tb[k];
-    if (it.unit_level >= 0) {
-        __syncthreads();
-        block_sum(tu, sh);
-        if (threadIdx.x == 0)
-            for (int k = 0; k < REC; ++k) rec[int64_t(it.rec2) * REC + k] = tu[k];
-    }
+    // (of single sites the last two sums follow from the others)
+    if (sites) site_record(tb, sh4, rec + int64_t(it.rec) * REC);
+    else block_record(tb, lv, sh, rec + int64_t(it.rec) * REC);
+    if (it.unit_level >= 0) site_record(tu, sh4, rec + int64_t(it.rec2) * REC);
     if (hist) {
         __syncthreads();
         hist_flush(shist, nh, H.counts + int64_t(it.level) * nh);
@@ -226,17 +250,17 @@ __global__ void __launch_bounds__(OBS_THREADS)
                     double* __restrict__ rec, const HistDev H) {
     constexpr int NW = OBS_THREADS / 32;
     __shared__ BlockSum<REC, OBS_THREADS> sh;
+    auto& sh4 = reinterpret_cast<BlockSum<4, OBS_THREADS>&>(sh);
     auto& sh2 = reinterpret_cast<BlockSum<2, OBS_THREADS>&>(sh);   // used before sh, a barrier apart
     extern __shared__ unsigned shist[];          // [block level | single-site level], nbins + 2 each
     const ObsPart it = items[blockIdx.x];
     const LevelDev lv = lvv[it.level];
     const SysDev& S = sysv[lv.sys];
     const double* ds = d + S.site_offset;
-    const double db = dbar[lv.sys];
-    const double inv_rbar = 1.0 / (S.rho_c + db);
-    const double inv_v = 1.0 / (double(lv.bx) * lv.by * lv.bz);
+    const double db = dbar[2 * lv.sys], inv_rbar = dbar[2 * lv.sys + 1];
     const int nh = H.nbins + 2;
     const bool hist = H.nbins > 0;
+    const double inv_v = hist ? 1.0 / block_volume(lv) : 0.0;
     if (hist) {
         hist_clear(shist, 2 * nh);
         __syncthreads();
@@ -250,7 +274,7 @@ __global__ void __launch_bounds__(OBS_THREADS)
     auto block_done = [&](int b, double s, double e) {
         Sg[lv.off + b] = s;
         Eg[lv.off + b] = e;
-        add_terms(tb, s, e, inv_v);
+        add_terms(tb, s, e);
         if (hist) atomicAdd(shist + hist_bin(s * inv_v, H), 1u);
     };
     for (int b = it.b0 + (by_warp ? warp : 0); b < it.b1; b += by_warp ? NW : 1) {
@@ -282,16 +306,8 @@ __global__ void __launch_bounds__(OBS_THREADS)
             __syncthreads();
         }
     }
-    finish_site_terms(tu);
-    if (it.part < 0) {
-        block_sum(tb, sh);
-        if (threadIdx.x == 0)
-            for (int k = 0; k < REC; ++k) rec[int64_t(it.rec) * REC + k] = tb[k];
-        __syncthreads();
-    }
-    block_sum(tu, sh);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < REC; ++k) rec[int64_t(it.rec2) * REC + k] = tu[k];
+    if (it.part < 0) block_record(tb, lv, sh, rec + int64_t(it.rec) * REC);
+    site_record(tu, sh4, rec + int64_t(it.rec2) * REC);
     if (hist) {
         __syncthreads();
         if (it.part < 0) hist_flush(shist, nh, H.counts + int64_t(it.level) * nh);
@@ -309,7 +325,6 @@ __global__ void __launch_bounds__(OBS_THREADS)
     __shared__ BlockSum<REC, OBS_THREADS> sh;
     const ObsBlocks it = items[blockIdx.x];
     const LevelDev lv = lvv[it.level];
-    const double inv_v = 1.0 / (double(lv.bx) * lv.by * lv.bz);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double tb[REC] = {0, 0, 0, 0, 0, 0};
     for (int b = it.b0 + warp; b < it.b1; b += NW) {
@@ -328,14 +343,12 @@ __global__ void __launch_bounds__(OBS_THREADS)
         if (lane == 0) {
             Sg[lv.off + b] = s;
             Eg[lv.off + b] = e;
-            add_terms(tb, s, e, inv_v);
+            add_terms(tb, s, e);
             if (H.nbins > 0)
-                atomicAdd(H.counts + int64_t(it.level) * (H.nbins + 2) + hist_bin(s * inv_v, H), 1ull);
+                atomicAdd(H.counts + int64_t(it.level) * (H.nbins + 2) + hist_bin(s * (1.0 / block_volume(lv)), H), 1ull);
         }
     }
-    block_sum(tb, sh);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < REC; ++k) rec[int64_t(it.rec) * REC + k] = tb[k];
+    block_record(tb, lv, sh, rec + int64_t(it.rec) * REC);
 }
 
 // Sums of phi and phi^2 of block b of level lv over its 2^d children (level
@@ -366,9 +379,9 @@ __global__ void __launch_bounds__(OBS_THREADS)
     const ObsItem it = items[blockIdx.x];
     const LevelDev lv = lvv[it.level];
     const LevelDev ch = lvv[lv.child];
-    const double inv_v = 1.0 / (double(lv.bx) * lv.by * lv.bz);
     const int nh = H.nbins + 2;
     const bool hist = H.nbins > 0;
+    const double inv_v = hist ? 1.0 / block_volume(lv) : 0.0;
     if (hist) {
         hist_clear(shist, nh);
         __syncthreads();
@@ -379,12 +392,10 @@ __global__ void __launch_bounds__(OBS_THREADS)
         children_sum(lv, ch, b, dims3, Sg, Eg, s, e);
         Sg[lv.off + b] = s;
         Eg[lv.off + b] = e;
-        add_terms(tb, s, e, inv_v);
+        add_terms(tb, s, e);
         if (hist) atomicAdd(shist + hist_bin(s * inv_v, H), 1u);
     }
-    block_sum(tb, sh);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < REC; ++k) rec[int64_t(it.rec) * REC + k] = tb[k];
+    block_record(tb, lv, sh, rec + int64_t(it.rec) * REC);
     if (hist) {
         __syncthreads();
         hist_flush(shist, nh, H.counts + int64_t(it.level) * nh);
@@ -420,42 +431,98 @@ __device__ __forceinline__ void accumulate_records(const LevelDev& lv, const dou
 }
 
 // The coarsest levels of one system per CTA: levels top - 1 .. 0 (level `top`
-// is complete), each behind a CTA barrier because it reads the block sums that
-// other threads of the CTA wrote; level l's six sums go straight into its
-// accumulators.  The other levels' records are accumulated by a warp each.
+// is complete), one after another in the first kTopChain threads, with the
+// block sums of the level below in shared memory (the first takes them from
+// memory) and levels of at most 32 blocks in one warp without a barrier; the
+// levels' sums are accumulated together at the end.  The other warps meanwhile
+// accumulate the records of the other levels.  A chain of latencies: 16^3, four
+// levels, 17 us (22 us with the block sums in memory and CTA-wide barriers).
 __global__ void __launch_bounds__(TOP_THREADS)
     pyr_top_kernel(const LevelDev* __restrict__ lvv, const ObsTop* __restrict__ tops, int dims3, double* Sg,
                    double* Eg, const double* __restrict__ rec, double* __restrict__ acc, int* status,
                    const HistDev H) {
-    constexpr int NW = TOP_THREADS / 32;
-    __shared__ BlockSum<REC, TOP_THREADS> sh;
+    constexpr int NC = TOP_THREADS / 2;
+    __shared__ BlockSum<REC, NC> sh;
+    __shared__ double bs[2][kTopBlocks], be[2][kTopBlocks];
+    __shared__ double sums[kMaxObsLevels][REC];
+    __shared__ LevelDev lvs[kMaxObsLevels];
     extern __shared__ unsigned shist[];
     const ObsTop T = tops[blockIdx.x];
-    const int nh = H.nbins + 2;
+    const int nh = H.nbins + 2, tid = threadIdx.x;
     const bool hist = H.nbins > 0;
-    for (int l = T.top + int(threadIdx.x >> 5); l < T.n_levels; l += NW)
-        accumulate_records(lvv[T.lv_first + l], rec, acc + int64_t(T.lv_first + l) * 7, status);
+    for (int l = tid; l < T.n_levels; l += TOP_THREADS) lvs[l] = lvv[T.lv_first + l];
+    __syncthreads();
+    double* const my_acc = acc + int64_t(T.lv_first) * 7;
+    if (tid >= NC) {
+        for (int l = T.top + (tid - NC) / 32; l < T.n_levels; l += NC / 32)
+            accumulate_records(lvs[l], rec, my_acc + 7 * l, status);
+        return;
+    }
     for (int l = T.top - 1; l >= 0; --l) {
-        const LevelDev lv = lvv[T.lv_first + l];
-        const LevelDev ch = lvv[T.lv_first + l + 1];
-        const double inv_v = 1.0 / (double(lv.bx) * lv.by * lv.bz);
+        const LevelDev& lv = lvs[l];
+        const LevelDev& ch = lvs[l + 1];
+        const int nb = int(lv.nblocks), src = (l + 1) & 1, dst = l & 1;
+        const double inv_v = hist ? 1.0 / block_volume(lv) : 0.0;
+        const bool warp_only = nb <= 32;
+        if (warp_only && tid >= 32) break;                // the remaining levels have no more blocks than this one
         if (hist) {
-            hist_clear(shist, nh);
-            __syncthreads();
+            for (int k = tid; k < nh; k += warp_only ? 32 : NC) shist[k] = 0u;
+            if (warp_only) __syncwarp();
+            else named_barrier(1, NC);
         }
         double tb[REC] = {0, 0, 0, 0, 0, 0};
-        for (int b = threadIdx.x; b < int(lv.nblocks); b += TOP_THREADS) {
-            double s, e;
-            children_sum(lv, ch, b, dims3, Sg, Eg, s, e);
-            Sg[lv.off + b] = s;
-            Eg[lv.off + b] = e;
-            add_terms(tb, s, e, inv_v);
+        for (int b = tid; b < nb; b += NC) {
+            double s = 0.0, e = 0.0;
+            if (l == T.top - 1) {
+                children_sum(lv, ch, b, dims3, Sg, Eg, s, e);
+            } else {
+                int X, Y, Z;
+                block_coords(lv, b, X, Y, Z);
+                const int nz = dims3 ? 2 : 1;
+                for (int dz = 0; dz < nz; ++dz)
+#pragma unroll
+                    for (int dy = 0; dy < 2; ++dy) {
+                        const int c = 2 * X + ch.gx * (2 * Y + dy + ch.gy * (nz * Z + dz));
+                        s += bs[src][c];
+                        e += be[src][c];
+                        s += bs[src][c + 1];
+                        e += be[src][c + 1];
+                    }
+            }
+            bs[dst][b] = s;
+            be[dst][b] = e;
+            add_terms(tb, s, e);
             if (hist) atomicAdd(shist + hist_bin(s * inv_v, H), 1u);
         }
-        block_sum(tb, sh, int(min(int64_t(TOP_THREADS), lv.nblocks)));      // its barrier also orders this level's block sums
-        if (threadIdx.x == 0) accumulate_level(acc + int64_t(T.lv_first + l) * 7, double(lv.nblocks), tb, status);
-        if (hist) hist_flush(shist, nh, H.counts + int64_t(T.lv_first + l) * nh);
-        __syncthreads();
+        if (warp_only) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int k = 0; k < REC; ++k) tb[k] += __shfl_down_sync(0xffffffffu, tb[k], o);
+        } else {
+            block_sum<REC, NC, 1>(tb, sh, min(NC, nb));   // its barriers also order this level's block sums
+        }
+        if (tid == 0) {
+#pragma unroll
+            for (int k = 0; k < REC; ++k) sums[l][k] = tb[k];
+        }
+        if (hist) {
+            if (warp_only) __syncwarp();
+            unsigned long long* g = H.counts + int64_t(T.lv_first + l) * nh;
+            for (int k = tid; k < nh; k += warp_only ? 32 : NC)
+                if (shist[k]) atomicAdd(g + k, (unsigned long long)shist[k]);
+        }
+        if (warp_only) __syncwarp();
+        else named_barrier(1, NC);
+    }
+    // warp 0, which has seen every level end: a lane per level adds its sums
+    if (tid < T.top) {
+        double t[REC];
+#pragma unroll
+        for (int k = 0; k < REC; ++k) t[k] = sums[tid][k];
+        const LevelDev& lv = lvs[tid];
+        finish_terms(t, 1.0 / block_volume(lv));
+        accumulate_level(my_acc + 7 * tid, double(lv.nblocks), t, status);
     }
 }
 

@@ -39,14 +39,13 @@ __global__ void sk_twiddle_kernel(double* __restrict__ tw, const int* __restrict
 // With dbar the input is phi = (d - dbar) / (rho_c + dbar); without (null) it
 // is the field d itself.
 __global__ void __launch_bounds__(AUX_THREADS)
-    sk_x_kernel(const SysDev* __restrict__ sysv, const SkSys* __restrict__ skv, const int4* __restrict__ items,
+    sk_x_kernel(const SkSys* __restrict__ skv, const int4* __restrict__ items,
                 const double* __restrict__ d, const double* __restrict__ dbar, const double* __restrict__ tw,
                 double* __restrict__ out) {
     const int4 it = items[blockIdx.x];
     const SkSys K = skv[it.x];
-    const SysDev& S = sysv[it.x];
-    const double db = dbar ? dbar[it.x] : 0.0;
-    const double inv_rbar = dbar ? 1.0 / (S.rho_c + db) : 1.0;
+    const double db = dbar ? dbar[2 * it.x] : 0.0;
+    const double inv_rbar = dbar ? dbar[2 * it.x + 1] : 1.0;
     for (int j = 0; j < SITES_PER_THREAD; ++j) {
         const int e = it.y + j * AUX_THREADS + threadIdx.x;
         if (e >= it.z) break;
@@ -201,7 +200,7 @@ __device__ __forceinline__ double2* fft_lines(double2* A, double2* B, int nl, in
 // as z_j = a_2j + i a_(2j+1), j < S/2 = h: with Z the transform of z,
 // F(k) = E + W_S^k O, E = (Z_k + conj Z_(h-k))/2, O = -i (Z_k - conj Z_(h-k))/2.
 __global__ void __launch_bounds__(FFT_THREADS)
-    fft_x_kernel(const SysDev* __restrict__ sysv, const SkSys* __restrict__ skv, const int4* __restrict__ items,
+    fft_x_kernel(const SkSys* __restrict__ skv, const int4* __restrict__ items,
                  const double* __restrict__ d, const double* __restrict__ dbar, const double* __restrict__ jf,
                  int64_t jstride, const double2* __restrict__ twv, double2* __restrict__ F, int64_t fstride) {
     extern __shared__ double2 fft_buf[];
@@ -214,8 +213,8 @@ __global__ void __launch_bounds__(FFT_THREADS)
     double db = 0.0, inv = 1.0;
     const double* src = it.w == 0 ? d : jf + (it.w - 1) * jstride;
     if (it.w == 0) {
-        db = dbar[it.x];
-        inv = 1.0 / (sysv[it.x].rho_c + db);
+        db = dbar[2 * it.x];
+        inv = dbar[2 * it.x + 1];
     }
     src += K.site_offset + int64_t(it.y) * S;
     // the samples in order: interleaved they are the packed complex line
@@ -493,7 +492,7 @@ cudaError_t launch_sk_twiddles(double* tw, const int* sides, const int* offs, in
 cudaError_t launch_sk_x(const SysDev* sys, const SkSys* sk, const int4* items, int n_items, const double* d,
                         const double* dbar, const double* tw, double* out, cudaStream_t st) {
     if (n_items == 0) return cudaSuccess;
-    sk_x_kernel<<<n_items, AUX_THREADS, 0, st>>>(sys, sk, items, d, dbar, tw, out);
+    sk_x_kernel<<<n_items, AUX_THREADS, 0, st>>>(sk, items, d, dbar, tw, out);
     return cudaGetLastError();
 }
 
@@ -524,7 +523,7 @@ cudaError_t launch_sk_fft(const FftLaunch& a, cudaStream_t st) {
     double2* F = reinterpret_cast<double2*>(a.F);
     // both line buffers of the largest item
     const size_t line = 2 * sizeof(double2);
-    fft_x_kernel<<<a.n_x, FFT_THREADS, line * a.max_x, st>>>(a.sys, a.sk, a.items, a.d, a.dbar, a.j, a.n_sites, tw, F,
+    fft_x_kernel<<<a.n_x, FFT_THREADS, line * a.max_x, st>>>(a.sk, a.items, a.d, a.dbar, a.j, a.n_sites, tw, F,
                                                             a.fstride);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && a.dims == 3) {

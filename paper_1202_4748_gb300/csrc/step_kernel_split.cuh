@@ -183,7 +183,9 @@ __global__ void __launch_bounds__(TX* TY, MINB)
 
     const int4 tl = A.tiles[blockIdx.x];
     const SysDev& S = A.sys[tl.x];
-    const SysPhys<Real>& P = A.phys[tl.x];
+    // fully relaxed: the few parameters it takes, in registers before the first wait
+    using Phys = typename std::conditional<MODE == 2, const SysPhys<Real>, const SysPhys<Real>&>::type;
+    Phys P = A.phys[tl.x];
     const int nx = S.nx, ny = S.ny, nz = S.nz, N = S.ns, pl = nx * ny;
     const int z0 = tl.w, z1 = min(z0 + A.zc, nz);
     const int tid = threadIdx.x;
@@ -298,7 +300,7 @@ __global__ void __launch_bounds__(TX* TY, MINB)
                 sites = site;
             }
             if constexpr (PULL && sizeof(Real) == 8) {
-                const FixedSum<19> fs(f);                // as density_of
+                const FixedSum<double, 19> fs(f);                // as density_of
                 sfor<0, 3>([&](auto C) {
                     constexpr int cc = C;
                     int64_t s = 0;
