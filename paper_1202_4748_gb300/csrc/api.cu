@@ -287,32 +287,34 @@ void choose_d3q19_row(const lb_system_desc* s, int n, int kind, bool quads, int&
 // Default row of the D2Q9 row-marching strips (modified equilibrium): the
 // number of rows per strip from the estimated step time, rows 0 (32 rows), 1
 // (16) and the shorter ones of the same kernel.  A strip forms the density of
-// two halo rows more than it collides.  A warp of paired FP32 strips takes
-// 0.9 us per row alone on its scheduler, 1.3 beside one other, 1.8 beside two
-// (3 CTAs of 4 warps per SM); the one-site strips (two warps per tile) keep 5
-// CTAs; in FP64 a CTA of 4 warps takes 8.3 us per row alone on its SM, and 6.4
-// beside others.  32 rows were the default of every ensemble: one 512^2
-// system 33 -> 8 us per step in FP32; in FP64, 64 CTAs on 152 SMs, 293 -> 128.
+// two halo rows more than it collides.  Two-site strips: 0.85 us per row while
+// the latency of a row bounds them, 0.51 us per row and warp of a scheduler when
+// loaded.  One-site strips (two warps per tile): shorter ones read each line
+// closer in time to the strips beside them (4001 x 3999: 32 rows 364 us, 16: 306,
+// 8: 272, 4: 296).  FP64: 7.8 us per row alone on a scheduler, 6.1 beside
+// others.  32 rows were once the default of every ensemble: one 512^2 system
+// 33 -> 8 us per step in FP32; in FP64, 64 CTAs on 152 SMs, 293 -> 98.
 void choose_d2q9_row(const lb_system_desc* s, int n, bool fp32, bool paired, int& tile_id) {
     const int sms = sm_count();
     int t[32][kVariantCols];
     const int nt = tile_table(LB_D2Q9, t);
     const int first = tile_id;
-    constexpr double row_us[6] = {0.0, 0.9, 1.3, 1.8, 1.8, 1.85};      // by warps per scheduler
     double best_us = INFINITY;
     for (int k = 0; k < nt; ++k) {
         if (t[k][5] != 2 || t[k][0] != t[first][0] || t[k][3] != t[first][3] || t[k][1] > t[first][1]) continue;
         const double warps = double(tiles_of(s, n, t[k])) * (paired ? 1 : 2), rows = t[k][1];
+        const double load = warps / (4.0 * sms);                          // warps per scheduler
         double us;
-        if (fp32) {
-            const int ctas = paired ? 3 : 5;
-            const double slots = 4.0 * ctas * sms, full = std::floor(warps / slots), rest = warps - full * slots;
-            us = (rows + 2) * (row_us[ctas] * full + row_us[int(std::ceil(rest / (4.0 * sms)))]);
+        if (paired) {
+            us = 1.5 + std::max(0.85 * (rows + 2), std::max(1.0, load + 0.5) * (0.51 * rows + 0.3));
+        } else if (fp32) {
+            const double filled = load <= 5.0 ? load + 0.5 : load + 1.5;  // 5 warps per scheduler at once
+            us = 1.0 + std::max(0.85 * (rows + 2), filled * (0.3 + 0.25 * rows + 0.0055 * rows * rows));
         } else {
-            const double load = warps / (4.0 * sms), ctas = load <= 4.0 ? std::ceil(load) : load + 0.5;
-            us = (rows + 2) * std::max(8.3, 6.4 * ctas);
+            const double filled = load <= 4.0 ? std::ceil(load) : load + 0.5;
+            us = 5.0 + std::max(7.8, 6.1 * filled) * rows;
         }
-        if (us < 0.98 * best_us) {
+        if (us < 0.99 * best_us) {
             best_us = us;
             tile_id = k;
         }

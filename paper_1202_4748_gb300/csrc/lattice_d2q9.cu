@@ -6,7 +6,8 @@ namespace lbf {
 
 namespace {
 // (x, y, 1, resident CTAs per SM (0 = default), producer warps (0: none), scheme,
-// sites per thread):
+// sites per thread); of the strips, whose CTAs are single warps, the resident
+// column only names the row: MINB below times four of them run per SM:
 // scheme 2 = row-marching warp strips of x sites x y rows (modified equilibrium
 // only; with 2 sites per thread each lane holds two x-adjacent sites, in
 // paired FP32, when every mode is at tau = 1, the run is FP32 and every x side
@@ -25,12 +26,12 @@ constexpr int kNumTiles = int(sizeof(kTiles) / sizeof(kTiles[0]));
 
 template <int CP, class Real, int MINB>
 cudaError_t strip_of(const StepLaunch& a, cudaStream_t st) {
-    if constexpr (CP == MODEQ) return step_strip<D2Q9, CP, Real, 4, MINB>(a, st);
+    if constexpr (CP == MODEQ) return step_strip<D2Q9, CP, Real, 4 * MINB>(a, st);
     return cudaErrorInvalidValue;            // the plan admits strips only with Eq. 65
 }
 template <int CP, class Real, int MINB>
 cudaError_t strip2_of(const StepLaunch& a, cudaStream_t st) {
-    if constexpr (CP == MODEQ) return step_strip2<D2Q9, CP, Real, 4, MINB>(a, st);
+    if constexpr (CP == MODEQ) return step_strip2<D2Q9, CP, Real, 4 * MINB>(a, st);
     return cudaErrorInvalidValue;
 }
 
@@ -41,7 +42,7 @@ cudaError_t step_tile(const StepLaunch& a, cudaStream_t st) {
         case 1:
         case 2:
         case 14:
-        case 15: return strip2_of<CP, Real, 3>(a, st);
+        case 15: return strip2_of<CP, Real, 5>(a, st);
         case 3: return strip2_of<CP, Real, 4>(a, st);
         case 4:
         case 5:

@@ -36,38 +36,37 @@ cudaError_t step_one_mode(const StepLaunch& a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// Row-marching strips (D2Q9, modified equilibrium): WPC warps per CTA, tiles
-// of SW sites x a.zc rows, one warp per 32 sites of a tile.
-template <class L, int CP, class Real, int WPC, int MINB, int MODE, int SW>
+// Row-marching strips (D2Q9, modified equilibrium): tiles of SW sites x a.zc
+// rows, a warp per 32 sites of a tile.  One warp per CTA: everything that is the
+// same in the warp's lanes (the system's records, the tile, the noise key) is
+// then the same in the CTA and needs no register per lane.  With four warps per
+// CTA the two-site kernel took 168 registers, now 92: 20 warps per SM instead
+// of 12.
+template <class L, int CP, class Real, int MINB, int MODE, int SW>
 cudaError_t step_strip_mode(const StepLaunch& a, cudaStream_t st) {
-    const StepArgs<Real> A = step_args<Real>(a);
-    const int warps = a.n_tiles * (SW / 32);
-    const int grid = (warps + WPC - 1) / WPC;
-    step_kernel_strip<L, CP, Real, WPC, MINB, MODE, SW><<<grid, 32 * WPC, 0, st>>>(A, a.n_tiles);
+    step_kernel_strip<L, CP, Real, MINB, MODE, SW><<<a.n_tiles * (SW / 32), 32, 0, st>>>(step_args<Real>(a));
     return cudaGetLastError();
 }
-template <class L, int CP, class Real, int WPC, int MINB, int SW = 32>
+template <class L, int CP, class Real, int MINB, int SW = 32>
 cudaError_t step_strip(const StepLaunch& a, cudaStream_t st) {
     constexpr int MB = sizeof(Real) == 4 && MINB > 0 ? MINB : 1;   // FP64 keeps its registers
-    if (a.bgk_only == 2) return step_strip_mode<L, CP, Real, WPC, MB, 2, SW>(a, st);
-    if (a.bgk_only == 1) return step_strip_mode<L, CP, Real, WPC, MB, 1, SW>(a, st);
-    return step_strip_mode<L, CP, Real, WPC, MB, 0, SW>(a, st);
+    if (a.bgk_only == 2) return step_strip_mode<L, CP, Real, MB, 2, SW>(a, st);
+    if (a.bgk_only == 1) return step_strip_mode<L, CP, Real, MB, 1, SW>(a, st);
+    return step_strip_mode<L, CP, Real, MB, 0, SW>(a, st);
 }
 
 // Two-site strips (D2Q9, modified equilibrium, FP32, every mode at tau = 1,
 // every x side a multiple of 4) on tiles of 64 sites x a.zc rows; any other run
 // of the same tiles takes the one-site strips, two warps per tile.
-template <class L, int CP, class Real, int WPC, int MINB>
+template <class L, int CP, class Real, int MINB>
 cudaError_t step_strip2(const StepLaunch& a, cudaStream_t st) {
     if constexpr (sizeof(Real) == 4 && CP == MODEQ) {
         if (a.bgk_only == 2 && a.pair_ok) {
-            const StepArgs<float> A = step_args<float>(a);
-            const int grid = (a.n_tiles + WPC - 1) / WPC;
-            step_kernel_strip_pair<WPC, MINB><<<grid, 32 * WPC, 0, st>>>(A, a.n_tiles);
+            step_kernel_strip_pair<MINB><<<a.n_tiles, 32, 0, st>>>(step_args<float>(a));
             return cudaGetLastError();
         }
     }
-    return step_strip<L, CP, Real, WPC, MINB, 64>(a, st);
+    return step_strip<L, CP, Real, MINB, 64>(a, st);
 }
 
 // z-marching launches (FP32, every mode at tau = 1): columns of TX x TY sites,

@@ -629,32 +629,51 @@ struct Nbr9 {
     __device__ __forceinline__ Real at() const { return v[1 + CY][1 + CX]; }
 };
 
+// Most rows a strip has.
+constexpr int kStripRows = 64;
+
+// Density deviations beside a strip of W columns from x0: halo[0][r] and
+// halo[1][r] of the sites x0 - 1 and x0 + W in row y0 - 1 + r, rows y0 - 1 .. y1,
+// a site per lane, before the strip's first row: two lanes in every row of the
+// march cost the whole warp's issue slots (and in FP64 its integer units).
+template <class L, int W, class Real>
+__device__ __forceinline__ void strip_halo(const Real* __restrict__ fb, int N, int nx, int ny, int x0, int y0, int y1,
+                                           Real (&halo)[2][kStripRows + 2]) {
+    const int rows = y1 - y0 + 2;
+    for (int t = threadIdx.x; t < 2 * rows; t += 32) {
+        const int side = t < rows ? 0 : 1, r = t - side * rows;
+        const Nbr nb(wrapm(side ? x0 + W : x0 - 1, nx), wrapm(y0 - 1 + r, ny), 0, nx, ny, 1, false);
+        Real g[L::Q];
+        pull_site<L, Real>(fb, N, nb, g);
+        halo[side][r] = density_of(g);
+    }
+    __syncwarp();
+}
+
 // Row-marching strips for the D2Q9 modified-equilibrium step (Eq. 65 needs
 // the density on the 3 x 3 neighbourhood only).  Each warp owns 32
 // consecutive sites of a row and walks A.zc rows; a tile (system, x0, y0) is SW
 // sites wide (32, or 64 for the tiles of the two-site kernel, whose one-site
 // form gives each tile two warps).  Per footprint row yy a lane pulls its
 // site's 9 populations, forms rho, and the neighbours' rho comes by warp
-// shuffles; lanes 0 and 31 also pull the halo sites x0 - 1 and x0 + 32.
+// shuffles, that of the sites x0 - 1 and x0 + 32 from shared memory (strip_halo).
 // Three density rows live in registers as (x - 1, x, x + 1) triples, and the
 // site of row yy - 1 collides from its populations pulled one iteration
 // earlier (with every mode at tau = 1, from its density and momentum only;
 // the collision is collide_d2q9_modeq for every relaxation setting).
-// No shared memory and no CTA barrier: every footprint value is formed once
+// No CTA barrier: every footprint value is formed once
 // per chunk (halo 2/32 in x, 2 rows in y).  Lanes past the system's last column
 // form the periodic image of their column for their neighbours and do not
 // collide.  (Colliding two rows behind, to overlap the next row's loads,
 // measured slower: 8 more registers per thread, fewer warps in flight.)
-template <class L, int CP, class Real, int WPC, int MINB, int MODE, int SW = 32>
-__global__ void __launch_bounds__(32 * WPC, MINB) step_kernel_strip(const StepArgs<Real> A, int n_tiles) {
+template <class L, int CP, class Real, int MINB, int MODE, int SW = 32>
+__global__ void __launch_bounds__(32, MINB) step_kernel_strip(const StepArgs<Real> A) {
     static_assert(L::D == 2 && CP == MODEQ, "row strips: D2Q9 with the modified equilibrium");
     constexpr bool TAU1 = MODE == 2;
     constexpr int Q = L::Q;
     constexpr int WPT = SW / 32;                     // warps per tile
-    const int lane = threadIdx.x & 31;
-    const int wg = blockIdx.x * WPC + int(threadIdx.x >> 5);
-    if (wg >= n_tiles * WPT) return;                 // the whole warp leaves together
-    const int4 tl = A.tiles[wg / WPT];
+    const int lane = threadIdx.x;
+    const int4 tl = A.tiles[blockIdx.x / WPT];
     // register copies of the per-system records: read once, not again after every row's stores
     const SysDev S = A.sys[tl.x];
     const SysPhys<Real> P = A.phys[tl.x];
@@ -662,17 +681,16 @@ __global__ void __launch_bounds__(32 * WPC, MINB) step_kernel_strip(const StepAr
     const bool sm = S.small != 0;
     const Real* __restrict__ fb = A.fin + S.pop_offset;
     Real* __restrict__ fo = A.fout + S.pop_offset;
-    const int x0 = tl.y + 32 * (wg % WPT);
+    const int x0 = tl.y + 32 * int(blockIdx.x % WPT);
     const int x = x0 + lane;
     const bool own = x < nx;
-    const bool extra = lane == 0 || lane == 31;
-    // pulled columns x - c_x for c_x = -1, 0, 1 (index 1 + c_x), of the lane's site and of its halo site
+    // pulled columns x - c_x for c_x = -1, 0, 1 (index 1 + c_x)
     const int xs = wrapm(x, nx);
-    const int xh = wrapm(lane == 0 ? x0 - 1 : x0 + 32, nx);
     const int xo[3] = {wrap1(xs + 1, nx), xs, wrap1(xs - 1, nx)};
-    const int ho[3] = {wrap1(xh + 1, nx), xh, wrap1(xh - 1, nx)};
     const int64_t step = *A.step_ptr + A.k;
     const int y0 = tl.z, y1 = min(y0 + A.zc, ny);
+    __shared__ Real halo[2][kStripRows + 2];
+    strip_halo<L, 32>(fb, N, nx, ny, x0, y0, y1, halo);
 
     Real fp[TAU1 ? 1 : Q];                           // pulled populations of row yy - 1
     Real pr = Real(0), pjx = Real(0), pjy = Real(0); // tau = 1: (drho, j) of row yy - 1
@@ -689,21 +707,12 @@ __global__ void __launch_bounds__(32 * WPC, MINB) step_kernel_strip(const StepAr
             constexpr int i = I;
             fc[i] = fb[i * N + ro[1 + L::c(i, 1)] + xo[1 + L::c(i, 0)]];
         });
-        Real re = Real(0);
-        if (extra) {
-            Real g[Q];
-            sfor<0, Q>([&](auto I) {
-                constexpr int i = I;
-                g[i] = fb[i * N + ro[1 + L::c(i, 1)] + ho[1 + L::c(i, 0)]];
-            });
-            re = density_of(g);
-        }
         Real rc, jx, jy;
         moments_d2q9<Real>(fc, rc, jx, jy);
         Real rl = __shfl_up_sync(0xffffffffu, rc, 1);
         Real rr = __shfl_down_sync(0xffffffffu, rc, 1);
-        if (lane == 0) rl = re;
-        if (lane == 31) rr = re;
+        if (lane == 0) rl = halo[0][yy - y0 + 1];
+        if (lane == 31) rr = halo[1][yy - y0 + 1];
         sfor<0, 3>([&](auto K) {
             constexpr int k = K;
             Rm[k] = R0[k];
