@@ -226,7 +226,7 @@ struct SplitCost {
 };
 SplitCost split_cost(int kind, bool quads) {
     if (kind == 2) return {11.4, 2.0, 14.7, 4.0, 7.4e-5};
-    if (kind == 1) return {0.72, 0.6, 1.15, 2.0, quads ? 1.6e-5 : 2.2e-5};
+    if (kind == 1) return {0.65, 0.55, 1.15, 2.0, quads ? 1.6e-5 : 2.2e-5};
     return {0.51, 0.43, 0.87, 2.0, quads ? 1.6e-5 : 2.2e-5};
 }
 
@@ -240,7 +240,7 @@ SplitCost split_cost(int kind, bool quads) {
 // every ensemble: 16^3 28.9 -> 5.3 us, 64^3 52 -> 14.4, 4 x 64^3 55 -> 46,
 // 16 x 64^3 157 -> 147 us per step; 2.6 M sites with odd sides 332 -> 137 us;
 // against the z-marching kernels that ran the other settings: 4 x 64^3 with a
-// rate per mode 181 -> 71 us, FP64 256^3 29.2 -> 11.1 ms (of which the integer
+// rate per mode 181 -> 61 us, FP64 256^3 29.2 -> 11.1 ms (of which the integer
 // noise 29.2 -> 14).
 double estimated_step_us(const lb_system_desc* s, int n, const int tdim[3], bool paired, int kind, int sms, bool quads) {
     const double ctas = double(tiles_of(s, n, tdim));

@@ -160,7 +160,7 @@ struct ZPlanes {
 // up to z + 2 W, and its copies land in density up to z + 3 W + 1 <= z + 7; no
 // warp is in an earlier iteration once they are issued, after the barrier.
 //
-// 16 x 8 columns, 128 threads: the Laplacian's halo costs 1.4, four or five
+// 16 x 8 columns, 128 threads: the Laplacian's halo costs 1.4, four
 // CTAs per SM decouple the phases.  FP32, tau = 1: bound by issue and, below a
 // CTA per SM, by the latency of a chunk (0.87 us per plane).  FP64: bound by
 // the FP64 units (two operations per clock and SM).
