@@ -53,6 +53,7 @@ struct Plan {
         jk_lap, jk_F, jk_acc, mom, total;
     int tdim[3] = {0, 0, 0};      // tile shape of the step kernel
     bool split = false, narrow = false;   // D3Q19: the split step (in 8 x 8 columns)
+    bool early = false;                   // whose kernels' CTAs fit on an SM each
     bool jk = false;
     int hist_bins = 0;
     double hist_range = 0.0;
@@ -406,6 +407,7 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
         P.spans_h.push_back(sp);
     }
     P.n_site_items = int(P.site_items_h.size());
+    P.early = P.split && P.n_tiles + P.n_site_items <= sm_count();
 
     // observable levels, items and records
     const int bchunk = OBS_THREADS * (spread ? 1 : BLOCKS_PER_THREAD);
@@ -894,6 +896,7 @@ cudaError_t launch_steps(lb_ctx* c, int64_t n) {
         a.zc = c->lattice == LB_D2Q9 ? P.tdim[1] : P.tdim[2];
         a.split = P.split ? 1 : 0;
         a.narrow = P.narrow ? 1 : 0;
+        a.early = P.early ? 1 : 0;
         a.mom = c->ws + P.mom;
         a.n_sites = P.n_sites;
         a.site_items = c->at<int4>(P.site_items);

@@ -26,6 +26,7 @@ StepArgs<Real> step_args(const StepLaunch& a) {
     A.k = a.k;
     A.status = a.status;
     A.zc = a.zc;
+    A.early = a.early;
     return A;
 }
 
@@ -163,13 +164,13 @@ cudaError_t step_moments(const StepLaunch& a, cudaStream_t st) {
         if (a.pair_ok) {
             if (a.small_items)
                 return launch_dependent(moments_quad_kernel<L, J, 64>, a.n_site_items, 64, st, a.sys, a.site_items, f,
-                                        mom, a.n_sites);
+                                        mom, a.n_sites, a.early);
             return launch_dependent(moments_quad_kernel<L, J, 256>, a.n_site_items, 256, st, a.sys, a.site_items, f,
-                                    mom, a.n_sites);
+                                    mom, a.n_sites, a.early);
         }
     }
     return launch_dependent(moments_kernel<L, Real, J, 256>, a.n_site_items, 256, st, a.sys, a.site_items, f, mom,
-                            a.n_sites);
+                            a.n_sites, a.early);
 }
 
 // Split step on D3Q19: the moment pass over the site items, then the collision

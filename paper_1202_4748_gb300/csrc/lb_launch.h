@@ -26,6 +26,7 @@ struct StepLaunch {
     int zc;                 // planes per chunk of the z-marching kernels, rows per strip on D2Q9
     int split;              // D3Q19: run the split step
     int narrow;             // in 8 x 8 columns (FP64)
+    int early;              // both kernels' CTAs fit on an SM each: each lets the next start at once
     void* mom;              // split step: density and momentum fields, one per n_sites values
     int64_t n_sites;        // sites of the ensemble
     const int4* site_items; // split step: the moment pass's work list

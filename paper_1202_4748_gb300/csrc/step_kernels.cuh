@@ -33,6 +33,7 @@ struct StepArgs {
     int k;                    // offset of this step inside the chunk
     int* status;
     int zc;                   // planes per tile of the z-marching kernels, rows per tile of the D2Q9 strips
+    int early;                // split step: let the next kernel's CTAs start at once
 };
 
 template <class L, int CP>
