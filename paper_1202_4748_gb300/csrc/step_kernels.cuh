@@ -287,14 +287,12 @@ __device__ __forceinline__ void collide_guo_bgk(Real (&f)[L::Q], const Real drho
     collide_guo_bgk_m<L, Real, TAU1>(f, drho, j, lv, S, P, site, step, status);
 }
 
-// Collision of one site given its pulled deviations f[], the density halo and
-// (Guo) the Laplacian halo.  Returns post-collision deviations in f[].
-// TAU1 (with BGK_ONLY): the single rate is 1, so f is replaced by the
-// equilibrium (plus force) and the noise amplitudes are the lattice constants.
-template <class L, int CP, class Real, bool BGK_ONLY, class RhoV, class LapV, bool TAU1 = false>
-__device__ __forceinline__ void collide_site(Real (&f)[L::Q], const Real drho, const RhoV& rv, const LapV& lv,
-                                             const SysDev& S, const SysPhys<Real>& P, const uint32_t site,
-                                             const int64_t step, int* status) {
+// Guo collision of one site at any relaxation rates, given its pulled deviations
+// f[] and the Laplacian halo.  Returns post-collision deviations in f[].
+template <class L, class Real, class LapV>
+__device__ __forceinline__ void collide_guo_modes(Real (&f)[L::Q], const Real drho, const LapV& lv, const SysDev& S,
+                                                  const SysPhys<Real>& P, const uint32_t site, const int64_t step,
+                                                  int* status) {
     constexpr int Q = L::Q;
     constexpr int K = Q - L::NC;
     const Real rho = P.rho_c + drho;
@@ -320,130 +318,57 @@ __device__ __forceinline__ void collide_site(Real (&f)[L::Q], const Real drho, c
     const Real p0 = rho * irc * df0 - f0;
     const Real cs2 = rho * irc * irc * (A_ + Real(3) * B_ * phi * phi);
 
-    Real feq[BGK_ONLY ? 1 : Q];
-    Real fsrc[BGK_ONLY ? 1 : Q];   // Guo population force
+    Real feq[Q], fsrc[Q];          // equilibrium, population force
     Real F[3] = {Real(0), Real(0), Real(0)};
-    // single-rate update f <- f - lam (f - f^eq) + (1 - lam/2) F_i done in the loops below
-    const Real lam_b = P.lam_bgk;
-    const Real fs_b = Real(1) - Real(0.5) * lam_b;
-    if constexpr (CP == MODEQ) {
-        // d_a rho = 3 sum_i t_i c_ia rho(r+c_i);  lap rho = 6 sum_i t_i (rho(r+c_i) - rho(r))
-        Real g[2] = {Real(0), Real(0)};
-        Real lap = Real(0);
-        sfor<1, Q>([&](auto I) {
-            constexpr int i = I;
-            const Real rn = rv.template at<L::c(i, 0), L::c(i, 1), L::c(i, 2)>();
-            if constexpr (L::c(i, 0) != 0) g[0] += Real(3.0 * L::w(i) * L::c(i, 0)) * rn;
-            if constexpr (L::c(i, 1) != 0) g[1] += Real(3.0 * L::w(i) * L::c(i, 1)) * rn;
-            lap += Real(6.0 * L::w(i)) * (rn - drho);
-        });
-        const Real ir = fast_rcp(rho);
-        const Real ux = j[0] * ir, uy = j[1] * ir;
-        const Real nu = P.nu;
-        const Real iso = p0 - kap * rho * lap;                     // p0 - kappa rho lap rho
-        const Real udg = ux * g[0] + uy * g[1];
-        // X_ab = rho u_a u_b + nu (u_a d_b rho + u_b d_a rho + u.grad rho delta_ab)
-        const Real Xxx = rho * ux * ux + nu * (Real(2) * ux * g[0] + udg);
-        const Real Xyy = rho * uy * uy + nu * (Real(2) * uy * g[1] + udg);
-        const Real Xxy = rho * ux * uy + nu * (ux * g[1] + uy * g[0]);
-        const Real gxx = kap * g[0] * g[0], gyy = kap * g[1] * g[1], gxy = kap * g[0] * g[1];
-        Real s = Real(0);
-        sfor<1, Q>([&](auto I) {
-            constexpr int i = I;
-            constexpr int cx = L::c(i, 0), cy = L::c(i, 1);
-            const Real xcc = Real(cx * cx - 1.0 / 3.0) * Xxx + Real(cy * cy - 1.0 / 3.0) * Xyy +
-                             Real(2.0 * cx * cy) * Xxy;
-            Real cu;
-            if constexpr (cx == 0) cu = Real(cy) * uy;
-            else if constexpr (cy == 0) cu = Real(cx) * ux;
-            else cu = Real(cx) * ux + Real(cy) * uy;
-            Real v = Real(pooley_w(i)) * (iso + rho * cu + Real(1.5) * xcc) + Real(pooley_wxx(i)) * gxx +
-                     Real(pooley_wyy(i)) * gyy;
-            if constexpr (pooley_wxy(i) != 0.0) v += Real(pooley_wxy(i)) * gxy;
-            s += v;
-            if constexpr (BGK_ONLY && TAU1) f[i] = v;
-            else if constexpr (BGK_ONLY) f[i] -= lam_b * (f[i] - v);
-            else feq[i] = v;
-        });
-        // deviation form of f_0 = rho - sum_{i>=1} f_i
-        if constexpr (BGK_ONLY && TAU1) f[0] = drho - s;
-        else if constexpr (BGK_ONLY) f[0] -= lam_b * (f[0] - (drho - s));
-        else feq[0] = drho - s;
-    } else {
-        // Guo body force F = kappa rho grad(lap rho)
-        Real gl[3] = {Real(0), Real(0), Real(0)};
-        sfor<1, Q>([&](auto I) {
-            constexpr int i = I;
-            const Real ln = lv.template at<L::c(i, 0), L::c(i, 1), L::c(i, 2)>();
-            sfor<0, L::D>([&](auto A) {
-                constexpr int a = A;
-                if constexpr (L::c(i, a) != 0) gl[a] += Real(3.0 * L::w(i) * L::c(i, a)) * ln;
-            });
-        });
-        const Real ir = Real(1) / rho;
-        Real u[3] = {Real(0), Real(0), Real(0)};
+    // Guo body force F = kappa rho grad(lap rho)
+    Real gl[3] = {Real(0), Real(0), Real(0)};
+    sfor<1, Q>([&](auto I) {
+        constexpr int i = I;
+        const Real ln = lv.template at<L::c(i, 0), L::c(i, 1), L::c(i, 2)>();
         sfor<0, L::D>([&](auto A) {
             constexpr int a = A;
-            F[a] = kap * rho * gl[a];
-            u[a] = (j[a] + Real(0.5) * F[a]) * ir;
+            if constexpr (L::c(i, a) != 0) gl[a] += Real(3.0 * L::w(i) * L::c(i, a)) * ln;
         });
-        const Real uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-        const Real uF = u[0] * F[0] + u[1] * F[1] + u[2] * F[2];
-        const Real p3 = Real(3) * p0;
-        Real s = Real(0);
-        sfor<1, Q>([&](auto I) {
-            constexpr int i = I;
-            Real cu = Real(0), cF = Real(0);
-            sfor<0, L::D>([&](auto A) {
-                constexpr int a = A;
-                if constexpr (L::c(i, a) == 1) {
-                    cu += u[a];
-                    cF += F[a];
-                }
-                if constexpr (L::c(i, a) == -1) {
-                    cu -= u[a];
-                    cF -= F[a];
-                }
-            });
-            constexpr double wi = L::w(i);
-            const Real v = Real(wi) * (p3 + rho * (Real(3) * cu + Real(4.5) * cu * cu - Real(1.5) * uu));
-            const Real src = Real(wi) * (Real(3) * (cF - uF) + Real(9) * cu * cF);
-            s += v;
-            if constexpr (BGK_ONLY) {
-                f[i] -= lam_b * (f[i] - v);
-                f[i] += fs_b * src;
-            } else {
-                feq[i] = v;
-                fsrc[i] = src;
+    });
+    const Real ir = Real(1) / rho;
+    Real u[3] = {Real(0), Real(0), Real(0)};
+    sfor<0, L::D>([&](auto A) {
+        constexpr int a = A;
+        F[a] = kap * rho * gl[a];
+        u[a] = (j[a] + Real(0.5) * F[a]) * ir;
+    });
+    const Real uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+    const Real uF = u[0] * F[0] + u[1] * F[1] + u[2] * F[2];
+    const Real p3 = Real(3) * p0;
+    Real s = Real(0);
+    sfor<1, Q>([&](auto I) {
+        constexpr int i = I;
+        Real cu = Real(0), cF = Real(0);
+        sfor<0, L::D>([&](auto A) {
+            constexpr int a = A;
+            if constexpr (L::c(i, a) == 1) {
+                cu += u[a];
+                cF += F[a];
+            }
+            if constexpr (L::c(i, a) == -1) {
+                cu -= u[a];
+                cF -= F[a];
             }
         });
-        if constexpr (BGK_ONLY) {
-            f[0] -= lam_b * (f[0] - (drho - s));
-            f[0] += fs_b * Real(-3.0 * L::w(0)) * uF;
-        } else {
-            feq[0] = drho - s;
-            fsrc[0] = Real(-3.0 * L::w(0)) * uF;
-        }
-    }
+        constexpr double wi = L::w(i);
+        const Real v = Real(wi) * (p3 + rho * (Real(3) * cu + Real(4.5) * cu * cu - Real(1.5) * uu));
+        const Real src = Real(wi) * (Real(3) * (cF - uF) + Real(9) * cu * cF);
+        s += v;
+        feq[i] = v;
+        fsrc[i] = src;
+    });
+    feq[0] = drho - s;
+    fsrc[0] = Real(-3.0 * L::w(0)) * uF;
 
     Real xi[K];
     sfor<0, K>([&](auto A) { xi[decltype(A)::value] = Real(0); });
-    if (P.kT > Real(0)) noise_modes<L, Real, BGK_ONLY && TAU1>(S, P, site, step, rho, cs2, xi, status);
+    if (P.kT > Real(0)) noise_modes<L, Real>(S, P, site, step, rho, cs2, xi, status);
 
-    if constexpr (BGK_ONLY) {
-        // f already relaxed and forced; add the noise through f_i += sum_a t_i T_ai xi_a / N_a
-        sfor<0, Q>([&](auto I) {
-            constexpr int i = I;
-            Real v = f[i];
-            sfor<L::NC, Q>([&](auto A) {
-                constexpr int a = A;
-                constexpr double coef = tinv<L>(i, a);
-                if constexpr (coef != 0.0) v += Real(coef) * xi[a - L::NC];
-            });
-            f[i] = v;
-        });
-        return;
-    } else {
     if (S.bgk) {
         // single relaxation rate: population-space update plus T^-1 xi
         const Real lam = P.lam_bgk;
@@ -451,7 +376,7 @@ __device__ __forceinline__ void collide_site(Real (&f)[L::Q], const Real drho, c
         sfor<0, Q>([&](auto I) {
             constexpr int i = I;
             Real v = f[i] - lam * (f[i] - feq[i]);
-            if constexpr (CP == GUO) v += fs * fsrc[i];
+            v += fs * fsrc[i];
             sfor<L::NC, Q>([&](auto A) {
                 constexpr int a = A;
                 constexpr double coef = tinv<L>(i, a);
@@ -488,25 +413,21 @@ __device__ __forceinline__ void collide_site(Real (&f)[L::Q], const Real drho, c
         });
         const Real lam = P.lam[a];
         m[a] -= lam * (m[a] - me);
-        if constexpr (CP == GUO) {
-            Real fh = Real(0);
-            sfor<0, Q>([&](auto I) {
-                constexpr int i = I;
-                constexpr int t = L::T(a, i);
-                if constexpr (t == 1) fh += fsrc[i];
-                else if constexpr (t == -1) fh -= fsrc[i];
-                else if constexpr (t != 0) fh += Real(t) * fsrc[i];
-            });
-            m[a] += (Real(1) - Real(0.5) * lam) * fh;
-        }
+        Real fh = Real(0);
+        sfor<0, Q>([&](auto I) {
+            constexpr int i = I;
+            constexpr int t = L::T(a, i);
+            if constexpr (t == 1) fh += fsrc[i];
+            else if constexpr (t == -1) fh -= fsrc[i];
+            else if constexpr (t != 0) fh += Real(t) * fsrc[i];
+        });
+        m[a] += (Real(1) - Real(0.5) * lam) * fh;
         m[a] += xi[a - L::NC];
     });
-    if constexpr (CP == GUO) {
-        sfor<0, L::D>([&](auto A) {
-            constexpr int a = A;
-            m[1 + a] += F[a];   // (T F)_a = F_a on the momentum rows
-        });
-    }
+    sfor<0, L::D>([&](auto A) {
+        constexpr int a = A;
+        m[1 + a] += F[a];   // (T F)_a = F_a on the momentum rows
+    });
     // back to populations: f_i = t_i sum_a T_ai m_a / N_a
     sfor<0, Q>([&](auto I) {
         constexpr int i = I;
@@ -518,14 +439,11 @@ __device__ __forceinline__ void collide_site(Real (&f)[L::Q], const Real drho, c
         });
         f[i] = s;
     });
-    }
 }
 
 template <class L, int CP, class Real, int TX, int TY, int TZ, int MODE>
 __global__ void __launch_bounds__(TX* TY* TZ)
     step_kernel(const StepArgs<Real> A) {
-    constexpr bool BGK_ONLY = MODE >= 1;
-    constexpr bool TAU1 = MODE == 2;
     constexpr int Q = L::Q;
     constexpr int H = HaloOf<L, CP>::H;
     constexpr int HZ = HaloOf<L, CP>::HZ;
@@ -603,16 +521,16 @@ __global__ void __launch_bounds__(TX* TY* TZ)
     const int64_t step = *A.step_ptr + A.k;
     const TileView<Real, SX, SY> rv{srho, cidx};
     const TileView<Real, LX, LY> lv{slap, lidx};
-    if constexpr (CP == MODEQ && L::D == 2) {
+    if constexpr (CP == MODEQ) {
         Real d0, jx, jy;
         moments_d2q9<Real>(f, d0, jx, jy);
         collide_d2q9_modeq<MODE, Real>(f, drho, jx, jy, rv, A.phys[tl.x], noise_key(S, step), uint32_t(site),
                                        A.status);
-    } else if constexpr (CP == GUO && BGK_ONLY)
-        collide_guo_bgk<L, Real, TAU1>(f, drho, lv, S, A.phys[tl.x], uint32_t(site), step, A.status);
-    else
-        collide_site<L, CP, Real, BGK_ONLY, TileView<Real, SX, SY>, TileView<Real, LX, LY>, TAU1>(
-            f, drho, rv, lv, S, A.phys[tl.x], uint32_t(site), step, A.status);
+    } else if constexpr (MODE >= 1) {
+        collide_guo_bgk<L, Real, MODE == 2>(f, drho, lv, S, A.phys[tl.x], uint32_t(site), step, A.status);
+    } else {
+        collide_guo_modes<L, Real>(f, drho, lv, S, A.phys[tl.x], uint32_t(site), step, A.status);
+    }
 
     Real* __restrict__ fo = A.fout + S.pop_offset;
     sfor<0, Q>([&](auto I) {
