@@ -52,6 +52,7 @@ KERNEL_SOURCES = ["paper_1202_4748_gb300/csrc/step_kernels.cuh", "paper_1202_474
                   "paper_1202_4748_gb300/csrc/step_kernel_pair.cuh", "paper_1202_4748_gb300/csrc/collide_d3q19.cuh",
                   "paper_1202_4748_gb300/csrc/vec2.cuh", "paper_1202_4748_gb300/csrc/collide_d2q9.cuh",
                   "paper_1202_4748_gb300/csrc/step_kernel_strip_pair.cuh", "paper_1202_4748_gb300/csrc/step_kernel_split.cuh",
+                  "paper_1202_4748_gb300/csrc/normal64.cuh",
                   "paper_1202_4748_gb300/csrc/lattice_tu.cuh",
                   "paper_1202_4748_gb300/csrc/lattice_d2q9.cu", "paper_1202_4748_gb300/csrc/lattice_d3q19.cu"]
 

@@ -3,7 +3,8 @@
 The header is plain C++ and is compiled here with the host compiler.  R, the
 cosine and the sine are formed to about 2^-58 relative and rounded once to
 double (at most 2^-53 relative), so each is within 1.1 x 2^-53 of the exact
-value over the words' whole range: random words, words near 0 and near 2^32
+value over the words' whole range; so are the integer roots and sums beside
+them.  The normals' words: random words, words near 0 and near 2^32
 (where -ln U is large and tiny), the edges of the table's intervals and of the
 octants.  numpy's long double (64-bit mantissa or more) is the exact side.
 """
@@ -11,6 +12,7 @@ import ctypes
 import os
 import shutil
 import subprocess
+from fractions import Fraction
 
 import numpy as np
 import pytest
@@ -27,6 +29,27 @@ extern "C" void normals(const uint32_t* a, const uint32_t* b, double* r, double*
         lbf::n64_angle(b[i], c[i], s[i]);
     }
 }
+extern "C" void roots(const double* x, double* r, double* q, long n) {
+    for (long i = 0; i < n; ++i) {
+        r[i] = lbf::n64_sqrt(x[i]);
+        q[i] = lbf::n64_inv_sqrt(x[i]);
+    }
+}
+template <class T> static int sums(const T* f, double* out, long n) {
+    int finite = 0;
+    for (long i = 0; i < n; ++i) {
+        T g[19];
+        for (int k = 0; k < 19; ++k) g[k] = f[19 * i + k];
+        const lbf::FixedSum<T, 19> s(g);
+        int64_t t = 0;
+        for (int k = 0; k < 19; ++k) t += k == 7 ? -s.m[k] : s.m[k];
+        out[i] = s.value(t);
+        finite += s.finite();
+    }
+    return finite;
+}
+extern "C" int sums64(const double* f, double* out, long n) { return sums(f, out, n); }
+extern "C" int sums32(const float* f, double* out, long n) { return sums(f, out, n); }
 """ % HEADER
 
 
@@ -65,3 +88,48 @@ def test_radius_and_angle_are_within_rounding_of_the_exact_values(lib):
     si = np.where(swap, np.cos(x), np.sin(x)) * np.where(octant >> 2, -1, 1)
     for have, want in zip(got, (radius, co, si)):
         assert np.max(np.abs((have.astype(L) - want) / want)) < 1.1 * 2.0 ** -53
+
+
+def test_roots_are_within_rounding_of_the_exact_values(lib):
+    """0.51 units in the last place, over every exponent of a normal double,
+    and the library's value for the rest."""
+    rng = np.random.default_rng(2)
+    x = np.ldexp(rng.uniform(0.5, 1.0, 300_000), rng.integers(-1000, 1000, 300_000))
+    x = np.concatenate([x, rng.uniform(0.5, 2.0, 300_000), [1.0, 4.0, 0.25, 2.0, np.nextafter(1, 0), np.nextafter(4, 5)]])
+    r, q = np.empty(x.size), np.empty(x.size)
+    p = [v.ctypes.data_as(ctypes.c_void_p) for v in (x, r, q)]
+    lib.roots(*p, ctypes.c_long(x.size))
+    want = np.sqrt(x.astype(np.longdouble))
+    assert np.max(np.abs((r - want) / want)) < 1.1 * 2.0 ** -53
+    assert np.max(np.abs(q * want - 1)) < 1.1 * 2.0 ** -53
+    x = np.array([0.0, np.inf, np.nan, -1.0, 5e-324])
+    lib.roots(*[v.ctypes.data_as(ctypes.c_void_p) for v in (x, r, q)], ctypes.c_long(x.size))
+    with np.errstate(all="ignore"):
+        np.testing.assert_array_equal(r[:5], np.sqrt(x))
+        np.testing.assert_array_equal(q[:5], 1.0 / np.sqrt(x))
+
+
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+def test_integer_sums(lib, dtype):
+    """Each of 19 values enters to half of 2^-57 of the largest's power of two,
+    and the sum is rounded once to double; infinities and NaNs are reported."""
+    rng = np.random.default_rng(3)
+    n = 20_000
+    f = rng.standard_normal((n, 19)) * np.exp(rng.uniform(-30, 30, (n, 1))) * np.exp(rng.uniform(-25, 0, (n, 19)))
+    f[: n // 4, 10:] = -f[: n // 4, :9]                    # cancelling
+    f[0], f[1, 1:] = 0.0, 0.0
+    f = np.ascontiguousarray(f.astype(dtype))
+    out = np.empty(n)
+    call = lib.sums64 if dtype == np.float64 else lib.sums32
+    assert call(f.ctypes.data_as(ctypes.c_void_p), out.ctypes.data_as(ctypes.c_void_p), ctypes.c_long(n)) == n
+    sign = np.ones(19)
+    sign[7] = -1
+    exact = [sum(map(Fraction, row)) for row in (f.astype(np.float64) * sign).tolist()]
+    off = np.array([float(abs(Fraction(o) - e)) for o, e in zip(out.tolist(), exact)])
+    want = np.array([float(e) for e in exact])
+    top = np.max(np.abs(f), axis=1).astype(np.float64)
+    assert np.all(off <= 19 * 2.0 ** -57 * top + 2.0 ** -53 * np.abs(want) * (1 + 2.0 ** -50))
+    for bad in (np.inf, -np.inf, np.nan):
+        g = f[:1].copy()
+        g[0, 5] = bad
+        assert call(g.ctypes.data_as(ctypes.c_void_p), out.ctypes.data_as(ctypes.c_void_p), ctypes.c_long(1)) == 0
