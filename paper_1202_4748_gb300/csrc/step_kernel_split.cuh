@@ -7,7 +7,10 @@
 // the field fits the scratch of a sample, which it shares).
 //
 // Each kernel is launched before its predecessor has ended and waits for it
-// behind its prologue.  It lets its successor's CTAs start when it has done its
+// behind its prologue, which reads only what no kernel writes (the plan's
+// records).  The buffers that kernels write are not `const __restrict__` here:
+// that promises read-only data for the whole kernel, which these are only behind
+// the wait.  It lets its successor's CTAs start when it has done its
 // work, or, where both fit on an SM each (`early`), as soon as it runs itself:
 // 16^3 5.8 -> 5.2 us per step.  With more CTAs those of the successor go to the
 // few SMs with room, several to each, and stay there (32^3 6.0 -> 8.2 us).
@@ -31,13 +34,13 @@ namespace lbf {
 // kernels (from 0, direction by direction).  One site per thread (any sides).
 template <class L, class Real, bool J, int NT>
 __global__ void __launch_bounds__(NT)
-    moments_kernel(const SysDev* __restrict__ sysv, const int4* __restrict__ items, const Real* __restrict__ fbuf,
-                   Real* __restrict__ mom, int64_t stride, int early) {
+    moments_kernel(const SysDev* __restrict__ sysv, const int4* __restrict__ items, const Real* fbuf,
+                   Real* mom, int64_t stride, int early) {
     const int4 it = items[blockIdx.x];
     const SysDev& S = sysv[it.x];
     const int nx = S.nx, ny = S.ny, nz = S.nz, N = S.ns;
-    const Real* __restrict__ fb = fbuf + S.pop_offset;
-    Real* __restrict__ out = mom + S.site_offset;
+    const Real* fb = fbuf + S.pop_offset;
+    Real* out = mom + S.site_offset;
     grid_wait();
     if (early) grid_release();
     for (int site = it.y + int(threadIdx.x); site < it.z; site += NT) {
@@ -63,12 +66,12 @@ __global__ void __launch_bounds__(NT)
 template <class L, bool J, int NT>
 __global__ void __launch_bounds__(NT)
     moments_quad_kernel(const SysDev* __restrict__ sysv, const int4* __restrict__ items,
-                        const float* __restrict__ fbuf, float* __restrict__ mom, int64_t stride, int early) {
+                        const float* fbuf, float* mom, int64_t stride, int early) {
     const int4 it = items[blockIdx.x];
     const SysDev& S = sysv[it.x];
     const int nx = S.nx, ny = S.ny, nz = S.nz, N = S.ns;
-    const float* __restrict__ fb = fbuf + S.pop_offset;
-    float* __restrict__ out = mom + S.site_offset;
+    const float* fb = fbuf + S.pop_offset;
+    float* out = mom + S.site_offset;
     const int lane = threadIdx.x & 31;
     grid_wait();
     if (early) grid_release();
@@ -174,7 +177,7 @@ struct ZPlanes {
 // the FP64 units (two operations per clock and SM).
 template <int MODE, int CP, class V, int TX, int TY, int MINB>
 __global__ void __launch_bounds__(TX* TY, MINB)
-    collide_march_kernel(const StepArgs<typename VT<V>::S> A, const typename VT<V>::S* __restrict__ mom,
+    collide_march_kernel(const StepArgs<typename VT<V>::S> A, const typename VT<V>::S* mom,
                          int64_t stride) {
     using Real = typename VT<V>::S;
     using L = D3Q19;
@@ -200,8 +203,8 @@ __global__ void __launch_bounds__(TX* TY, MINB)
     const int lx = tid % TX, ly = tid / TX;
     const int x = tl.y + lx, y = tl.z + ly;
     const bool own = x < nx && y < ny;
-    const Real* __restrict__ rho_g = mom + S.site_offset;
-    const Real* __restrict__ jg = rho_g + stride + (y * nx + x);
+    const Real* rho_g = mom + S.site_offset;
+    const Real* jg = rho_g + stride + (y * nx + x);
     Real* __restrict__ fo = A.fout + S.pop_offset + (y * nx + x);
 
     // wrapped in-plane offset of the thread's footprint sites (-1: not needed)

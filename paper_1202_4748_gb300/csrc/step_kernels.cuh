@@ -90,8 +90,9 @@ struct RingView {          // three planes (z - 1, z, z + 1) at arbitrary offset
 };
 
 // Pull all q populations of the site described by `nb` (f_i(r) = buf_i(r - c_i)).
+// (No promise about fb here: the split step's kernels call it behind a grid_wait.)
 template <class L, class Real>
-__device__ __forceinline__ void pull_site(const Real* __restrict__ fb, int N, const Nbr& nb, Real (&f)[L::Q]) {
+__device__ __forceinline__ void pull_site(const Real* fb, int N, const Nbr& nb, Real (&f)[L::Q]) {
     sfor<0, L::Q>([&](auto I) {
         constexpr int i = I;
         f[i] = fb[i * N + nb.template at<-L::c(i, 0), -L::c(i, 1), -L::c(i, 2)>()];
