@@ -183,24 +183,45 @@ __global__ void __launch_bounds__(AUX_THREADS)
         Real(in[int64_t(blockIdx.y) * S.n_sites + site] - (i == 0 ? S.rho_c : 0.0));
 }
 
-// Sums of the pulled populations of a site to FP64 accuracy, rv = sum_i f_i,
-// mv = sum_i c_i f_i, by integer additions (FixedSum): the per-population work
-// and the conversions stay off the FP64 units, which do two operations per clock
-// and SM.  (Compensated FP64 sums took 0.39 ms for 573,440 FP64 sites; compensated
-// FP32 sums with eight conversions per site 57 us for 2^20 FP32 sites, now 47.)
+// Sums of the pulled populations of a site, rv = sum_i f_i, mv = sum_i c_i f_i, by
+// integer additions: the per-population work and the conversions stay off the FP64
+// units, which do two operations per clock and SM.  FP32 fields to 2^-57 of the
+// largest population (FixedSum; compensated FP32 sums with eight conversions per
+// site took 57 us for 2^20 sites, now 47), FP64 fields to 2^-116 (WideSum;
+// compensated FP64 sums, to 2^-106, took 0.39 ms for 573,440 sites).
 template <class L, class Real>
 __device__ __forceinline__ void site_sums(const Real (&f)[L::Q], double& rv, double (&mv)[3]) {
-    const FixedSum<Real, L::Q> s(f);
-    int64_t r = 0, m[3] = {0, 0, 0};
+    bool finite;
+    if constexpr (sizeof(Real) == 8) {
+        const WideSum<L::Q> s(f);
+        __int128 r = 0, m[3] = {0, 0, 0};
 #pragma unroll
-    for (int i = 0; i < L::Q; ++i) {
-        r += s.m[i];
+        for (int i = 0; i < L::Q; ++i) {
+            const __int128 v = s.add(i);
+            r += v;
 #pragma unroll
-        for (int a = 0; a < 3; ++a) m[a] += L::c(i, a) * s.m[i];
+            for (int a = 0; a < 3; ++a) {
+                if (L::c(i, a) == 1) m[a] += v;
+                if (L::c(i, a) == -1) m[a] -= v;
+            }
+        }
+        rv = s.value(r);
+        for (int a = 0; a < 3; ++a) mv[a] = s.value(m[a]);
+        finite = s.finite();
+    } else {
+        const FixedSum<Real, L::Q> s(f);
+        int64_t r = 0, m[3] = {0, 0, 0};
+#pragma unroll
+        for (int i = 0; i < L::Q; ++i) {
+            r += s.m[i];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) m[a] += L::c(i, a) * s.m[i];
+        }
+        rv = s.value(r);
+        for (int a = 0; a < 3; ++a) mv[a] = s.value(m[a]);
+        finite = s.finite();
     }
-    rv = s.value(r);
-    for (int a = 0; a < 3; ++a) mv[a] = s.value(m[a]);
-    if (!s.finite()) {
+    if (!finite) {
         rv = mv[0] = mv[1] = mv[2] = 0.0;
         for (int i = 0; i < L::Q; ++i) {
             rv += double(f[i]);

@@ -198,6 +198,52 @@ struct FixedSum {
     }
 };
 
+// Sums of N doubles to about 2^-116 of the largest, rounded once (to nearest,
+// ties to even): as FixedSum with 122 bits, for sums whose cancellation has to
+// keep its digits (a site's momentum is often far below its populations).  The
+// integers are formed one by one, add(i) at a time, so that a site needs no array
+// of them.  (Compensated FP64 sums, to 2^-106, cost six FP64 operations an addend.)
+template <int N>
+struct WideSum {
+    static_assert(N <= 31, "headroom");
+    const double (&f)[N];
+    uint32_t top;                  // largest exponent field, in place
+    static LB_HD uint64_t bits(double x) {
+        uint64_t u;
+        memcpy(&u, &x, 8);
+        return u;
+    }
+    LB_HD explicit WideSum(const double (&v)[N]) : f(v), top(0) {
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int i = 0; i < N; ++i) {
+            const uint32_t e = uint32_t(bits(f[i]) >> 32) & 0x7ff00000u;
+            top = e > top ? e : top;
+        }
+    }
+    LB_HD bool finite() const { return top != 0x7ff00000u; }
+    // f[i] as an integer multiple of 2^(top - bias - 121)
+    LB_HD __int128 add(int i) const {
+        const uint64_t u = bits(f[i]), one = uint64_t(1) << 52;
+        const uint32_t e = uint32_t(u >> 32) & 0x7ff00000u, sh = (top - e) >> 20;
+        if (e == 0 || sh > 121) return 0;                  // zeros and subnormals count as 0
+        const __int128 v = __int128((unsigned __int128)((u & (one - 1)) | one) << 69 >> sh);
+        return int64_t(u) < 0 ? -v : v;
+    }
+    LB_HD double value(__int128 s) const {
+        if (s == 0) return 0.0;
+        unsigned __int128 a = s < 0 ? -(unsigned __int128)s : (unsigned __int128)s;
+        const int nl = uint64_t(a >> 64) ? n64_clz(uint64_t(a >> 64)) : 64 + n64_clz(uint64_t(a));
+        a <<= nl;
+        const uint64_t m = uint64_t(a >> 64), rest = (m & 0x3ff) | (uint64_t(a) != 0) | ((m >> 11) & 1);
+        const int e = int(top >> 20) - 1023 + 1 - 121 + 127 - nl;                          // (m / 2^64) 2^e
+        if (e < -1020) return 0.0;
+        const double d = n64_bits((uint64_t(e + 1021) << 52) + (m >> 11) + (((m >> 10) & 1) & (rest != 0)));
+        return s < 0 ? -d : d;
+    }
+};
+
 // sqrt(-2 ln U), U = (w + 1/2) 2^-32; tab holds the 64 entries of kLogTable
 template <class Table>
 LB_HD double n64_radius(uint32_t w, const Table& tab) {
