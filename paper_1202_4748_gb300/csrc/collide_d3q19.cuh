@@ -120,16 +120,20 @@ __device__ __forceinline__ float sfu_sqrt(float x) {
 }
 
 // Factor that the draws of a lane precision expect in the variance from which
-// their scale is formed (draw4): 2 ln 2 in float, 1 in double.
+// their scale is formed (draw4): 2 ln 2 in float, 1 in double; and the mean square
+// of the normals that this gives: the special functions' logarithm, root, sine and
+// cosine come out low in the mean (1.3e9 draws on GB300).
 template <class S>
 struct DrawScale;
 template <>
 struct DrawScale<float> {
     static constexpr double v = 1.3862943611198906;
+    static constexpr double mean_square = 1.0 - 2.55e-7;
 };
 template <>
 struct DrawScale<double> {
     static constexpr double v = 1.0;
+    static constexpr double mean_square = 1.0;
 };
 
 // Four normals of draw d for every lane: n0, n1 from the words (w0, w1)
@@ -463,9 +467,9 @@ __device__ __forceinline__ void d3q19_gradient(const RhoV& rv, V (&g)[3]) {
     g[2] = vfma(dfz, vk<V>(1.0 / 6.0), vmul(vadd(vsub(exz, ezm), vsub(eyz, eym)), vk<V>(1.0 / 12.0)));
 }
 
-// h_4 .. h_9 and h_16 (m_a / (36 N_a)) of the modified equilibrium below.
+// m_4 .. m_9 and m_16 of the modified equilibrium below.
 template <class V>
-__device__ __forceinline__ void d3q19_modeq_second(V (&h)[19], const V drho, const V rho, const V jx, const V jy,
+__device__ __forceinline__ void d3q19_modeq_second(V (&m)[19], const V drho, const V rho, const V jx, const V jy,
                                                    const V jz, const V ir, const V p0, const V lap, const V (&g)[3],
                                                    const SysPhys<typename VT<V>::S>& P) {
     const V ux = vmul(jx, ir), uy = vmul(jy, ir), uz = vmul(jz, ir);
@@ -483,16 +487,14 @@ __device__ __forceinline__ void d3q19_modeq_second(V (&h)[19], const V drho, con
     const V Ksum = vadd(vadd(Kxx, Kyy), Kzz);
     const V trX = vadd(vadd(Xxx, Xyy), Xzz);
 
-    // h_a = m_a / (36 N_a); N = (1, 1/3 x3, 2/3, 4/3, 4/9, 1/9 x3, ..., 2 for mode 16)
-    h[4] = vmul(vfma(Ksum, vk<V>(-0.5), vfma(iso, vk<V>(3.0), vsub(trX, drho))), vk<V>(1.0 / 24.0));
-    h[5] = vmul(vadd(vfma(Xxx, vk<V>(2.0), vsub(vk<V>(0.0), vadd(Xyy, Xzz))),
-                     vfma(Kxx, vk<V>(2.0), vsub(vk<V>(0.0), vadd(Kyy, Kzz)))),
-                vk<V>(1.0 / 48.0));
-    h[6] = vmul(vadd(vsub(Xyy, Xzz), vsub(Kyy, Kzz)), vk<V>(1.0 / 16.0));
-    h[7] = vmul(vfma(kgx, g[1], Xxy), vk<V>(1.0 / 4.0));
-    h[8] = vmul(vfma(kgy, g[2], Xyz), vk<V>(1.0 / 4.0));
-    h[9] = vmul(vfma(kgz, g[0], Xzx), vk<V>(1.0 / 4.0));
-    h[16] = vmul(vfma(Ksum, vk<V>(-1.5), vfma(iso, vk<V>(-3.0), drho)), vk<V>(1.0 / 72.0));
+    m[4] = vfma(Ksum, vk<V>(-0.5), vfma(iso, vk<V>(3.0), vsub(trX, drho)));
+    m[5] = vadd(vfma(Xxx, vk<V>(2.0), vsub(vk<V>(0.0), vadd(Xyy, Xzz))),
+                vfma(Kxx, vk<V>(2.0), vsub(vk<V>(0.0), vadd(Kyy, Kzz))));
+    m[6] = vadd(vsub(Xyy, Xzz), vsub(Kyy, Kzz));
+    m[7] = vfma(kgx, g[1], Xxy);
+    m[8] = vfma(kgy, g[2], Xyz);
+    m[9] = vfma(kgz, g[0], Xzx);
+    m[16] = vfma(Ksum, vk<V>(-1.5), vfma(iso, vk<V>(-3.0), drho));
 }
 
 // The modified equilibrium carried to D3Q19 (Eq. 65's structure with the
@@ -536,6 +538,14 @@ __device__ __forceinline__ void collide_d3q19_modeq_tau1(V (&f)[19], const V drh
     const V ir = vmap(rho, [](S x) { return fast_rcp(x); });
     V h[19];
     d3q19_modeq_second<V>(h, drho, rho, jx, jy, jz, ir, p0, lap, g, P);
+    // h_a = m_a / (36 N_a); N = (1, 1/3 x3, 2/3, 4/3, 4/9, 1/9 x3, ..., 2 for mode 16)
+    h[4] = vmul(h[4], vk<V>(1.0 / 24.0));
+    h[5] = vmul(h[5], vk<V>(1.0 / 48.0));
+    h[6] = vmul(h[6], vk<V>(1.0 / 16.0));
+    h[7] = vmul(h[7], vk<V>(1.0 / 4.0));
+    h[8] = vmul(h[8], vk<V>(1.0 / 4.0));
+    h[9] = vmul(h[9], vk<V>(1.0 / 4.0));
+    h[16] = vmul(h[16], vk<V>(1.0 / 72.0));
     h[0] = vmul(drho, vk<V>(1.0 / 36.0));
     h[1] = vmul(jx, vk<V>(1.0 / 12.0));
     h[2] = vmul(jy, vk<V>(1.0 / 12.0));
@@ -543,29 +553,41 @@ __device__ __forceinline__ void collide_d3q19_modeq_tau1(V (&f)[19], const V drh
     d3q19_tau1_noise_and_populations<V>(h, f, rho, cs2, P, key, site, status);
 }
 
-// x / N, N = 36 or 12, with the part of 1 / N that its rounding loses: the error
-// of the constant alone would scale the conserved moments by the same factor in
-// every step, which rates that keep fluctuations long add up (FP64, one rate,
-// 100 steps: block moments 3.3e-15 from an FP64 reference, now 2.8e-15).
-template <int N, class V>
-__device__ __forceinline__ V over(const V x) {
+// x / (36 N_a) of mode a, with the part that the rounding of 1 / 24, 1 / 48 or
+// 1 / 72 loses: the error of the constant alone would scale a mode's rate and noise
+// by the same factor in every step.
+template <int A, class V>
+__device__ __forceinline__ V over_norm(const V x) {
     using S = typename VT<V>::S;
-    static_assert(N == 36 || N == 12, "N fl64(1 / N) = 1 - 2^-54");
+    constexpr int N = (A >= 7 && A <= 9) ? 4 : (A >= 13 && A <= 15) ? 8 : (A == 6 || A == 18) ? 16
+                      : (A == 5 || A == 17) ? 48 : A == 16 ? 72 : 24;
+    static_assert(A >= 4 && A < 19, "non-conserved modes");
     constexpr double hi = double(S(1.0 / N));
+    // double: N fl64(1 / N) = 1 - 2^-54 for N = 3 or 9 times a power of two
     constexpr double lo = sizeof(S) == 8 ? 5.551115123125783e-17 / N : 1.0 / N - hi;
-    return vfma(x, vk<V>(hi), vmul(x, vk<V>(lo)));
+    if constexpr ((N & (N - 1)) == 0) return vmul(x, vk<V>(hi));
+    else return vfma(x, vk<V>(hi), vmul(x, vk<V>(lo)));
 }
 
-// Collision with any relaxation rates, either coupling: with k_a = w_a / (36 N_a),
-//   w_a = m_a + lambda_a (m^eq_a - m_a) + (1 - lambda_a / 2) S_a + xi_a
-// on the non-conserved modes, m^eq as in the fully relaxed collisions above
-// (Guo: with E_bc = rho u_b u_c alone) and S the Guo source, S_4 = 2 u.F,
-// S_5 = 2 (3 u_x F_x - u.F), S_6 = 2 (u_y F_y - u_z F_z), S_7 = u_x F_y + u_y F_x,
-// S_8, S_9 likewise, 0 on the ghosts.  MODE 0: a rate per mode, m_a from the
-// sums the modes share; MODE 1: one rate lambda, f' = (1 - lambda) f + 36 t_i
-// sum_a T_ai (lambda k^eq + (1 - lambda / 2) k^S + k^xi).  f holds the
-// pre-collision deviations on entry; nv views the density (MODEQ) or its
-// Laplacian (GUO) around the site(s).
+// Collision with any relaxation rates, either coupling, as an increment of the
+// populations: f_i' = f_i + t_i sum_a T_ai w_a / N_a,
+//   w_a = lambda_a (m^eq_a - m_a) + (1 - lambda_a / 2) S_a + xi_a
+// on the non-conserved modes, m_a from the sums of f that the modes share, m^eq
+// as in the fully relaxed collisions above (Guo: with E_bc = rho u_b u_c alone)
+// and S the Guo source, S_4 = 2 u.F, S_5 = 2 (3 u_x F_x - u.F), S_6 = 2 (u_y F_y -
+// u_z F_z), S_7 = u_x F_y + u_y F_x, S_8, S_9 likewise, 0 on the ghosts; w_0 = 0
+// and w_a = F_a on the momentum.  MODE 0: a rate per mode; MODE 1: one rate.
+// f holds the pre-collision deviations on entry; nv views the density (MODEQ) or
+// its Laplacian (GUO) around the site(s).
+//
+// The conserved moments do not pass through the scaled moments, whose rounding a
+// slow mode adds up step after step, f is rounded once, and neither the constants
+// nor the draws' mean square bias a mode's rate or noise.  Against exact arithmetic
+// (16 x 16 x 8, 50 steps) FP32 populations are off by 4.3e-7 of their size with a
+// rate per mode, 5.4e-7 with one rate (Guo), 3.3e-7 and 3.7e-7 (modified
+// equilibrium); transforming relaxed moments back leaves 6.1e-7 to 7.7e-7 and
+// 4.0e-7 to 4.7e-7.  It costs 4 to 7 % of the step (4 x 64^3, a rate per mode: 63.7
+// us for 61.4): f stays in registers to the end.
 template <int MODE, int CP, class V, class NV>
 __device__ __forceinline__ void collide_d3q19_rates(V (&f)[19], const V drho, const V jx, const V jy, const V jz,
                                                     const NV& nv, const SysPhys<typename VT<V>::S>& P,
@@ -587,9 +609,9 @@ __device__ __forceinline__ void collide_d3q19_rates(V (&f)[19], const V drho, co
     const V rr = vmul(rho, vbc<V>(P.inv_rho_c));
     const V p0 = vsub(vmul(rr, df0), f0);
     const V cs2 = vmul(vmul(rr, vbc<V>(P.inv_rho_c)), vfma(vbc<V>(S(3) * P.b), phi2, vbc<V>(P.a)));
-    const V ir = vmap(rho, [](S x) { return fast_rcp(x); });
+    const V ir = vmap(rho, [](S x) { return S(1) / x; });
 
-    // k: equilibrium moments over 36 N_a (0 .. 9 and 16); s: the Guo source likewise (4 .. 9)
+    // k: equilibrium moments (4 .. 9 and 16); s: the Guo source (4 .. 9)
     V k[19], s[6] = {}, F[3] = {};
     if constexpr (CP == GUO) {
         V gx, gy, gz;
@@ -605,46 +627,29 @@ __device__ __forceinline__ void collide_d3q19_rates(V (&f)[19], const V drho, co
         const V Exx = vmul(ux, mx), Eyy = vmul(uy, my), Ezz = vmul(uz, mz);
         const V tr = vadd(vadd(Exx, Eyy), Ezz);
         const V iso = vfma(p0, vk<V>(-3.0), drho);
-        k[4] = vmul(vsub(tr, iso), vk<V>(1.0 / 24.0));
-        k[5] = vmul(vfma(Exx, vk<V>(3.0), vsub(vk<V>(0.0), tr)), vk<V>(1.0 / 48.0));
-        k[6] = vmul(vsub(Eyy, Ezz), vk<V>(1.0 / 16.0));
-        k[7] = vmul(vmul(ux, my), vk<V>(1.0 / 4.0));
-        k[8] = vmul(vmul(uy, mz), vk<V>(1.0 / 4.0));
-        k[9] = vmul(vmul(uz, mx), vk<V>(1.0 / 4.0));
-        k[16] = vmul(iso, vk<V>(1.0 / 72.0));
+        k[4] = vsub(tr, iso);
+        k[5] = vfma(Exx, vk<V>(3.0), vsub(vk<V>(0.0), tr));
+        k[6] = vsub(Eyy, Ezz);
+        k[7] = vmul(ux, my);
+        k[8] = vmul(uy, mz);
+        k[9] = vmul(uz, mx);
+        k[16] = iso;
         const V gxx = vmul(ux, F[0]), gyy = vmul(uy, F[1]), gzz = vmul(uz, F[2]);
         const V uF = vadd(vadd(gxx, gyy), gzz);
-        s[0] = vmul(uF, vk<V>(1.0 / 12.0));
-        s[1] = vmul(vfma(gxx, vk<V>(3.0), vsub(vk<V>(0.0), uF)), vk<V>(1.0 / 24.0));
-        s[2] = vmul(vsub(gyy, gzz), vk<V>(1.0 / 8.0));
-        s[3] = vmul(vfma(ux, F[1], vmul(uy, F[0])), vk<V>(1.0 / 4.0));
-        s[4] = vmul(vfma(uy, F[2], vmul(uz, F[1])), vk<V>(1.0 / 4.0));
-        s[5] = vmul(vfma(uz, F[0], vmul(ux, F[2])), vk<V>(1.0 / 4.0));
+        s[0] = vadd(uF, uF);
+        s[1] = vmul(vfma(gxx, vk<V>(3.0), vsub(vk<V>(0.0), uF)), vk<V>(2.0));
+        s[2] = vmul(vsub(gyy, gzz), vk<V>(2.0));
+        s[3] = vfma(ux, F[1], vmul(uy, F[0]));
+        s[4] = vfma(uy, F[2], vmul(uz, F[1]));
+        s[5] = vfma(uz, F[0], vmul(ux, F[2]));
     } else {
         V g[3];
         d3q19_gradient<V>(nv, g);
         const V lap = lap_d3q19<V>(nv);
         d3q19_modeq_second<V>(k, drho, rho, jx, jy, jz, ir, p0, lap, g, P);
     }
-    k[0] = over<36>(drho);
-    k[1] = over<12>(jx);
-    k[2] = over<12>(jy);
-    k[3] = over<12>(jz);
-
-    if constexpr (MODE == 1) {
-        const V lam = vbc<V>(P.lam_bgk), half = vbc<V>(S(1) - S(0.5) * P.lam_bgk);
-#pragma unroll
-        for (int a = 0; a < 10; ++a) k[a] = vmul(lam, k[a]);
-        k[16] = vmul(lam, k[16]);
-        if constexpr (CP == GUO) {
-#pragma unroll
-            for (int a = 0; a < 6; ++a) k[4 + a] = vfma(half, s[a], k[4 + a]);
-        }
-#pragma unroll
-        for (int a = 10; a < 16; ++a) k[a] = vk<V>(0.0);
-        k[17] = k[18] = vk<V>(0.0);
-    } else {
-        // m_a / (36 N_a) of f: sums and differences of opposite velocities, faces and edges
+    {
+        // m_a of f: sums and differences of opposite velocities, faces and edges
         const V sx = vadd(f[1], f[2]), sy = vadd(f[3], f[4]), sz = vadd(f[5], f[6]);
         const V dx = vsub(f[1], f[2]), dy = vsub(f[3], f[4]), dz = vsub(f[5], f[6]);
         const V a1 = vadd(f[7], f[8]), a2 = vadd(f[9], f[10]), e1 = vsub(f[7], f[8]), e2 = vsub(f[9], f[10]);
@@ -657,49 +662,42 @@ __device__ __forceinline__ void collide_d3q19_rates(V (&f)[19], const V drho, co
         const V Xxy = vadd(e1, e2), Yxy = vsub(e1, e2), Xxz = vadd(g1, g2), Zxz = vsub(g1, g2);
         const V Yyz = vadd(h1, h2), Zyz = vsub(h1, h2);
         V m[19];
-        m[4] = vmul(vsub(ee, f[0]), vk<V>(1.0 / 24.0));
-        m[5] = vmul(vadd(f5, e5), vk<V>(1.0 / 48.0));
-        m[6] = vmul(vadd(f6, e6), vk<V>(1.0 / 16.0));
-        m[7] = vmul(vsub(a1, a2), vk<V>(1.0 / 4.0));
-        m[8] = vmul(vsub(c1, c2), vk<V>(1.0 / 4.0));
-        m[9] = vmul(vsub(b1, b2), vk<V>(1.0 / 4.0));
-        m[10] = vmul(vfma(dx, vk<V>(-2.0), vadd(Xxy, Xxz)), vk<V>(1.0 / 24.0));
-        m[11] = vmul(vfma(dy, vk<V>(-2.0), vadd(Yxy, Yyz)), vk<V>(1.0 / 24.0));
-        m[12] = vmul(vfma(dz, vk<V>(-2.0), vadd(Zxz, Zyz)), vk<V>(1.0 / 24.0));
-        m[13] = vmul(vsub(Xxy, Xxz), vk<V>(1.0 / 8.0));
-        m[14] = vmul(vsub(Yyz, Yxy), vk<V>(1.0 / 8.0));
-        m[15] = vmul(vsub(Zxz, Zyz), vk<V>(1.0 / 8.0));
-        m[16] = vmul(vadd(vfma(vadd(sx, fyz), vk<V>(-2.0), f[0]), ee), vk<V>(1.0 / 72.0));
-        m[17] = vmul(vsub(e5, f5), vk<V>(1.0 / 48.0));
-        m[18] = vmul(vsub(e6, f6), vk<V>(1.0 / 16.0));
+        m[4] = vsub(ee, f[0]);
+        m[5] = vadd(f5, e5);
+        m[6] = vadd(f6, e6);
+        m[7] = vsub(a1, a2);
+        m[8] = vsub(c1, c2);
+        m[9] = vsub(b1, b2);
+        m[10] = vfma(dx, vk<V>(-2.0), vadd(Xxy, Xxz));
+        m[11] = vfma(dy, vk<V>(-2.0), vadd(Yxy, Yyz));
+        m[12] = vfma(dz, vk<V>(-2.0), vadd(Zxz, Zyz));
+        m[13] = vsub(Xxy, Xxz);
+        m[14] = vsub(Yyz, Yxy);
+        m[15] = vsub(Zxz, Zyz);
+        m[16] = vadd(vfma(vadd(sx, fyz), vk<V>(-2.0), f[0]), ee);
+        m[17] = vsub(e5, f5);
+        m[18] = vsub(e6, f6);
         sfor<4, 19>([&](auto A) {
             constexpr int a = A;
-            const V lam = vbc<V>(P.lam[a]);
-            if constexpr (a < 10 || a == 16) k[a] = vfma(lam, vsub(k[a], m[a]), m[a]);
-            else k[a] = vmul(vbc<V>(S(1) - P.lam[a]), m[a]);
-            if constexpr (CP == GUO && a < 10) k[a] = vfma(vbc<V>(S(1) - S(0.5) * P.lam[a]), s[a - 4], k[a]);
+            const S l = MODE == 1 ? P.lam_bgk : P.lam[a];
+            if constexpr (a < 10 || a == 16) k[a] = vmul(vbc<V>(l), vsub(k[a], m[a]));
+            else k[a] = vmul(vbc<V>(-l), m[a]);
+            if constexpr (CP == GUO && a < 10) k[a] = vfma(vbc<V>(S(1) - S(0.5) * l), s[a - 4], k[a]);
         });
     }
-    if constexpr (CP == GUO) {
-        // (T F)_a = F_a on the momentum rows
-        k[1] = vfma(F[0], vk<V>(1.0 / 12.0), k[1]);
-        k[2] = vfma(F[1], vk<V>(1.0 / 12.0), k[2]);
-        k[3] = vfma(F[2], vk<V>(1.0 / 12.0), k[3]);
-    }
-
     if (P.kT > S(0)) {
         // as in the fully relaxed collisions, with g_ab = 1 - gamma_a gamma_b on the
         // amplitudes: M = [[(2/3 + om) g_44, -om g_4,16], [., (2 + om) g_16,16]]
-        const V sc = vsqrt_pos(vmul(vbc<V>(vmul(S(3.0 * DrawScale<S>::v), P.kT)), rho));
+        const V sc = vsqrt_pos(vmul(vbc<V>(vmul(S(3.0 * DrawScale<S>::v / DrawScale<S>::mean_square), P.kT)), rho));
         const V om = vfma(cs2, vk<V>(-3.0), vk<V>(1.0));
         const V mpp = vmul(vadd(vk<V>(2.0 / 3.0), om), vbc<V>(P.g_diag[4]));
         const V mpr = vmul(om, vbc<V>(-P.g_pair));
         const V mrr = vmul(vadd(vk<V>(2.0), om), vbc<V>(P.g_diag[16]));
         const V det = vsub(vmul(mpp, mrr), vmul(mpr, mpr));
         const V q = vrsqrt(mpp);
-        V k11 = vmul(vmul(mpp, q), vk<V>(1.0 / 24.0));
-        V k21 = vmul(vmul(mpr, q), vk<V>(1.0 / 72.0));
-        V k22 = vmul(vmul(det, vrsqrt(vmul(det, mpp))), vk<V>(1.0 / 72.0));
+        V k11 = vmul(mpp, q);
+        V k21 = vmul(mpr, q);
+        V k22 = vmul(det, vrsqrt(vmul(det, mpp)));
         auto bad = [&](int l) { return !(lane(det, l) > S(0)) || !(lane(mpp, l) > S(0)); };
         bool bad_noise = false;
 #pragma unroll
@@ -715,39 +713,40 @@ __device__ __forceinline__ void collide_d3q19_rates(V (&f)[19], const V drho, co
             }
             atomicOr(status, ST_NOISE);
         }
-        // sqrt(N_a g_aa) / (36 N_a), 36 N_a as above
-        auto amp = [&](int a, double inv) { return vbc<V>(vmul(P.namp[a], S(inv))); };
+        auto amp = [&](int a) { return vbc<V>(P.namp[a]); };       // sqrt(N_a g_aa)
         V n[4];
         draw4<19>(key, site, 0u, sc, sc, n, true);
         const V n4 = n[0];
         k[4] = vfma(k11, n4, k[4]);
-        k[5] = vfma(n[1], amp(5, 1.0 / 48.0), k[5]);
-        k[6] = vfma(n[2], amp(6, 1.0 / 16.0), k[6]);
-        k[7] = vfma(n[3], amp(7, 1.0 / 4.0), k[7]);
+        k[5] = vfma(n[1], amp(5), k[5]);
+        k[6] = vfma(n[2], amp(6), k[6]);
+        k[7] = vfma(n[3], amp(7), k[7]);
         draw4<19>(key, site, 1u, sc, sc, n, true);
-        k[8] = vfma(n[0], amp(8, 1.0 / 4.0), k[8]);
-        k[9] = vfma(n[1], amp(9, 1.0 / 4.0), k[9]);
-        k[10] = vfma(n[2], amp(10, 1.0 / 24.0), k[10]);
-        k[11] = vfma(n[3], amp(11, 1.0 / 24.0), k[11]);
+        k[8] = vfma(n[0], amp(8), k[8]);
+        k[9] = vfma(n[1], amp(9), k[9]);
+        k[10] = vfma(n[2], amp(10), k[10]);
+        k[11] = vfma(n[3], amp(11), k[11]);
         draw4<19>(key, site, 2u, sc, sc, n, true);
-        k[12] = vfma(n[0], amp(12, 1.0 / 24.0), k[12]);
-        k[13] = vfma(n[1], amp(13, 1.0 / 8.0), k[13]);
-        k[14] = vfma(n[2], amp(14, 1.0 / 8.0), k[14]);
-        k[15] = vfma(n[3], amp(15, 1.0 / 8.0), k[15]);
+        k[12] = vfma(n[0], amp(12), k[12]);
+        k[13] = vfma(n[1], amp(13), k[13]);
+        k[14] = vfma(n[2], amp(14), k[14]);
+        k[15] = vfma(n[3], amp(15), k[15]);
         draw4<19>(key, site, 3u, sc, sc, n, false);
         k[16] = vfma(k22, n[0], vfma(k21, n4, k[16]));
-        k[17] = vfma(n[1], amp(17, 1.0 / 48.0), k[17]);
-        k[18] = vfma(n[2], amp(18, 1.0 / 16.0), k[18]);
+        k[17] = vfma(n[1], amp(17), k[17]);
+        k[18] = vfma(n[2], amp(18), k[18]);
     }
-    if constexpr (MODE == 1) {
-        V g[19];
-        d3q19_populations<V>(k, g);
-        const V oml = vbc<V>(S(1) - P.lam_bgk);
+    // w_a / (36 N_a); (T F)_a = F_a on the momentum rows
+    sfor<4, 19>([&](auto A) { k[decltype(A)::value] = over_norm<decltype(A)::value>(k[decltype(A)::value]); });
+    k[0] = vk<V>(0.0);
+    sfor<0, 3>([&](auto C) {
+        constexpr int c = C;
+        k[1 + c] = CP == GUO ? vmul(F[c], vk<V>(1.0 / 12.0)) : vk<V>(0.0);
+    });
+    V g[19];
+    d3q19_populations<V>(k, g);
 #pragma unroll
-        for (int i = 0; i < 19; ++i) f[i] = vfma(oml, f[i], g[i]);
-    } else {
-        d3q19_populations<V>(k, f);
-    }
+    for (int i = 0; i < 19; ++i) f[i] = vadd(f[i], g[i]);
 }
 
 }  // namespace lbf
