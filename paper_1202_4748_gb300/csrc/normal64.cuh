@@ -107,9 +107,9 @@ LB_HD uint64_t n64_root(uint64_t v) {
     return r << 2;
 }
 
-// sqrt(x) and 1/sqrt(x) of a positive normal x, within 0.51 units in the last
-// place (16 and 10 FP64 operations of the library become integer ones);
-// anything else through the library.
+// sqrt(x) of a positive normal x, correctly rounded, and 1/sqrt(x), within 0.51
+// units in the last place (16 and 10 FP64 operations of the library become integer
+// ones); anything else through the library.
 LB_HD bool n64_split(double x, uint64_t& v, int& h) {
     uint64_t u;
     memcpy(&u, &x, 8);
@@ -126,7 +126,14 @@ LB_HD double n64_sqrt(double x) {
     uint64_t v;
     int h;
     if (!n64_split(x, v, h)) return sqrt(x);
-    return n64_double(n64_root(v), h);
+    // the nearest 53-bit N of the root to 2^-58, then of the exact one: the root
+    // lies below N + 1/2 (N - 1/2) where v 2^44 does below (2N + 1)^2 ((2N - 1)^2),
+    // all modulo 2^64 (the differences are below 2^57; no root of 53 bits is a half)
+    const uint64_t r = n64_root(v);
+    uint64_t N = (r >> 11) + ((r >> 10) & 1);
+    const int64_t d = int64_t((v << 44) - 4 * N * N);
+    N += uint64_t(d > int64_t(4 * N)) - uint64_t(d < -int64_t(4 * N));
+    return n64_bits((uint64_t(h + 1021) << 52) + N);
 }
 LB_HD double n64_inv_sqrt(double x) {
     uint64_t v;

@@ -26,6 +26,12 @@ extern "C" int wide(const double* f, double* out, long n) {
     }
     return finite;
 }
+extern "C" void roots(const double* x, double* r, double* q, long n) {
+    for (long i = 0; i < n; ++i) {
+        r[i] = lbf::n64_sqrt(x[i]);
+        q[i] = lbf::n64_inv_sqrt(x[i]);
+    }
+}
 """ % HEADER
 
 
@@ -72,3 +78,28 @@ def test_wide_sums_keep_what_a_cancellation_leaves(lib):
         g = f[4:5].copy()
         g[0, 5] = bad
         assert call(lib.wide, g)[0] == 0
+
+
+def test_roots_over_every_exponent(lib):
+    """sqrt rounds like the library's (correctly), 1/sqrt to 0.51 units in the last
+    place, from the smallest normal double to the largest: random mantissas, those
+    next to squares of 27-bit numbers, and those whose root lies closest to half of
+    a last place, N + 1/2 with x the double nearest to its square."""
+    rng = np.random.default_rng(6)
+    n = 400_000
+    mant = rng.uniform(0.5, 1.0, n)
+    sq = rng.integers(1 << 26, 1 << 27, n).astype(np.float64) ** 2 * 2.0 ** -54
+    half = (rng.integers(1 << 52, 1 << 53, n).astype(np.longdouble) + np.longdouble(0.5)) * np.longdouble(2.0) ** -53
+    mant = np.concatenate([mant, sq, np.nextafter(sq, 0), np.nextafter(sq, 1), (half * half).astype(np.float64),
+                           0.5 * np.nextafter(1, 2) * np.ones(1), [0.5, np.nextafter(1, 0)]])
+    mant = np.where(mant >= 1, 0.5, np.where(mant < 0.5, mant * 2, mant))
+    x = np.ldexp(mant, rng.integers(-1021, 1025, mant.size))
+    for e in (-1021, -1020, 1023, 1024):
+        x = np.concatenate([x, np.ldexp(mant[-3000:], e)])
+    x = np.concatenate([x, [np.finfo(float).tiny, np.nextafter(np.finfo(float).tiny, 1), np.finfo(float).max]])
+    assert np.all(np.isfinite(x)) and x.min() == np.finfo(float).tiny
+    r, q = np.empty(x.size), np.empty(x.size)
+    lib.roots(*[v.ctypes.data_as(ctypes.c_void_p) for v in (x, r, q)], ctypes.c_long(x.size))
+    np.testing.assert_array_equal(r, np.sqrt(x))
+    want = np.sqrt(x.astype(np.longdouble))
+    assert np.max(np.abs(q * want - 1)) < 1.1 * 2.0 ** -53
