@@ -43,7 +43,7 @@ __device__ __forceinline__ float density_of(const float (&f)[Q]) {
 template <int Q>
 __device__ __forceinline__ double density_of(const double (&f)[Q]) {
     const FixedSum<double, Q> s(f);
-    if (s.finite()) {
+    if (s.in_range()) {
         int64_t v = 0;
 #pragma unroll
         for (int i = 0; i < Q; ++i) v += s.m[i];
@@ -61,7 +61,7 @@ template <class V>
 __device__ __forceinline__ void moments_d2q9(const V (&f)[9], V& drho, V& jx, V& jy) {
     if constexpr (VT<V>::W == 1 && sizeof(V) == 8) {
         const FixedSum<double, 9> s(f);
-        if (s.finite()) {
+        if (s.in_range()) {
             const int64_t(&m)[9] = s.m;
             const int64_t a = m[5] - m[6], b = m[7] - m[8];
             drho = s.value(((m[0] + m[1]) + (m[2] + m[3])) + ((m[4] + m[5]) + (m[6] + m[7])) + m[8]);

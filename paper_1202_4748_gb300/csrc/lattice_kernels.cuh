@@ -188,10 +188,11 @@ __global__ void __launch_bounds__(AUX_THREADS)
 // units, which do two operations per clock and SM.  FP32 fields to 2^-57 of the
 // largest population (FixedSum; compensated FP32 sums with eight conversions per
 // site took 57 us for 2^20 sites, now 47), FP64 fields to 2^-116 (WideSum;
-// compensated FP64 sums, to 2^-106, took 0.39 ms for 573,440 sites).
+// compensated FP64 sums, to 2^-106, took 0.39 ms for 573,440 sites).  Outside
+// their range: FP64 sums, compensated (Knuth's TwoSum).
 template <class L, class Real>
 __device__ __forceinline__ void site_sums(const Real (&f)[L::Q], double& rv, double (&mv)[3]) {
-    bool finite;
+    bool in_range;
     if constexpr (sizeof(Real) == 8) {
         const WideSum<L::Q> s(f);
         __int128 r = 0, m[3] = {0, 0, 0};
@@ -207,7 +208,7 @@ __device__ __forceinline__ void site_sums(const Real (&f)[L::Q], double& rv, dou
         }
         rv = s.value(r);
         for (int a = 0; a < 3; ++a) mv[a] = s.value(m[a]);
-        finite = s.finite();
+        in_range = s.in_range();
     } else {
         const FixedSum<Real, L::Q> s(f);
         int64_t r = 0, m[3] = {0, 0, 0};
@@ -219,14 +220,23 @@ __device__ __forceinline__ void site_sums(const Real (&f)[L::Q], double& rv, dou
         }
         rv = s.value(r);
         for (int a = 0; a < 3; ++a) mv[a] = s.value(m[a]);
-        finite = s.finite();
+        in_range = s.in_range();
     }
-    if (!finite) {
-        rv = mv[0] = mv[1] = mv[2] = 0.0;
+    if (!in_range) {
+        double v[4] = {0.0, 0.0, 0.0, 0.0}, c[4] = {0.0, 0.0, 0.0, 0.0};
+        auto add = [&](int k, double x) {
+            const double t = v[k] + x, y = t - v[k];
+            c[k] += (v[k] - (t - y)) + (x - y);
+            v[k] = t;
+        };
         for (int i = 0; i < L::Q; ++i) {
-            rv += double(f[i]);
-            for (int a = 0; a < 3; ++a) mv[a] += L::c(i, a) * double(f[i]);
+            add(0, double(f[i]));
+            for (int a = 0; a < 3; ++a)
+                if (L::c(i, a) != 0) add(1 + a, L::c(i, a) * double(f[i]));
         }
+        auto sum = [&](int k) { return v[k] - v[k] == 0.0 ? v[k] + c[k] : v[k]; };    // (an overflow has no remainder)
+        rv = sum(0);
+        for (int a = 0; a < 3; ++a) mv[a] = sum(1 + a);
     }
 }
 

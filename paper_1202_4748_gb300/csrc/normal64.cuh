@@ -152,8 +152,10 @@ LB_HD double n64_inv_sqrt(double x) {
 // Sums of N floats or doubles to about 2^-57 of the largest: the mantissas
 // aligned to the largest exponent as integers of 58 bits, so that a sum of up to
 // 31 of them fits 63 bits and every sum costs integer additions (floats within
-// 2^-34 of the largest enter exactly).  finite() is false when a value is
-// infinite or NaN (the sums are then the caller's in FP64).
+// 2^-34 of the largest enter exactly).  Subnormal values count as 0 and a sum has
+// to be a normal double, which holds in_range(): where the largest value is so
+// small that subnormal ones matter beside it, so large that a sum may overflow,
+// infinite or NaN (finite() is false), the sums are the caller's in FP64.
 template <class T, int N>
 struct FixedSum {
     static_assert(N <= 31, "headroom");
@@ -194,12 +196,16 @@ struct FixedSum {
         }
     }
     LB_HD bool finite() const { return top != kTop; }
+    // largest value from 2^63 times the subnormal ones (doubles: and its 2^-57 a normal double) to 2^-5 of overflow
+    LB_HD bool in_range() const {
+        constexpr uint32_t low = 64u << kExp, high = sizeof(T) == 8 ? 2040u << kExp : kTop;
+        return top - low < high - low;
+    }
     // the double nearest to s 2^(top - bias - 57)
     LB_HD double value(int64_t s) const {
         if (s == 0) return 0.0;
         const uint64_t a = s < 0 ? uint64_t(0) - uint64_t(s) : uint64_t(s);
         const int nl = n64_clz(a), e = int(top >> kExp) - kBias + 1 - 57 + 63 - nl;      // (m / 2^64) 2^e
-        if (e < -1020) return 0.0;
         const double d = n64_double(a << nl, e);
         return s < 0 ? -d : d;
     }
@@ -230,6 +236,11 @@ struct WideSum {
         }
     }
     LB_HD bool finite() const { return top != 0x7ff00000u; }
+    // as FixedSum: 2^-121 of the largest value is a normal double, 2^5 times it too
+    LB_HD bool in_range() const {
+        constexpr uint32_t low = 160u << 20, high = 2040u << 20;
+        return top - low < high - low;
+    }
     // f[i] as an integer multiple of 2^(top - bias - 121)
     LB_HD __int128 add(int i) const {
         const uint64_t u = bits(f[i]), one = uint64_t(1) << 52;
@@ -245,7 +256,6 @@ struct WideSum {
         a <<= nl;
         const uint64_t m = uint64_t(a >> 64), rest = (m & 0x3ff) | (uint64_t(a) != 0) | ((m >> 11) & 1);
         const int e = int(top >> 20) - 1023 + 1 - 121 + 127 - nl;                          // (m / 2^64) 2^e
-        if (e < -1020) return 0.0;
         const double d = n64_bits((uint64_t(e + 1021) << 52) + (m >> 11) + (((m >> 10) & 1) & (rest != 0)));
         return s < 0 ? -d : d;
     }

@@ -322,9 +322,9 @@ __global__ void __launch_bounds__(TX* TY, MINB)
                         if constexpr (L::c(i, cc) == 1) s += fs.m[i];
                         if constexpr (L::c(i, cc) == -1) s -= fs.m[i];
                     });
-                    if (!fs.finite())
+                    if (!fs.in_range())
                         sfor<1, 19>([&](auto I) { d += double(L::c(decltype(I)::value, cc)) * f[decltype(I)::value]; });
-                    jm[cc] = fs.finite() ? fs.value(s) : d;
+                    jm[cc] = fs.in_range() ? fs.value(s) : d;
                 });
             } else if constexpr (PULL) {
                 sfor<0, 3>([&](auto C) {

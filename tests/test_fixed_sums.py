@@ -26,6 +26,29 @@ extern "C" int wide(const double* f, double* out, long n) {
     }
     return finite;
 }
+// the sum through the fixed-point form where it says it holds, ok[i] = 0 elsewhere
+template <class T> static void ranged(const T* f, double* out, int* ok, long n) {
+    for (long i = 0; i < n; ++i) {
+        T g[19];
+        for (int k = 0; k < 19; ++k) g[k] = f[19 * i + k];
+        const lbf::FixedSum<T, 19> s(g);
+        int64_t t = 0;
+        for (int k = 0; k < 19; ++k) t += s.m[k];
+        out[i] = (ok[i] = s.in_range()) ? s.value(t) : 0.0;
+    }
+}
+extern "C" void ranged64(const double* f, double* out, int* ok, long n) { ranged(f, out, ok, n); }
+extern "C" void ranged32(const float* f, double* out, int* ok, long n) { ranged(f, out, ok, n); }
+extern "C" void ranged128(const double* f, double* out, int* ok, long n) {
+    for (long i = 0; i < n; ++i) {
+        double g[19];
+        for (int k = 0; k < 19; ++k) g[k] = f[19 * i + k];
+        const lbf::WideSum<19> s(g);
+        __int128 t = 0;
+        for (int k = 0; k < 19; ++k) t += s.add(k);
+        out[i] = (ok[i] = s.in_range()) ? s.value(t) : 0.0;
+    }
+}
 extern "C" void roots(const double* x, double* r, double* q, long n) {
     for (long i = 0; i < n; ++i) {
         r[i] = lbf::n64_sqrt(x[i]);
@@ -103,3 +126,30 @@ def test_roots_over_every_exponent(lib):
     np.testing.assert_array_equal(r, np.sqrt(x))
     want = np.sqrt(x.astype(np.longdouble))
     assert np.max(np.abs(q * want - 1)) < 1.1 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("name,dtype,cut", [("ranged64", np.float64, 57), ("ranged32", np.float32, 57),
+                                            ("ranged128", np.float64, 121)])
+def test_sums_over_every_exponent(lib, name, dtype, cut):
+    """Wherever the sum claims to hold it is within 19 x 2^-cut of the largest
+    addend and a rounding of the exact one, at every exponent of the type; the
+    ordinary ones (1e-200 to 1e200, FP32 1e-18 up) are all claimed."""
+    rng = np.random.default_rng(8)
+    n = 30_000
+    info = np.finfo(dtype)
+    top = rng.integers(info.minexp - info.nmant, info.maxexp + 1, n)
+    f = rng.uniform(-1, 1, (n, 19)) * np.exp2(rng.uniform(-80, 0, (n, 19)) * rng.integers(0, 2, (n, 1)))
+    f[np.arange(n), rng.integers(0, 19, n)] = rng.uniform(0.5, 1, n) * rng.choice([-1, 1], n)
+    f[: n // 3] = np.abs(f[: n // 3])                          # sums that overflow
+    f = np.ascontiguousarray(np.ldexp(f, top[:, None]).astype(dtype))
+    assert np.all(np.isfinite(f))
+    out, ok = np.empty(n), np.empty(n, dtype=np.int32)
+    getattr(lib, name)(*[v.ctypes.data_as(ctypes.c_void_p) for v in (f, out, ok)], ctypes.c_long(n))
+    big = np.max(np.abs(f.astype(np.longdouble)), axis=1)
+    ordinary = (big > (1e-200 if dtype == np.float64 else 1e-18)) & (big < 1e200)
+    assert np.all(ok[ordinary]) and not np.all(ok)
+    for row, o, held in zip(f.astype(np.float64).tolist(), out.tolist(), ok.tolist()):
+        if held:
+            exact = sum(map(Fraction, row))
+            bound = 19 * Fraction(2) ** -cut * Fraction(max(map(abs, row))) + Fraction(2) ** -53 * abs(exact) * (1 + Fraction(2) ** -50)
+            assert np.isfinite(o) and abs(Fraction(o) - exact) <= bound
