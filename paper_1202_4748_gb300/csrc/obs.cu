@@ -22,12 +22,20 @@
 //                      after another behind CTA barriers (a launch per level
 //                      before: these levels are microseconds of latency each),
 //                      and the sums of the records the kernels above wrote
+#include "../../include/lbfluct.h"
 #include "lattice_kernels.cuh"
 #include "lb_launch.h"
 
 namespace lbf {
 
 namespace {
+
+// Histogram counts are dynamic shared memory beside the kernels' own, together
+// within what a launch gets without asking for more.
+constexpr size_t kPlainShared = 48 * 1024;
+constexpr size_t hist_shared(int nbins, int levels) { return sizeof(unsigned) * levels * size_t(nbins + 2); }
+static_assert(sizeof(BlockSum<REC, OBS_THREADS>) + hist_shared(LB_MAX_HIST_BINS, 2) <= kPlainShared,
+              "pyr_bottom_kernel, pyr_part_kernel, pyr_up_kernel");
 
 __global__ void __launch_bounds__(AUX_THREADS)
     init_noise_kernel(const SysDev* __restrict__ sysv, const int4* __restrict__ items, double amp,
@@ -430,6 +438,17 @@ __device__ __forceinline__ void accumulate_records(const LevelDev& lv, const dou
     if (lane == 0) accumulate_level(a, double(lv.nblocks), t, status);
 }
 
+// Block sums of alternate levels: the first has up to kTopBlocks blocks, every
+// next one at most a quarter of the one below it.
+template <int NC>
+struct TopShared {
+    BlockSum<REC, NC> sh;
+    double bs0[kTopBlocks], be0[kTopBlocks], bs1[kTopBlocks / 4], be1[kTopBlocks / 4];
+    double sums[kMaxObsLevels][REC];
+    LevelDev lvs[kMaxObsLevels];
+};
+static_assert(sizeof(TopShared<TOP_THREADS / 2>) + hist_shared(LB_MAX_HIST_BINS, 1) <= kPlainShared, "pyr_top_kernel");
+
 // The coarsest levels of one system per CTA: levels top - 1 .. 0 (level `top`
 // is complete), one after another in the first kTopChain threads, with the
 // block sums of the level below in shared memory (the first takes them from
@@ -442,10 +461,10 @@ __global__ void __launch_bounds__(TOP_THREADS)
                    double* Eg, const double* __restrict__ rec, double* __restrict__ acc, int* status,
                    const HistDev H) {
     constexpr int NC = TOP_THREADS / 2;
-    __shared__ BlockSum<REC, NC> sh;
-    __shared__ double bs[2][kTopBlocks], be[2][kTopBlocks];
-    __shared__ double sums[kMaxObsLevels][REC];
-    __shared__ LevelDev lvs[kMaxObsLevels];
+    __shared__ TopShared<NC> sm;
+    auto& sh = sm.sh;
+    auto& sums = sm.sums;
+    auto& lvs = sm.lvs;
     extern __shared__ unsigned shist[];
     const ObsTop T = tops[blockIdx.x];
     const int nh = H.nbins + 2, tid = threadIdx.x;
@@ -461,7 +480,11 @@ __global__ void __launch_bounds__(TOP_THREADS)
     for (int l = T.top - 1; l >= 0; --l) {
         const LevelDev& lv = lvs[l];
         const LevelDev& ch = lvs[l + 1];
-        const int nb = int(lv.nblocks), src = (l + 1) & 1, dst = l & 1;
+        const int nb = int(lv.nblocks), dst = (T.top - 1 - l) & 1;       // (0: the first level, the largest)
+        double* const bs = dst ? sm.bs1 : sm.bs0;
+        double* const be = dst ? sm.be1 : sm.be0;
+        const double* const cs = dst ? sm.bs0 : sm.bs1;                  // the level below
+        const double* const ce = dst ? sm.be0 : sm.be1;
         const double inv_v = hist ? 1.0 / block_volume(lv) : 0.0;
         const bool warp_only = nb <= 32;
         if (warp_only && tid >= 32) break;                // the remaining levels have no more blocks than this one
@@ -483,14 +506,14 @@ __global__ void __launch_bounds__(TOP_THREADS)
 #pragma unroll
                     for (int dy = 0; dy < 2; ++dy) {
                         const int c = 2 * X + ch.gx * (2 * Y + dy + ch.gy * (nz * Z + dz));
-                        s += bs[src][c];
-                        e += be[src][c];
-                        s += bs[src][c + 1];
-                        e += be[src][c + 1];
+                        s += cs[c];
+                        e += ce[c];
+                        s += cs[c + 1];
+                        e += ce[c + 1];
                     }
             }
-            bs[dst][b] = s;
-            be[dst][b] = e;
+            bs[b] = s;
+            be[b] = e;
             add_terms(tb, s, e);
             if (hist) atomicAdd(shist + hist_bin(s * inv_v, H), 1u);
         }
@@ -575,7 +598,7 @@ cudaError_t launch_pyr_bottom(const SysDev* sys, const LevelDev* lv, const ObsIt
                               const double* d, const double* dbar, double* S, double* E, double* rec,
                               const HistDev& hist, cudaStream_t st) {
     if (n_items == 0) return cudaSuccess;
-    const size_t shm = hist.nbins > 0 ? 2 * sizeof(unsigned) * (hist.nbins + 2) : 0;
+    const size_t shm = hist.nbins > 0 ? hist_shared(hist.nbins, 2) : 0;
     pyr_bottom_kernel<<<n_items, OBS_THREADS, shm, st>>>(sys, lv, items, d, dbar, S, E, rec, hist);
     return cudaGetLastError();
 }
@@ -584,7 +607,7 @@ cudaError_t launch_pyr_part(const SysDev* sys, const LevelDev* lv, const ObsPart
                             const double* d, const double* dbar, double* S, double* E, double2* parts, double* rec,
                             const HistDev& hist, cudaStream_t st) {
     if (n_items == 0) return cudaSuccess;
-    const size_t shm = hist.nbins > 0 ? 2 * sizeof(unsigned) * (hist.nbins + 2) : 0;
+    const size_t shm = hist.nbins > 0 ? hist_shared(hist.nbins, 2) : 0;
     pyr_part_kernel<<<n_items, OBS_THREADS, shm, st>>>(sys, lv, items, d, dbar, S, E, parts, rec, hist);
     return cudaGetLastError();
 }
@@ -598,7 +621,7 @@ cudaError_t launch_pyr_blocks(const LevelDev* lv, const ObsBlocks* items, int n_
 
 cudaError_t launch_pyr_top(const LevelDev* lv, const ObsTop* tops, int n_sys, int dims3, double* S, double* E,
                            const double* rec, double* acc, int* status, const HistDev& hist, cudaStream_t st) {
-    const size_t shm = hist.nbins > 0 ? sizeof(unsigned) * (hist.nbins + 2) : 0;
+    const size_t shm = hist.nbins > 0 ? hist_shared(hist.nbins, 1) : 0;
     pyr_top_kernel<<<n_sys, TOP_THREADS, shm, st>>>(lv, tops, dims3, S, E, rec, acc, status, hist);
     return cudaGetLastError();
 }
@@ -606,7 +629,7 @@ cudaError_t launch_pyr_top(const LevelDev* lv, const ObsTop* tops, int n_sys, in
 cudaError_t launch_pyr_up(const LevelDev* lv, const ObsItem* items, int n_items, int dims3,
                           double* S, double* E, double* rec, const HistDev& hist, cudaStream_t st) {
     if (n_items == 0) return cudaSuccess;
-    const size_t shm = hist.nbins > 0 ? sizeof(unsigned) * (hist.nbins + 2) : 0;
+    const size_t shm = hist.nbins > 0 ? hist_shared(hist.nbins, 1) : 0;
     pyr_up_kernel<<<n_items, OBS_THREADS, shm, st>>>(lv, items, dims3, S, E, rec, hist);
     return cudaGetLastError();
 }
