@@ -335,7 +335,8 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
     }
     st = choose_tile(s[0].lattice, s[0].coupling, o, tile_id);
     if (st != LB_OK) return st;
-    if (o->variant == 0 && o->tile[0] <= 0 && o->occupancy <= 0) {
+    const bool by_default = o->variant == 0 && o->tile[0] <= 0 && o->occupancy <= 0;
+    if (by_default) {
         if (d3) choose_d3q19_row(s, n, !fp32 ? 2 : (relaxed ? 0 : 1), quads, tile_id);
         else if (s[0].coupling == LB_MODEQ) choose_d2q9_row(s, n, fp32, fp32 && relaxed && quads, tile_id);
     }
@@ -581,8 +582,9 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
     };
     P.sys = take(sizeof(SysDev) * n);
     P.phys = take(sizeof(SysPhys<double>) * n);
-    // (room for the shortest default tiles, so that the layout does not depend on the choice)
-    const int short_tile[3] = {d3 ? 16 : 64, d3 ? 8 : 4, d3 ? 2 : 1};
+    // (room for the smallest default tiles, and below for the split step's field, so that
+    // the size does not depend on the row that the current device's SMs make the default)
+    const int short_tile[3] = {d3 ? 8 : 64, d3 ? 8 : 4, d3 ? 2 : 1};
     P.tiles = take(sizeof(int4) * std::max<int64_t>(P.n_tiles, tiles_of(s, n, short_tile)));
     P.pop0 = take(es * q * P.n_sites);
     P.pop1 = take(es * q * P.n_sites);
@@ -600,7 +602,8 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
     P.d = take(sizeof(double) * P.n_sites);
     P.S = take(sizeof(double) * P.n_blocks_pyr);
     P.E = take(sizeof(double) * P.n_blocks_pyr);
-    if (P.split) off = std::max(off, align_up(P.mom + (fp32 && relaxed ? 16 : es) * P.n_sites));
+    if (P.split || (d3 && by_default))
+        off = std::max(off, align_up(P.mom + (fp32 && relaxed ? 16 : es) * P.n_sites));
     P.bottom_items = take(sizeof(ObsItem) * P.n_bottom);
     P.part_items = take(sizeof(ObsPart) * P.part_h.size());
     P.block_items = take(sizeof(ObsBlocks) * P.block_h.size());
