@@ -94,16 +94,17 @@ cudaError_t step_ws(const StepLaunch& a, cudaStream_t st) {
     size_t dyn = 0;
     if constexpr (STG == 1) {
         dyn = BulkStage<L, TX, TY, PW>::bytes;
-        static bool attr = false;              // once per instantiation
-        if (!attr) {
+        static PerDevice attr;                 // once per instantiation and device
+        cudaError_t e = cudaSuccess;
+        const int set = attr.get(current_device(), [&] {
             auto k = step_kernel_ws<L, TX, TY, PW, MINB, STG>;
-            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dyn));
+            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dyn));
             if (e == cudaSuccess)
                 e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
                                          int(cudaSharedmemCarveoutMaxShared));
-            if (e != cudaSuccess) return e;
-            attr = true;
-        }
+            return e == cudaSuccess ? 1 : 0;
+        });
+        if (!set) return e;
     }
     step_kernel_ws<L, TX, TY, PW, MINB, STG><<<a.n_tiles, TX * TY + 32 * PW, dyn, st>>>(A);
     return cudaGetLastError();
@@ -118,18 +119,20 @@ template <int TX, int TY, int PW, int MINB, int R, int STG, int CP = GUO>
 cudaError_t step_pair(const StepLaunch& a, cudaStream_t st) {
     const StepArgs<float> A = step_args<float>(a);
     constexpr size_t dyn = PairSmem<TX, TY, PW, R, STG, CP>::bytes;
-    static int state = 0;                      // once per instantiation: 1 usable, -1 not
-    if (state == 0) {
+    static PerDevice usable;                   // once per instantiation and device: 1 usable, -1 not
+    cudaError_t e = cudaSuccess;
+    const int state = usable.get(current_device(), [&] {
         auto k = step_kernel_pair<TX, TY, PW, MINB, R, STG, CP>;
         cudaFuncAttributes fa;
-        cudaError_t e = cudaFuncGetAttributes(&fa, k);
+        e = cudaFuncGetAttributes(&fa, k);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dyn));
         // (no carve-out preference: the rings need a fraction of the SM's
         // shared memory, and the producers' load misses are staged in L1)
-        if (e != cudaSuccess) return e;
+        if (e != cudaSuccess) return 0;
         // the register split must balance against the launch count it assumes
-        state = (!PairRegs<TX, TY, PW, MINB, STG>::split || fa.numRegs == PairRegs<TX, TY, PW, MINB, STG>::launch) ? 1 : -1;
-    }
+        return !PairRegs<TX, TY, PW, MINB, STG>::split || fa.numRegs == PairRegs<TX, TY, PW, MINB, STG>::launch ? 1 : -1;
+    });
+    if (!state) return e;
     if (state < 0) {
         if constexpr (CP == MODEQ) return step_zm<D3Q19, TX, TY, MINB>(a, st);
         else return step_ws<D3Q19, TX, TY, PW, 1, 0>(a, st);

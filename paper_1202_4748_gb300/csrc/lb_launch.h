@@ -6,11 +6,18 @@
 #include <cuda_runtime.h>
 
 #include "lb_device.cuh"
+#include "per_device.h"
 
 namespace lbf {
 
 constexpr int AUX_THREADS = 256;        // threads of the auxiliary (non-step) kernels
 constexpr int SITES_PER_THREAD = 4;     // sites per thread in a site-pass item
+
+// The calling thread's device (-1: none).
+inline int current_device() {
+    int d = -1;
+    return cudaGetDevice(&d) == cudaSuccess ? d : -1;
+}
 
 struct StepLaunch {
     const SysDev* sys;

@@ -509,23 +509,24 @@ cudaError_t launch_sk_fft(const FftLaunch& a, cudaStream_t st) {
     // two buffers of kSkFftMaxElems values; the last pass holds every field of a
     // line, three of kSkFftMaxElems in 2-D (192 KB), four of at most 483 in 3-D
     constexpr int kMaxBytes = int(2 * kSkFftMaxElems * sizeof(double2));
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(fft_x_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxBytes);
+    static PerDevice attr;
+    cudaError_t e = cudaSuccess;
+    const int set = attr.get(current_device(), [&] {
+        e = cudaFuncSetAttribute(fft_x_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxBytes);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(fft_y_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxBytes);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(fft_last_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * kMaxBytes);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+        return e == cudaSuccess ? 1 : 0;
+    });
+    if (!set) return e;
     const double2* tw = reinterpret_cast<const double2*>(a.tw);
     double2* F = reinterpret_cast<double2*>(a.F);
     // both line buffers of the largest item
     const size_t line = 2 * sizeof(double2);
     fft_x_kernel<<<a.n_x, FFT_THREADS, line * a.max_x, st>>>(a.sk, a.items, a.d, a.dbar, a.j, a.n_sites, tw, F,
                                                             a.fstride);
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e == cudaSuccess && a.dims == 3) {
         fft_y_kernel<<<a.n_y, FFT_THREADS, line * a.max_y, st>>>(a.sk, a.items + a.n_x, tw, F, a.fstride);
         e = cudaGetLastError();
