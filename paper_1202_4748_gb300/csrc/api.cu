@@ -79,6 +79,7 @@ struct Plan {
     std::vector<int4> fft_items_h;
     int n_fft_x = 0, n_fft_y = 0, n_fft_last = 0, fft_max_x = 0, fft_max_y = 0, fft_max_last = 0, n_fields = 1;
     int64_t half_total = 0;     // values of one field's half spectra
+    int64_t half_stride = 0;    // between the fields' half spectra
     size_t fft_items = 0;
 };
 
@@ -622,17 +623,21 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
     P.sk_tw = take(sizeof(double) * 2 * P.tw_total);
     P.fft_items = take(sizeof(int4) * P.fft_items_h.size());
     P.sk_acc = take(sizeof(double) * skn);
-    // half spectra of every field (line FFTs), or two complex fields (direct sums)
-    P.sk_b0 = take(sizeof(double) * 2 * (P.sk_fft ? P.half_total * P.n_fields : skn));
-    P.sk_b1 = take(sizeof(double) * 2 * (P.sk_fft ? 0 : skn));
-    P.sk_bins = take(sizeof(double) * 6 * P.sk_max_bins);
-    // momentum spectra: j (3 fields), Laplacian scratch (Guo), transforms (3 complex
-    // fields of the direct sums; the layout has them whichever way a side goes), accumulators
+    // line FFTs: half spectra of every field, the momentum's in the room of the
+    // transforms that the direct sums take, one stride apart from the first field's
+    // (half <= n: 3 half spectra fit 3 complex fields); direct sums: two complex fields
     P.jk = P.sk && o->jk_spectra == 1;
     const int64_t jkn = P.jk ? P.n_sites : 0;
+    P.sk_b0 = take(sizeof(double) * 2 * (P.sk_fft ? P.half_total : skn));
+    P.jk_F = off;
+    P.half_stride = int64_t(P.jk_F - P.sk_b0) / int64_t(sizeof(double2));
+    take(std::max<size_t>(sizeof(double) * 6 * jkn,
+                          P.sk_fft && P.jk ? sizeof(double2) * (P.half_stride * (P.n_fields - 2) + P.half_total) : 0));
+    P.sk_b1 = take(sizeof(double) * 2 * (P.sk_fft ? 0 : skn));
+    P.sk_bins = take(sizeof(double) * 6 * P.sk_max_bins);
+    // momentum spectra: j (3 fields), Laplacian scratch (Guo), accumulators
     P.jk_j = take(sizeof(double) * 3 * jkn);
     P.jk_lap = take(sizeof(double) * jkn);
-    P.jk_F = take(sizeof(double) * 6 * jkn);
     P.jk_acc = take(sizeof(double) * 3 * jkn);
     P.total = off;
     return LB_OK;
@@ -809,7 +814,6 @@ cudaError_t add_half_force(lb_ctx* c) {
 cudaError_t sample_sk_direct(lb_ctx* c) {
     const Plan& P = c->P;
     cudaError_t e = cudaSuccess;
-    const SysDev* sys = c->at<SysDev>(P.sys);
     const SkSys* sk = c->at<SkSys>(P.sk_sys);
     const int4* items = c->at<int4>(P.site_items);
     const int n_items = P.n_site_items;
@@ -820,7 +824,7 @@ cudaError_t sample_sk_direct(lb_ctx* c) {
     const bool d3 = c->lattice == LB_D3Q19;
     // in: real field (with dbar: the order parameter); the transform lands in b0 (3-D) or out
     auto transform = [&](const double* in, const double* dbar, double* out) {
-        cudaError_t r = launch_sk_x(sys, sk, items, n_items, in, dbar, tw, b0, c->stream);
+        cudaError_t r = launch_sk_x(sk, items, n_items, in, dbar, tw, b0, c->stream);
         if (r == cudaSuccess) r = launch_sk_pass(sk, items, n_items, 1, tw, b0, d3 ? b1 : out, c->stream);
         if (r == cudaSuccess && d3) r = launch_sk_pass(sk, items, n_items, 2, tw, b1, out, c->stream);
         c->launches += d3 ? 3 : 2;
@@ -857,7 +861,6 @@ cudaError_t sample_sk(lb_ctx* c, int buf, bool have_d) {
     if (e != cudaSuccess) return e;
     if (!P.sk_fft) return sample_sk_direct(c);
     FftLaunch a;
-    a.sys = c->at<SysDev>(P.sys);
     a.sk = c->at<SkSys>(P.sk_sys);
     a.items = c->at<int4>(P.fft_items);
     a.n_x = P.n_fft_x;
@@ -873,7 +876,7 @@ cudaError_t sample_sk(lb_ctx* c, int buf, bool have_d) {
     a.j = c->at<double>(P.jk_j);
     a.tw = c->at<double>(P.sk_tw);
     a.F = c->at<double>(P.sk_b0);
-    a.fstride = P.half_total;
+    a.fstride = P.half_stride;
     a.n_sites = P.n_sites;
     a.acc = c->at<double>(P.sk_acc);
     a.jacc = c->at<double>(P.jk_acc);

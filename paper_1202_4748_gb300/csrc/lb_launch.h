@@ -182,7 +182,7 @@ struct SkSys {             // per system: sides, twiddle-table offsets, site off
 cudaError_t launch_sk_twiddles(double* tw, const int* sides, const int* offs, int n_tables, int max_n,
                                cudaStream_t st);
 // x pass (real phi -> complex), then y and z passes (complex -> complex), then accumulate |F|^2 / N.
-cudaError_t launch_sk_x(const SysDev* sys, const SkSys* sk, const int4* items, int n_items, const double* d,
+cudaError_t launch_sk_x(const SkSys* sk, const int4* items, int n_items, const double* d,
                         const double* dbar, const double* tw, double* out, cudaStream_t st);
 cudaError_t launch_sk_pass(const SkSys* sk, const int4* items, int n_items, int axis, const double* tw,
                            const double* in, double* out, cudaStream_t st);
@@ -196,7 +196,6 @@ constexpr int kSkFftMaxElems = 2048;
 constexpr int FFT_THREADS = 128;
 bool sk_fft_side(int n);
 struct FftLaunch {
-    const SysDev* sys;
     const SkSys* sk;
     const int4* items;
     int n_x, n_y, n_last, max_x, max_y, max_last;

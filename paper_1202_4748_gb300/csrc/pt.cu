@@ -175,12 +175,11 @@ cudaError_t pt_eval(PtCtx& c, double m, double kappa, bool want_s2, double& S1, 
                                                                      c.at<double>(P.part2));
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && want_s2) {
-        const SysDev* sys = c.at<SysDev>(P.sys);
         const SkSys* sk = c.at<SkSys>(P.sk);
         const double* tw = c.at<double>(P.tw);
         double* b0 = c.at<double>(P.b0);
         double* b1 = c.at<double>(P.b1);
-        e = launch_sk_x(sys, sk, items, P.n_items, c.at<double>(P.G), nullptr, tw, b0, c.st);
+        e = launch_sk_x(sk, items, P.n_items, c.at<double>(P.G), nullptr, tw, b0, c.st);
         if (e == cudaSuccess) e = launch_sk_pass(sk, items, P.n_items, 1, tw, b0, b1, c.st);
         const double* fin = b1;
         if (e == cudaSuccess && P.dims == 3) {

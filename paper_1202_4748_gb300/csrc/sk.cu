@@ -489,7 +489,7 @@ cudaError_t launch_sk_twiddles(double* tw, const int* sides, const int* offs, in
     return cudaGetLastError();
 }
 
-cudaError_t launch_sk_x(const SysDev* sys, const SkSys* sk, const int4* items, int n_items, const double* d,
+cudaError_t launch_sk_x(const SkSys* sk, const int4* items, int n_items, const double* d,
                         const double* dbar, const double* tw, double* out, cudaStream_t st) {
     if (n_items == 0) return cudaSuccess;
     sk_x_kernel<<<n_items, AUX_THREADS, 0, st>>>(sk, items, d, dbar, tw, out);

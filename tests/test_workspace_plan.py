@@ -32,3 +32,18 @@ def test_default_size_covers_every_row_the_default_may_be(precision, coupling, s
         for r, row in enumerate(lb.kernel_variants("D2Q9")):
             if coup2 == "modeq" and row[0] == 64 and row[5] == 2:
                 assert lb.workspace_bytes(flat, precision=precision, obs_every=1, variant=r + 1) <= have2, row
+
+
+@pytest.mark.parametrize("lattice,n", [("D3Q19", 64), ("D3Q19", 45), ("D3Q19", 2), ("D2Q9", 512), ("D2Q9", 33),
+                                       ("D2Q9", 2100)])
+def test_momentum_spectra_share_their_transforms_room(lattice, n):
+    """Beside what the structure factor needs: the momentum (3 fields), a Laplacian,
+    3 complex transforms and 3 accumulators, 104 bytes a site; the half spectra of
+    the line FFTs are those transforms, not a region of their own."""
+    import paper_1202_4748_gb300 as lb
+    s = synth.system(lattice, n=n)
+    sites = s["nx"] * s["ny"] * s["nz"]
+    a = lb.workspace_bytes([s], precision="fp32", sk_every=5)
+    b = lb.workspace_bytes([s], precision="fp32", sk_every=5, jk_spectra=True)
+    lines = 16 * 40 * sites // n                       # longer work lists (16 bytes per few lines)
+    assert 13 * 8 * sites - 2048 <= b - a <= 13 * 8 * sites + lines // 8 + 8192
