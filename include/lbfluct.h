@@ -103,6 +103,10 @@ typedef struct {
  *               counter is a multiple of graph_chunk; 0 = plain launches.
  *   tile        tile shape of the step kernel (0 = library default): (x, y, 1)
  *               on D2Q9; on D3Q19 (x, y, z-chunk) of the z-marching kernel.
+ *               Has to match a compiled variant.  On D3Q19 an FP64 run, or
+ *               one with a relaxation time other than 1, takes only the
+ *               z-chunk from it: its columns are 16 x 8, or 8 x 8 in FP64
+ *               where those leave fewer lanes outside the systems.
  *   occupancy   resident CTAs per SM the step kernel was compiled for (its
  *               register budget); 0 = the tile's default.  Must match a
  *               compiled variant, else LB_ERR_UNSUPPORTED.
@@ -391,7 +395,8 @@ lb_status lb_load(lb_ctx* ctx, const char* path);
  * kernel forms the density and momentum of every site, a second collides the
  * tile columns (in FP32 two sites stacked in z per thread).  On D3Q19, FP64 runs
  * and runs with a relaxation time other than 1 take the split step whatever the
- * row, in 16 x 8 columns with the row's z-chunk.
+ * row, with the row's z-chunk, in 16 x 8 columns (FP64: 8 x 8 where they cover the
+ * systems with at least 5 % fewer lanes).
  * Row 0 is the default; where the coupling cannot run it (scheme 2 with the
  * Guo form) the first row it can run is.  Selecting a row the coupling cannot
  * run gives LB_ERR_UNSUPPORTED.  Used by the autotuner; no device call. */
@@ -406,6 +411,8 @@ int lb_kernel_variants(int lattice, int32_t* out, int max_rows);
  * on D3Q19, ensembles too small for that, those with an nx that is not a
  * multiple of 4, FP64 runs and runs with a relaxation time other than 1 take
  * the row of the lowest estimated step time among the paired and split rows.
+ * A row asked for is returned as asked for; where the run takes the split step
+ * whatever the row (see lb_kernel_variants), its z-chunk is what runs.
  * Errors: LB_ERR_ARG. */
 lb_status lb_kernel_variant(lb_ctx* ctx, int* row);
 

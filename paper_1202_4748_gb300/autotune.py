@@ -2,7 +2,8 @@
 
 For a given ensemble, every step-kernel variant compiled into the library for
 its lattice (tile shape, register budget, producer warps; listed by
-``lb_kernel_variants``) is timed on the device (CUDA events around a plain run
+``lb_kernel_variants``) that runs something else than the ones before it
+(``candidates``) is timed on the device (CUDA events around a plain run
 of step launches, after a warm-up) through the public API, and the fastest is
 returned.  Results are cached in a JSON file keyed by lattice, coupling,
 precision and the multiset of system sizes, so a later run of the same ensemble
@@ -13,7 +14,7 @@ selects it.
 import json
 import os
 
-from . import Ensemble, LBError, LB_ERR_UNSUPPORTED, kernel_variants
+from . import Ensemble, LBError, LB_D3Q19, LB_ERR_UNSUPPORTED, LB_FP32_DEVIATION, kernel_variants
 
 DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "lbfluct_tiles.json")
 
@@ -26,6 +27,22 @@ def variants(lattice):
 def variant_index(lattice, row):
     """The ``variant`` option (1-based) that selects a compiled variant row."""
     return variants(lattice).index(tuple(row)) + 1
+
+
+def candidates(systems, precision):
+    """Indices of the rows to time: all of them, but on D3Q19 in FP64 or with a
+    relaxation time other than 1, where every row runs the split step with its
+    z-chunk, one per z-chunk (a row of the split step where there is one)."""
+    rows = variants(systems[0]["lattice"])
+    relaxed = all(float(t) == 1.0 for s in systems for t in s["tau"][4:19])
+    if systems[0]["lattice"] not in ("D3Q19", LB_D3Q19) or (precision in ("fp32", LB_FP32_DEVIATION) and relaxed):
+        return list(range(len(rows)))
+    by_chunk = {}
+    for i, row in enumerate(rows):
+        split = row[:2] == (16, 8) and row[3:6] == (4, 0, 0)
+        if split or row[2] not in by_chunk:
+            by_chunk[row[2]] = i
+    return sorted(by_chunk.values())
 
 
 def ensemble_key(systems, precision):
@@ -72,7 +89,8 @@ def tune(systems, precision="fp32", cache=DEFAULT_CACHE, steps=20, warmup=5, ref
         if ent is not None and tuple(ent["best"]) in rows:
             return tuple(ent["best"]), {tuple(map(int, k.split("x"))): v for k, v in ent["ms"].items()}
     results = {}
-    for i, row in enumerate(rows):
+    for i in candidates(systems, precision):
+        row = rows[i]
         try:
             results[row] = time_variant(systems, precision, i, steps, warmup)
         except LBError as e:
