@@ -185,13 +185,14 @@ int64_t tiles_of(const lb_system_desc* s, int n, const int tdim[3]) {
     return c;
 }
 
-// SMs of the current device (152 when none is visible).
+// SMs of the current device (GB300's when none is visible).
+constexpr int kGb300Sms = 152;
 int sm_count() {
     int sms = 0, dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) {
         cudaGetLastError();
-        sms = 152;
+        sms = kGb300Sms;
     }
     return sms;
 }
@@ -544,12 +545,13 @@ lb_status make_plan(const lb_system_desc* s, int n, const lb_run_opts* o, std::v
             if (!sk_fft_side(h.d.nx)) P.sk_fft = false;
         if (P.sk_fft) {
             // lines per item: eight (whole warps of butterflies, 128-byte runs of
-            // kx), more where that leaves several items per SM, in kSkFftMaxElems
+            // kx), more where that leaves eight items per SM, in kSkFftMaxElems (a
+            // GB300's SMs, not the current device's: the list is part of the workspace)
             const bool d3 = s[0].lattice == LB_D3Q19;
             P.n_fields = o->jk_spectra == 1 ? (d3 ? 4 : 3) : 1;
             int64_t lines_all = 0;
             for (auto& h : sys) lines_all += h.n / h.d.nx * P.n_fields;
-            const int want = int(std::min<int64_t>(64, std::max<int64_t>(8, lines_all / (8 * 152))));
+            const int want = int(std::min<int64_t>(64, std::max<int64_t>(8, lines_all / (8 * kGb300Sms))));
             auto add = [&](int k, int lines, int len, int field, int in_cta, int& count, int& mx) {
                 const int per = std::max(1, std::min(std::max(want / in_cta, 2), kSkFftMaxElems / (len * in_cta)));
                 for (int l = 0; l < lines; l += per, ++count) {
