@@ -222,6 +222,14 @@ __device__ __forceinline__ float2 vsqrt_pos(float2 x) {
     return make_float2(sfu_sqrt(fmaxf(x.x, 0.0f)), sfu_sqrt(fmaxf(x.y, 0.0f)));
 }
 __device__ __forceinline__ double vsqrt_pos(double x) { return n64_sqrt(x > 0.0 ? x : 0.0); }
+// The same with subnormal variances (kT below 4e-39 in float) kept.
+__device__ __forceinline__ float sqrt_any(float x) {
+    float y;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(fmaxf(x, 0.0f)));
+    return y;
+}
+__device__ __forceinline__ float2 vsqrt_any(float2 x) { return make_float2(sqrt_any(x.x), sqrt_any(x.y)); }
+__device__ __forceinline__ double vsqrt_any(double x) { return vsqrt_pos(x); }
 
 // Laplacian of the density, lap rho = 6 sum_i t_i (rho(r + c_i) - rho(r))
 // = (1/3) (sum of the 6 face neighbours) + (1/6) (sum of the 12 edge
@@ -688,7 +696,7 @@ __device__ __forceinline__ void collide_d3q19_rates(V (&f)[19], const V drho, co
     if (P.kT > S(0)) {
         // as in the fully relaxed collisions, with g_ab = 1 - gamma_a gamma_b on the
         // amplitudes: M = [[(2/3 + om) g_44, -om g_4,16], [., (2 + om) g_16,16]]
-        const V sc = vsqrt_pos(vmul(vbc<V>(vmul(S(3.0 * DrawScale<S>::v / DrawScale<S>::mean_square), P.kT)), rho));
+        const V sc = vsqrt_any(vmul(vbc<V>(vmul(S(3.0 * DrawScale<S>::v / DrawScale<S>::mean_square), P.kT)), rho));
         const V om = vfma(cs2, vk<V>(-3.0), vk<V>(1.0));
         const V mpp = vmul(vadd(vk<V>(2.0 / 3.0), om), vbc<V>(P.g_diag[4]));
         const V mpr = vmul(om, vbc<V>(-P.g_pair));

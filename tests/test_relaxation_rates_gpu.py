@@ -42,3 +42,26 @@ def test_populations_stay_as_close_to_fp64(coupling, rates):
     off = np.linalg.norm(got - want, axis=1) / np.linalg.norm(want, axis=1)
     rms = np.sqrt(np.mean(off * off))
     assert rms <= BAR[coupling, rates], rms
+
+
+@pytest.mark.parametrize("coupling,rates", sorted(BAR))
+def test_noise_of_a_subnormal_temperature(coupling, rates):
+    """kT = 2^-130 is a subnormal float, its noise of 2^-65 is not: one step from rest
+    is that of kT = 2^-90 times 2^-20, the same draws on a scale whose variance keeps
+    21 bits (its root 22, and a few FP32 roundings after it)."""
+    import paper_1202_4748_gb300 as lb
+
+    def one(kT):
+        systems = [synth.system("D3Q19", coupling, n=8, a=0.0, kT=kT, tau=[1.0] * 4 + RATES[rates], seed=k)
+                   for k in range(3)]
+        e = lb.Ensemble(systems, precision="fp32")
+        e.init(amplitude=0.0)
+        e.step(1)
+        e.sync()
+        f = np.array([e.read_fields(k)[1:] for k in range(3)])
+        e.close()
+        return f
+
+    got, want = one(2.0 ** -130), one(2.0 ** -90) * 2.0 ** -20
+    assert np.max(np.abs(want)) > 2.0 ** -67
+    assert np.max(np.abs(got - want)) <= 2.0 ** -20 * np.max(np.abs(want))
