@@ -244,7 +244,7 @@ SplitCost split_cost(int kind, bool quads) {
 // every ensemble: 16^3 28.9 -> 5.3 us, 64^3 52 -> 14.4, 4 x 64^3 55 -> 46,
 // 16 x 64^3 157 -> 147 us per step; 2.6 M sites with odd sides 332 -> 137 us;
 // against the z-marching kernels that ran the other settings: 4 x 64^3 with a
-// rate per mode 181 -> 61 us, FP64 256^3 29.2 -> 11.1 ms (of which the integer
+// rate per mode 181 -> 64 us, FP64 256^3 29.2 -> 11.1 ms (of which the integer
 // noise 29.2 -> 14).
 double estimated_step_us(const lb_system_desc* s, int n, const int tdim[3], bool paired, int kind, int sms, bool quads) {
     const double ctas = double(tiles_of(s, n, tdim));

@@ -591,11 +591,11 @@ __device__ __forceinline__ V over_norm(const V x) {
 // The conserved moments do not pass through the scaled moments, whose rounding a
 // slow mode adds up step after step, f is rounded once, and neither the constants
 // nor the draws' mean square bias a mode's rate or noise.  Against exact arithmetic
-// (16 x 16 x 8, 50 steps) FP32 populations are off by 4.3e-7 of their size with a
-// rate per mode, 5.4e-7 with one rate (Guo), 3.3e-7 and 3.7e-7 (modified
-// equilibrium); transforming relaxed moments back leaves 6.1e-7 to 7.7e-7 and
-// 4.0e-7 to 4.7e-7.  It costs 4 to 7 % of the step (4 x 64^3, a rate per mode: 63.7
-// us for 61.4): f stays in registers to the end.
+// (16 x 16 x 8, 50 steps) FP32 populations are off by 4.1e-7 of their size with a
+// rate per mode, 5.2e-7 with one rate (Guo), 3.0e-7 and 3.4e-7 (modified
+// equilibrium); transforming relaxed moments back leaves 6.3e-7, 7.7e-7, 4.1e-7 and
+// 4.7e-7.  It costs 4 to 7 % of the step (4 x 64^3, a rate per mode: 63.5 us for
+// 61.4): f stays in registers to the end.
 template <int MODE, int CP, class V, class NV>
 __device__ __forceinline__ void collide_d3q19_rates(V (&f)[19], const V drho, const V jx, const V jy, const V jz,
                                                     const NV& nv, const SysPhys<typename VT<V>::S>& P,

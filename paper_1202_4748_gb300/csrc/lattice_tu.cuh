@@ -178,11 +178,12 @@ cudaError_t step_moments(const StepLaunch& a, cudaStream_t st) {
 
 // Split step on D3Q19: the moment pass over the site items, then the collision
 // of 16 x 8 columns (FP64: 8 x 8 where they leave fewer lanes outside the
-// systems) in chunks of a.zc planes.  4 resident CTAs, 128 registers, no spills:
-// FP32 with a rate per mode takes 4 x 64^3 in 61 us (3 CTAs, 166 registers: 69),
-// 160^3 in 219 (232); fully relaxed, 5 CTAs spill 8 bytes and give 134.5 us for
-// 136.5 on 2.6 M odd-sided sites but 198 for 192 on 4 x 99^3; FP64 hides its
-// latencies better with 4 than with 2 (64^3 190 -> 173 us).
+// systems) in chunks of a.zc planes.  4 resident CTAs, 128 registers: no spills
+// fully relaxed; other rates, which keep the populations to the end, spill 12 to 60
+// bytes, and FP32 with a rate per mode takes 4 x 64^3 in 63.5 us (3 CTAs, 168
+// registers, no spills: 67.3), 160^3 in 229 (233).  Fully relaxed, 5 CTAs spill 8
+// bytes and give 134.5 us for 136.5 on 2.6 M odd-sided sites but 198 for 192 on
+// 4 x 99^3; FP64 hides its latencies better with 4 than with 2 (64^3 190 -> 173 us).
 template <int MODE, int CP, class Real, int TX>
 cudaError_t step_split_columns(const StepLaunch& a, cudaStream_t st) {
     using V = typename std::conditional<std::is_same<Real, float>::value, float2, double>::type;
