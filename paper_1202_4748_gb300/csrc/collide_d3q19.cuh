@@ -594,8 +594,10 @@ __device__ __forceinline__ V over_norm(const V x) {
 // (16 x 16 x 8, 50 steps) FP32 populations are off by 4.1e-7 of their size with a
 // rate per mode, 5.2e-7 with one rate (Guo), 3.0e-7 and 3.4e-7 (modified
 // equilibrium); transforming relaxed moments back leaves 6.3e-7, 7.7e-7, 4.1e-7 and
-// 4.7e-7.  It costs 4 to 7 % of the step (4 x 64^3, a rate per mode: 63.5 us for
-// 61.4): f stays in registers to the end.
+// 4.7e-7.  In FP32 it costs 4 to 7 % of the step (4 x 64^3, a rate per mode: 63.5
+// us for 61.4): f stays in registers to the end.  In FP64, bound by its operations,
+// a rate per mode gains (64^3: 252 us to 241) and one rate loses (211 to 239), being
+// the same operations then; block moments come 2 to 4 times closer.
 template <int MODE, int CP, class V, class NV>
 __device__ __forceinline__ void collide_d3q19_rates(V (&f)[19], const V drho, const V jx, const V jy, const V jz,
                                                     const NV& nv, const SysPhys<typename VT<V>::S>& P,

@@ -209,7 +209,6 @@ struct FftLaunch {
 cudaError_t launch_sk_fft(const FftLaunch& a, cudaStream_t st);
 cudaError_t launch_sk_accum(const SkSys* sk, const int4* items, int n_items, const double* F, double* acc,
                             cudaStream_t st);
-// per-shell sums of the accumulated C(k) of one system (one CTA per shell)
 // Momentum spectra (see sk.cu): accumulate the x, longitudinal and transverse
 // spectra of the transforms F0..F2 (F2 unused in 2-D) into acc + c * stride.
 cudaError_t launch_jk_accum(const SkSys* sk, const int4* items, int n_items, int dims, const double* F0,
